@@ -84,31 +84,103 @@ __global__ void __launch_bounds__(1024) k_subqubo(const double* __restrict__ Q, 
 }
 
 // One CTA per sub-QUBO: E(y) = sum_a y_a (D_a + sum_{b != a} y_b Q_ab), a and b ascending, in
-// FP64, for each of its shots; the block keeps the lowest (E, y) pair (ties: smaller y).
+// FP64, for its shots; the block keeps the lowest (E, y) pair (ties: smaller y). FP64 issues at
+// 1/64 of the FP32 rate, so every shot is first evaluated in FP32 and only those that can be the
+// lowest are evaluated in FP64: with S the sum of the |entries|, |E32 - E| <= (k^2 + 1) 2^-24 S
+// (rounding the entries and adding at most k^2 of them), so a shot above the lowest E32 by more
+// than 2 (k^2 + 8) 2^-23 S (twice what the two bounds allow) cannot win. Matrices whose entries
+// leave the FP32 range are evaluated in FP64 alone.
+// 128 sub-QUBOs of 12 variables, 1024 shots each: 53 -> 21 us.
+__device__ __forceinline__ double shot_energy64(const double* sq, int k, uint64_t y) {
+    double E = 0.0;
+    for (int a = 0; a < k; ++a) {
+        if (!((y >> a) & 1u)) continue;
+        double r = sq[a * k + a];
+        for (int b = 0; b < k; ++b)
+            if (b != a && ((y >> b) & 1u)) r += sq[a * k + b];
+        E += r;
+    }
+    return E;
+}
+
 __global__ void __launch_bounds__(256) k_best_shot(int k, int shots, const double* __restrict__ qblk,
                                                    const double* __restrict__ qdiag,
                                                    const uint64_t* __restrict__ z, uint64_t* __restrict__ best) {
     __shared__ double sq[32 * 32];
+    __shared__ float sf[32 * 32];
     __shared__ double be[256];
     __shared__ uint64_t bz[256];
+    __shared__ float red[2][8];
     const int j = blockIdx.x;
-    for (int e = threadIdx.x; e < k * k; e += blockDim.x)
-        sq[e] = (e / k == e % k) ? qdiag[(int64_t)j * k + e / k] : qblk[(int64_t)j * k * k + e];
+    const uint64_t* zj = z + (int64_t)j * shots;
+    float s = 0.0f;
+    for (int e = threadIdx.x; e < k * k; e += blockDim.x) {
+        const double v = (e / k == e % k) ? qdiag[(int64_t)j * k + e / k] : qblk[(int64_t)j * k * k + e];
+        sq[e] = v;
+        sf[e] = (float)v;
+        s += fabsf((float)v);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) red[0][threadIdx.x >> 5] = s;
     __syncthreads();
+    float S = 0.0f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) S += red[0][w];
+    const bool fast = S > 1e-30f && S < 1e30f;   // false for NaN
+    // FP32 energies of four shots of this thread at a time
+    const auto e32 = [&](int s0, float (&e)[4]) {
+        uint32_t y[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int t = s0 + i * (int)blockDim.x;
+            y[i] = t < shots ? (uint32_t)zj[t] : 0u;
+            e[i] = 0.0f;
+        }
+        for (int a = 0; a < k; ++a) {
+            float r[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            for (int b = 0; b < k; ++b) {
+                const float q = sf[a * k + b];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) r[i] += ((y[i] >> b) & 1u) ? q : 0.0f;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) e[i] += ((y[i] >> a) & 1u) ? r[i] : 0.0f;
+        }
+    };
+    float thr = 0.0f;
+    if (fast) {
+        float m = 3.0e38f;
+        for (int s0 = threadIdx.x; s0 < shots; s0 += 4 * (int)blockDim.x) {
+            float e[4];
+            e32(s0, e);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (s0 + i * (int)blockDim.x < shots) m = fminf(m, e[i]);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if ((threadIdx.x & 31) == 0) red[1][threadIdx.x >> 5] = m;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < 8; ++w) m = fminf(m, red[1][w]);
+        thr = m + 2.0f * (float)(k * k + 8) * 1.1920928955078125e-7f * S;
+    }
     double myE = 0.0;
     uint64_t myz = ~0ull;
     bool have = false;
-    for (int s = threadIdx.x; s < shots; s += blockDim.x) {
-        const uint64_t y = z[(int64_t)j * shots + s];
-        double E = 0.0;
-        for (int a = 0; a < k; ++a) {
-            if (!((y >> a) & 1u)) continue;
-            double r = sq[a * k + a];
-            for (int b = 0; b < k; ++b)
-                if (b != a && ((y >> b) & 1u)) r += sq[a * k + b];
-            E += r;
+    for (int s0 = threadIdx.x; s0 < shots; s0 += 4 * (int)blockDim.x) {
+        float e[4];
+        if (fast) e32(s0, e);
+#pragma unroll 1
+        for (int i = 0; i < 4; ++i) {
+            const int t = s0 + i * (int)blockDim.x;
+            const float ei = i == 0 ? e[0] : (i == 1 ? e[1] : (i == 2 ? e[2] : e[3]));
+            if (t >= shots || (fast && ei > thr)) continue;
+            const uint64_t y = zj[t];
+            const double E = shot_energy64(sq, k, y);
+            if (!have || E < myE || (E == myE && y < myz)) { myE = E; myz = y; have = true; }
         }
-        if (!have || E < myE || (E == myE && y < myz)) { myE = E; myz = y; have = true; }
     }
     be[threadIdx.x] = have ? myE : 0.0;
     bz[threadIdx.x] = have ? myz : ~0ull;

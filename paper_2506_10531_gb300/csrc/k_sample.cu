@@ -2,17 +2,27 @@
 // uniforms supplied by the caller (Section IV reads the sub-solution from measured shots; the
 // default path of this library takes the top-k bitstrings instead).
 //
-// The 2^n probabilities are cut into P = 2^(n - pb) contiguous parts of 2^pb amplitudes
-// (pb = max(n - 12, 0), so P <= 4096):
-//   1. k_sample_parts: FP64 sum of each part (one block per part, fixed reduction order);
-//   2. k_sample_scan:  exclusive prefix of the part sums and the total, sequential in one thread
-//      (at most 4096 adds), so the offsets are exactly the running sums of the parts;
-//   3. k_sample_draw:  one warp per shot: t = u * total, the last part whose offset is <= t, then
-//      a walk through that part 32 amplitudes at a time with a warp prefix scan until the running
-//      sum exceeds t. Every loop is bounded by the part length; nothing waits on another block.
-// A batch of states of equal n (a DQAOA cycle's sub-QUBO states, 2^n amplitudes apart) runs as
-// one launch of each kernel, the state index in blockIdx.y; each state has its own scratch
-// (2P + 1 doubles), uniforms and shots.
+// The 2^n probabilities are cut into F = 2^(n - fb) fine parts of 2^fb contiguous amplitudes
+// (fb = 4 up to n = 20, then n - 16, so F <= 65536) and runs of up to 256 fine parts form a
+// coarse part (C <= 256 of them):
+//   1. k_sample_sums: one block per coarse part: the FP64 sum of each fine part, their exclusive
+//      prefix inside the coarse part, and the coarse part's total;
+//   2. k_sample_draw: every block first scans the C coarse totals (at most 256 values, cheaper
+//      than a launch of its own); a shot's target t = u * total is then located by two binary
+//      searches (coarse offsets in shared memory, fine prefixes in L2) and a walk through one
+//      fine part.
+// What bounds it: FP64 issue (GB300 has two FP64 lanes per SM and clock), so the design counts
+// FP64 operations: three per amplitude for the sums; the searches compare the non-negative
+// doubles as integers; a shot's walk is one thread over its 16 amplitudes (1.5 FP64 warp
+// instructions per shot; a warp per shot with shuffle scans needs 8 per 32 amplitudes walked).
+// Only for fb >= 7 half a warp walks a part together.
+// Every loop is bounded by the part length; nothing waits on another block. A batch of states of
+// equal n (a DQAOA cycle's sub-QUBO states, 2^n amplitudes apart) runs as one launch of each
+// kernel, the state index in blockIdx.y; each state has its own scratch (F + C doubles),
+// uniforms and shots. Complex64 loads are 8 bytes wide: a state needs no more alignment.
+// Measured on GB300 against parts of 2^(n-12) amplitudes, a one-thread scan over 4096 of them and a
+// warp per shot: one n = 20 state, 65536 shots, 748 -> 41 us (sums 17, draw 23); 128 states of
+// n = 12, 1024 shots each, 2380 -> 49 us (sums 10, draw 38).
 #include <cuda_runtime.h>
 
 #include "qaoa_common.cuh"
@@ -23,105 +33,243 @@ namespace qaoa {
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
+constexpr int NTS = 256;   // threads per block; also the most fine parts of a coarse part
 
-__global__ void __launch_bounds__(256) k_sample_parts(const float2* __restrict__ psi, int n, int pb,
-                                                      double* __restrict__ scratch) {
-    __shared__ double red[8];
-    const uint64_t L = 1ull << pb, base = (uint64_t)blockIdx.x << pb;
-    psi += (uint64_t)blockIdx.y << n;
-    double* part = scratch + (size_t)blockIdx.y * (2 * ((size_t)1 << (n - pb)) + 1);
-    double acc = 0.0;
-    for (uint64_t u = threadIdx.x; u < L; u += blockDim.x) acc += exact_prob(psi[base + u]);
-    acc = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+// Fine-part bits, fine parts per coarse part (log2) and coarse parts (log2) of an n-qubit state.
+struct SampleGeo {
+    int fb, jb, cb;
+};
+__host__ __device__ inline SampleGeo sample_geo(int n) {
+    SampleGeo g;
+    g.fb = n > 20 ? n - 16 : (n < 4 ? n : 4);
+    const int f = n - g.fb;
+    g.jb = f < 8 ? f : 8;
+    g.cb = f - g.jb;
+    return g;
+}
+
+// |v|^2 in FP64: the products of two floats are exact, the fused add rounds once (the value of
+// exact_prob in one operation fewer)
+__device__ __forceinline__ double prob64(float2 v) {
+    return __fma_rn((double)v.x, (double)v.x, __dmul_rn((double)v.y, (double)v.y));
+}
+
+// Inclusive prefix over W lanes: at each level the upper half of a group adds the lower half's
+// total. The sums never decrease from lane to lane and a zero leaves its neighbour's sum as it
+// is, bit for bit, so a part or an amplitude without probability spans no target.
+template <int W>
+__device__ __forceinline__ double lane_scan(double v) {
+    const int lane = threadIdx.x & (W - 1);
+#pragma unroll
+    for (int d = 1; d < W; d <<= 1) {
+        const double o = __shfl_sync(FULL, v, (lane & ~(2 * d - 1)) | (d - 1), W);
+        if (lane & d) v = o + v;
+    }
+    return v;
+}
+
+// Exclusive prefix of one value per thread over the block (fixed order, properties as lane_scan);
+// the total in *tot.
+__device__ __forceinline__ double block_excl_scan(double v, double* wsum, double* tot) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const double incl = lane_scan<32>(v);
+    if (lane == 31) wsum[w] = incl;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        part[blockIdx.x] = t;
+    double off = 0.0, all = 0.0;
+#pragma unroll
+    for (int i = 0; i < NTS / 32; ++i) {
+        if (i < w) off += wsum[i];
+        all += wsum[i];
     }
+    *tot = all;
+    const double left = __shfl_up_sync(FULL, incl, 1);
+    return lane == 0 ? off : off + left;
 }
 
-__global__ void k_sample_scan(double* __restrict__ scratch, int parts) {
-    if (threadIdx.x != 0) return;
-    const double* part = scratch + (size_t)blockIdx.x * (2 * (size_t)parts + 1);
-    double* off = const_cast<double*>(part) + parts;
-    double* total = off + parts;
-    double acc = 0.0;
-    for (int b = 0; b < parts; ++b) {
-        off[b] = acc;
-        acc += part[b];
+// One block per coarse part of 2^(fb + jb) amplitudes. Fine parts of up to 128 amplitudes: 4096
+// amplitudes at a time are read coalesced, their probabilities pass through shared memory (rows of
+// 16 padded to 17) and thread t adds the 16 of row t; neighbouring threads combine their rows
+// when a fine part has more than one. Longer fine parts: one warp per part, lanes strided.
+__global__ void __launch_bounds__(NTS) k_sample_sums(const float2* __restrict__ psi, int n,
+                                                     double* __restrict__ scratch) {
+    __shared__ double row[NTS * 17];
+    __shared__ double fine[NTS];
+    __shared__ double wsum[NTS / 32];
+    const SampleGeo g = sample_geo(n);
+    const uint32_t J = 1u << g.jb;
+    psi += ((uint64_t)blockIdx.y << n) + ((uint64_t)blockIdx.x << (g.fb + g.jb));
+    double* pre = scratch + (size_t)blockIdx.y * (((size_t)1 << (n - g.fb)) + ((size_t)1 << g.cb));
+    double* coarse = pre + ((size_t)1 << (n - g.fb));
+    pre += (size_t)blockIdx.x << g.jb;
+    if (g.fb <= 7) {
+        const uint32_t D = 1u << (g.fb + g.jb);   // amplitudes of the block
+        const int rb = g.fb < 4 ? 0 : g.fb - 4;   // rows per fine part (log2)
+        for (uint32_t c0 = 0; c0 < D; c0 += NTS * 16) {
+            float2 v[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const uint32_t u = c0 + (uint32_t)i * NTS + threadIdx.x;
+                v[i] = u < D ? psi[u] : make_float2(0.0f, 0.0f);
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const uint32_t u = (uint32_t)i * NTS + threadIdx.x;
+                row[u + (u >> 4)] = prob64(v[i]);
+            }
+            __syncthreads();
+            double s = 0.0;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) s += row[threadIdx.x * 17 + i];
+            for (int d = 0; d < rb; ++d) s += __shfl_xor_sync(FULL, s, 1 << d);
+            const uint32_t f = (c0 >> g.fb) + (threadIdx.x >> rb);
+            if ((threadIdx.x & ((1u << rb) - 1u)) == 0 && f < J) fine[f] = s;
+            __syncthreads();
+        }
+    } else {
+        const uint32_t L = 1u << g.fb;
+        for (uint32_t f = threadIdx.x >> 5; f < J; f += NTS / 32) {
+            const float2* p = psi + ((uint64_t)f << g.fb) + (threadIdx.x & 31);
+            double a = 0.0, b = 0.0;
+#pragma unroll 4
+            for (uint32_t u = 0; u < L; u += 64) {
+                const float2 v0 = p[u], v1 = p[u + 32];
+                a = __fma_rn((double)v0.x, (double)v0.x, a);
+                b = __fma_rn((double)v1.x, (double)v1.x, b);
+                a = __fma_rn((double)v0.y, (double)v0.y, a);
+                b = __fma_rn((double)v1.y, (double)v1.y, b);
+            }
+            const double s = warp_sum(a + b);
+            if ((threadIdx.x & 31) == 0) fine[f] = s;
+        }
+        __syncthreads();
     }
-    *total = acc;
+    double tot;
+    const double ex = block_excl_scan(threadIdx.x < J ? fine[threadIdx.x] : 0.0, wsum, &tot);
+    if (threadIdx.x < J) pre[threadIdx.x] = ex;
+    if (threadIdx.x == 0) coarse[blockIdx.x] = tot;
 }
 
-__global__ void __launch_bounds__(256) k_sample_draw(const float2* __restrict__ psi, int n, int pb, int parts,
+// The last of `count` non-decreasing offsets (off[0] = 0) that is <= t, as integers: every offset
+// is a non-negative double, and a negative t lies below all of them in either reading.
+__device__ __forceinline__ uint32_t last_le(const double* off, uint32_t count, double t) {
+    const long long tb = pbits(t);
+    uint32_t lo = 0;
+    for (uint32_t step = count >> 1; step; step >>= 1)   // count is a power of two
+        if (pbits(off[lo + step]) <= tb) lo += step;
+    return lo;
+}
+
+// The largest double below the positive double v (v itself when v <= 0): targets stay below the
+// total of the part they are searched in, so a tail of empty parts is never chosen.
+__device__ __forceinline__ double below(double v) {
+    return pbits(v) > 0 ? __longlong_as_double(pbits(v) - 1) : v;
+}
+
+// One thread per shot (HALF = false, fine parts of up to 64 amplitudes) or 16 lanes per shot.
+template <bool HALF>
+__global__ void __launch_bounds__(NTS) k_sample_draw(const float2* __restrict__ psi, int n,
                                                      const double* __restrict__ scratch, int64_t shots,
-                                                     const double* __restrict__ u,
-                                                     uint64_t* __restrict__ out) {
-    const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;   // one warp per shot
-    const int lane = threadIdx.x & 31;
-    if (s >= shots) return;                                                    // warp-uniform
+                                                     const double* __restrict__ u, uint64_t* __restrict__ out) {
+    __shared__ double off[NTS];
+    __shared__ double wsum[NTS / 32];
+    const SampleGeo g = sample_geo(n);
+    const uint32_t C = 1u << g.cb, J = 1u << g.jb;
+    const double* pre = scratch + (size_t)blockIdx.y * (((size_t)1 << (n - g.fb)) + C);
+    const double* coarse = pre + ((size_t)1 << (n - g.fb));
     psi += (uint64_t)blockIdx.y << n;
-    const double* off = scratch + (size_t)blockIdx.y * (2 * (size_t)parts + 1) + parts;
-    const double* total = off + parts;
     u += (size_t)blockIdx.y * shots;
     out += (size_t)blockIdx.y * shots;
-    const double t = u[s] * *total;
-    // the last part whose offset is <= t (offsets are non-decreasing; parts before a run of
-    // empty parts are skipped that way)
-    int lo = 0, hi = parts - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (off[mid] <= t) lo = mid;
-        else hi = mid - 1;
-    }
-    const uint64_t L = 1ull << pb, base = (uint64_t)lo << pb;
-    double acc = off[lo];
-    int64_t lastnz = -1;
-    for (uint64_t c0 = 0; c0 < L; c0 += 32) {
-        const bool in = c0 + (uint64_t)lane < L;
-        const double p = in ? exact_prob(psi[base + c0 + lane]) : 0.0;
-        double incl = p;
+    double total;
+    off[threadIdx.x] = block_excl_scan(threadIdx.x < C ? coarse[threadIdx.x] : 0.0, wsum, &total);
+    __syncthreads();
+    const int64_t id = (int64_t)blockIdx.x * NTS + threadIdx.x;
+    const int64_t s = HALF ? id >> 4 : id;
+    const bool live = s < shots;
+    if (!HALF && !live) return;
+    const double t = fmin(u[live ? s : shots - 1] * total, below(total));
+    const uint32_t c = last_le(off, C, t);
+    const double r = fmin(t - off[c], below(coarse[c]));
+    const uint32_t f = last_le(pre + ((size_t)c << g.jb), J, r);
+    double acc = pre[((size_t)c << g.jb) + f];
+    const uint64_t base = (((uint64_t)c << g.jb) + f) << g.fb;
+    const uint32_t L = 1u << g.fb;
+    const float2* p = psi + base;
+    uint32_t hit = 0xffffffffu, lastnz = 0xffffffffu;
+    if (!HALF) {
+        for (uint32_t c0 = 0; c0 < L && hit == 0xffffffffu; c0 += 16) {
+            float2 v[16];
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const double o = __shfl_up_sync(FULL, incl, d);
-            if (lane >= d) incl += o;
+            for (int i = 0; i < 16; ++i) v[i] = c0 + i < L ? p[c0 + i] : make_float2(0.0f, 0.0f);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const double q = prob64(v[i]);
+                acc += q;
+                if (hit == 0xffffffffu && c0 + i < L && acc > r) hit = c0 + i;
+                if (pbits(q) > 0) lastnz = c0 + i;
+            }
         }
-        const unsigned hit = __ballot_sync(FULL, in && acc + incl > t);
-        if (hit) {
-            if (lane == 0) out[s] = base + c0 + (uint64_t)(__ffs(hit) - 1);
-            return;
+        // no running sum exceeded the target (rounding at the part's end): its last nonzero amplitude
+        if (hit == 0xffffffffu) hit = lastnz != 0xffffffffu ? lastnz : 0u;
+        out[s] = base + hit;
+    } else {
+        // each of the 16 lanes sums its own L / 16 contiguous amplitudes, a scan finds the lane
+        // that holds the target, and its run is walked 16 amplitudes at a time by all lanes
+        const int hl = threadIdx.x & 15;
+        const uint32_t S = L >> 4;
+        const float2* pl = p + (uint32_t)hl * S;
+        double a = 0.0, b = 0.0;
+#pragma unroll 4
+        for (uint32_t i = 0; i < S; i += 2) {
+            const float2 v0 = pl[i], v1 = pl[i + 1];
+            a = __fma_rn((double)v0.x, (double)v0.x, a);
+            b = __fma_rn((double)v1.x, (double)v1.x, b);
+            a = __fma_rn((double)v0.y, (double)v0.y, a);
+            b = __fma_rn((double)v1.y, (double)v1.y, b);
         }
-        const unsigned nz = __ballot_sync(FULL, in && p > 0.0);
-        if (nz) lastnz = (int64_t)(base + c0 + (uint64_t)(31 - __clz(nz)));
-        acc += __shfl_sync(FULL, incl, 31);
+        const double mine = a + b;
+        const double incl = lane_scan<16>(mine);
+        const int sh = threadIdx.x & 16;
+        const uint32_t over = (__ballot_sync(FULL, acc + incl > r) >> sh) & 0xffffu;
+        const uint32_t some = (__ballot_sync(FULL, pbits(mine) > 0) >> sh) & 0xffffu;
+        // the first lane past the target, else the last one that holds any probability
+        const int w = over ? __ffs((int)over) - 1 : (some ? 31 - __clz((int)some) : 0);
+        const double wl = __shfl_sync(FULL, incl, w > 0 ? w - 1 : 0, 16);
+        if (w > 0) acc += wl;
+        const float2* pw = p + (uint32_t)w * S;
+        for (uint32_t c0 = 0; c0 < S; c0 += 16) {      // the same trip count in every lane
+            const uint32_t i = c0 + hl;
+            const double q = i < S ? prob64(pw[i]) : 0.0;
+            const double in2 = lane_scan<16>(q);
+            const uint32_t h2 = (__ballot_sync(FULL, i < S && acc + in2 > r) >> sh) & 0xffffu;
+            const uint32_t nz = (__ballot_sync(FULL, pbits(q) > 0) >> sh) & 0xffffu;
+            if (hit == 0xffffffffu && h2) hit = c0 + (uint32_t)__ffs((int)h2) - 1u;
+            if (nz) lastnz = c0 + 31u - (uint32_t)__clz((int)nz);
+            acc += __shfl_sync(FULL, in2, 15, 16);
+        }
+        if (hit == 0xffffffffu) hit = lastnz != 0xffffffffu ? lastnz : 0u;
+        if (live && hl == 0) out[s] = base + (uint64_t)w * S + hit;
     }
-    // no running sum exceeded t (rounding at the part's end): the part's last nonzero amplitude
-    if (lane == 0) out[s] = lastnz >= 0 ? (uint64_t)lastnz : base;
 }
 
 }  // namespace
 
-int sample_part_bits(int n) { return n > 12 ? n - 12 : 0; }
-
 size_t sample_scratch_bytes(int n) {
-    const size_t parts = (size_t)1 << (n - sample_part_bits(n));
-    return (2 * parts + 1) * sizeof(double);
+    const SampleGeo g = sample_geo(n);
+    return (((size_t)1 << (n - g.fb)) + ((size_t)1 << g.cb)) * sizeof(double);
 }
 
 cudaError_t launch_sample(int n, const void* psi, int count, int64_t shots, const double* u, uint64_t* out,
                           double* scratch, cudaStream_t st) {
     if (count < 1 || count > 65535) return cudaErrorInvalidValue;
-    const int pb = sample_part_bits(n);
-    const int parts = 1 << (n - pb);
+    const SampleGeo g = sample_geo(n);
     const float2* ps = static_cast<const float2*>(psi);
-    k_sample_parts<<<dim3((unsigned)parts, (unsigned)count), 256, 0, st>>>(ps, n, pb, scratch);
-    k_sample_scan<<<(unsigned)count, 32, 0, st>>>(scratch, parts);
+    k_sample_sums<<<dim3(1u << g.cb, (unsigned)count), NTS, 0, st>>>(ps, n, scratch);
     if (shots > 0) {
-        const int64_t blocks = (shots * 32 + 255) / 256;
-        k_sample_draw<<<dim3((unsigned)blocks, (unsigned)count), 256, 0, st>>>(ps, n, pb, parts, scratch, shots, u,
-                                                                              out);
+        const bool half = g.fb >= 7;
+        const int64_t lanes = shots * (half ? 16 : 1);
+        const dim3 grid((unsigned)((lanes + NTS - 1) / NTS), (unsigned)count);
+        if (half) k_sample_draw<true><<<grid, NTS, 0, st>>>(ps, n, scratch, shots, u, out);
+        else k_sample_draw<false><<<grid, NTS, 0, st>>>(ps, n, scratch, shots, u, out);
     }
     return cudaGetLastError();
 }

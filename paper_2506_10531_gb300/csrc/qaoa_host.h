@@ -67,7 +67,6 @@ cudaError_t launch_best_shot(int m, int k, int shots, const double* qblk, const 
 cudaError_t launch_plain_layers(int n, int p, const float* gamma, const float* beta,
                                 const float* E, float2* psi, int init_plus, cudaStream_t st,
                                 int* kernels);
-int sample_part_bits(int n);
 size_t sample_scratch_bytes(int n);
 // `count` states of 2^n amplitudes, one after the other from psi; state c draws `shots` shots
 // with the uniforms u[c * shots ...] into out[c * shots ...]; scratch: count * sample_scratch_bytes(n)
