@@ -136,7 +136,6 @@ __device__ void run_cluster_instance(cg::cluster_group& cl, const InstDesc<float
     const int G = num_windows(0, L, R);
     const int S = snake_len(G, p);
     const float amp0 = (float)exp2(-0.5 * (double)n);
-    auto nofin = [](uint32_t, int, bool) {};
     for (int si = 0; si < S; ++si) {
         SubPass sp;
         snake_step(si, G, p, 0, started ? 0 : 1, 0, L, L, R, sp);
@@ -150,7 +149,7 @@ __device__ void run_cluster_instance(cg::cluster_group& cl, const InstDesc<float
             cl.sync();
         }
         sp.post = (si == S - 1);
-        subpass_fwd<float, R>(tile, sp, s.lc, si == 0 && !started, amp0, __popc(r), nofin);
+        subpass_fwd<float, R>(tile, sp, s.lc, si == 0 && !started, amp0, __popc(r));
         __syncthreads();
     }
     // ---- per-CTA reductions, then rank 0 merges the CTAs (rank order for <C>) ----

@@ -129,12 +129,11 @@ __device__ void stream_tile(const StreamPass& P, const StreamInst<T>& I, uint64_
     const int nl = P.lb - P.la + 1;
     const int S = snake_len(G, nl);
     const T amp0 = (T)I.amp0;
-    auto nofin = [](uint32_t, int, bool) {};
     for (int si = 0; si < S; ++si) {
         SubPass sp;
         snake_step(si, G, nl, P.la, P.ph_first, m0, P.tb, P.tb, R, sp);
         sp.post = P.fin && (si == S - 1);
-        subpass_fwd<T, R>(tile, sp, s.lc, P.init && si == 0, amp0, __popcll(tau), nofin);
+        subpass_fwd<T, R>(tile, sp, s.lc, P.init && si == 0, amp0, __popcll(tau));
         __syncthreads();
     }
     // ---- shared -> HBM (16-byte accesses on both sides). Between passes the state stays in

@@ -218,50 +218,108 @@ struct SwzLayout {
     __device__ __forceinline__ static uint32_t e(uint32_t u) { return swz<T>(u); }
 };
 
-// Element addresses of a group. The swizzle is linear over GF(2) and a group's base index and
-// its window offsets (i << A) have disjoint bits, so
-//   swz(base | (i << A)) = swz(base) ^ swz(i << A),
-// one XOR of a per-thread value with a compile-time constant per element.
-template <typename T, int A>
-__device__ __forceinline__ uint32_t woff(int i) { return swz<T>((uint32_t)i << A); }
-
-// Load / store the 2^R amplitudes of a group (window start A). complex64 windows starting at
-// bit 0 move aligned pairs with one 16-byte shared access (the swizzle keeps pairs adjacent).
-template <int R, int A, typename Lay = SwzLayout<float>>
-__device__ __forceinline__ void load_group(const float2* psi, uint32_t sb, float2 (&v)[1 << R]) {
-    if (A == 0 && R >= 1) {
+// Element addresses of a group. Both maps are linear over GF(2) and a group's base index and its
+// window offsets (i << A) have disjoint bits, so
+//   p(base | (i << A)) = p(base) ^ p(i << A),   p(i << A) = xor of p(1 << (A + j)) over the set
+// bits j of i: walking i in Gray-code order, each element's byte offset is the last one XOR one
+// of R per-window values. The window start A is a run-time value, so that one copy of a sub-pass
+// serves every window: with a copy per window start the sub-passes waited for instructions (GB300,
+// stall "no instruction": 17.8 of 22 cycles per issue in a single n = 8 run, 4.5 of 14 in a batch
+// of 500 instances of n = 12). One copy: that batch 76.6 -> 72.1 us, an uneven training step
+// (48 instances, n = 8..24) 10.30 -> 10.02 ms, serving ticks 4% shorter.
+template <int R>
+struct WinSteps {
+    uint32_t s[R];   // byte steps
+};
+template <int R, typename Map>
+__device__ __forceinline__ WinSteps<R> win_steps(int a, uint32_t bytes, Map&& map) {
+    WinSteps<R> w;
 #pragma unroll
-        for (int i = 0; i < (1 << R); i += 2) {
-            const float4 t = *reinterpret_cast<const float4*>(psi + (sb ^ Lay::p((uint32_t)i << A)));
+    for (int j = 0; j < R; ++j) w.s[j] = map(1u << (a + j)) * bytes;
+    return w;
+}
+// Element of step k of the Gray walk, and the byte step from step k - 1 to step k (of the window
+// bits from `from` on; steps are compile-time indices of unrolled loops).
+__host__ __device__ constexpr int gray_elem(int k) { return k ^ (k >> 1); }
+template <int R>
+__device__ __forceinline__ uint32_t gray_step(const WinSteps<R>& w, int k, int from = 0) {
+    int j = from;
+    while (j < R - 1 && !((k >> (j - from)) & 1)) ++j;
+    return w.s[j];
+}
+
+// Load / store the 2^R elements of a group whose element 0 lies b0 bytes into the tile. complex64
+// windows starting at bit 0 move aligned pairs with one 16-byte shared access (the swizzle keeps
+// pairs adjacent; conflict-free that way).
+template <int R>
+__device__ __forceinline__ void load_group(const float2* psi, uint32_t b0, bool pairs, const WinSteps<R>& w,
+                                           float2 (&v)[1 << R]) {
+    const char* p = reinterpret_cast<const char*>(psi);
+    if (pairs) {
+#pragma unroll
+        for (int k = 0; k < (1 << (R - 1)); ++k) {
+            if (k) b0 ^= gray_step(w, k, 1);
+            const int i = 2 * gray_elem(k);
+            const float4 t = *reinterpret_cast<const float4*>(p + b0);
             v[i] = make_float2(t.x, t.y);
             v[i + 1] = make_float2(t.z, t.w);
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < (1 << R); ++i) v[i] = psi[sb ^ Lay::p((uint32_t)i << A)];
+        for (int k = 0; k < (1 << R); ++k) {
+            if (k) b0 ^= gray_step(w, k);
+            v[gray_elem(k)] = *reinterpret_cast<const float2*>(p + b0);
+        }
     }
 }
-template <int R, int A, typename Lay = SwzLayout<float>>
-__device__ __forceinline__ void store_group(float2* psi, uint32_t sb, const float2 (&v)[1 << R]) {
-    if (A == 0 && R >= 1) {
+template <int R>
+__device__ __forceinline__ void store_group(float2* psi, uint32_t b0, bool pairs, const WinSteps<R>& w,
+                                            const float2 (&v)[1 << R]) {
+    char* p = reinterpret_cast<char*>(psi);
+    if (pairs) {
 #pragma unroll
-        for (int i = 0; i < (1 << R); i += 2)
-            *reinterpret_cast<float4*>(psi + (sb ^ Lay::p((uint32_t)i << A))) =
-                make_float4(v[i].x, v[i].y, v[i + 1].x, v[i + 1].y);
+        for (int k = 0; k < (1 << (R - 1)); ++k) {
+            if (k) b0 ^= gray_step(w, k, 1);
+            const int i = 2 * gray_elem(k);
+            *reinterpret_cast<float4*>(p + b0) = make_float4(v[i].x, v[i].y, v[i + 1].x, v[i + 1].y);
+        }
     } else {
 #pragma unroll
-        for (int i = 0; i < (1 << R); ++i) psi[sb ^ Lay::p((uint32_t)i << A)] = v[i];
+        for (int k = 0; k < (1 << R); ++k) {
+            if (k) b0 ^= gray_step(w, k);
+            *reinterpret_cast<float2*>(p + b0) = v[gray_elem(k)];
+        }
     }
 }
-template <int R, int A, typename Lay = SwzLayout<double>>
-__device__ __forceinline__ void load_group(const double2* psi, uint32_t sb, double2 (&v)[1 << R]) {
+template <int R>
+__device__ __forceinline__ void load_group(const double2* psi, uint32_t b0, bool, const WinSteps<R>& w,
+                                           double2 (&v)[1 << R]) {
+    const char* p = reinterpret_cast<const char*>(psi);
 #pragma unroll
-    for (int i = 0; i < (1 << R); ++i) v[i] = psi[sb ^ Lay::p((uint32_t)i << A)];
+    for (int k = 0; k < (1 << R); ++k) {
+        if (k) b0 ^= gray_step(w, k);
+        v[gray_elem(k)] = *reinterpret_cast<const double2*>(p + b0);
+    }
 }
-template <int R, int A, typename Lay = SwzLayout<double>>
-__device__ __forceinline__ void store_group(double2* psi, uint32_t sb, const double2 (&v)[1 << R]) {
+template <int R>
+__device__ __forceinline__ void store_group(double2* psi, uint32_t b0, bool, const WinSteps<R>& w,
+                                            const double2 (&v)[1 << R]) {
+    char* p = reinterpret_cast<char*>(psi);
 #pragma unroll
-    for (int i = 0; i < (1 << R); ++i) psi[sb ^ Lay::p((uint32_t)i << A)] = v[i];
+    for (int k = 0; k < (1 << R); ++k) {
+        if (k) b0 ^= gray_step(w, k);
+        *reinterpret_cast<double2*>(p + b0) = v[gray_elem(k)];
+    }
+}
+// fn(i, e) for every element i of a group with its energy e (element 0 lies b0 bytes into E)
+template <int R, typename T, typename Fn>
+__device__ __forceinline__ void for_energies(const T* E, uint32_t b0, const WinSteps<R>& w, Fn&& fn) {
+    const char* p = reinterpret_cast<const char*>(E);
+#pragma unroll
+    for (int k = 0; k < (1 << R); ++k) {
+        if (k) b0 ^= gray_step(w, k);
+        fn(gray_elem(k), *reinterpret_cast<const T*>(p + b0));
+    }
 }
 
 // Shared state of one tile.
@@ -273,126 +331,51 @@ struct TileRef {
     int tb;                    // tile bits
 };
 
-// Forward sub-pass with a compile-time window start A (see subpass_fwd).
-template <typename T, int R, int A, typename Fin>
-__device__ __forceinline__ void subpass_fwd_a(const TileRef<T>& t, const SubPass& sp,
-                                              const LayerConst<T>* lc, bool init, T amp0, int pc0,
-                                              Fin&& fin) {
-    using C = typename Num<T>::C;
-    const uint32_t ngroups = 1u << (t.tb - R);
-    for (uint32_t g0 = 0; g0 < ngroups; g0 += blockDim.x) {
-        const uint32_t g = g0 + threadIdx.x;
-        const bool valid = g < ngroups;
-        const uint32_t base = group_base<R>(valid ? g : 0u, A);
-        const uint32_t sb = swz<T>(base);
-        C v[1 << R];
-        if (valid) {
-            if (init) {
-                // |+> in the rotated frame: amp0 i^{|z|}, |z| = pc0 + |base| + |i|; the four
-                // values i^m amp0 are formed once and picked by the compile-time |i|
-                const int pb = pc0 + __popc(base);
-                C a;
-                a.x = amp0;
-                a.y = T(0);
-                const C q0 = times_i_pow(a, pb), q1 = times_i_pow(a, pb + 1);
-                const C q2 = times_i_pow(a, pb + 2), q3 = times_i_pow(a, pb + 3);
-#pragma unroll
-                for (int i = 0; i < (1 << R); ++i) {
-                    const int m = __popc(i) & 3;
-                    v[i] = m == 0 ? q0 : (m == 1 ? q1 : (m == 2 ? q2 : q3));
-                }
-            } else {
-                load_group<R, A>(t.psi, sb, v);
-            }
-            for (int l = sp.la; l <= sp.lb; ++l) {
-                if (l > sp.la || sp.ph_first) {
-                    const T gp = lc[l].gpi, pre = lc[l].pre;
-#pragma unroll
-                    for (int i = 0; i < (1 << R); ++i) {
-                        T s, c;
-                        sincos_phase(gp, t.E[sb ^ woff<T, A>(i)], s, c);
-                        rot_neg(v[i], s * pre, c * pre);
-                    }
-                }
-                mix_layer<R>(v, sp.mask, lc[l]);
-            }
-            if (sp.post && lc[sp.lb].shear) scale_group<R>(v, lc[sp.lb].post);
-            store_group<R, A>(t.psi, sb, v);
-        }
-        fin(base, A, valid);
-    }
-}
-
 // Forward sub-pass over all groups of the tile.
 //   init:  amplitudes start as |+> (amp0 i^{|z|} in the rotated frame; pc0 = number of set
 //          global bits that the tile index itself fixes) instead of being read
-//   fin:   called once per group slot after the group has been written back, by every thread
-//          of the block (warp-uniform trip count), as fin(base, a, valid); it re-reads the
-//          group from shared memory, which keeps the final reductions out of the register
-//          budget of the butterflies.
-// The window start is dispatched to a compile-time constant (0 <= a <= tb - R <= 9).
-template <typename T, int R, typename Fin>
+template <typename T, int R>
 __device__ __forceinline__ void subpass_fwd(const TileRef<T>& t, const SubPass& sp,
-                                            const LayerConst<T>* lc, bool init, T amp0, int pc0,
-                                            Fin&& fin) {
-    switch (sp.a) {
-        case 0: subpass_fwd_a<T, R, 0>(t, sp, lc, init, amp0, pc0, fin); break;
-        case 1: subpass_fwd_a<T, R, 1>(t, sp, lc, init, amp0, pc0, fin); break;
-        case 2: subpass_fwd_a<T, R, 2>(t, sp, lc, init, amp0, pc0, fin); break;
-        case 3: subpass_fwd_a<T, R, 3>(t, sp, lc, init, amp0, pc0, fin); break;
-        case 4: subpass_fwd_a<T, R, 4>(t, sp, lc, init, amp0, pc0, fin); break;
-        case 5: subpass_fwd_a<T, R, 5>(t, sp, lc, init, amp0, pc0, fin); break;
-        case 6: subpass_fwd_a<T, R, 6>(t, sp, lc, init, amp0, pc0, fin); break;
-        case 7: subpass_fwd_a<T, R, 7>(t, sp, lc, init, amp0, pc0, fin); break;
-        case 8: subpass_fwd_a<T, R, 8>(t, sp, lc, init, amp0, pc0, fin); break;
-        default: subpass_fwd_a<T, R, 9>(t, sp, lc, init, amp0, pc0, fin); break;
-    }
-}
-
-// Adjoint sub-pass with a compile-time window start A (see subpass_adj).
-template <typename T, int R, int A, typename Lay = SwzLayout<T>>
-__device__ __forceinline__ void subpass_adj_a(const TileRef<T>& t, const SubPass& sp,
-                                              const LayerConst<T>* lc, bool lam_from_E,
-                                              T (&acc_b)[2], T (&acc_g)[2]) {
+                                            const LayerConst<T>* lc, bool init, T amp0, int pc0) {
     using C = typename Num<T>::C;
+    const auto map = [](uint32_t u) { return swz<T>(u); };
+    const WinSteps<R> ws = win_steps<R>(sp.a, sizeof(C), map), we = win_steps<R>(sp.a, sizeof(T), map);
     const uint32_t ngroups = 1u << (t.tb - R);
     for (uint32_t g = threadIdx.x; g < ngroups; g += blockDim.x) {
-        const uint32_t base = group_base<R>(g, A);
-        const uint32_t sb = Lay::p(base), eb = Lay::e(base);
-        C v[1 << R], u[1 << R];
-        load_group<R, A, Lay>(t.psi, sb, v);
-        if (lam_from_E) {
+        const uint32_t base = group_base<R>(g, sp.a);
+        const uint32_t sb = swz<T>(base);
+        C v[1 << R];
+        if (init) {
+            // |+> in the rotated frame: amp0 i^{|z|}, |z| = pc0 + |base| + |i|; the four
+            // values i^m amp0 are formed once and picked by the compile-time |i|
+            const int pb = pc0 + __popc(base);
+            C a;
+            a.x = amp0;
+            a.y = T(0);
+            const C q0 = times_i_pow(a, pb), q1 = times_i_pow(a, pb + 1);
+            const C q2 = times_i_pow(a, pb + 2), q3 = times_i_pow(a, pb + 3);
 #pragma unroll
             for (int i = 0; i < (1 << R); ++i) {
-                const T e = t.E[eb ^ Lay::e((uint32_t)i << A)];
-                u[i].x = e * v[i].x;
-                u[i].y = e * v[i].y;
+                const int m = __popc(i) & 3;
+                v[i] = m == 0 ? q0 : (m == 1 ? q1 : (m == 2 ? q2 : q3));
             }
         } else {
-            load_group<R, A, Lay>(t.lam, sb, u);
+            load_group<R>(t.psi, sb * (uint32_t)sizeof(C), sp.a == 0, ws, v);
         }
-        for (int l = sp.lb; l >= sp.la; --l) {
-            const int j = sp.lb - l;
-            const T ab = mix_group_adj<R>(v, u, sp.mask, lc[l].c, lc[l].s);
-            if (j == 0) acc_b[0] += ab; else acc_b[1] += ab;
+#pragma unroll 1
+        for (int l = sp.la; l <= sp.lb; ++l) {
             if (l > sp.la || sp.ph_first) {
-                const T gp = -lc[l].gpi;
-                T ag[4] = {T(0), T(0), T(0), T(0)};
-#pragma unroll
-                for (int i = 0; i < (1 << R); ++i) {
-                    const T e = t.E[eb ^ Lay::e((uint32_t)i << A)];
-                    ag[i & 3] = fma(e, im_conj_mul(u[i], v[i]), ag[i & 3]);
+                const T gp = lc[l].gpi, pre = lc[l].pre;
+                for_energies<R>(t.E, sb * (uint32_t)sizeof(T), we, [&](int i, T e) {
                     T s, c;
                     sincos_phase(gp, e, s, c);
-                    rot_neg(v[i], s, c);
-                    rot_neg(u[i], s, c);
-                }
-                const T agt = (ag[0] + ag[1]) + (ag[2] + ag[3]);
-                if (j == 0) acc_g[0] += agt; else acc_g[1] += agt;
+                    rot_neg(v[i], s * pre, c * pre);
+                });
             }
+            mix_layer<R>(v, sp.mask, lc[l]);
         }
-        store_group<R, A, Lay>(t.psi, sb, v);
-        store_group<R, A, Lay>(t.lam, sb, u);
+        if (sp.post && lc[sp.lb].shear) scale_group<R>(v, lc[sp.lb].post);
+        store_group<R>(t.psi, sb * (uint32_t)sizeof(C), sp.a == 0, ws, v);
     }
 }
 
@@ -404,55 +387,44 @@ template <typename T, int R, typename Lay = SwzLayout<T>>
 __device__ __forceinline__ void subpass_adj(const TileRef<T>& t, const SubPass& sp,
                                             const LayerConst<T>* lc, bool lam_from_E,
                                             T (&acc_b)[2], T (&acc_g)[2]) {
-    switch (sp.a) {
-        case 0: subpass_adj_a<T, R, 0, Lay>(t, sp, lc, lam_from_E, acc_b, acc_g); break;
-        case 1: subpass_adj_a<T, R, 1, Lay>(t, sp, lc, lam_from_E, acc_b, acc_g); break;
-        case 2: subpass_adj_a<T, R, 2, Lay>(t, sp, lc, lam_from_E, acc_b, acc_g); break;
-        case 3: subpass_adj_a<T, R, 3, Lay>(t, sp, lc, lam_from_E, acc_b, acc_g); break;
-        case 4: subpass_adj_a<T, R, 4, Lay>(t, sp, lc, lam_from_E, acc_b, acc_g); break;
-        case 5: subpass_adj_a<T, R, 5, Lay>(t, sp, lc, lam_from_E, acc_b, acc_g); break;
-        case 6: subpass_adj_a<T, R, 6, Lay>(t, sp, lc, lam_from_E, acc_b, acc_g); break;
-        case 7: subpass_adj_a<T, R, 7, Lay>(t, sp, lc, lam_from_E, acc_b, acc_g); break;
-        case 8: subpass_adj_a<T, R, 8, Lay>(t, sp, lc, lam_from_E, acc_b, acc_g); break;
-        default: subpass_adj_a<T, R, 9, Lay>(t, sp, lc, lam_from_E, acc_b, acc_g); break;
-    }
-}
-
-// Final reductions of one group (2^R amplitudes of window start a, already written back):
-// <C> partial (FP32 over the group, FP64 across groups) and the warp's top-k list. Before
-// offering, the list threshold is raised to the k-th largest of the lanes' group maxima: the k
-// lanes with the largest maxima hold k distinct elements at least that probable, so every
-// element of the final top-k passes the FP32 filter (margins as in WarpTopK::offer), while
-// most elements are rejected without an insertion. zmap(u) gives the global index of tile
-// index u. Called by every thread of the warp.
-template <typename T, int R, typename ZMap>
-__device__ __forceinline__ void reduce_group(const TileRef<T>& t, uint32_t base, int a, bool valid,
-                                             int k, WarpTopK& top, double& ex, ZMap&& zmap) {
     using C = typename Num<T>::C;
-    T accp = T(0);
-    float pmax = -1.0f;
-#pragma unroll 1
-    for (int i = 0; i < (1 << R); ++i) {
-        if (valid) {
-            const uint32_t ix = swz<T>(base | ((uint32_t)i << a));
-            const C v = t.psi[ix];
-            const T pr = v.x * v.x + v.y * v.y;
-            accp += pr * t.E[ix];
-            pmax = fmaxf(pmax, (float)pr);
+    const WinSteps<R> ws = win_steps<R>(sp.a, sizeof(C), [](uint32_t u) { return Lay::p(u); });
+    const WinSteps<R> we = win_steps<R>(sp.a, sizeof(T), [](uint32_t u) { return Lay::e(u); });
+    const uint32_t ngroups = 1u << (t.tb - R);
+    for (uint32_t g = threadIdx.x; g < ngroups; g += blockDim.x) {
+        const uint32_t base = group_base<R>(g, sp.a);
+        const uint32_t sb = Lay::p(base) * (uint32_t)sizeof(C), eb = Lay::e(base) * (uint32_t)sizeof(T);
+        C v[1 << R], u[1 << R];
+        load_group<R>(t.psi, sb, sp.a == 0, ws, v);
+        if (lam_from_E) {
+            for_energies<R>(t.E, eb, we, [&](int i, T e) {
+                u[i].x = e * v[i].x;
+                u[i].y = e * v[i].y;
+            });
+        } else {
+            load_group<R>(t.lam, sb, sp.a == 0, ws, u);
         }
-    }
-    ex += (double)accp;
-    if (k <= 0) return;
-    const float kth = warp_kth_largest(pmax, k);
-    if (kth > 0.0f) top.raise_threshold(kth * 0.99999904632568359375f);   // (1 - 2^-20)
 #pragma unroll 1
-    for (int i = 0; i < (1 << R); ++i) {
-        const uint32_t u = base | ((uint32_t)i << a);
-        C v;
-        v.x = T(0);
-        v.y = T(0);
-        if (valid) v = t.psi[swz<T>(u)];
-        top.offer(v, zmap(u), valid);
+        for (int l = sp.lb; l >= sp.la; --l) {
+            const int j = sp.lb - l;
+            const T ab = mix_group_adj<R>(v, u, sp.mask, lc[l].c, lc[l].s);
+            if (j == 0) acc_b[0] += ab; else acc_b[1] += ab;
+            if (l > sp.la || sp.ph_first) {
+                const T gp = -lc[l].gpi;
+                T ag[4] = {T(0), T(0), T(0), T(0)};
+                for_energies<R>(t.E, eb, we, [&](int i, T e) {
+                    ag[i & 3] = fma(e, im_conj_mul(u[i], v[i]), ag[i & 3]);
+                    T s, c;
+                    sincos_phase(gp, e, s, c);
+                    rot_neg(v[i], s, c);
+                    rot_neg(u[i], s, c);
+                });
+                const T agt = (ag[0] + ag[1]) + (ag[2] + ag[3]);
+                if (j == 0) acc_g[0] += agt; else acc_g[1] += agt;
+            }
+        }
+        store_group<R>(t.psi, sb, sp.a == 0, ws, v);
+        store_group<R>(t.lam, sb, sp.a == 0, ws, u);
     }
 }
 
