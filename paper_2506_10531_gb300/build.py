@@ -10,7 +10,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libqaoa.so")
 BUILD = os.path.join(HERE, "_build")
-SOURCES = ["qaoa_api.cu", "k_resident.cu", "k_cluster.cu", "k_stream.cu", "k_plain.cu", "k_dqaoa.cu",
+SOURCES = ["qaoa_api.cu", "k_resident.cu", "k_cluster.cu", "k_stream.cu", "k_plain.cu", "k_reduce.cu", "k_dqaoa.cu",
            "k_noalloc.cu", "k_cstream.cu", "k_tstream.cu", "qaoa_server.cu", "qaoa_tune.cu", "k_sample.cu", "dqaoa_host.cpp", "cobyla.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # host code without FP contraction: the host merge rounds the same way on every architecture

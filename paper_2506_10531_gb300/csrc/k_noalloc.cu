@@ -1,5 +1,5 @@
 // k_noalloc.cu -- <C> and top-k of a complex64 state with no allocation at all: the standalone
-// reduction kernels of k_stream.cu run on a fixed scratch array that lives in this file, in
+// reduction kernels of k_reduce.cu run on a fixed scratch array that lives in this file, in
 // device memory reserved when the library is loaded (every GPU that loads the library holds it
 // until the process exits). The paper has no counterpart; this is an interface addition for
 // callers that cannot allocate device memory.

@@ -77,6 +77,7 @@ __device__ void forward_run(const InstDesc<T>& d, const Smem<T>& s, bool started
     }
     // <C> and the top-k list of the final state (the list is unique under (probability desc,
     // index asc), whatever the order of the reduction)
+    if (!d.expect && d.k == 0) return;   // the state alone is wanted
     double ex = 0.0;
     tile_reduce<T>(tile, d.k, [](uint32_t u) { return u; }, s.tk, ex);
     const double tot = block_sum(ex, s.red);

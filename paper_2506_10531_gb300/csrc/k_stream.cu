@@ -1,5 +1,5 @@
 // k_stream.cu -- HBM-streaming tier for states larger than one SM's shared memory, plus the
-// standalone energy build and the standalone <C> / top-k reductions over a state in HBM.
+// standalone energy build.
 //
 // A layer of Eq. 2 (Section IV) on a 2^n state is split into HBM passes. Each pass moves
 // tiles of 2^tb amplitudes between HBM and shared memory and runs the tile engine on them:
@@ -14,6 +14,7 @@
 #include "qaoa_engine.cuh"
 #include "qaoa_kernels.h"
 #include "qaoa_stream.h"
+#include "qaoa_topk.cuh"
 
 namespace qaoa {
 
@@ -251,34 +252,6 @@ __global__ void __launch_bounds__(256, 2) k_stream_pass(const StreamPass P,
     }
 }
 
-// Merge the top-k lists of `nl` lists (list j at tile slot j * stride) into one list of the k
-// best (probability desc, index asc; unique, so any merge order gives the same list): each warp
-// takes a strided share of the entries, then warp 0 merges the warps' lists. The result is in
-// lanes 0..k-1 of warp 0 (f.p, f.z).
-__device__ __forceinline__ void merge_lists(const double* topp, const uint32_t* topz, uint64_t nl,
-                                            uint64_t stride, int k, TopEnt* tops, WarpTopK& f) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    WarpTopK top;
-    top.init(k);
-    const uint64_t nent = nl * (uint64_t)k;
-    for (uint64_t e0 = (uint64_t)warp * 32; e0 < nent; e0 += (uint64_t)(blockDim.x >> 5) * 32) {
-        const uint64_t e = e0 + lane;
-        const bool ok = e < nent;
-        const uint64_t a = ok ? (e / k) * stride * k + e % k : 0;
-        top.offer_exact(ok ? topp[a] : -1.0, ok ? topz[a] : 0u, ok);
-    }
-    if (lane < k) tops[warp * 32 + lane] = TopEnt{top.p, top.z};
-    __syncthreads();
-    if (warp == 0) {
-        f.init(k);
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            const bool ok = lane < k;
-            const TopEnt e = ok ? tops[w * 32 + lane] : TopEnt{-1.0, 0xffffffffu};
-            f.offer_exact(e.p, e.z, ok);
-        }
-    }
-}
-
 // First merge level for instances with many tiles: block (c, i) merges the lists of tiles
 // [c * FIN_CHUNK, (c + 1) * FIN_CHUNK) of instance i and writes the result over the list of the
 // chunk's first tile (only this block reads the chunk, and it reads everything first).
@@ -288,18 +261,20 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_stream_topk_chunks(const StreamInst<T>* __restrict__ insts,
                                                            int count, uint64_t ntiles, int k,
                                                            const StreamInst<T> one) {
-    __shared__ TopEnt tops[8 * 32];
+    __shared__ TopScratch ts;
     const int ii = blockIdx.y;
     if (ii >= count) return;
     const StreamInst<T>& I = insts ? insts[ii] : one;
     const uint64_t t0 = (uint64_t)blockIdx.x * FIN_CHUNK;
     const uint64_t nl = (ntiles - t0) < FIN_CHUNK ? (ntiles - t0) : FIN_CHUNK;
-    WarpTopK f;
-    merge_lists(I.part_topp + t0 * k, I.part_topz + t0 * k, nl, 1, k, tops, f);
-    __syncthreads();   // every read of the chunk is done before its first list is overwritten
+    // merge_entries ends with a barrier: every read of the chunk is done before its first list is
+    // overwritten
+    double* topp = I.part_topp + t0 * k;
+    uint32_t* topz = I.part_topz + t0 * k;
+    merge_entries(nl * k, k, ts, [=](uint64_t e) { return TopEnt{topp[e], topz[e]}; });
     if (threadIdx.x < (unsigned)k) {
-        I.part_topp[t0 * k + threadIdx.x] = f.p;
-        I.part_topz[t0 * k + threadIdx.x] = f.z;
+        topp[threadIdx.x] = ts.run[threadIdx.x].p;
+        topz[threadIdx.x] = ts.run[threadIdx.x].z;
     }
 }
 
@@ -311,7 +286,7 @@ __global__ void __launch_bounds__(256) k_stream_finalize(const StreamInst<T>* __
                                                          int count, uint64_t ntiles, int k,
                                                          uint64_t stride, const StreamInst<T> one) {
     __shared__ double red[32];
-    __shared__ TopEnt tops[8 * 32];
+    __shared__ TopScratch ts;
     const int ii = blockIdx.x;
     if (ii >= count) return;
     const StreamInst<T>& I = insts ? insts[ii] : one;
@@ -324,11 +299,15 @@ __global__ void __launch_bounds__(256) k_stream_finalize(const StreamInst<T>* __
     if (threadIdx.x == 0 && I.expect) *I.expect = tot;
     if (k > 0) {
         const uint64_t nl = (ntiles + stride - 1) / stride;
-        WarpTopK f;
-        merge_lists(I.part_topp, I.part_topz, nl, stride, k, tops, f);
+        const double* topp = I.part_topp;
+        const uint32_t* topz = I.part_topz;
+        merge_entries(nl * k, k, ts, [=](uint64_t e) {
+            const uint64_t a = (e / k) * stride * k + e % k;
+            return TopEnt{topp[a], topz[a]};
+        });
         if (threadIdx.x < (unsigned)k) {
-            if (I.topk_idx) I.topk_idx[threadIdx.x] = (uint64_t)f.z;
-            if (I.topk_prob) I.topk_prob[threadIdx.x] = f.p;
+            if (I.topk_idx) I.topk_idx[threadIdx.x] = (uint64_t)ts.run[threadIdx.x].z;
+            if (I.topk_prob) I.topk_prob[threadIdx.x] = ts.run[threadIdx.x].p;
         }
     }
 }
@@ -623,101 +602,6 @@ __global__ void __launch_bounds__(256) k_energy(int n, int m, const T* __restric
     }
 }
 
-// ---- standalone <C> and top-k over a state in HBM ----------------------------------------
-// Grid-stride over elements; each thread accumulates FP32 products over at most 32 elements
-// before adding them to its FP64 partial; per-CTA partials and top-k lists go to the
-// caller-provided scratch and are merged by k_stream_finalize-style reduction.
-template <typename T>
-__global__ void __launch_bounds__(256) k_reduce_state(int n, const typename Num<T>::C* __restrict__ psi,
-                                                      const T* __restrict__ E, int k,
-                                                      double* part_expect, double* part_topp,
-                                                      uint32_t* part_topz) {
-    __shared__ double red[32];
-    __shared__ TopEnt tops[8 * 32];
-    const uint64_t D = 1ull << n;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    WarpTopK top;
-    top.init(k > 0 ? k : 1);
-    double ex = 0.0;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    // chunks of 32 consecutive strides so that the FP32 partial has at most 32 terms
-    for (uint64_t c0 = (uint64_t)blockIdx.x * blockDim.x; c0 < D; c0 += stride * 32) {
-        T acc = T(0);
-        for (int r = 0; r < 32; ++r) {
-            const uint64_t z = c0 + (uint64_t)r * stride + threadIdx.x;
-            const bool ok = z < D;
-            typename Num<T>::C v;
-            v.x = T(0); v.y = T(0);
-            if (ok) {
-                v = psi[z];
-                if (E) acc += (v.x * v.x + v.y * v.y) * E[z];
-            }
-            if (k > 0) top.offer(v, (uint32_t)z, ok);
-        }
-        ex += (double)acc;
-    }
-    const double tot = block_sum(ex, red);
-    if (threadIdx.x == 0) part_expect[blockIdx.x] = tot;
-    if (k > 0) {
-        if (lane < k) tops[warp * 32 + lane] = TopEnt{top.p, top.z};
-        __syncthreads();
-        if (warp == 0) {
-            WarpTopK f;
-            f.init(k);
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-                const bool ok = lane < k;
-                const TopEnt e = ok ? tops[w * 32 + lane] : TopEnt{-1.0, 0xffffffffu};
-                f.offer_exact(e.p, e.z, ok);
-            }
-            if (lane < k) {
-                part_topp[(uint64_t)blockIdx.x * k + lane] = f.p;
-                part_topz[(uint64_t)blockIdx.x * k + lane] = f.z;
-            }
-        }
-    }
-}
-
-__global__ void __launch_bounds__(256) k_reduce_finalize(int nparts, const double* part_expect,
-                                                         const double* part_topp,
-                                                         const uint32_t* part_topz, int k,
-                                                         double* expect, uint64_t* topk_idx,
-                                                         double* topk_prob) {
-    __shared__ double red[32];
-    __shared__ TopEnt tops[8 * 32];
-    double acc = 0.0;
-    const int per = (nparts + blockDim.x - 1) / blockDim.x;
-    for (int t = threadIdx.x * per; t < (int)(threadIdx.x + 1) * per && t < nparts; ++t)
-        acc += part_expect[t];
-    const double tot = block_sum(acc, red);
-    if (threadIdx.x == 0 && expect) *expect = tot;
-    if (k > 0) {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        WarpTopK top;
-        top.init(k);
-        const int nent = nparts * k;
-        for (int e0 = warp * 32; e0 < nent; e0 += (int)(blockDim.x >> 5) * 32) {
-            const int e = e0 + lane;
-            const bool ok = e < nent;
-            top.offer_exact(ok ? part_topp[e] : -1.0, ok ? part_topz[e] : 0u, ok);
-        }
-        if (lane < k) tops[warp * 32 + lane] = TopEnt{top.p, top.z};
-        __syncthreads();
-        if (warp == 0) {
-            WarpTopK f;
-            f.init(k);
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-                const bool ok = lane < k;
-                const TopEnt e = ok ? tops[w * 32 + lane] : TopEnt{-1.0, 0xffffffffu};
-                f.offer_exact(e.p, e.z, ok);
-            }
-            if (lane < k) {
-                if (topk_idx) topk_idx[lane] = (uint64_t)f.z;
-                if (topk_prob) topk_prob[lane] = f.p;
-            }
-        }
-    }
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------
@@ -921,19 +805,6 @@ cudaError_t launch_stream_grad_reduce(bool dbl, const StreamPass* passes, int S,
     for (int i = 0; i < S; ++i) { pl.la[i] = passes[i].la; pl.lb[i] = passes[i].lb; }
     if (dbl) k_stream_grad_reduce<double><<<count, 256, 0, st>>>(pl, S, static_cast<const StreamInst<double>*>(insts), count, ntiles, one_of<double>(one));
     else k_stream_grad_reduce<float><<<count, 256, 0, st>>>(pl, S, static_cast<const StreamInst<float>*>(insts), count, ntiles, one_of<float>(one));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_reduce_state(bool dbl, int n, const void* psi, const void* E, int k,
-                                double* part_expect, double* part_topp, uint32_t* part_topz,
-                                double* expect, uint64_t* topk_idx, double* topk_prob,
-                                cudaStream_t st) {
-    const int parts = reduce_parts(n);
-    if (dbl) k_reduce_state<double><<<parts, 256, 0, st>>>(n, static_cast<const double2*>(psi), static_cast<const double*>(E), k, part_expect, part_topp, part_topz);
-    else k_reduce_state<float><<<parts, 256, 0, st>>>(n, static_cast<const float2*>(psi), static_cast<const float*>(E), k, part_expect, part_topp, part_topz);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_reduce_finalize<<<1, 256, 0, st>>>(parts, part_expect, part_topp, part_topz, k, expect, topk_idx, topk_prob);
     return cudaGetLastError();
 }
 

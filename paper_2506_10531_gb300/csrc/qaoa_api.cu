@@ -104,8 +104,11 @@ template <typename T>
 qaoa_status run_resident_one(qaoa_ctx* c, const InstDesc<T>& d, cudaStream_t st) {
     const bool dbl = is_dbl<T>();
     const bool grad = (d.flags & F_GRAD) != 0;
-    // the descriptor travels by value as a kernel parameter
-    CK(launch_resident(dbl, nullptr, 1, d.n, d.p, grad, nullptr, 1, st, &d));
+    // the descriptor travels by value as a kernel parameter. One block runs alone, so it takes as
+    // many threads as the narrowest windows that suit n give it (n = 8, p = 1 on GB300: 32 us with
+    // 5-qubit windows, 8 of 32 threads busy; 17.5 us with 3-qubit ones)
+    const int rmax = dbl ? RES_RMAX : (d.n <= 12 ? 3 : (d.n == 13 ? 4 : RES_RMAX));
+    CK(launch_resident(dbl, nullptr, 1, d.n, d.p, grad, nullptr, 1, st, &d, rmax));
     return QAOA_OK;
 }
 
