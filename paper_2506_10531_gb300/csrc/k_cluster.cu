@@ -28,7 +28,7 @@ struct ClusterSmem {
     float2* psi;
     float* E;
     float* Q;
-    LayerConst<float>* lc;
+    FwdConst<float>* lc;
     double* red;     // 32
     double* cex;     // this CTA's <C> partial
     TileTopk tk;     // top-k scratch; tk.out is this CTA's list (read by rank 0)
@@ -46,7 +46,7 @@ __host__ __device__ inline size_t cluster_layout(int n, int L, int p, int thread
     off[0] = o; o = cl_align(o + D * sizeof(float2));
     off[1] = o; o = cl_align(o + D * sizeof(float));
     off[2] = o; o = cl_align(o + (size_t)n * n * sizeof(float));
-    off[3] = o; o = cl_align(o + (size_t)p * sizeof(LayerConst<float>));
+    off[3] = o; o = cl_align(o + (size_t)p * sizeof(FwdConst<float>));
     off[4] = o; o = cl_align(o + 32 * sizeof(double));
     // top-k scratch (used after the last sub-pass) and energy tables (used before the first)
     // share one region
@@ -66,7 +66,7 @@ __host__ __device__ inline size_t cluster_layout(int n, int L, int p, int thread
 // takes NP = 16 / C slab positions at once so that 16 remote loads are in flight together.
 template <int CB>
 __device__ void global_subpass(cg::cluster_group& cl, const ClusterSmem& s, int L, uint32_t r,
-                               const LayerConst<float>& lc) {
+                               const FwdConst<float>& lc) {
     constexpr int C = 1 << CB;
     constexpr int NP = (16 / C) > 0 ? (16 / C) : 1;
     float2* rp[C];
@@ -110,7 +110,7 @@ __device__ void run_cluster_instance(cg::cluster_group& cl, const InstDesc<float
     s.psi = reinterpret_cast<float2*>(sm + off[0]);
     s.E = reinterpret_cast<float*>(sm + off[1]);
     s.Q = reinterpret_cast<float*>(sm + off[2]);
-    s.lc = reinterpret_cast<LayerConst<float>*>(sm + off[3]);
+    s.lc = reinterpret_cast<FwdConst<float>*>(sm + off[3]);
     s.red = reinterpret_cast<double*>(sm + off[4]);
     s.tk.wlists = reinterpret_cast<TopEnt*>(sm + off[5]);
     s.cex = reinterpret_cast<double*>(sm + off[6]);
@@ -121,7 +121,7 @@ __device__ void run_cluster_instance(cg::cluster_group& cl, const InstDesc<float
     s.escr = reinterpret_cast<float*>(sm + off[10]);
     const uint32_t D = 1u << L;
 
-    set_layer_consts<float>(s.lc, d.gamma, d.beta, p, n, true);
+    set_fwd_consts(s.lc, d.gamma, d.beta, p, n);
     for (int i = threadIdx.x; i < n * n; i += blockDim.x) s.Q[i] = d.Q[i];
     __syncthreads();
     const FusedInit<float> fi{s.psi, (float)exp2(-0.5 * (double)n),
@@ -134,11 +134,10 @@ __device__ void run_cluster_instance(cg::cluster_group& cl, const InstDesc<float
     // ---- forward: local snake with the global sub-pass before each layer's last window ----
     const TileRef<float> tile{s.psi, nullptr, s.E, L};
     const int G = num_windows(0, L, R);
-    const int S = snake_len(G, p);
     const float amp0 = (float)exp2(-0.5 * (double)n);
-    for (int si = 0; si < S; ++si) {
-        SubPass sp;
-        snake_step(si, G, p, 0, started ? 0 : 1, 0, L, L, R, sp);
+    Snake sn(p, 0, started ? 0 : 1, 0, L, L, R);
+    for (int si = 0;; ++si, sn.next()) {
+        SubPass sp = sn.get();
         // sub-pass (l+1)(G-1) holds layer l's last local window (fused with the cost and the
         // first window of layer l+1); the global qubits of layer l are mixed just before it,
         // after the cost of layer l (G >= 2: L >= 10 is required by the host)
@@ -148,9 +147,10 @@ __device__ void run_cluster_instance(cg::cluster_group& cl, const InstDesc<float
             global_subpass<CB>(cl, s, L, r, s.lc[sp.la]);
             cl.sync();
         }
-        sp.post = (si == S - 1);
+        sp.post = sn.last();
         subpass_fwd<float, R>(tile, sp, s.lc, si == 0 && !started, amp0, __popc(r));
         __syncthreads();
+        if (sn.last()) break;
     }
     // ---- per-CTA reductions, then rank 0 merges the CTAs (rank order for <C>) ----
     double ex = 0.0;

@@ -124,12 +124,13 @@ __device__ __forceinline__ void w2_store(float2* sp, const float2 (&v)[32]) {
 }
 template <int R>
 __device__ __forceinline__ void phase_group(float2 (&v)[1 << R], const float* sE, uint32_t e0, int eshift,
-                                            const LayerConst<float>& k) {
+                                            int parity, const LayerConst<float>& k) {
+    const Pending<float> pre(k.pre, k.pcot, parity);
 #pragma unroll
     for (int i = 0; i < (1 << R); ++i) {
         float s, c;
-        sincos_phase(k.gpi, sE[e0 + ((uint32_t)i << eshift)], s, c);
-        rot_neg(v[i], s * k.pre, c * k.pre);
+        sincos_phase(k.ph, sE[e0 + ((uint32_t)i << eshift)], s, c);
+        rot_neg(v[i], s * pre.f[__popc(i) & 1], c * pre.f[__popc(i) & 1]);
     }
 }
 // W1: bits [4, 8). Group g < 512 (thread t: g = t and t + 256): base = (g & 15) | (g >> 4) << 8,
@@ -343,7 +344,7 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
             // thread l reads back only its own staged gamma_l, beta_l; the Q stores are ordered
             // before their readers by the barriers that end set_layer_consts
             set_layer_consts<float>(reinterpret_cast<LayerConst<float>*>(sm + o.lc[sl]), gst, bst, p, n,
-                                    true);
+                                    false);
         }
     };
     refill(0);
@@ -441,7 +442,7 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
 #pragma unroll
                         for (int i = 0; i < 32; ++i) {
                             float s, c;
-                            sincos_phase(lc[0].gpi, ev[i], s, c);
+                            sincos_phase(lc[0].ph, ev[i], s, c);
                             float2 a = make_float2(I.amp0 * c, -I.amp0 * s);
                             v[i] = times_i_pow(a, pc + __popc(i));
                         }
@@ -460,10 +461,10 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
                         w2_load(sp, v);
                         mix_layer<5>(v, 31, lc[pass - 1]);
                         if (!fin) {
-                            phase_group<5>(v, sE, threadIdx.x, 8, lc[pass]);
+                            phase_group<5>(v, sE, threadIdx.x, 8, __popc(threadIdx.x) + __popc(tau), lc[pass]);
                             mix_layer<5>(v, 31, lc[pass]);
                         } else {
-                            if (lc[p - 1].shear) scale_group<5>(v, lc[p - 1].post);
+                            scale_group<5>(v, Pending<float>(lc[p - 1].post, lc[p - 1].cot, __popc(threadIdx.x) + __popc(tau)));
 #pragma unroll
                             for (int i = 0; i < 32; ++i) {
                                 const float pr = v[i].x * v[i].x + v[i].y * v[i].y;
@@ -489,10 +490,10 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
                         for (int i = 0; i < (1 << H); ++i) v[i] = sp[b + ((uint32_t)i << CB)];
                         mix_layer<H>(v, (1 << H) - 1, lc[pass - 1]);
                         if (!fin) {
-                            phase_group<H>(v, sE, lo, CB, lc[pass]);
+                            phase_group<H>(v, sE, lo, CB, __popc(lo) + __popc(tau), lc[pass]);
                             mix_layer<H>(v, (1 << H) - 1, lc[pass]);
                         } else {
-                            if (lc[p - 1].shear) scale_group<H>(v, lc[p - 1].post);
+                            scale_group<H>(v, Pending<float>(lc[p - 1].post, lc[p - 1].cot, __popc(lo) + __popc(tau)));
 #pragma unroll
                             for (int i = 0; i < (1 << H); ++i) {
                                 const float pr = v[i].x * v[i].x + v[i].y * v[i].y;

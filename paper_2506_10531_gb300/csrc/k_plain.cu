@@ -19,7 +19,7 @@ __global__ void k_plain_phase(uint64_t D, const float* __restrict__ E, const flo
     const uint64_t z = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (z >= D) return;
     float s, c;
-    sincos_phase(gamma[l] / 3.14159265358979323846f, E[z], s, c);
+    sincos_gpi(gamma[l] / 3.14159265358979323846f, E[z], s, c);
     float2 v = psi[z];
     rot_neg(v, s, c);
     psi[z] = v;

@@ -24,9 +24,8 @@ struct Smem {
     typename Num<T>::C* lam;
     T* E;
     T* Q;
-    LayerConst<T>* lc;
-    double* red;       // 32 doubles
-    double* acc;       // 2 p doubles: d gamma, d beta accumulators
+    LayerConst<T>* lc;     // adjoint; the forward run's FwdConst<T> occupy the same place
+    double* red;       // 64 doubles
     TileTopk tk;       // top-k scratch
     T* escr;           // energy-build tables
 };
@@ -43,8 +42,7 @@ __host__ __device__ inline size_t smem_layout(int n, int p, bool grad, int threa
     off[2] = o; o = align_up(o + D * sizeof(T), 16);                       // E
     off[3] = o; o = align_up(o + (size_t)n * n * sizeof(T), 16);           // Q
     off[4] = o; o = align_up(o + (size_t)p * sizeof(LayerConst<T>), 16);   // layer consts
-    off[5] = o; o = align_up(o + 32 * sizeof(double), 16);                 // reduction
-    off[6] = o; o = align_up(o + 2 * (size_t)p * sizeof(double), 16);      // grad accum
+    off[5] = o; o = align_up(o + 64 * sizeof(double), 16);                 // reduction
     // the energy-build tables are used before the first sub-pass and the top-k scratch after
     // the last one: both live in one region
     const size_t nw = (size_t)(threads + 31) / 32;
@@ -60,19 +58,38 @@ __host__ __device__ inline size_t smem_layout(int n, int p, bool grad, int threa
 }
 
 template <typename T, int R>
-__device__ void forward_run(const InstDesc<T>& d, const Smem<T>& s, bool started) {
+__device__ void forward_run(const InstDesc<T>& d, const Smem<T>& s, const WinSched& ws, bool started) {
     const int n = d.n, p = d.p;
     const TileRef<T> tile{s.psi, s.lam, s.E, n};
     // started: the energy build already wrote |+> after the first cost layer
     const bool init = !(d.flags & F_INIT_PSI) && !started;
     const T amp0 = (T)exp2(-0.5 * (double)n);
-    const int G = num_windows(0, n, R);
-    const int S = snake_len(G, p);
-    for (int si = 0; si < S; ++si) {
+    const FwdConst<T>* lc = reinterpret_cast<const FwdConst<T>*>(s.lc);
+    // layer by layer through the windows in the schedule's order; when a layer's last window is the
+    // next one's first, both share a sub-pass around the cost phase
+    bool opens = !started, first = true;
+    int pos = 0;
+    for (int l = 0; l < p;) {
         SubPass sp;
-        snake_step(si, G, p, 0, started ? 0 : 1, 0, n, n, R, sp);
-        sp.post = (si == S - 1);
-        subpass_fwd<T, R>(tile, sp, s.lc, init && si == 0, amp0, 0);
+        const int w = (l & 1) ? ws.odd[pos] : pos;
+        sp.a = ws.a[w];
+        sp.mask = ws.mask[w];
+        sp.la = sp.lb = l;
+        sp.ph_first = opens;
+        opens = false;
+        if (++pos == ws.nw) {
+            pos = 0;
+            opens = true;
+            ++l;
+            if (l < p && w == ((l & 1) ? ws.odd[0] : 0)) {
+                sp.lb = l;
+                opens = false;
+                if (++pos == ws.nw) { pos = 0; opens = true; ++l; }
+            }
+        }
+        sp.post = l == p;
+        subpass_fwd<T, R>(tile, sp, lc, init && first, amp0, 0);
+        first = false;
         __syncthreads();
     }
     // <C> and the top-k list of the final state (the list is unique under (probability desc,
@@ -94,30 +111,41 @@ template <typename T, int R>
 __device__ void adjoint_run(const InstDesc<T>& d, const Smem<T>& s) {
     const int n = d.n, p = d.p;
     const TileRef<T> tile{s.psi, s.lam, s.E, n};
-    const int G = num_windows(0, n, R);
-    const int S = snake_len(G, p);
-    for (int l = threadIdx.x; l < 2 * p; l += blockDim.x) s.acc[l] = 0.0;
-    __syncthreads();
-    for (int si = S - 1; si >= 0; --si) {
-        SubPass sp;
-        snake_step(si, G, p, 0, 1, 0, n, n, R, sp);
-        T ab[2] = {T(0), T(0)}, ag[2] = {T(0), T(0)};
-        subpass_adj<T, R>(tile, sp, s.lc, si == S - 1, ab, ag);
-        __syncthreads();
-        for (int j = 0; j <= sp.lb - sp.la; ++j) {
-            const int l = sp.lb - j;
-            const double sb = block_sum((double)ab[j], s.red);
-            const double sg = block_sum((double)ag[j], s.red);
-            if (threadIdx.x == 0) {
-                s.acc[p + l] += sb;
-                if (l > sp.la || sp.ph_first) s.acc[l] += sg;
-            }
+    // A thread adds its FP32 terms of a layer in FP64 (db, dg: of layer `cur` and of the one below);
+    // a layer's block sum is taken once, when the sweep has left the layer.
+    double db[2] = {0.0, 0.0}, dg[2] = {0.0, 0.0};
+    int cur = p - 1;
+    set_layer_consts<T>(s.lc, d.gamma, d.beta, p, n, true);
+    Snake sn(p, 0, 1, 0, n, n, R);
+    sn.to_last();
+    bool first = true;
+    for (;; sn.prev()) {
+        const SubPass sp = sn.get();
+        while (sp.lb < cur) {   // uniform: layer cur is complete
+            const double v = block_sum4(db[0], dg[0], 0.0, 0.0, s.red);
+            if (threadIdx.x == 0 && d.dbeta) d.dbeta[cur] = 2.0 * v;
+            if (threadIdx.x == 1 && d.dgamma) d.dgamma[cur] = 2.0 * v;
+            db[0] = db[1]; dg[0] = dg[1];
+            db[1] = dg[1] = 0.0;
+            --cur;
         }
+        T acc[4] = {T(0), T(0), T(0), T(0)};
+        subpass_adj<T, R>(tile, sp, s.lc, first, cur, acc);
+        first = false;
+        db[0] += (double)acc[0];
+        db[1] += (double)acc[1];
+        dg[0] += (double)acc[2];
+        dg[1] += (double)acc[3];
         __syncthreads();
+        if (sn.first()) break;
     }
-    for (int l = threadIdx.x; l < p; l += blockDim.x) {
-        if (d.dgamma) d.dgamma[l] = 2.0 * s.acc[l];
-        if (d.dbeta) d.dbeta[l] = 2.0 * s.acc[p + l];
+    while (cur >= 0) {
+        const double v = block_sum4(db[0], dg[0], 0.0, 0.0, s.red);
+        if (threadIdx.x == 0 && d.dbeta) d.dbeta[cur] = 2.0 * v;
+        if (threadIdx.x == 1 && d.dgamma) d.dgamma[cur] = 2.0 * v;
+        db[0] = db[1]; dg[0] = dg[1];
+        db[1] = dg[1] = 0.0;
+        --cur;
     }
     __syncthreads();
 }
@@ -129,11 +157,11 @@ __host__ __device__ inline int resident_window(int n, int rb, int rmax) {
     return n < r ? n : r;
 }
 
-template <typename T, int R, int RA>
-__device__ void run_instance(const InstDesc<T>& d, unsigned char* sm) {
+template <typename T, int R, int RA, bool GRAD>
+__device__ void run_instance(const InstDesc<T>& d, unsigned char* sm, const WinSched& ws) {
     using C = typename Num<T>::C;
     const int n = d.n, p = d.p;
-    const bool grad = (d.flags & F_GRAD) != 0;
+    const bool grad = GRAD && (d.flags & F_GRAD) != 0;
     size_t off[12];
     smem_layout<T>(n, p, grad, blockDim.x, off);
     Smem<T> s;
@@ -143,7 +171,6 @@ __device__ void run_instance(const InstDesc<T>& d, unsigned char* sm) {
     s.Q = reinterpret_cast<T*>(sm + off[3]);
     s.lc = reinterpret_cast<LayerConst<T>*>(sm + off[4]);
     s.red = reinterpret_cast<double*>(sm + off[5]);
-    s.acc = reinterpret_cast<double*>(sm + off[6]);
     s.tk.wlists = reinterpret_cast<TopEnt*>(sm + off[7]);
     s.tk.cand = reinterpret_cast<TopEnt*>(sm + off[8]);
     s.tk.out = reinterpret_cast<TopEnt*>(sm + off[9]);
@@ -152,7 +179,8 @@ __device__ void run_instance(const InstDesc<T>& d, unsigned char* sm) {
     s.escr = reinterpret_cast<T*>(sm + off[11]);
     const uint32_t D = 1u << n;
 
-    set_layer_consts<T>(s.lc, d.gamma, d.beta, p, n, true);
+    static_assert(sizeof(FwdConst<T>) <= sizeof(LayerConst<T>), "the forward constants share the adjoint's place");
+    set_fwd_consts(reinterpret_cast<FwdConst<T>*>(s.lc), d.gamma, d.beta, p, n);
     bool started = false;
     if (d.Q) {
         for (int i = threadIdx.x; i < n * n; i += blockDim.x) s.Q[i] = d.Q[i];
@@ -176,38 +204,42 @@ __device__ void run_instance(const InstDesc<T>& d, unsigned char* sm) {
     if (d.E_out)
         for (uint32_t z = threadIdx.x; z < D; z += blockDim.x) d.E_out[z] = s.E[swz<T>(z)];
 
-    forward_run<T, R>(d, s, started);
+    forward_run<T, R>(d, s, ws, started);
 
     if (d.psi_out) {              // back from the rotated frame: psi = (-i)^{|z|} psi~
         C* pout = reinterpret_cast<C*>(d.psi_out);
         for (uint32_t z = threadIdx.x; z < D; z += blockDim.x)
             pout[z] = times_i_pow(s.psi[swz<T>(z)], -__popc(z));
     }
-    if (grad) adjoint_run<T, RA>(d, s);
+    if constexpr (GRAD) {
+        if (grad) adjoint_run<T, RA>(d, s);
+    }
 }
 
-template <typename T>
-__device__ void dispatch_instance(const InstDesc<T>& d, unsigned char* sm, int rmax) {
+template <typename T, bool GRAD>
+__device__ void dispatch_instance(const InstDesc<T>& d, unsigned char* sm, int rmax, const WinSched& ws) {
     constexpr int RBF = Num<T>::RB, RBA = Num<T>::RB_ADJ;
     // register windows: RB (forward, or rmax when the launch asks for narrower ones) and RB_ADJ
     // (adjoint) qubits, fewer when n is smaller
     const int rf = resident_window(d.n, RBF, rmax), ra = min(d.n, RBA);
-    if (rf == RBF && ra == RBA) run_instance<T, RBF, RBA>(d, sm);
-    else if (rf == 4 && ra == 4) run_instance<T, 4, 4>(d, sm);
-    else if (rf == 3) run_instance<T, 3, 3>(d, sm);
-    else if (rf == 2) run_instance<T, 2, 2>(d, sm);
-    else run_instance<T, 1, 1>(d, sm);
+    if (rf == RBF && ra == RBA) run_instance<T, RBF, RBA, GRAD>(d, sm, ws);
+    else if (rf == 4 && ra == 4) run_instance<T, 4, 4, GRAD>(d, sm, ws);
+    else if (rf == 3) run_instance<T, 3, 3, GRAD>(d, sm, ws);
+    else if (rf == 2) run_instance<T, 2, 2, GRAD>(d, sm, ws);
+    else run_instance<T, 1, 1, GRAD>(d, sm, ws);
 }
 
 // Persistent walk over `count` descriptors (queue: device counter zeroed before the launch);
 // with desc == nullptr the single instance `one` (passed by value) is run by block 0.
-template <typename T>
+// GRAD: a kernel of its own with the adjoint sweep, so that forward launches do not carry its
+// registers and code.
+template <typename T, bool GRAD>
 __global__ void __launch_bounds__(512) k_resident(const InstDesc<T>* __restrict__ desc, int count,
-                                                  int* queue, const InstDesc<T> one, int rmax) {
+                                                  int* queue, const InstDesc<T> one, int rmax, const WinSched ws) {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ int s_next;
     if (desc == nullptr) {
-        if (blockIdx.x == 0) dispatch_instance<T>(one, sm, rmax);
+        if (blockIdx.x == 0) dispatch_instance<T, GRAD>(one, sm, rmax, ws);
         return;
     }
     for (;;) {
@@ -217,7 +249,7 @@ __global__ void __launch_bounds__(512) k_resident(const InstDesc<T>* __restrict_
         __syncthreads();
         if (ii >= count) break;
         const InstDesc<T> d = desc[ii];
-        dispatch_instance<T>(d, sm, rmax);
+        dispatch_instance<T, GRAD>(d, sm, rmax, ws);
         __syncthreads();
     }
 }
@@ -242,37 +274,34 @@ int resident_max_blocks_per_sm(bool dbl, int n, int pmax, bool grad, int rmax) {
     const size_t sm = resident_smem_bytes(dbl, n, pmax, grad, rmax);
     // the occupancy query counts a block that needs more than 48 KB of dynamic shared memory only
     // once the kernel may use that much, so the limit is raised first (the launch sets it again)
-    if (dbl) {
-        if (cudaFuncSetAttribute(k_resident<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_resident<double>, th, sm) != cudaSuccess)
+    const auto query = [&](auto kern) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, th, sm) != cudaSuccess)
             nb = 0;
-    } else {
-        if (cudaFuncSetAttribute(k_resident<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_resident<float>, th, sm) != cudaSuccess)
-            nb = 0;
-    }
+    };
+    if (dbl) { if (grad) query(k_resident<double, true>); else query(k_resident<double, false>); }
+    else { if (grad) query(k_resident<float, true>); else query(k_resident<float, false>); }
     return nb;
 }
 
 cudaError_t launch_resident(bool dbl, const void* desc, int count, int n, int pmax, bool grad,
-                            int* queue, int grid, cudaStream_t st, const void* one, int rmax) {
+                            int* queue, int grid, cudaStream_t st, const void* one, int rmax, bool block5) {
     const int th = resident_threads(dbl, n, rmax);
     const size_t sm = resident_smem_bytes(dbl, n, pmax, grad, rmax);
-    cudaError_t e;
-    if (dbl) {
-        e = cudaFuncSetAttribute(k_resident<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const int R = resident_window(n, dbl ? Num<double>::RB : Num<float>::RB, rmax);
+    // the qubit order of blocks of the window itself, or of 5 qubits for narrower windows of a
+    // single complex64 instance
+    const WinSched ws = win_sched(n, block5 ? Num<float>::RB : R, R);
+    const auto go = [&](auto kern, auto inst) -> cudaError_t {
+        using D = decltype(inst);
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
-        InstDesc<double> o{};
-        if (one) o = *static_cast<const InstDesc<double>*>(one);
-        k_resident<double><<<grid, th, sm, st>>>(static_cast<const InstDesc<double>*>(desc), count, queue, o, rmax);
-    } else {
-        e = cudaFuncSetAttribute(k_resident<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        InstDesc<float> o{};
-        if (one) o = *static_cast<const InstDesc<float>*>(one);
-        k_resident<float><<<grid, th, sm, st>>>(static_cast<const InstDesc<float>*>(desc), count, queue, o, rmax);
-    }
-    return cudaGetLastError();
+        if (one) inst = *static_cast<const D*>(one);
+        kern<<<grid, th, sm, st>>>(static_cast<const D*>(desc), count, queue, inst, rmax, ws);
+        return cudaGetLastError();
+    };
+    if (dbl) return grad ? go(k_resident<double, true>, InstDesc<double>{}) : go(k_resident<double, false>, InstDesc<double>{});
+    return grad ? go(k_resident<float, true>, InstDesc<float>{}) : go(k_resident<float, false>, InstDesc<float>{});
 }
 
 }  // namespace qaoa

@@ -35,6 +35,7 @@ __device__ __forceinline__ uint64_t global_index(const StreamPass& P, uint64_t t
 // B, any for kind A) has global index global_index(P, tau, u0) + j * gstep. Returns false when
 // kind B's contiguous run is longer than the step (then the index is formed per element).
 __device__ __forceinline__ bool linear_walk(const StreamPass& P, uint32_t step, uint64_t& gstep) {
+    if (step < 512u) return false;   // the swizzle permutes bits 1..8: a shorter stride would not advance linearly
     if (P.kind == 0) { gstep = step; return true; }
     if (step & ((1u << P.c) - 1u)) return false;
     gstep = (uint64_t)(step >> P.c) << P.s;
@@ -102,40 +103,53 @@ template <typename T>
 struct StreamSmem {
     typename Num<T>::C* psi;
     T* E;
-    LayerConst<T>* lc;
+    FwdConst<T>* lc;
     double* red;
     TileTopk tk;
     TopEnt* run;     // running top-k of the state's tiles this block reduced (last pass)
 };
 
-// have_run: this block reduced tile prev_tau of the same state just before (last pass, k >= 1);
-// s.run then holds the top-k of all the state's tiles it reduced so far.
-template <typename T, int R>
+// The tile's copies HBM -> shared: asynchronous, all in flight before the wait in stream_tile
+// (tile bit 0 is global bit 0 and c >= 1, so aligned pairs stay adjacent in both layouts).
+template <typename T>
+__device__ __forceinline__ void stream_stage(const StreamPass& P, const StreamInst<T>& I, uint64_t tau,
+                                             const StreamSmem<T>& s) {
+    using C = typename Num<T>::C;
+    if (!P.init) stage_tile<T>(P, tau, reinterpret_cast<C*>(I.psi), s.psi, P.need_e ? I.E : nullptr, s.E);
+    else if (P.need_e) stage_tile<T>(P, tau, nullptr, nullptr, I.E, s.E);
+}
+
+// One staged tile. have_run: this block reduced tile prev_tau of the same state just before (last
+// pass, k >= 1); s.run then holds the top-k of all the state's tiles it reduced so far. TOPK:
+// the instantiation serves passes with a top-k.
+template <typename T, int R, bool TOPK>
 __device__ void stream_tile(const StreamPass& P, const StreamInst<T>& I, uint64_t tau,
                             const StreamSmem<T>& s, bool have_run, uint64_t prev_tau) {
     using C = typename Num<T>::C;
     const uint32_t TD = 1u << P.tb;
-    const bool needE = P.need_e;
     C* gpsi = reinterpret_cast<C*>(I.psi);
-    // ---- HBM -> shared: asynchronous 16-byte copies, all in flight before the wait ----
-    // (tile bit 0 is global bit 0 and c >= 1, so aligned pairs stay adjacent in both layouts)
-    if (!P.init) stage_tile<T>(P, tau, gpsi, s.psi, needE ? I.E : nullptr, s.E);
-    else if (needE) stage_tile<T>(P, tau, nullptr, nullptr, I.E, s.E);
     cp_async_wait_all();
     __syncthreads();
     // ---- tile engine: snake over the local windows of the mixed bits, layers [la, lb] ----
     const TileRef<T> tile{s.psi, nullptr, s.E, P.tb};
     const int m0 = (P.kind == 0) ? 0 : P.c;
-    const int G = num_windows(m0, P.tb, R);
-    const int nl = P.lb - P.la + 1;
-    const int S = snake_len(G, nl);
     const T amp0 = (T)I.amp0;
-    for (int si = 0; si < S; ++si) {
-        SubPass sp;
-        snake_step(si, G, nl, P.la, P.ph_first, m0, P.tb, P.tb, R, sp);
-        sp.post = P.fin && (si == S - 1);
-        subpass_fwd<T, R>(tile, sp, s.lc, P.init && si == 0, amp0, __popcll(tau));
-        __syncthreads();
+    if (P.nsub > 0) {              // listed sub-passes (a single state's small tiles)
+        for (int i = 0; i < P.nsub; ++i) {
+            const StreamSub& b = P.sub[i];
+            SubPass sp{b.a, b.mask, P.la + b.l0, P.la + b.l1, b.phase, P.fin && i == P.nsub - 1};
+            subpass_fwd<T, R>(tile, sp, s.lc, P.init && i == 0, amp0, __popcll(tau));
+            __syncthreads();
+        }
+    } else {
+        Snake sn(P.lb - P.la + 1, P.la, P.ph_first, m0, P.tb, P.tb, R);
+        for (;; sn.next()) {
+            SubPass sp = sn.get();
+            sp.post = P.fin && sn.last();
+            subpass_fwd<T, R>(tile, sp, s.lc, P.init && sn.first(), amp0, __popcll(tau));
+            __syncthreads();
+            if (sn.last()) break;
+        }
     }
     // ---- shared -> HBM (16-byte accesses on both sides). Between passes the state stays in
     // the rotated frame; the last pass converts back with (-i)^{|z|} (|z| = |tau| + |u|: the
@@ -164,7 +178,14 @@ __device__ void stream_tile(const StreamPass& P, const StreamInst<T>& I, uint64_
                 gpsi[global_index(P, tau, u)] = times_i_pow(s.psi[swz<T>(u)], -(pt + __popc(u)));
         }
     }
-    if (P.fin) {
+    if (P.fin && !TOPK) {
+        if (I.expect) {                        // <C> alone, and only where somebody reads it
+            double ex = 0.0;
+            tile_expect<T>(tile, ex);
+            const double tot = block_sum(ex, s.red);
+            if (threadIdx.x == 0) I.part_expect[tau] = tot;
+        }
+    } else if (P.fin) {
         double ex = 0.0;
         const StreamPass Pm = P;   // by value: the lambda then holds no address of a kernel parameter
         const auto zmap = [Pm, tau](uint32_t u) { return (uint32_t)global_index(Pm, tau, u); };
@@ -194,8 +215,8 @@ __device__ void stream_tile(const StreamPass& P, const StreamInst<T>& I, uint64_
     __syncthreads();
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256, 2) k_stream_pass(const StreamPass P,
+template <typename T, int R, int NTH, bool TOPK>
+__global__ void __launch_bounds__(NTH, 2) k_stream_pass(const StreamPass P,
                                                      const StreamInst<T>* __restrict__ insts,
                                                      int count, const StreamInst<T> one) {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -205,7 +226,7 @@ __global__ void __launch_bounds__(256, 2) k_stream_pass(const StreamPass P,
     size_t o = 0;
     s.psi = reinterpret_cast<C*>(sm + o); o += (size_t)TD * sizeof(C);
     s.E = reinterpret_cast<T*>(sm + o); o += (size_t)TD * sizeof(T);
-    s.lc = reinterpret_cast<LayerConst<T>*>(sm + o); o += 64 * sizeof(LayerConst<T>);
+    s.lc = reinterpret_cast<FwdConst<T>*>(sm + o); o += 64 * sizeof(LayerConst<T>);
     o = (o + 15) & ~(size_t)15;
     s.red = reinterpret_cast<double*>(sm + o); o += 32 * sizeof(double);
     s.tk.wlists = reinterpret_cast<TopEnt*>(sm + o); o += 8 * 32 * sizeof(TopEnt);
@@ -234,19 +255,17 @@ __global__ void __launch_bounds__(256, 2) k_stream_pass(const StreamPass P,
     int run_ii = -1;
     uint64_t run_tau = 0;
     for (; b < bend; b += bstep) {
-        const int ii = (int)(b / ntiles);
-        const uint64_t tau = b % ntiles;
+        const int ii = (int)(b >> (P.n - P.tb));
+        const uint64_t tau = b & (ntiles - 1);
         const StreamInst<T>& I = insts ? insts[ii] : one;
+        stream_stage<T>(P, I, tau, s);   // the copies run while the constants are formed
         if (I.gamma != cur_g || I.beta != cur_b || I.p != cur_p) {
-            __syncthreads();
-            set_layer_consts<T>(s.lc, I.gamma, I.beta, I.p, P.n, true);
-            __syncthreads();
+            set_fwd_consts(s.lc, I.gamma, I.beta, I.p, P.n);
             cur_g = I.gamma;
             cur_b = I.beta;
             cur_p = I.p;
         }
-        constexpr int RB = Num<T>::RB;
-        stream_tile<T, RB>(P, I, tau, s, run_ii == ii, run_tau);
+        stream_tile<T, R, TOPK>(P, I, tau, s, run_ii == ii, run_tau);
         run_ii = ii;
         run_tau = tau;
     }
@@ -323,43 +342,29 @@ constexpr int ADJ_THREADS = 256;
 template <typename T, int RA>
 __device__ void stream_adj_tile(const StreamPass& P, int si, bool lam_first, bool store,
                                 const StreamInst<T>& I, uint64_t tau, const StreamSmem<T>& s,
-                                typename Num<T>::C* slam) {
+                                typename Num<T>::C* slam, const LayerConst<T>* lc) {
     using C = typename Num<T>::C;
     C* gpsi = reinterpret_cast<C*>(I.psi);
     C* glam = reinterpret_cast<C*>(I.lam);
-    stage_tile<T>(P, tau, gpsi, s.psi, I.E, s.E);
-    if (!lam_first) stage_tile<T>(P, tau, glam, slam, nullptr, nullptr);
     cp_async_wait_all();
     __syncthreads();
     const TileRef<T> tile{s.psi, slam, s.E, P.tb};
     const int m0 = (P.kind == 0) ? 0 : P.c;
-    const int G = num_windows(m0, P.tb, RA);
-    const int nl = P.lb - P.la + 1;
-    const int S = snake_len(G, nl);
-    // tile accumulators by the pass's layer slot (0: layer lb, 1: layer la); a local
-    // sub-pass reports relative to its own last layer, mapped here
-    T ab[2] = {T(0), T(0)}, ag[2] = {T(0), T(0)};
-    for (int k = S - 1; k >= 0; --k) {
-        SubPass sp;
-        snake_step(k, G, nl, P.la, P.ph_first, m0, P.tb, P.tb, RA, sp);
-        T lb_[2] = {T(0), T(0)}, lg_[2] = {T(0), T(0)};
-        subpass_adj<T, RA>(tile, sp, s.lc, lam_first && k == S - 1, lb_, lg_);
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int slot = P.lb - (sp.lb - j);
-            if (j <= sp.lb - sp.la) {
-                if (slot == 0) { ab[0] += lb_[j]; ag[0] += lg_[j]; }
-                else { ab[1] += lb_[j]; ag[1] += lg_[j]; }
-            }
-        }
+    Snake sn(P.lb - P.la + 1, P.la, P.ph_first, m0, P.tb, P.tb, RA);
+    sn.to_last();
+    bool first = lam_first;
+    // tile accumulators by the pass's layer slot (0: layer lb, 1: layer la)
+    T acc[4] = {T(0), T(0), T(0), T(0)};
+    for (;; sn.prev()) {
+        const SubPass sp = sn.get();
+        subpass_adj<T, RA>(tile, sp, lc, first, P.lb, acc);
+        first = false;
         __syncthreads();
+        if (sn.first()) break;
     }
     double* out = I.part_grad + ((uint64_t)si << (P.n - P.tb)) * 4 + tau * 4;
-    const double v0 = block_sum((double)ab[0], s.red);
-    const double v1 = block_sum((double)ab[1], s.red);
-    const double v2 = block_sum((double)ag[0], s.red);
-    const double v3 = block_sum((double)ag[1], s.red);
-    if (threadIdx.x == 0) { out[0] = v0; out[1] = v1; out[2] = v2; out[3] = v3; }
+    const double v = block_sum4((double)acc[0], (double)acc[1], (double)acc[2], (double)acc[3], s.red);
+    if (threadIdx.x < 4) out[threadIdx.x] = v;
     if (store) {
         store_tile<T>(P, tau, s.psi, gpsi);
         store_tile<T>(P, tau, slam, glam);
@@ -367,8 +372,8 @@ __device__ void stream_adj_tile(const StreamPass& P, int si, bool lam_first, boo
     __syncthreads();
 }
 
-template <typename T>
-__global__ void __launch_bounds__(ADJ_THREADS, 2) k_stream_adj_pass(const StreamPass P, int si, int lam_first,
+template <typename T, int RA, int NTH>
+__global__ void __launch_bounds__(NTH, 2) k_stream_adj_pass(const StreamPass P, int si, int lam_first,
                                                          int store,
                                                          const StreamInst<T>* __restrict__ insts,
                                                          int count, const StreamInst<T> one) {
@@ -380,31 +385,32 @@ __global__ void __launch_bounds__(ADJ_THREADS, 2) k_stream_adj_pass(const Stream
     s.psi = reinterpret_cast<C*>(sm + o); o += (size_t)TD * sizeof(C);
     C* slam = reinterpret_cast<C*>(sm + o); o += (size_t)TD * sizeof(C);
     s.E = reinterpret_cast<T*>(sm + o); o += (size_t)TD * sizeof(T);
-    s.lc = reinterpret_cast<LayerConst<T>*>(sm + o); o += 64 * sizeof(LayerConst<T>);
+    LayerConst<T>* lc = reinterpret_cast<LayerConst<T>*>(sm + o); o += 64 * sizeof(LayerConst<T>);
     o = (o + 15) & ~(size_t)15;
-    s.red = reinterpret_cast<double*>(sm + o);
+    s.red = reinterpret_cast<double*>(sm + o);   // 64 doubles
     const uint64_t ntiles = 1ull << (P.n - P.tb);
     const uint64_t total = ntiles * (uint64_t)count;
     const T *cur_g = nullptr, *cur_b = nullptr;
     int cur_p = 0;
     for (uint64_t b = blockIdx.x; b < total; b += gridDim.x) {
-        const int ii = (int)(b / ntiles);
-        const uint64_t tau = b % ntiles;
+        const int ii = (int)(b >> (P.n - P.tb));
+        const uint64_t tau = b & (ntiles - 1);
         const StreamInst<T>& I = insts ? insts[ii] : one;
+        stage_tile<T>(P, tau, reinterpret_cast<C*>(I.psi), s.psi, I.E, s.E);
+        if (!lam_first) stage_tile<T>(P, tau, reinterpret_cast<C*>(I.lam), slam, nullptr, nullptr);
         if (I.gamma != cur_g || I.beta != cur_b || I.p != cur_p) {
-            __syncthreads();
-            set_layer_consts<T>(s.lc, I.gamma, I.beta, I.p, P.n, false);
+            set_layer_consts<T>(lc, I.gamma, I.beta, I.p, P.n, true);
             cur_g = I.gamma;
             cur_b = I.beta;
             cur_p = I.p;
         }
-        constexpr int RA = Num<T>::RB_ADJ;
-        stream_adj_tile<T, RA>(P, si, lam_first != 0, store != 0, I, tau, s, slam);
+        stream_adj_tile<T, RA>(P, si, lam_first != 0, store != 0, I, tau, s, slam, lc);
     }
 }
 
-// Per instance: dgamma_l = 2 sum of the gamma slots of layer l, dbeta_l = 2 sum of the beta
-// slots, over passes in order and tiles in fixed contiguous chunks per thread.
+// Block (i, l): dgamma_l = 2 sum of the gamma slots of layer l of instance i, dbeta_l = 2 sum of the
+// beta slots, over passes in order and tiles in fixed contiguous chunks per thread. (One block per
+// instance, its layers one after the other: 15 us at n = 20, p = 4; a layer per block: 6 us.)
 struct PassLayers {
     int la[256], lb[256];
 };
@@ -418,7 +424,8 @@ __global__ void __launch_bounds__(256) k_stream_grad_reduce(const PassLayers pl,
     if (ii >= count) return;
     const StreamInst<T>& I = insts ? insts[ii] : one;
     const uint64_t per = (ntiles + blockDim.x - 1) / blockDim.x;
-    for (int l = 0; l < I.p; ++l) {
+    const int l = blockIdx.y;
+    if (l < I.p) {
         double gb = 0.0, gg = 0.0;
         for (int s = 0; s < S; ++s) {
             const bool hb = pl.lb[s] == l, ha = pl.la[s] == l && pl.lb[s] != pl.la[s];
@@ -430,12 +437,9 @@ __global__ void __launch_bounds__(256) k_stream_grad_reduce(const PassLayers pl,
                 if (ha) { gb += q[1]; gg += q[3]; }
             }
         }
-        const double sb = block_sum(gb, red);
-        const double sg = block_sum(gg, red);
-        if (threadIdx.x == 0) {
-            if (I.dbeta) I.dbeta[l] = 2.0 * sb;
-            if (I.dgamma) I.dgamma[l] = 2.0 * sg;
-        }
+        const double v = block_sum4(gb, gg, 0.0, 0.0, red);
+        if (threadIdx.x == 0 && I.dbeta) I.dbeta[l] = 2.0 * v;
+        if (threadIdx.x == 1 && I.dgamma) I.dgamma[l] = 2.0 * v;
     }
 }
 
@@ -549,56 +553,164 @@ __global__ void __launch_bounds__(256) k_energy_rows(int n, int nh, const T* __r
     }
 }
 
-// ---- energy build into HBM --------------------------------------------------------------
-// Thread t of 2^m fixes the low m bits of z and walks the high n - m bits in Gray-code order
-// (same increment rule as the resident tier); every step writes one coalesced row of E.
-// blockIdx.y selects the instance when insts != nullptr (then Q and E come from it).
+// ---- energy build into HBM, direct form ---------------------------------------------------
+// The row form without a walk (nh = 0: a single instance of up to 20 qubits), the same additions in
+// the same order: E is what qaoa_build_energies has always returned, and what states and shots
+// follow from. Bits 2..9 belong to the thread, the bits above to the block, so the loops over the
+// block's set bits are uniform and the thread's bits act as masks on unrolled additions, where
+// the row form tests every pair of bits (n = 19: 9.4 -> 6.8 us).
+__device__ __forceinline__ float keep(float x, uint32_t m) { return __uint_as_float(__float_as_uint(x) & m); }
+__device__ __forceinline__ double keep(double x, uint32_t m) { return m ? x : 0.0; }
+
 template <typename T>
-__global__ void __launch_bounds__(256) k_energy(int n, int m, const T* __restrict__ Q,
-                                                T* __restrict__ E, const StreamInst<T>* insts) {
-    __shared__ T Qs[32 * 32];
+__global__ void __launch_bounds__(256) k_energy_direct(int n, const T* __restrict__ Q, T* __restrict__ E) {
+    __shared__ T W[32 * 32];      // zero beyond n
+    for (int x = threadIdx.x; x < 32 * 32; x += blockDim.x) {
+        const int i = x >> 5, j = x & 31;
+        T w = T(0);
+        if (i < n && j < n) w = (i == j) ? Q[i * n + i] : Q[i * n + j] + Q[j * n + i];
+        W[x] = w;
+    }
+    __syncthreads();
+    uint32_t m[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) m[i] = 0u - ((threadIdx.x >> i) & 1u);
+    T eb = T(0), f0 = W[0], f1 = W[33];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const T* row = W + (2 + i) * 32;
+        T r = row[2 + i];
+#pragma unroll
+        for (int j = 0; j < i; ++j) r += keep(row[2 + j], m[j]);
+        eb += keep(r, m[i]);
+        f0 += keep(row[0], m[i]);
+        f1 += keep(row[1], m[i]);
+    }
+    const uint32_t hi = blockIdx.x;
+    for (uint32_t b = hi; b; b &= b - 1u) {
+        const int i = 10 + __ffs((int)b) - 1;
+        const T* row = W + i * 32;
+        T r = row[i];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) r += keep(row[2 + j], m[j]);
+        for (uint32_t d = hi & ((b & (0u - b)) - 1u); d; d &= d - 1u) r += row[10 + __ffs((int)d) - 1];
+        eb += r;
+        f0 += row[0];
+        f1 += row[1];
+    }
+    T* dst = E + (((uint64_t)hi << 10) | ((uint64_t)threadIdx.x << 2));
+    const T e0 = eb, e1 = eb + f0, e2 = eb + f1, e3 = eb + f0 + f1 + W[1];
+    if constexpr (sizeof(T) == 4) {       // E is 8-byte aligned
+        reinterpret_cast<float2*>(dst)[0] = make_float2(e0, e1);
+        reinterpret_cast<float2*>(dst)[1] = make_float2(e2, e3);
+    } else {
+        dst[0] = e0; dst[1] = e1; dst[2] = e2; dst[3] = e3;
+    }
+}
+
+// ---- energy build into HBM, tile form ----------------------------------------------------
+// A block builds the 2^11 energies of one value hi of the bits above 11 (all 2^n for n < 11). With
+// W_ij = Q_ij + Q_ji and S the set bits of hi,
+//   E(z) = E_S + sum_{i in lo} d_i + sum_{i<k in lo} W_ik,   d_i = Q_ii + sum_{s in S} W_is,
+// the block's d_i and E_S are summed by warps (a lane per bit of hi), a thread adds the terms
+// of its low eight bits once and forms its eight energies by subset doubling over bits 8..10,
+// against a sum over all bit pairs per energy quadruple in the row form, whose walk over hi is
+// too short to pay for its start below about 2^23 energies (n = 20 on GB300: 14.6 us in the row form, 8.4 us
+// here). The energies of
+// batched instances; single instances keep the row form's sums (k_energy_direct). Sums are
+// compensated (Acc: TwoSum, the rounding errors added separately), so that an energy is off by
+// little more than its own last rounding (relative 2-norm at n = 19: 9e-8 in the row form,
+// 2.5e-8 here): phases gamma E inherit that error. Stores are 4 (8) bytes per lane, coalesced: any
+// alignment.
+constexpr int ETB = 11;
+
+template <typename T>
+struct Acc {
+    T s, c;   // value s + c
+    __device__ __forceinline__ void add(T x) {
+        const T t = s + x, z = t - s;
+        c += (s - (t - z)) + (x - z);
+        s = t;
+    }
+    __device__ __forceinline__ void add(const Acc& o) {
+        add(o.s);
+        c += o.c;
+    }
+};
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_energy_tile(int n, const T* __restrict__ Q, T* __restrict__ E,
+                                                     const StreamInst<T>* insts) {
+    __shared__ T W[32 * 32];      // zero beyond n
+    __shared__ Acc<T> d[16];
     if (insts) {
         Q = insts[blockIdx.y].Q;
         E = const_cast<T*>(insts[blockIdx.y].E);
     }
-    for (int i = threadIdx.x; i < n * n; i += blockDim.x) Qs[i] = Q[i];
+#pragma unroll
+    for (int x = threadIdx.x; x < 32 * 32; x += 256) {
+        const int i = x >> 5, j = x & 31;
+        T w = T(0);
+        if (i < n && j < n) w = (i == j) ? Q[i * n + i] : Q[i * n + j] + Q[j * n + i];
+        W[x] = w;
+    }
+    const uint32_t hi = blockIdx.x;
+    const int nhi = n > ETB ? n - ETB : 0, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __syncthreads();
-    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (1ull << m)) return;
-    const int nh = n - m;
-    T e = T(0);
-    for (int i = 0; i < m; ++i) {
-        if (!((t >> i) & 1u)) continue;
-        for (int j = 0; j < m; ++j)
-            if ((t >> j) & 1u) e += Qs[i * n + j];
+    const bool on = lane < nhi && ((hi >> lane) & 1u);
+    for (int b = warp; b <= ETB; b += 8) {          // d_0 .. d_10, and E_S as entry 11
+        Acc<T> v{T(0), T(0)};
+        if (b < ETB) {
+            if (on) v.s = W[b * 32 + ETB + lane];
+        } else if (on) {
+            const T* row = W + (ETB + lane) * 32 + ETB;
+            v.s = row[lane];
+            for (int s = 0; s < lane; ++s)
+                if ((hi >> s) & 1u) v.add(row[s]);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const Acc<T> w{__shfl_xor_sync(0xffffffffu, v.s, o), __shfl_xor_sync(0xffffffffu, v.c, o)};
+            v.add(w);
+        }
+        if (b < ETB) v.add(W[b * 32 + b]);
+        if (lane == 0) d[b] = v;
     }
-    constexpr int MAXH = 12;
-    T F[MAXH];
+    __syncthreads();
+    const uint32_t t = threadIdx.x;
+    T f[8];
 #pragma unroll
-    for (int h = 0; h < MAXH; ++h) {
-        T f = T(0);
-        if (h < nh)
-            for (int j = 0; j < m; ++j)
-                if ((t >> j) & 1u) f += Qs[(m + h) * n + j];
-        F[h] = f;
+    for (int i = 0; i < 8; ++i) f[i] = T((t >> i) & 1u);
+    Acc<T> base = d[ETB], w8[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) w8[b] = d[8 + b];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const Acc<T> di = d[i];
+        base.add(f[i] * di.s);
+        base.c = fma(f[i], di.c, base.c);
+#pragma unroll
+        for (int k = i + 1; k < 8; ++k) base.add(f[i] * f[k] * W[i * 32 + k]);
+#pragma unroll
+        for (int b = 0; b < 3; ++b) w8[b].add(f[i] * W[i * 32 + 8 + b]);
     }
-    uint64_t z = t;
-    E[z] = e;
-    const uint32_t steps = 1u << nh;
-    for (uint32_t k = 1; k < steps; ++k) {
-        const int b = __ffs((int)k) - 1;
-        const int hb = m + b;
-        const T d = ((z >> hb) & 1ull) ? T(-1) : T(1);
-        T fb = T(0);
+    const T w01 = W[8 * 32 + 9], w02 = W[8 * 32 + 10], w12 = W[9 * 32 + 10];
+    Acc<T> x[8];
+    x[0] = base;
 #pragma unroll
-        for (int h = 0; h < MAXH; ++h)
-            if (h == b) fb = F[h];
-        e += d * (Qs[hb * n + hb] + T(2) * fb);
-        z ^= 1ull << hb;
+    for (int j = 1; j < 8; ++j) {
+        const int top = j >= 4 ? 2 : (j >= 2 ? 1 : 0);   // x[j] from x[j without its top bit]
+        x[j] = x[j ^ (1 << top)];
+        x[j].add(w8[top]);
+        if (top == 1 && (j & 1)) x[j].add(w01);
+        if (top == 2 && (j & 1)) x[j].add(w02);
+        if (top == 2 && (j & 2)) x[j].add(w12);
+    }
+    const uint64_t z0 = ((uint64_t)hi << ETB) | t;
 #pragma unroll
-        for (int h = 0; h < MAXH; ++h)
-            if (h < nh && h != b) F[h] += d * Qs[(m + h) * n + hb];
-        E[z] = e;
+    for (int j = 0; j < 8; ++j) {
+        const uint64_t z = z0 + ((uint64_t)j << 8);
+        if (n >= ETB || z < (1ull << n)) E[z] = x[j].s + x[j].c;
     }
 }
 
@@ -608,15 +720,87 @@ __global__ void __launch_bounds__(256) k_energy(int n, int m, const T* __restric
 // host side
 // ---------------------------------------------------------------------------------------------
 
+// Passes of a single complex64 state of 15..21 qubits. With the batched tiles (2^13 forward, 2^12
+// adjoint) such a state is a few dozen tiles, one per CTA and pass, and a pass lasts as long as
+// one tile does on a CTA of 256 threads that runs a thousand unrolled instructions once.
+//   qaoa_run_layers: qubits 0..12 in the batched tiles, qubits 13..n-1 in tiles of 2^10 or 2^11
+//   amplitudes (runs of at least 8), eight amplitudes per thread, the windows of a pass listed on
+//   the host so that the qubit order stays that of 5-qubit windows over 0..12 and 13..n-1 (see
+//   FwdConst: shots are drawn from these states, and that order is why the contiguous tiles
+//   keep 13 qubits; 1024 threads on one of them took as long as 256).
+//   qaoa_grad (whose states stay inside): tb = (n + 4) / 2 bits forward and adjoint, runs of at
+//   least 8 amplitudes, 16 amplitudes per thread.
+// GB300: qaoa_run_layers at n = 19, p = 3, passes of 22 to 29 us -> 14 to 18 (qubits 0..12) and 8 to
+// 10 us; qaoa_grad at n = 20, p = 4, forward passes 23 to 32 -> 10 to 15 us.
+constexpr int SMALL_R = 3, SMALL_NMIN = 15, SMALL_NMAX = 21, SMALL_LOW = 13, SMALL_RA = 4;
+static bool small_tiles(bool dbl, int n, int tb) { return !dbl && n >= 14 && n <= SMALL_NMAX && tb == (n + 4) / 2; }
+
 int stream_tile_bits(bool dbl) { return dbl ? 12 : 13; }
 int stream_adj_tile_bits(bool dbl) { return dbl ? 11 : 12; }
+int stream_one_grad_tile_bits(bool dbl, int n, bool adjoint) {
+    if (!dbl && n >= 14 && n <= SMALL_NMAX) return (n + 4) / 2;
+    return adjoint ? stream_adj_tile_bits(dbl) : stream_tile_bits(dbl);
+}
+uint64_t stream_one_max_tiles(bool dbl, int n) {
+    if (!dbl && n >= SMALL_NMIN && n <= SMALL_NMAX) return 1ull << (n - 10);
+    return n > stream_tile_bits(dbl) ? 1ull << (n - stream_tile_bits(dbl)) : 0;
+}
+
+// The forward passes of a single state (see above); other sizes and types: the batched plan.
+int stream_plan_one(bool dbl, int n, int p, int k, StreamPass* out, int max_out) {
+    if (dbl || n < SMALL_NMIN || n > SMALL_NMAX || k > 0) return stream_plan(dbl, n, p, k, out, max_out);
+    if (p + 1 > max_out) return -1;
+    // blocks of qubits, each cut into windows of at most SMALL_R
+    struct Blk { int q, size; };
+    Blk up[2];
+    int nu = 0;
+    for (int q = SMALL_LOW; q < n; q += 5) up[nu++] = Blk{q, n - q < 5 ? n - q : 5};
+    const int tbA = SMALL_LOW, h = n - SMALL_LOW, tbB = n < 19 ? 10 : 11, c = tbB - h;
+    for (int si = 0; si <= p; ++si) {
+        StreamPass P{};
+        P.n = n;
+        P.la = si > 0 ? si - 1 : 0;
+        P.lb = si < p ? si : p - 1;
+        if (si == 0) P.lb = 0;
+        P.init = P.ph_first = si == 0 ? 1 : 0;
+        P.fin = si == p ? 1 : 0;
+        const bool lower = (si & 1) == 0;
+        P.kind = lower ? 0 : 1;
+        P.tb = lower ? tbA : tbB;
+        P.c = lower ? tbA : c;
+        P.s = lower ? tbA : SMALL_LOW;
+        P.h = lower ? 0 : h;
+        P.need_e = (P.ph_first || P.lb > P.la || P.fin) ? 1 : 0;
+        const int shift = c - SMALL_LOW;                  // tile bit of qubit q: q + shift
+        for (int l = P.la; !lower && l <= P.lb; ++l)
+            for (int i = 0; i < nu; ++i) {
+                const Blk& b = up[l > P.la ? nu - 1 - i : i];
+                for (int q = b.q; q < b.q + b.size; q += SMALL_R) {
+                    const int size = b.q + b.size - q < SMALL_R ? b.q + b.size - q : SMALL_R;
+                    const int lo = q + shift, a = lo + SMALL_R <= P.tb ? lo : P.tb - SMALL_R;
+                    StreamSub sb{a, ((1 << size) - 1) << (lo - a), l - P.la, l - P.la, 0};
+                    const bool opens = i == 0 && q == b.q;
+                    sb.phase = opens && (l > P.la || P.ph_first) ? 1 : 0;
+                    if (opens && l > P.la && P.sub[P.nsub - 1].a == sb.a && P.sub[P.nsub - 1].mask == sb.mask) {
+                        P.sub[P.nsub - 1].l1 = sb.l1;      // shared around the cost phase
+                        continue;
+                    }
+                    if (P.nsub == STREAM_MAX_SUB) return -1;
+                    P.sub[P.nsub++] = sb;
+                }
+            }
+        out[si] = P;
+    }
+    return p + 1;
+}
 
 // HBM windows of a layer: window 0 = kind A (qubits 0..tb-1); windows 1.. = kind B chunks of
-// the qubits [tb, n), as equal as possible, each at most tb - 4 qubits.
+// the qubits [tb, n), as equal as possible, each at most tb - 4 qubits (tb - 3 for the small adjoint
+// tiles of a single state).
 int stream_plan(bool dbl, int n, int p, int k, StreamPass* out, int max_out, int tb) {
     if (tb < 0) tb = stream_tile_bits(dbl);
     if (n <= tb) return -1;
-    const int hmax = tb - 4;
+    const int hmax = tb - (small_tiles(dbl, n, tb) ? 3 : 4);
     const int rest = n - tb;
     const int nB = (rest + hmax - 1) / hmax;
     int chunk_s[16], chunk_h[16];
@@ -659,8 +843,8 @@ int stream_plan(bool dbl, int n, int p, int k, StreamPass* out, int max_out, int
     return S;
 }
 
-size_t stream_smem_bytes(bool dbl) {
-    const size_t TD = (size_t)1 << stream_tile_bits(dbl);
+static size_t stream_smem_bytes(bool dbl, int tb) {
+    const size_t TD = (size_t)1 << tb;
     const size_t c = dbl ? 16 : 8, r = dbl ? 8 : 4, lcs = dbl ? sizeof(LayerConst<double>) : sizeof(LayerConst<float>);
     size_t o = TD * c + TD * r + 64 * lcs;
     o = (o + 15) & ~(size_t)15;
@@ -675,20 +859,24 @@ static StreamInst<T> one_of(const void* one) {
     return o;
 }
 
+template <typename T, int R, int NTH, bool TOPK>
+static cudaError_t pass_t(const StreamPass& P, const void* insts, int count, int grid, int threads, cudaStream_t st,
+                          const void* one) {
+    const size_t sm = stream_smem_bytes(sizeof(T) == 8, P.tb);
+    const cudaError_t e = cudaFuncSetAttribute(k_stream_pass<T, R, NTH, TOPK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    k_stream_pass<T, R, NTH, TOPK><<<grid, threads, sm, st>>>(P, static_cast<const StreamInst<T>*>(insts), count, one_of<T>(one));
+    return cudaGetLastError();
+}
+
 cudaError_t launch_stream_pass(bool dbl, const StreamPass& P, const void* insts, int count,
                                int grid, cudaStream_t st, const void* one) {
-    const size_t sm = stream_smem_bytes(dbl);
-    cudaError_t e;
-    if (dbl) {
-        e = cudaFuncSetAttribute(k_stream_pass<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        k_stream_pass<double><<<grid, 256, sm, st>>>(P, static_cast<const StreamInst<double>*>(insts), count, one_of<double>(one));
-    } else {
-        e = cudaFuncSetAttribute(k_stream_pass<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        k_stream_pass<float><<<grid, 256, sm, st>>>(P, static_cast<const StreamInst<float>*>(insts), count, one_of<float>(one));
-    }
-    return cudaGetLastError();
+    if (dbl) return pass_t<double, Num<double>::RB, 256, true>(P, insts, count, grid, 256, st, one);
+    if (P.nsub > 0) return pass_t<float, SMALL_R, 256, false>(P, insts, count, grid, 1 << (P.tb - SMALL_R), st, one);
+    if (small_tiles(dbl, P.n, P.tb) && P.k == 0)
+        return pass_t<float, SMALL_RA, 256, false>(P, insts, count, grid, 1 << (P.tb - SMALL_RA), st, one);
+    if (P.k == 0) return pass_t<float, Num<float>::RB, 256, false>(P, insts, count, grid, 256, st, one);
+    return pass_t<float, Num<float>::RB, 256, true>(P, insts, count, grid, 256, st, one);
 }
 
 bool stream_finalize_two_level(uint64_t ntiles, int k) { return k > 0 && ntiles > FIN_CHUNK; }
@@ -707,15 +895,6 @@ cudaError_t launch_stream_finalize(bool dbl, const void* insts, int count, uint6
     if (dbl) k_stream_finalize<double><<<count, 256, 0, st>>>(static_cast<const StreamInst<double>*>(insts), count, ntiles, k, stride, one_of<double>(one));
     else k_stream_finalize<float><<<count, 256, 0, st>>>(static_cast<const StreamInst<float>*>(insts), count, ntiles, k, stride, one_of<float>(one));
     return cudaGetLastError();
-}
-
-static int energy_split(int n) {
-    // low bits fixed per thread: enough threads to fill the GPU, at most 2^12 Gray steps each
-    int m = n - 6;
-    if (m < 0) m = 0;
-    if (m > 20) m = 20;
-    if (n - m > 12) m = n - 12;
-    return m;
 }
 
 // Top bits walked per thread by the row form: enough threads in total (instances x 2^(n-2-nh))
@@ -746,65 +925,83 @@ static cudaError_t launch_rows(int n, int count, const void* Q, void* E, const v
     return cudaSuccess;
 }
 
-cudaError_t launch_energy(bool dbl, int n, const void* Q, void* E, cudaStream_t st) {
-    if (n >= 2 && (reinterpret_cast<uintptr_t>(E) & 7u) == 0)
-        return dbl ? launch_rows<double>(n, 1, Q, E, nullptr, st) : launch_rows<float>(n, 1, Q, E, nullptr, st);
-    const int m = energy_split(n);
-    const uint64_t threads = 1ull << m;
-    const int block = threads < 256 ? (int)threads : 256;
-    const uint64_t grid = (threads + block - 1) / block;
-    if (dbl) k_energy<double><<<(unsigned)grid, block, 0, st>>>(n, m, static_cast<const double*>(Q), static_cast<double*>(E), nullptr);
-    else k_energy<float><<<(unsigned)grid, block, 0, st>>>(n, m, static_cast<const float*>(Q), static_cast<float*>(E), nullptr);
+// Batches: tile form up to 2^22 energies per instance, row form above.
+constexpr int ENERGY_TILE_NMAX = 22;
+
+template <typename T>
+static cudaError_t launch_tiles(int n, int count, const void* Q, void* E, const void* insts, cudaStream_t st) {
+    const unsigned gx = n > ETB ? 1u << (n - ETB) : 1u;
+    const StreamInst<T>* in = static_cast<const StreamInst<T>*>(insts);
+    for (int c0 = 0; c0 < count; c0 += 65535) {          // grid.y limit
+        const int cy = count - c0 < 65535 ? count - c0 : 65535;
+        k_energy_tile<T><<<dim3(gx, (unsigned)cy), 256, 0, st>>>(n, static_cast<const T*>(Q), static_cast<T*>(E),
+                                                                 in ? in + c0 : nullptr);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+template <typename T>
+static cudaError_t launch_one(int n, const void* Q, void* E, cudaStream_t st) {
+    // one qubit, or an address the wider stores cannot take
+    if (n < 2 || (reinterpret_cast<uintptr_t>(E) & 7u) != 0) return launch_tiles<T>(n, 1, Q, E, nullptr, st);
+    if (rows_nh(n, 1) > 0) return launch_rows<T>(n, 1, Q, E, nullptr, st);
+    const unsigned blocks = n > 10 ? 1u << (n - 10) : 1u, threads = n > 10 ? 256u : 1u << (n - 2);
+    k_energy_direct<T><<<blocks, threads, 0, st>>>(n, static_cast<const T*>(Q), static_cast<T*>(E));
     return cudaGetLastError();
+}
+
+cudaError_t launch_energy(bool dbl, int n, const void* Q, void* E, cudaStream_t st) {
+    return dbl ? launch_one<double>(n, Q, E, st) : launch_one<float>(n, Q, E, st);
 }
 
 cudaError_t launch_energy_batch(bool dbl, int n, const void* insts, int count, cudaStream_t st) {
     // every instance's E is at least 8-byte aligned (plan validation)
-    if (n >= 2)
-        return dbl ? launch_rows<double>(n, count, nullptr, nullptr, insts, st)
-                   : launch_rows<float>(n, count, nullptr, nullptr, insts, st);
-    const int m = energy_split(n);
-    const uint64_t threads = 1ull << m;
-    const int block = threads < 256 ? (int)threads : 256;
-    const dim3 grid((unsigned)((threads + block - 1) / block), (unsigned)count);
-    if (dbl) k_energy<double><<<grid, block, 0, st>>>(n, m, nullptr, nullptr, static_cast<const StreamInst<double>*>(insts));
-    else k_energy<float><<<grid, block, 0, st>>>(n, m, nullptr, nullptr, static_cast<const StreamInst<float>*>(insts));
-    return cudaGetLastError();
+    if (n <= ENERGY_TILE_NMAX)
+        return dbl ? launch_tiles<double>(n, count, nullptr, nullptr, insts, st)
+                   : launch_tiles<float>(n, count, nullptr, nullptr, insts, st);
+    return dbl ? launch_rows<double>(n, count, nullptr, nullptr, insts, st)
+               : launch_rows<float>(n, count, nullptr, nullptr, insts, st);
 }
 
-size_t stream_adj_smem_bytes(bool dbl) {
-    const size_t TD = (size_t)1 << stream_adj_tile_bits(dbl);
+static size_t stream_adj_smem_bytes(bool dbl, int tb) {
+    const size_t TD = (size_t)1 << tb;
     const size_t c = dbl ? 16 : 8, r = dbl ? 8 : 4;
     const size_t lcs = dbl ? sizeof(LayerConst<double>) : sizeof(LayerConst<float>);
     size_t o = 2 * TD * c + TD * r + 64 * lcs;
     o = (o + 15) & ~(size_t)15;
-    return o + 32 * sizeof(double);
+    return o + 64 * sizeof(double);
+}
+
+template <typename T, int RA, int NTH>
+static cudaError_t adj_t(const StreamPass& P, int si, bool lam_first, bool store, const void* insts, int count, int grid,
+                         int threads, cudaStream_t st, const void* one) {
+    const size_t sm = stream_adj_smem_bytes(sizeof(T) == 8, P.tb);
+    const cudaError_t e = cudaFuncSetAttribute(k_stream_adj_pass<T, RA, NTH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    k_stream_adj_pass<T, RA, NTH><<<grid, threads, sm, st>>>(P, si, lam_first, store, static_cast<const StreamInst<T>*>(insts),
+                                                            count, one_of<T>(one));
+    return cudaGetLastError();
 }
 
 cudaError_t launch_stream_adj_pass(bool dbl, const StreamPass& P, int si, bool lam_first, bool store,
                                    const void* insts, int count, int grid, cudaStream_t st,
                                    const void* one) {
-    const size_t sm = stream_adj_smem_bytes(dbl);
-    cudaError_t e;
-    if (dbl) {
-        e = cudaFuncSetAttribute(k_stream_adj_pass<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        k_stream_adj_pass<double><<<grid, ADJ_THREADS, sm, st>>>(P, si, lam_first, store, static_cast<const StreamInst<double>*>(insts), count, one_of<double>(one));
-    } else {
-        e = cudaFuncSetAttribute(k_stream_adj_pass<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        k_stream_adj_pass<float><<<grid, ADJ_THREADS, sm, st>>>(P, si, lam_first, store, static_cast<const StreamInst<float>*>(insts), count, one_of<float>(one));
-    }
-    return cudaGetLastError();
+    if (dbl) return adj_t<double, Num<double>::RB_ADJ, ADJ_THREADS>(P, si, lam_first, store, insts, count, grid, ADJ_THREADS, st, one);
+    if (small_tiles(dbl, P.n, P.tb))
+        return adj_t<float, SMALL_RA, 256>(P, si, lam_first, store, insts, count, grid, 1 << (P.tb - SMALL_RA), st, one);
+    return adj_t<float, Num<float>::RB_ADJ, ADJ_THREADS>(P, si, lam_first, store, insts, count, grid, ADJ_THREADS, st, one);
 }
 
 cudaError_t launch_stream_grad_reduce(bool dbl, const StreamPass* passes, int S, const void* insts,
                                       int count, uint64_t ntiles, cudaStream_t st, const void* one) {
     if (S > 256) return cudaErrorInvalidValue;
     PassLayers pl;
-    for (int i = 0; i < S; ++i) { pl.la[i] = passes[i].la; pl.lb[i] = passes[i].lb; }
-    if (dbl) k_stream_grad_reduce<double><<<count, 256, 0, st>>>(pl, S, static_cast<const StreamInst<double>*>(insts), count, ntiles, one_of<double>(one));
-    else k_stream_grad_reduce<float><<<count, 256, 0, st>>>(pl, S, static_cast<const StreamInst<float>*>(insts), count, ntiles, one_of<float>(one));
+    int p = 1;   // layers of the group (uniform for a launch)
+    for (int i = 0; i < S; ++i) { pl.la[i] = passes[i].la; pl.lb[i] = passes[i].lb; p = pl.lb[i] + 1 > p ? pl.lb[i] + 1 : p; }
+    if (dbl) k_stream_grad_reduce<double><<<dim3((unsigned)count, (unsigned)p), 256, 0, st>>>(pl, S, static_cast<const StreamInst<double>*>(insts), count, ntiles, one_of<double>(one));
+    else k_stream_grad_reduce<float><<<dim3((unsigned)count, (unsigned)p), 256, 0, st>>>(pl, S, static_cast<const StreamInst<float>*>(insts), count, ntiles, one_of<float>(one));
     return cudaGetLastError();
 }
 

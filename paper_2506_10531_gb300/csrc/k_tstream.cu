@@ -137,7 +137,7 @@ __device__ __forceinline__ void wgroup(float2* sp, uint32_t g, const Geo& geo, c
 #pragma unroll
         for (int i = 0; i < (1 << R); ++i) {
             float s, c;
-            sincos_phase(lc[0].gpi, sE[base + ((uint32_t)i << A)], s, c);
+            sincos_phase(lc[0].ph, sE[base + ((uint32_t)i << A)], s, c);
             v[i] = times_i_pow(make_float2(amp0 * c, -amp0 * s), pc + __popc(i));
         }
         mix_layer<R>(v, (1 << R) - 1, lc[0]);
@@ -146,16 +146,17 @@ __device__ __forceinline__ void wgroup(float2* sp, uint32_t g, const Geo& geo, c
         if (op.mix_la) mix_layer<R>(v, (1 << R) - 1, lc[op.la]);
         if (op.phase) {
             const LayerConst<float>& k = lc[op.lb];
+            const Pending<float> pre(k.pre, k.pcot, __popc(base) + __popcll(geo.zt));
 #pragma unroll
             for (int i = 0; i < (1 << R); ++i) {
                 float s, c;
-                sincos_phase(k.gpi, sE[base + ((uint32_t)i << A)], s, c);
-                rot_neg(v[i], s * k.pre, c * k.pre);
+                sincos_phase(k.ph, sE[base + ((uint32_t)i << A)], s, c);
+                rot_neg(v[i], s * pre.f[__popc(i) & 1], c * pre.f[__popc(i) & 1]);
             }
             mix_layer<R>(v, (1 << R) - 1, k);
         }
         if (op.fin) {
-            if (lc[op.la].shear) scale_group<R>(v, lc[op.la].post);
+            scale_group<R>(v, Pending<float>(lc[op.la].post, lc[op.la].cot, __popc(base) + __popcll(geo.zt)));
 #pragma unroll
             for (int i = 0; i < (1 << R); ++i) {
                 const float pr = v[i].x * v[i].x + v[i].y * v[i].y;
@@ -341,7 +342,8 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const StreamPass P, cons
         for (int s = 0; s < NSTAGE; ++s) mbar_init(&mbar[s], 1);
     __syncthreads();
 
-    const uint64_t ntiles = 1ull << (P.n - TB);
+    const int tbits = P.n - TB;                 // tiles of an instance: 2^tbits
+    const uint64_t ntiles = 1ull << tbits;
     const uint64_t total = ntiles * (uint64_t)count;
     const uint64_t first = blockIdx.x, step = gridDim.x;
     const int nmine = first < total ? (int)((total - 1 - first) / step + 1) : 0;
@@ -354,8 +356,8 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const StreamPass P, cons
     // has read the state buffer (wait_store), the state
     auto issue = [&](int k, bool wait_store) {
         const uint64_t q = first + (uint64_t)k * step;
-        const int ii = (int)(q / ntiles);
-        const uint64_t tau = q % ntiles;
+        const int ii = (int)(q >> tbits);
+        const uint64_t tau = q & (ntiles - 1);
         const int s = k % NSTAGE;
         const CUtensorMap* m = maps + (size_t)ii * T.maps_per_inst;
         mbar_expect_tx(&mbar[s], (P.init ? 0u : TD * 8) + (P.need_e ? TD * 4 : 0u));
@@ -368,9 +370,9 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const StreamPass P, cons
         // that store no state: with the state stores in flight it slowed the others down)
         if (pf && k + 1 < nmine) {
             const uint64_t q1 = q + step;
-            const CUtensorMap* m1 = maps + (size_t)(q1 / ntiles) * T.maps_per_inst;
-            if (P.need_e) tile_prefetch(T, m1 + T.emap, q1 % ntiles);
-            if (!P.init) tile_prefetch(T, m1 + T.map, q1 % ntiles);
+            const CUtensorMap* m1 = maps + (size_t)(q1 >> tbits) * T.maps_per_inst;
+            if (P.need_e) tile_prefetch(T, m1 + T.emap, q1 & (ntiles - 1));
+            if (!P.init) tile_prefetch(T, m1 + T.map, q1 & (ntiles - 1));
         }
     };
     if (loads && nmine > 0 && threadIdx.x == 0) issue(0, false);
@@ -380,13 +382,13 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const StreamPass P, cons
     bool run_valid = false;   // the run list holds this CTA's best k of the current instance so far
     for (int k = 0; k < nmine; ++k) {
         const uint64_t q = first + (uint64_t)k * step;
-        const int ii = (int)(q / ntiles);
-        const uint64_t tau = q % ntiles;
+        const int ii = (int)(q >> tbits);
+        const uint64_t tau = q & (ntiles - 1);
         const int s = k % NSTAGE;
         const StreamInst<float>& I = insts[ii];
         if (I.gamma != cur_g || I.beta != cur_b || I.p != cur_p) {
             __syncthreads();
-            set_layer_consts<float>(lc, I.gamma, I.beta, I.p, P.n, true);
+            set_layer_consts<float>(lc, I.gamma, I.beta, I.p, P.n, false);
             cur_g = I.gamma;
             cur_b = I.beta;
             cur_p = I.p;
@@ -502,7 +504,7 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const StreamPass P, cons
                 }
                 // this tile's slot: the list when it is the CTA's last tile of the instance
                 const uint64_t qn = q + step;
-                const bool last_of_inst = k + 1 >= nmine || (int)(qn / ntiles) != ii;
+                const bool last_of_inst = k + 1 >= nmine || (int)(qn >> tbits) != ii;
                 if (threadIdx.x < (unsigned)kk) {
                     const TopEnt e = last_of_inst ? run[threadIdx.x] : TopEnt{-1.0, 0xffffffffu};
                     I.part_topp[tau * kk + threadIdx.x] = e.p;
@@ -584,83 +586,67 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_adj_pass(const StreamPass P, 
     __syncthreads();
 
     constexpr int RA = Num<float>::RB_ADJ;
-    const uint64_t ntiles = 1ull << (P.n - TSA_TB);
-    const uint64_t total = ntiles * (uint64_t)count;
-    const uint64_t first = blockIdx.x, step = gridDim.x;
-    const int nmine = first < total ? (int)((total - 1 - first) / step + 1) : 0;
+    const int tbits = P.n - TSA_TB;             // tiles of an instance: 2^tbits (fewer than 2^32 in all)
+    const uint32_t total = (uint32_t)count << tbits, tmask = (1u << tbits) - 1u;
     const bool need_e = lam_first || P.ph_first || P.lb > P.la;
     uint32_t parity = 0;
     bool ok = true;
     // the energies first (never stored from), then, once the last tile's stores have read the
     // state buffers (wait_store), psi and lam
-    auto issue = [&](int k, bool wait_store) {
-        const uint64_t q = first + (uint64_t)k * step;
-        const int ii = (int)(q / ntiles);
-        const uint64_t tau = q % ntiles;
-        const CUtensorMap* m = maps + (size_t)ii * T.maps_per_inst;
+    auto issue = [&](uint32_t q, bool wait_store) {
+        const uint32_t tau = q & tmask;
+        const CUtensorMap* m = maps + (size_t)(q >> tbits) * T.maps_per_inst;
         mbar_expect_tx(mbar, TDA * 8 + (lam_first ? 0u : TDA * 8) + (need_e ? TDA * 4 : 0u));
         if (need_e) tile_load(T, m + T.emap, sE, tau, mbar);
         if (wait_store) bulk_wait_read();
         tile_load(T, m + T.map, spsi, tau, mbar);
         if (!lam_first) tile_load(T, m + T.map + 1, slam, tau, mbar);
         // the tile after it towards L2, a tile's compute ahead of its own loads
-        if (k + 1 < nmine) {
-            const uint64_t q1 = q + step;
-            const CUtensorMap* m1 = maps + (size_t)(q1 / ntiles) * T.maps_per_inst;
-            if (need_e) tile_prefetch(T, m1 + T.emap, q1 % ntiles);
-            tile_prefetch(T, m1 + T.map, q1 % ntiles);
-            if (!lam_first) tile_prefetch(T, m1 + T.map + 1, q1 % ntiles);
+        const uint32_t q1 = q + gridDim.x;
+        if (q1 < total) {
+            const CUtensorMap* m1 = maps + (size_t)(q1 >> tbits) * T.maps_per_inst;
+            if (need_e) tile_prefetch(T, m1 + T.emap, q1 & tmask);
+            tile_prefetch(T, m1 + T.map, q1 & tmask);
+            if (!lam_first) tile_prefetch(T, m1 + T.map + 1, q1 & tmask);
         }
     };
-    if (nmine > 0 && threadIdx.x == 0) issue(0, false);
-    const float *cur_g = nullptr, *cur_b = nullptr;
-    int cur_p = 0;
+    if (blockIdx.x < total && threadIdx.x == 0) issue(blockIdx.x, false);
+    // the parameters the constants belong to, in shared memory: the sub-passes need the registers
+    __shared__ const float *cur_g, *cur_b;
+    __shared__ int cur_p;
+    if (threadIdx.x == 0) cur_p = 0;
+    __syncthreads();
     const TileRef<float> tile{spsi, slam, sE, TSA_TB};
-    const int m0 = (P.kind == 0) ? 0 : P.c;
-    const int G = num_windows(m0, TSA_TB, RA);
-    const int nl = P.lb - P.la + 1;
-    const int S = snake_len(G, nl);
-    for (int k = 0; k < nmine; ++k) {
-        const uint64_t q = first + (uint64_t)k * step;
-        const int ii = (int)(q / ntiles);
-        const uint64_t tau = q % ntiles;
-        const StreamInst<float>& I = insts[ii];
-        if (I.gamma != cur_g || I.beta != cur_b || I.p != cur_p) {
+    for (uint32_t q = blockIdx.x; q < total; q += gridDim.x) {
+        const uint32_t tau = q & tmask;
+        const StreamInst<float>& I = insts[q >> tbits];
+        if (I.p != cur_p || I.gamma != cur_g || I.beta != cur_b) {
             __syncthreads();
-            set_layer_consts<float>(lc, I.gamma, I.beta, I.p, P.n, false);
-            cur_g = I.gamma;
-            cur_b = I.beta;
-            cur_p = I.p;
+            set_layer_consts<float>(lc, I.gamma, I.beta, I.p, P.n, true);
+            if (threadIdx.x == 0) { cur_g = I.gamma; cur_b = I.beta; cur_p = I.p; }
+            __syncthreads();
         }
         if (ok) ok = mbar_wait_bounded(mbar, parity);
         parity ^= 1u;
-        float ab[2] = {0.0f, 0.0f}, ag[2] = {0.0f, 0.0f};
-        for (int kk = S - 1; kk >= 0; --kk) {
-            SubPass sp;
-            snake_step(kk, G, nl, P.la, P.ph_first, m0, TSA_TB, TSA_TB, RA, sp, true);
-            float lb_[2] = {0.0f, 0.0f}, lg_[2] = {0.0f, 0.0f};
-            subpass_adj<float, RA, TmaLayout>(tile, sp, lc, lam_first && kk == S - 1, lb_, lg_);
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int slot = P.lb - (sp.lb - j);
-                if (j <= sp.lb - sp.la) {
-                    if (slot == 0) { ab[0] += lb_[j]; ag[0] += lg_[j]; }
-                    else { ab[1] += lb_[j]; ag[1] += lg_[j]; }
-                }
-            }
+        float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        bool first_sub = lam_first;
+        Snake sn(P.lb - P.la + 1, P.la, P.ph_first, P.kind == 0 ? 0 : P.c, TSA_TB, TSA_TB, RA, true);
+        sn.to_last();
+        for (;; sn.prev()) {
+            const SubPass sp = sn.get();
+            subpass_adj<float, RA, TmaLayout>(tile, sp, lc, first_sub, P.lb, acc);
+            first_sub = false;
             __syncthreads();
+            if (sn.first()) break;
         }
-        double* out = I.part_grad + ((uint64_t)si << (P.n - TSA_TB)) * 4 + tau * 4;
-        const double v0 = block_sum((double)ab[0], red);
-        const double v1 = block_sum((double)ab[1], red);
-        const double v2 = block_sum((double)ag[0], red);
-        const double v3 = block_sum((double)ag[1], red);
-        if (threadIdx.x == 0) { out[0] = v0; out[1] = v1; out[2] = v2; out[3] = v3; }
+        double* out = I.part_grad + (((uint64_t)si << tbits) + tau) * 4;
+        const double v = block_sum4((double)acc[0], (double)acc[1], (double)acc[2], (double)acc[3], red);
+        if (threadIdx.x < 4) out[threadIdx.x] = v;
         if (store) {
             fence_async_smem();
             __syncthreads();
             if (threadIdx.x == 0) {
-                const CUtensorMap* m = maps + (size_t)ii * T.maps_per_inst;
+                const CUtensorMap* m = maps + (size_t)(q >> tbits) * T.maps_per_inst;
                 tile_store(T, m + T.map, spsi, tau);
                 tile_store(T, m + T.map + 1, slam, tau);
                 bulk_commit();
@@ -671,7 +657,7 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_adj_pass(const StreamPass P, 
         }
         // the next tile's loads: the energies at once, psi and lam once this tile's stores have
         // read the buffers
-        if (k + 1 < nmine && threadIdx.x == 0 && ok) issue(k + 1, true);
+        if (q + gridDim.x < total && threadIdx.x == 0 && ok) issue(q + gridDim.x, true);
     }
     if (threadIdx.x == 0) {
         bulk_wait_all();

@@ -62,9 +62,8 @@ constexpr int PLAN_STATUS_SLOT = 62;
 // Scratch of one streaming instance: per-tile <C> partials and top-k lists, laid out as
 // [expect (nt doubles)] [probabilities (nt*k doubles)] [indices (nt*k uint32)], each 256-aligned.
 size_t stream_scratch_bytes(bool dbl, int n, int k) {
-    const int tb = stream_tile_bits(dbl);
-    if (n <= tb) return 0;
-    const size_t nt = (size_t)1 << (n - tb), kk = (size_t)std::max(k, 1);
+    const size_t nt = (size_t)stream_one_max_tiles(dbl, n), kk = (size_t)std::max(k, 1);
+    if (nt == 0) return 0;
     return align256(nt * sizeof(double)) + align256(nt * kk * sizeof(double)) +
            align256(nt * kk * sizeof(uint32_t));
 }
@@ -81,8 +80,8 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 // Workspace of a streaming gradient: psi and lam (2^n complex each), the forward scratch and the
 // per-pass, per-tile gradient partials of the adjoint plan (4 doubles).
 size_t stream_grad_bytes(bool dbl, int n, int p) {
-    const int tb = stream_tile_bits(dbl), tba = stream_adj_tile_bits(dbl);
-    if (n <= tb) return 0;
+    const int tba = stream_one_grad_tile_bits(dbl, n, true);
+    if (n <= stream_tile_bits(dbl)) return 0;
     StreamPass tmp[256];
     const int S = stream_plan(dbl, n, p, 0, tmp, 256, tba);
     if (S < 0) return 0;
@@ -107,9 +106,15 @@ qaoa_status run_resident_one(qaoa_ctx* c, const InstDesc<T>& d, cudaStream_t st)
     // the descriptor travels by value as a kernel parameter. One block runs alone, so it takes as
     // many threads as the narrowest windows that suit n give it (n = 8, p = 1 on GB300: 32 us with
     // 5-qubit windows, 8 of 32 threads busy; 17.5 us with 3-qubit ones)
-    const int rmax = dbl ? RES_RMAX : (d.n <= 12 ? 3 : (d.n == 13 ? 4 : RES_RMAX));
-    CK(launch_resident(dbl, nullptr, 1, d.n, d.p, grad, nullptr, 1, st, &d, rmax));
+    const int rmax = (dbl || d.n > 12) ? RES_RMAX : 3;
+    CK(launch_resident(dbl, nullptr, 1, d.n, d.p, grad, nullptr, 1, st, &d, rmax, !dbl));
     return QAOA_OK;
+}
+
+// Blocks of one pass of a single state: one per tile for the small tiles, else a persistent grid.
+int one_grid(const qaoa_ctx* c, bool dbl, const StreamPass& P) {
+    const uint64_t nt = 1ull << (P.n - P.tb);
+    return (int)(P.tb < stream_tile_bits(dbl) ? nt : std::min<uint64_t>(nt, (uint64_t)c->nsm * 2));
 }
 
 // ---- streaming single instance -----------------------------------------------------------
@@ -121,10 +126,9 @@ qaoa_status run_stream_one(qaoa_ctx* c, int n, int p, const T* gamma, const T* b
     if (!init_plus)
         return fail(QAOA_E_UNSUPPORTED, "streaming tier (n=%d) starts from |+> only", n);
     StreamPass passes[256];
-    const int S = stream_plan(dbl, n, p, k, passes, 256);
+    const int S = stream_plan_one(dbl, n, p, k, passes, 256);
     if (S < 0) return fail(QAOA_E_INVALID, "no streaming plan for n=%d p=%d", n, p);
-    const int tb = stream_tile_bits(dbl);
-    const uint64_t nt = 1ull << (n - tb);
+    const uint64_t nt = 1ull << (n - passes[S - 1].tb);   // tiles of the last pass
     char* w = static_cast<char*>(c->ws) + ws_off;
     StreamInst<T> I{};
     I.p = p;
@@ -140,8 +144,7 @@ qaoa_status run_stream_one(qaoa_ctx* c, int n, int p, const T* gamma, const T* b
     I.expect = expect;
     I.topk_idx = tidx;
     I.topk_prob = tprob;
-    const int grid = (int)std::min<uint64_t>(nt, (uint64_t)c->nsm * 2);
-    for (int s = 0; s < S; ++s) CK(launch_stream_pass(dbl, passes[s], nullptr, 1, grid, st, &I));
+    for (int s = 0; s < S; ++s) CK(launch_stream_pass(dbl, passes[s], nullptr, 1, one_grid(c, dbl, passes[s]), st, &I));
     if (expect || (k > 0 && tidx)) CK(launch_stream_finalize(dbl, nullptr, 1, nt, k, st, &I));
     return QAOA_OK;
 }
@@ -153,10 +156,10 @@ qaoa_status grad_stream_one(qaoa_ctx* c, int n, int p, const T* gamma, const T* 
     qaoa_status q = ensure_ws(c, stream_grad_bytes(dbl, n, p));
     if (q) return q;
     StreamPass passes[256];
-    const int S = stream_plan(dbl, n, p, 0, passes, 256);
+    const int tb = stream_one_grad_tile_bits(dbl, n, false);
+    const int S = stream_plan(dbl, n, p, 0, passes, 256, tb);
     if (S < 0) return fail(QAOA_E_INVALID, "no streaming plan for n=%d p=%d", n, p);
     passes[S - 1].keep_frame = 1;
-    const int tb = stream_tile_bits(dbl);
     const uint64_t nt = 1ull << (n - tb), D = 1ull << n;
     const size_t cs = sizeof(typename qaoa::Num<T>::C);
     char* w = static_cast<char*>(c->ws);
@@ -177,13 +180,12 @@ qaoa_status grad_stream_one(qaoa_ctx* c, int n, int p, const T* gamma, const T* 
     I.dgamma = dgamma;
     I.dbeta = dbeta;
     StreamPass apasses[256];
-    const int tba = stream_adj_tile_bits(dbl);
+    const int tba = stream_one_grad_tile_bits(dbl, n, true);
     const int SA = stream_plan(dbl, n, p, 0, apasses, 256, tba);
     if (SA < 0) return fail(QAOA_E_INVALID, "no adjoint plan for n=%d p=%d", n, p);
     const uint64_t nta = 1ull << (n - tba);
-    const int grid = (int)std::min<uint64_t>(nt, (uint64_t)c->nsm * 2);
-    const int agrid = (int)std::min<uint64_t>(nta, (uint64_t)c->nsm * 2);
-    for (int s = 0; s < S; ++s) CK(launch_stream_pass(dbl, passes[s], nullptr, 1, grid, st, &I));
+    const int agrid = (int)std::min<uint64_t>(nta, (uint64_t)c->nsm * (tba < stream_adj_tile_bits(dbl) ? 4 : 2));
+    for (int s = 0; s < S; ++s) CK(launch_stream_pass(dbl, passes[s], nullptr, 1, one_grid(c, dbl, passes[s]), st, &I));
     if (expect) CK(launch_stream_finalize(dbl, nullptr, 1, nt, 0, st, &I));
     for (int s = SA - 1; s >= 0; --s)
         CK(launch_stream_adj_pass(dbl, apasses[s], s, s == SA - 1, s > 0, nullptr, 1, agrid, st, &I));

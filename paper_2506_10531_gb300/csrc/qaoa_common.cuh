@@ -65,17 +65,41 @@ __device__ __forceinline__ void adam_update(float& theta, float& m, float& v, do
 
 // ---- complex helpers ---------------------------------------------------------------------
 
-__device__ __forceinline__ void sincos_phase(float g_over_pi, float e, float& s, float& c) {
-    // theta = gamma E = pi t with t = (gamma / pi) E. Periodicity: r = t - 2 rint(t / 2) lies in
-    // [-1, 1] and is computed exactly (t and 2 rint(t/2) are within 1 of each other), so
-    // theta' = pi r in [-pi, pi] has the same sine and cosine; the hardware sin/cos is then
-    // evaluated on its accurate range (absolute error below 1e-6).
+// The cost phase theta = gamma E in turns. complex64: gamma / 2 pi is kept as the unevaluated sum
+// hi + lo of two floats; m = rint(hi E) (by adding and taking off 1.5 2^23) is a whole number of
+// turns, r = hi E - m is rounded once (|r| <= 1/2 for |hi E| < 2^22) and lo E corrects it, so the
+// phase is as exact as E itself; the hardware sine and cosine are evaluated on [-pi, pi]
+// (absolute error below 1e-6). The rounding of a single-float product gamma E was the largest
+// error of a state: n = 19, p = 3, 2.1e-6 (relative, 2-norm) with it and with powers of a rounded
+// cosine, 0.9e-6 without both.
+template <typename T> struct PhaseK;
+template <> struct PhaseK<float> {
+    float hi, lo;
+};
+template <> struct PhaseK<double> {
+    double g;   // gamma / pi
+};
+__device__ __forceinline__ void make_phase(float gamma, PhaseK<float>& k) {
+    constexpr double inv = 0.15915494309189533577;   // 1 / 2 pi
+    constexpr float ih = (float)inv, il = (float)(inv - (double)ih);
+    k.hi = gamma * ih;
+    k.lo = fmaf(gamma, il, fmaf(gamma, ih, -k.hi));
+}
+__device__ __forceinline__ void make_phase(double gamma, PhaseK<double>& k) { k.g = gamma * 0.31830988618379067154; }
+__device__ __forceinline__ void sincos_phase(const PhaseK<float>& k, float e, float& s, float& c) {
+    const float m = __fadd_rn(__fadd_rn(k.hi * e, 12582912.0f), -12582912.0f);
+    const float r = fmaf(k.lo, e, fmaf(k.hi, e, -m));
+    __sincosf(6.28318530717958647693f * r, &s, &c);
+}
+// The same from a single-float gamma / pi (FwdConst): t = (gamma / pi) E, r = t - 2 rint(t / 2) in
+// [-1, 1] exactly.
+__device__ __forceinline__ void sincos_gpi(float g_over_pi, float e, float& s, float& c) {
     const float t = g_over_pi * e;
     const float r = fmaf(-2.0f, rintf(0.5f * t), t);
     __sincosf(3.14159265358979323846f * r, &s, &c);
 }
-__device__ __forceinline__ void sincos_phase(double g_over_pi, double e, double& s, double& c) {
-    sincospi(g_over_pi * e, &s, &c);
+__device__ __forceinline__ void sincos_phase(const PhaseK<double>& k, double e, double& s, double& c) {
+    sincospi(k.g * e, &s, &c);
 }
 
 __device__ __forceinline__ void sincos_full(float x, float& s, float& c) { sincosf(x, &s, &c); }
@@ -99,13 +123,6 @@ __device__ __forceinline__ void rot_neg(C& v, T s, T c) {
 // psi is converted back with (-i)^{|z|} only where a state leaves the library.
 
 // Packed FP32 pair arithmetic (one instruction for both components).
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
-    float2 d;
-    asm("{\n .reg .b64 ra, rb, rd;\n mov.b64 ra, {%2, %3};\n mov.b64 rb, {%4, %5};\n"
-        " mul.rn.f32x2 rd, ra, rb;\n mov.b64 {%0, %1}, rd;\n}"
-        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return d;
-}
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
     float2 d;
     asm("{\n .reg .b64 ra, rb, rc, rd;\n mov.b64 ra, {%2, %3};\n mov.b64 rb, {%4, %5};\n"
@@ -115,48 +132,54 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
     return d;
 }
 
-// Mixer coefficients of one layer in the rotated frame.
-template <typename T> struct RotCoef;
-template <> struct RotCoef<float> {
-    float2 cc, ss, ns;   // (c, c), (s, s), (-s, -s)
-    __device__ __forceinline__ RotCoef(float c, float s)
-        : cc(make_float2(c, c)), ss(make_float2(s, s)), ns(make_float2(-s, -s)) {}
-};
-template <> struct RotCoef<double> {
-    double c, s;
-    __device__ __forceinline__ RotCoef(double c_, double s_) : c(c_), s(s_) {}
-};
-
-// exp(-i beta X) on the pair (a, b) = (psi~[z], psi~[z | 2^q]) in the rotated frame.
-__device__ __forceinline__ void butterfly(float2& a, float2& b, const RotCoef<float>& k) {
-    const float2 t = mul2(b, k.ns);    // -s b
-    const float2 u = mul2(a, k.ss);    //  s a
-    a = fma2(a, k.cc, t);
-    b = fma2(b, k.cc, u);
-}
-__device__ __forceinline__ void butterfly(double2& a, double2& b, const RotCoef<double>& k) {
-    const double2 a0 = a, b0 = b;
-    a.x = k.c * a0.x - k.s * b0.x;
-    a.y = k.c * a0.y - k.s * b0.y;
-    b.x = k.s * a0.x + k.c * b0.x;
-    b.y = k.s * a0.y + k.c * b0.y;
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n .reg .b64 ra, rb, rd;\n mov.b64 ra, {%2, %3};\n mov.b64 rb, {%4, %5};\n"
+        " mul.rn.f32x2 rd, ra, rb;\n mov.b64 {%0, %1}, rd;\n}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
 }
 
-// Unscaled shear form of the same rotation, used when |cos b| >= |sin b|:
-//   [[c, -s], [s, c]] = c [[1, -t], [t, 1]],  t = tan b,
-// so a' = a - t b, b' = b + t a (two packed FMAs per pair) and every qubit of the layer leaves
-// a factor c that is applied once per amplitude (c^n) at the next cost phase or at the end.
-__device__ __forceinline__ void butterfly_shear(float2& a, float2& b, float t) {
-    const float2 a0 = a;
-    a = fma2(b, make_float2(-t, -t), a);
-    b = fma2(a0, make_float2(t, t), b);
+// The rotation [[c, -s], [s, c]] in unscaled shear form: with |t| <= 1,
+//   |c| >= |s|:  c [[1, -t], [t, 1]], t = s / c:                     a' = a - t b, b' = b + t a;
+//   |c| <  |s|:  s [[t, -1], [1, t]], t = c / s, its first row taken
+//                with the opposite sign:                             a' = b - t a, b' = a + t b.
+// Two packed FMAs per pair either way; each qubit leaves a factor c, or s with the sign -1
+// where its bit is 0, that is applied once per amplitude at the next cost phase or at the end.
+__device__ __forceinline__ float2 fma_s(float2 a, float t, float2 b) { return fma2(a, make_float2(t, t), b); }
+__device__ __forceinline__ double2 fma_s(double2 a, double t, double2 b) {
+    return make_double2(fma(a.x, t, b.x), fma(a.y, t, b.y));
 }
-__device__ __forceinline__ void butterfly_shear(double2& a, double2& b, double t) {
-    const double2 a0 = a;
-    a.x = fma(-t, b.x, a0.x);
-    a.y = fma(-t, b.y, a0.y);
-    b.x = fma(t, a0.x, b.x);
-    b.y = fma(t, a0.y, b.y);
+__device__ __forceinline__ float2 fma_v(float2 a, float2 b, float2 c) { return fma2(a, b, c); }
+__device__ __forceinline__ double2 fma_v(double2 a, double2 b, double2 c) {
+    return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
+}
+template <bool COT, typename C, typename T>
+__device__ __forceinline__ void butterfly(C& a, C& b, T t) {
+    const C a0 = a, b0 = b;
+    a = COT ? fma_s(a0, -t, b0) : fma_s(b0, -t, a0);
+    b = COT ? fma_s(b0, t, a0) : fma_s(a0, t, b0);
+}
+
+// The scaled rotation, four packed operations (the tile engine's complex64 forward runs use it where
+// |c| < |s|, see FwdConst).
+__device__ __forceinline__ void butterfly_scaled(float2& a, float2& b, float c, float s) {
+    const float2 t = mul2(b, make_float2(-s, -s));
+    const float2 u = mul2(a, make_float2(s, s));
+    a = fma2(a, make_float2(c, c), t);
+    b = fma2(b, make_float2(c, c), u);
+}
+
+// The inverse rotation [[c, s], [-s, c]] (0 <= c) in three shears, u = tan(beta / 2), |u| <= 1:
+// a += u b, b -= s a, a += u b. One FMA more per pair than the unscaled form, but every step is in
+// place: the adjoint holds two states in registers and chooses its qubits at run time, where a
+// result in a new register costs a move wherever the branches meet (at n = 24 the unscaled form
+// spent 94 of 285 instructions per amplitude of a two-layer pass on them, and spilled).
+template <typename C, typename T>
+__device__ __forceinline__ void lift_inverse(C& a, C& b, T u, T s) {
+    a = fma_s(b, u, a);
+    b = fma_s(a, -s, b);
+    a = fma_s(b, u, a);
 }
 
 // Multiply by i^m (m mod 4): the frame change of an amplitude with m set bits. Branch-free

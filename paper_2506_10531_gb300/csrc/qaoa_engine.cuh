@@ -19,18 +19,31 @@
 
 namespace qaoa {
 
-// Per-layer constants staged in shared memory: cost uses gamma/pi, the mixer (cos b, sin b).
-// A layer with |cos b| >= |sin b| mixes with unscaled shears (t = tan b); the factor
-// (cos b)^n it leaves is applied by the next layer's cost phase (`pre`) or, for the last layer,
-// by the last sub-pass (`post`).
+// Per-layer constants staged in shared memory. Every layer mixes with unscaled shears (see
+// butterfly); the factor its n qubits leave is post (-1)^(cot |z|), |z| the set bits of the global
+// index, applied by the next layer's cost phase (pre, pcot) or, for the last layer, by the last
+// sub-pass. The adjoint undoes the mixers with three in-place shears instead (lift_inverse), which
+// leave no factor: t is then tan(beta / 2) and sn sin(beta), beta taken modulo pi into
+// [-pi/2, pi/2] (a sign that both of its states share).
 template <typename T>
 struct LayerConst {
-    T gpi;     // gamma_l / pi
-    T c, s;    // cos(beta_l), sin(beta_l)
-    T t;       // tan(beta_l) when shear != 0
-    T pre;     // scale applied with this layer's cost phase (pending factor of layer l-1)
-    T post;    // scale still pending after this layer (used for the last layer)
-    int shear;
+    PhaseK<T> ph;   // gamma_l
+    T t;            // tan(beta_l), or cot(beta_l) with cot; adjoint: tan(beta_l / 2)
+    T sn;           // adjoint: sin(beta_l)
+    T pre;          // factor of layer l - 1, applied with this layer's cost phase
+    T post;         // factor this layer leaves
+    int cot, pcot;  // this layer's and layer l - 1's form
+};
+
+// A pending factor on the elements of a group: f0 on those with an even number of set window
+// bits, f1 on the others (parity: of the set bits of the group's base index).
+template <typename T>
+struct Pending {
+    T f[2];
+    __device__ __forceinline__ Pending(T post, int cot, int parity) {
+        f[0] = (cot && (parity & 1)) ? -post : post;
+        f[1] = cot ? -f[0] : f[0];
+    }
 };
 
 // x^n by repeated squaring in the working precision (no FP64 on the complex64 path).
@@ -45,27 +58,109 @@ __device__ __forceinline__ T ipow(T x, int n) {
     return r;
 }
 
+// (1 + t^2)^(-n/2): the factor n shears with the rounded t leave, so that a layer keeps the norm.
+// In complex64 as a product of two-float numbers: the n-th power of a factor rounded to float
+// put up to n 2^-24 on every amplitude.
+struct Two {
+    float h, l;
+    __device__ __forceinline__ Two mul(const Two& o) const {
+        const float p = h * o.h;
+        const float e = fmaf(h, o.l, fmaf(l, o.h, fmaf(h, o.h, -p)));
+        const float s = p + e;
+        return Two{s, e - (s - p)};
+    }
+};
+__device__ __forceinline__ float shear_norm(float t, int n) {
+    const float qh = fmaf(t, t, 1.0f), ql = fmaf(t, t, 1.0f - qh);      // 1 + t^2 = qh + ql
+    const float r0 = rsqrtf(qh), s = r0 * r0, se = fmaf(r0, r0, -s);
+    float d = fmaf(-qh, s, 1.0f);                                       // 1 - (1 + t^2) r0^2
+    d = fmaf(-qh, se, fmaf(-ql, s, d));
+    Two x{r0, 0.5f * r0 * d}, r{1.0f, 0.0f};
+    for (; n; n >>= 1) {
+        if (n & 1) r = r.mul(x);
+        x = x.mul(x);
+    }
+    return r.h + r.l;
+}
+__device__ __forceinline__ double shear_norm(double t, int n) { return ipow(rsqrt(fma(t, t, 1.0)), n); }
+
 // Fill the constants of p layers of an n-qubit instance (one thread per layer; contains a
-// __syncthreads, so every thread of the block calls it).
+// __syncthreads, so every thread of the block calls it). The factor of a cot layer is
+// (sign(s) / sqrt(1 + t^2))^n (-1)^(n - |z|): everything but (-1)^|z| is folded into post.
 template <typename T>
 __device__ __forceinline__ void set_layer_consts(LayerConst<T>* lc, const T* gamma, const T* beta,
-                                                 int p, int n, bool allow_shear) {
+                                                 int p, int n, bool adjoint) {
     for (int l = threadIdx.x; l < p; l += blockDim.x) {
         T sb, cb;
         sincos_full(beta[l], sb, cb);
         LayerConst<T> k;
-        k.gpi = gamma[l] * T(0.31830988618379067154);   // 1 / pi
+        make_phase(gamma[l], k.ph);
+        k.pre = k.post = T(1);
+        k.sn = T(0);
+        k.cot = k.pcot = 0;
+        if (adjoint) {
+            if (cb < T(0)) { sb = -sb; cb = -cb; }
+            k.t = sb / (T(1) + cb);
+            k.sn = sb;
+        } else {
+            k.cot = fabs(cb) < fabs(sb) ? 1 : 0;
+            const T f = k.cot ? sb : cb;
+            k.t = (k.cot ? cb : sb) / f;
+            const bool neg = k.cot ? f > T(0) : f < T(0);     // the sign of -s or c
+            k.post = shear_norm(k.t, n);
+            if (neg && (n & 1)) k.post = -k.post;
+        }
+        lc[l] = k;
+    }
+    __syncthreads();
+    for (int l = 1 + (int)threadIdx.x; l < p; l += blockDim.x) {
+        lc[l].pre = lc[l - 1].post;
+        lc[l].pcot = lc[l - 1].cot;
+    }
+    __syncthreads();
+}
+
+// Constants of the engine's forward runs. complex128 uses LayerConst. complex64 states of the
+// resident tier and of the single-instance calls are what measured shots are drawn from, and
+// a shot is a whole number that moves when a probability moves by one rounding: these runs
+// keep one arithmetic (gamma / pi in one float, shears where |cos| >= |sin| and scaled
+// rotations elsewhere, factors as powers of the rounded cosine) and one order of the qubits in a
+// layer (blocks of `block` qubits ascending in even layers, descending in odd ones, ascending
+// inside a block) whatever windows, tiles or block sizes a launch takes.
+struct FwdConst32 {
+    float gpi;     // gamma_l / pi
+    float c, s;    // cos(beta_l), sin(beta_l)
+    float t;       // tan(beta_l) when shear != 0
+    float pre;     // scale applied with this layer's cost phase (pending factor of layer l-1)
+    float post;    // scale still pending after this layer (used for the last layer)
+    int shear;
+};
+template <typename T> struct FwdOf;
+template <> struct FwdOf<float> { using K = FwdConst32; };
+template <> struct FwdOf<double> { using K = LayerConst<double>; };
+template <typename T> using FwdConst = typename FwdOf<T>::K;
+
+__device__ __forceinline__ void set_fwd_consts(FwdConst32* lc, const float* gamma, const float* beta, int p, int n) {
+    for (int l = threadIdx.x; l < p; l += blockDim.x) {
+        float sb, cb;
+        sincosf(beta[l], &sb, &cb);
+        FwdConst32 k;
+        k.gpi = gamma[l] * 0.31830988618379067154f;   // 1 / pi
         k.c = cb;
         k.s = sb;
-        k.shear = (allow_shear && fabs(cb) >= fabs(sb)) ? 1 : 0;
-        k.t = k.shear ? sb / cb : T(0);
-        k.post = k.shear ? ipow(cb, n) : T(1);
-        k.pre = T(1);
+        k.shear = fabsf(cb) >= fabsf(sb) ? 1 : 0;
+        k.t = k.shear ? sb / cb : 0.0f;
+        k.post = k.shear ? ipow(cb, n) : 1.0f;
+        k.pre = 1.0f;
         lc[l] = k;
     }
     __syncthreads();
     for (int l = 1 + (int)threadIdx.x; l < p; l += blockDim.x) lc[l].pre = lc[l - 1].post;
     __syncthreads();
+}
+__device__ __forceinline__ void set_fwd_consts(LayerConst<double>* lc, const double* gamma, const double* beta, int p,
+                                               int n) {
+    set_layer_consts<double>(lc, gamma, beta, p, n, false);
 }
 
 // One sub-pass: window start a, butterfly mask over the window bits, layers [la, lb]
@@ -89,42 +184,70 @@ __device__ __forceinline__ void window_of(int w, int m0, int m1, int tb, int R, 
 
 __device__ __forceinline__ int num_windows(int m0, int m1, int R) { return (m1 - m0 + R - 1) / R; }
 
-// Number of sub-passes of the snake schedule for layers [L0, L1] over G windows.
-__device__ __forceinline__ int snake_len(int G, int nl) {
-    return (G <= 1) ? nl : 1 + nl * (G - 1);
-}
-
-// The s-th sub-pass of the snake over layers L0..L0+nl-1 (ph_first of the very first one is
-// given by `first_ph`). Returns window index w plus the SubPass fields. top_phase: a single
-// layer that opens with its cost phase runs its windows top down, so the phase shares the top
-// window (the mixer windows of one layer commute); the TMA adjoint keeps every energy read in a
-// window whose lanes cover the low tile bits that way.
-__device__ __forceinline__ void snake_step(int s, int G, int nl, int L0, int first_ph, int m0,
-                                           int m1, int tb, int R, SubPass& sp, bool top_phase = false) {
-    int w, la, lb, phf;
-    if (G <= 1) {
-        w = 0;
-        la = lb = L0 + s;
-        phf = (s == 0) ? first_ph : 1;
-    } else {
-        // sub-pass 0 is window order[0] of layer 0; afterwards layer l has G-1 sub-passes
-        int l, pos;
-        if (s < G) { l = 0; pos = s; }
-        else { l = 1 + (s - G) / (G - 1); pos = 1 + (s - G) % (G - 1); }
-        const bool fwd = (l % 2) == 0 && !(top_phase && nl == 1 && first_ph);
-        w = fwd ? pos : (G - 1 - pos);
-        la = L0 + l;
-        lb = (pos == G - 1 && l + 1 < nl) ? la + 1 : la;
-        phf = (l == 0 && pos == 0) ? first_ph : 0;
+// Walk of the snake over layers L0..L0+nl-1, forward from begin() or backward from end(): sub-pass
+// 0 is window order[0] of layer 0, afterwards layer l has G - 1 sub-passes, so the position is
+// advanced without a division (a thread's sub-pass is a few hundred instructions; forming the
+// position from its number took a fifth of that). ph_first of the very first sub-pass is given
+// by first_ph. top_phase: a single layer that opens with its cost phase runs its windows top
+// down, so the phase shares the top window (the mixer windows of one layer commute); the TMA
+// adjoint keeps every energy read in a window whose lanes cover the low tile bits that way.
+struct Snake {
+    int G, nl, L0, first_ph, m0, m1, tb, R;
+    bool top;
+    int l, pos;
+    __device__ __forceinline__ Snake(int nl_, int L0_, int first_ph_, int m0_, int m1_, int tb_, int R_,
+                                     bool top_phase = false)
+        : G(num_windows(m0_, m1_, R_)), nl(nl_), L0(L0_), first_ph(first_ph_), m0(m0_), m1(m1_), tb(tb_), R(R_),
+          top(top_phase && nl_ == 1 && first_ph_), l(0), pos(0) {}
+    __device__ __forceinline__ void to_last() {
+        l = nl - 1;
+        pos = G > 1 ? G - 1 : 0;
     }
-    int a, mask;
-    window_of(w, m0, m1, tb, R, a, mask);
-    sp.a = a;
-    sp.mask = mask;
-    sp.la = la;
-    sp.lb = lb;
-    sp.ph_first = phf;
-    sp.post = 0;
+    __device__ __forceinline__ bool first() const { return l == 0 && pos == 0; }
+    __device__ __forceinline__ bool last() const { return l == nl - 1 && pos == (G > 1 ? G - 1 : 0); }
+    __device__ __forceinline__ void next() {
+        if (G <= 1 || pos == G - 1) { ++l; pos = G > 1 ? 1 : 0; }
+        else ++pos;
+    }
+    __device__ __forceinline__ void prev() {
+        if (G <= 1) --l;
+        else if (pos == 1 && l > 0) { --l; pos = G - 1; }
+        else --pos;
+    }
+    __device__ __forceinline__ SubPass get() const {
+        SubPass sp;
+        const bool fwd = (l & 1) == 0 && !top;
+        const int w = fwd ? pos : G - 1 - pos;
+        sp.la = L0 + l;
+        sp.lb = (G > 1 && pos == G - 1 && l + 1 < nl) ? sp.la + 1 : sp.la;
+        sp.ph_first = first() ? first_ph : (G <= 1 ? 1 : 0);
+        window_of(w, m0, m1, tb, R, sp.a, sp.mask);
+        sp.post = 0;
+        return sp;
+    }
+};
+
+// Register windows of a layer over bits [0, n) that keep the qubit order of blocks of `block` qubits
+// (FwdConst): each block is cut into windows of at most R qubits; odd layers take the blocks top
+// down, and the windows of a block always upwards (odd: their order). Made on the host.
+struct WinSched {
+    int nw;
+    signed char a[10], mask[10], odd[10];
+};
+inline WinSched win_sched(int n, int block, int R) {
+    WinSched w{};
+    for (int b = 0; b < n; b += block)
+        for (int q = b; q < n && q < b + block; q += R) {
+            const int size = (b + block < n ? b + block : n) - q < R ? (b + block < n ? b + block : n) - q : R;
+            const int a = q + R <= n ? q : (n > R ? n - R : 0);
+            w.a[w.nw] = (signed char)a;
+            w.mask[w.nw++] = (signed char)(((1 << size) - 1) << (q - a));
+        }
+    const int per = (block + R - 1) / R;
+    int k = 0;
+    for (int b = (w.nw + per - 1) / per - 1; b >= 0; --b)
+        for (int i = b * per; i < (b + 1) * per && i < w.nw; ++i) w.odd[k++] = (signed char)i;
+    return w;
 }
 
 // Local index of element i of group g for window start a (R window bits).
@@ -135,78 +258,128 @@ __device__ __forceinline__ uint32_t group_base(uint32_t g, int a) {
     return low | (high << (a + R));
 }
 
-// Mixer of one layer on the masked window bits of a register group (rotated frame).
-template <int R, typename C, typename T>
-__device__ __forceinline__ void mix_group(C (&v)[1 << R], int mask, T c, T s) {
-    const RotCoef<T> k(c, s);
+// Mixer of layer constants k on the masked window bits of a register group (rotated frame,
+// unscaled).
+template <int R, bool COT, bool FULL, typename C, typename T>
+__device__ __forceinline__ void mix_group(C (&v)[1 << R], int mask, T t) {
 #pragma unroll
     for (int j = 0; j < R; ++j) {
-        if (mask & (1 << j)) {
+        if (FULL || (mask & (1 << j))) {
 #pragma unroll
             for (int i = 0; i < (1 << R); ++i)
-                if (!(i & (1 << j))) butterfly(v[i], v[i | (1 << j)], k);
+                if (!(i & (1 << j))) butterfly<COT>(v[i], v[i | (1 << j)], t);
         }
     }
 }
-
-// Shear-form mixer (see LayerConst): a' = a - t b, b' = b + t a on the masked window bits.
-template <int R, typename C, typename T>
-__device__ __forceinline__ void mix_group_shear(C (&v)[1 << R], int mask, T t) {
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-        if (mask & (1 << j)) {
-#pragma unroll
-            for (int i = 0; i < (1 << R); ++i)
-                if (!(i & (1 << j))) butterfly_shear(v[i], v[i | (1 << j)], t);
-        }
-    }
-}
-
-// Scale every amplitude of a group.
-template <int R, typename C, typename T>
-__device__ __forceinline__ void scale_group(C (&v)[1 << R], T f) {
-#pragma unroll
-    for (int i = 0; i < (1 << R); ++i) {
-        v[i].x *= f;
-        v[i].y *= f;
-    }
-}
-
-// Mixer of layer constants k on a register group (shear or full rotation).
+// Whole windows have a path of their own without the qubit tests: a butterfly's result lands in
+// new registers, and every point where branches meet moves them back.
 template <int R, typename C, typename T>
 __device__ __forceinline__ void mix_layer(C (&v)[1 << R], int mask, const LayerConst<T>& k) {
-    if (k.shear) mix_group_shear<R>(v, mask, k.t);
-    else mix_group<R>(v, mask, k.c, k.s);
+    constexpr int ALL = (1 << R) - 1;
+    if (k.cot) {
+        if (mask == ALL) mix_group<R, true, true>(v, mask, k.t);
+        else mix_group<R, true, false>(v, mask, k.t);
+    } else {
+        if (mask == ALL) mix_group<R, false, true>(v, mask, k.t);
+        else mix_group<R, false, false>(v, mask, k.t);
+    }
+}
+
+template <int R, typename Fn>
+__device__ __forceinline__ void each_pair(float2 (&v)[1 << R], int mask, Fn&& fn) {
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        if (mask & (1 << j)) {
+#pragma unroll
+            for (int i = 0; i < (1 << R); ++i)
+                if (!(i & (1 << j))) fn(v[i], v[i | (1 << j)]);
+        }
+    }
+}
+template <int R>
+__device__ __forceinline__ void mix_layer(float2 (&v)[1 << R], int mask, const FwdConst32& k) {
+    if (k.shear) {
+        const float t = k.t;
+        if (mask == (1 << R) - 1) each_pair<R>(v, (1 << R) - 1, [t](float2& a, float2& b) { butterfly<false>(a, b, t); });
+        else each_pair<R>(v, mask, [t](float2& a, float2& b) { butterfly<false>(a, b, t); });
+    } else {
+        const float c = k.c, s = k.s;
+        each_pair<R>(v, mask, [c, s](float2& a, float2& b) { butterfly_scaled(a, b, c, s); });
+    }
+}
+// The cost phase of a forward layer with the factor the layer before left, on one amplitude: i,
+// parity as in Pending.
+struct FwdPhase32 {
+    float g, pre;
+    __device__ __forceinline__ FwdPhase32(const FwdConst32& k, int) : g(k.gpi), pre(k.pre) {}
+    __device__ __forceinline__ void apply(float2& v, int, float e) const {
+        float s, c;
+        sincos_gpi(g, e, s, c);
+        rot_neg(v, s * pre, c * pre);
+    }
+};
+struct FwdPhase64 {
+    PhaseK<double> ph;
+    Pending<double> pre;
+    __device__ __forceinline__ FwdPhase64(const LayerConst<double>& k, int parity) : ph(k.ph), pre(k.pre, k.pcot, parity) {}
+    __device__ __forceinline__ void apply(double2& v, int i, double e) const {
+        double s, c;
+        sincos_phase(ph, e, s, c);
+        rot_neg(v, s * pre.f[__popc(i) & 1], c * pre.f[__popc(i) & 1]);
+    }
+};
+__device__ __forceinline__ FwdPhase32 fwd_phase(const FwdConst32& k, int parity) { return FwdPhase32(k, parity); }
+__device__ __forceinline__ FwdPhase64 fwd_phase(const LayerConst<double>& k, int parity) { return FwdPhase64(k, parity); }
+
+// Apply a pending factor to every amplitude of a group.
+template <int R, typename C, typename T>
+__device__ __forceinline__ void scale_group(C (&v)[1 << R], const Pending<T>& f) {
+#pragma unroll
+    for (int i = 0; i < (1 << R); ++i) {
+        v[i].x *= f.f[__popc(i) & 1];
+        v[i].y *= f.f[__popc(i) & 1];
+    }
+}
+
+// The factor the last layer leaves.
+template <int R>
+__device__ __forceinline__ void finish_group(float2 (&v)[1 << R], const FwdConst32& k, int) {
+    if (!k.shear) return;
+#pragma unroll
+    for (int i = 0; i < (1 << R); ++i) {
+        v[i].x *= k.post;
+        v[i].y *= k.post;
+    }
+}
+template <int R>
+__device__ __forceinline__ void finish_group(double2 (&v)[1 << R], const LayerConst<double>& k, int parity) {
+    scale_group<R>(v, Pending<double>(k.post, k.cot, parity));
 }
 
 // Mixer inverse on two states with the accumulation of Im <lam| X_q |psi> over the masked
 // qubits. Any point of the layer's mixer gives the same value (X_q commutes with every
 // exp(-i beta X_q')). In the rotated frame X_q becomes Y_q, so over the pairs (a, b)
-//   Im <lam|X_q|psi> = sum Re(conj(lam~_b) psi~_a) - Re(conj(lam~_a) psi~_b).
-// Four independent partial sums keep the accumulation off the FMA latency chain.
+//   Im <lam|X_q|psi> = sum Re(conj(lam~_b) psi~_a) - Re(conj(lam~_a) psi~_b),
+// two packed FMAs per pair.
 template <int R, typename C, typename T>
-__device__ __forceinline__ T mix_group_adj(C (&v)[1 << R], C (&u)[1 << R], int mask, T c, T s) {
-    const RotCoef<T> k(c, -s);
-    T acc[4] = {T(0), T(0), T(0), T(0)};
+__device__ __forceinline__ T mix_group_adj(C (&v)[1 << R], C (&u)[1 << R], int mask, T tu, T s) {
+    C p, m;
+    p.x = p.y = m.x = m.y = T(0);
 #pragma unroll
     for (int j = 0; j < R; ++j) {
         if (mask & (1 << j)) {
-            int slot = 0;
 #pragma unroll
             for (int i = 0; i < (1 << R); ++i)
                 if (!(i & (1 << j))) {
                     const int b = i | (1 << j);
-                    T& a = acc[slot++ & 3];
-                    a = fma(u[b].x, v[i].x, a);
-                    a = fma(u[b].y, v[i].y, a);
-                    a = fma(-u[i].x, v[b].x, a);
-                    a = fma(-u[i].y, v[b].y, a);
-                    butterfly(v[i], v[b], k);
-                    butterfly(u[i], u[b], k);
+                    p = fma_v(u[b], v[i], p);
+                    m = fma_v(u[i], v[b], m);
+                    lift_inverse(v[i], v[b], tu, s);
+                    lift_inverse(u[i], u[b], tu, s);
                 }
         }
     }
-    return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    return (p.x + p.y) - (m.x + m.y);
 }
 
 // Shared-memory layout of a tile: position of amplitude u (p) and of energy u (e). The engine's
@@ -248,77 +421,97 @@ __device__ __forceinline__ uint32_t gray_step(const WinSteps<R>& w, int k, int f
     return w.s[j];
 }
 
-// Load / store the 2^R elements of a group whose element 0 lies b0 bytes into the tile. complex64
-// windows starting at bit 0 move aligned pairs with one 16-byte shared access (the swizzle keeps
-// pairs adjacent; conflict-free that way).
+// 32-bit shared-memory accesses (the tile pointers reach the sub-passes through structs, where the
+// compiler would fall back to generic 64-bit addressing).
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void lds(uint32_t a, float& v) { asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory"); }
+__device__ __forceinline__ void lds(uint32_t a, double& v) { asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory"); }
+__device__ __forceinline__ void lds(uint32_t a, float2& v) {
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void lds(uint32_t a, double2& v) {
+    asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void lds2(uint32_t a, float2& v, float2& w) {
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(w.x), "=f"(w.y) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void sts(uint32_t a, const float2& v) {
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void sts(uint32_t a, const double2& v) {
+    asm volatile("st.shared.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(v.x), "d"(v.y) : "memory");
+}
+__device__ __forceinline__ void sts2(uint32_t a, const float2& v, const float2& w) {
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(w.x), "f"(w.y) : "memory");
+}
+
+// Load / store the 2^R elements of a group whose element 0 lies b0 bytes into the tile at shared
+// address p. complex64 windows starting at bit 0 (pairs) move aligned pairs with one 16-byte shared
+// access (the swizzle keeps pairs adjacent; conflict-free that way).
 template <int R>
-__device__ __forceinline__ void load_group(const float2* psi, uint32_t b0, bool pairs, const WinSteps<R>& w,
+__device__ __forceinline__ void load_group(uint32_t p, uint32_t b0, bool pairs, const WinSteps<R>& w,
                                            float2 (&v)[1 << R]) {
-    const char* p = reinterpret_cast<const char*>(psi);
     if (pairs) {
 #pragma unroll
         for (int k = 0; k < (1 << (R - 1)); ++k) {
             if (k) b0 ^= gray_step(w, k, 1);
             const int i = 2 * gray_elem(k);
-            const float4 t = *reinterpret_cast<const float4*>(p + b0);
-            v[i] = make_float2(t.x, t.y);
-            v[i + 1] = make_float2(t.z, t.w);
+            lds2(p + b0, v[i], v[i + 1]);
         }
     } else {
 #pragma unroll
         for (int k = 0; k < (1 << R); ++k) {
             if (k) b0 ^= gray_step(w, k);
-            v[gray_elem(k)] = *reinterpret_cast<const float2*>(p + b0);
+            lds(p + b0, v[gray_elem(k)]);
         }
     }
 }
 template <int R>
-__device__ __forceinline__ void store_group(float2* psi, uint32_t b0, bool pairs, const WinSteps<R>& w,
+__device__ __forceinline__ void store_group(uint32_t p, uint32_t b0, bool pairs, const WinSteps<R>& w,
                                             const float2 (&v)[1 << R]) {
-    char* p = reinterpret_cast<char*>(psi);
     if (pairs) {
 #pragma unroll
         for (int k = 0; k < (1 << (R - 1)); ++k) {
             if (k) b0 ^= gray_step(w, k, 1);
             const int i = 2 * gray_elem(k);
-            *reinterpret_cast<float4*>(p + b0) = make_float4(v[i].x, v[i].y, v[i + 1].x, v[i + 1].y);
+            sts2(p + b0, v[i], v[i + 1]);
         }
     } else {
 #pragma unroll
         for (int k = 0; k < (1 << R); ++k) {
             if (k) b0 ^= gray_step(w, k);
-            *reinterpret_cast<float2*>(p + b0) = v[gray_elem(k)];
+            sts(p + b0, v[gray_elem(k)]);
         }
     }
 }
 template <int R>
-__device__ __forceinline__ void load_group(const double2* psi, uint32_t b0, bool, const WinSteps<R>& w,
+__device__ __forceinline__ void load_group(uint32_t p, uint32_t b0, bool, const WinSteps<R>& w,
                                            double2 (&v)[1 << R]) {
-    const char* p = reinterpret_cast<const char*>(psi);
 #pragma unroll
     for (int k = 0; k < (1 << R); ++k) {
         if (k) b0 ^= gray_step(w, k);
-        v[gray_elem(k)] = *reinterpret_cast<const double2*>(p + b0);
+        lds(p + b0, v[gray_elem(k)]);
     }
 }
 template <int R>
-__device__ __forceinline__ void store_group(double2* psi, uint32_t b0, bool, const WinSteps<R>& w,
+__device__ __forceinline__ void store_group(uint32_t p, uint32_t b0, bool, const WinSteps<R>& w,
                                             const double2 (&v)[1 << R]) {
-    char* p = reinterpret_cast<char*>(psi);
 #pragma unroll
     for (int k = 0; k < (1 << R); ++k) {
         if (k) b0 ^= gray_step(w, k);
-        *reinterpret_cast<double2*>(p + b0) = v[gray_elem(k)];
+        sts(p + b0, v[gray_elem(k)]);
     }
 }
-// fn(i, e) for every element i of a group with its energy e (element 0 lies b0 bytes into E)
+// fn(i, e) for every element i of a group with its energy e (element 0 lies b0 bytes into the
+// energies at shared address p)
 template <int R, typename T, typename Fn>
-__device__ __forceinline__ void for_energies(const T* E, uint32_t b0, const WinSteps<R>& w, Fn&& fn) {
-    const char* p = reinterpret_cast<const char*>(E);
+__device__ __forceinline__ void for_energies(uint32_t p, uint32_t b0, const WinSteps<R>& w, Fn&& fn) {
 #pragma unroll
     for (int k = 0; k < (1 << R); ++k) {
         if (k) b0 ^= gray_step(w, k);
-        fn(gray_elem(k), *reinterpret_cast<const T*>(p + b0));
+        T e;
+        lds(p + b0, e);
+        fn(gray_elem(k), e);
     }
 }
 
@@ -336,9 +529,10 @@ struct TileRef {
 //          global bits that the tile index itself fixes) instead of being read
 template <typename T, int R>
 __device__ __forceinline__ void subpass_fwd(const TileRef<T>& t, const SubPass& sp,
-                                            const LayerConst<T>* lc, bool init, T amp0, int pc0) {
+                                            const FwdConst<T>* lc, bool init, T amp0, int pc0) {
     using C = typename Num<T>::C;
     const auto map = [](uint32_t u) { return swz<T>(u); };
+    const uint32_t apsi = smem_addr(t.psi), aE = smem_addr(t.E);
     const WinSteps<R> ws = win_steps<R>(sp.a, sizeof(C), map), we = win_steps<R>(sp.a, sizeof(T), map);
     const uint32_t ngroups = 1u << (t.tb - R);
     for (uint32_t g = threadIdx.x; g < ngroups; g += blockDim.x) {
@@ -360,34 +554,30 @@ __device__ __forceinline__ void subpass_fwd(const TileRef<T>& t, const SubPass& 
                 v[i] = m == 0 ? q0 : (m == 1 ? q1 : (m == 2 ? q2 : q3));
             }
         } else {
-            load_group<R>(t.psi, sb * (uint32_t)sizeof(C), sp.a == 0, ws, v);
+            load_group<R>(apsi, sb * (uint32_t)sizeof(C), sp.a == 0, ws, v);
         }
 #pragma unroll 1
         for (int l = sp.la; l <= sp.lb; ++l) {
             if (l > sp.la || sp.ph_first) {
-                const T gp = lc[l].gpi, pre = lc[l].pre;
-                for_energies<R>(t.E, sb * (uint32_t)sizeof(T), we, [&](int i, T e) {
-                    T s, c;
-                    sincos_phase(gp, e, s, c);
-                    rot_neg(v[i], s * pre, c * pre);
-                });
+                const auto ph = fwd_phase(lc[l], pc0 + __popc(base));
+                for_energies<R, T>(aE, sb * (uint32_t)sizeof(T), we, [&](int i, T e) { ph.apply(v[i], i, e); });
             }
             mix_layer<R>(v, sp.mask, lc[l]);
         }
-        if (sp.post && lc[sp.lb].shear) scale_group<R>(v, lc[sp.lb].post);
-        store_group<R>(t.psi, sb * (uint32_t)sizeof(C), sp.a == 0, ws, v);
+        if (sp.post) finish_group<R>(v, lc[sp.lb], pc0 + __popc(base));
+        store_group<R>(apsi, sb * (uint32_t)sizeof(C), sp.a == 0, ws, v);
     }
 }
 
-// Adjoint sub-pass: the forward sub-pass `sp` undone on psi and lam, accumulating
-//   acc_b[j] += Im <lam| sum_q X_q |psi> (window qubits) for layer lb - j,
-//   acc_g[j] += Im <lam| E |psi>                          for layer lb - j (its cost op).
-// lam_from_E: lam = E psi is formed on load (first adjoint sub-pass).
+// Adjoint sub-pass: the forward sub-pass `sp` undone on psi and lam, accumulating for layer l,
+// slot = top - l (0 or 1),
+//   acc[slot] += Im <lam| sum_q X_q |psi> (window qubits),  acc[2 + slot] += Im <lam| E |psi> (its
+// cost phase). lam_from_E: lam = E psi is formed on load (first adjoint sub-pass).
 template <typename T, int R, typename Lay = SwzLayout<T>>
 __device__ __forceinline__ void subpass_adj(const TileRef<T>& t, const SubPass& sp,
-                                            const LayerConst<T>* lc, bool lam_from_E,
-                                            T (&acc_b)[2], T (&acc_g)[2]) {
+                                            const LayerConst<T>* lc, bool lam_from_E, int top, T (&acc)[4]) {
     using C = typename Num<T>::C;
+    const uint32_t apsi = smem_addr(t.psi), alam = smem_addr(t.lam), aE = smem_addr(t.E);
     const WinSteps<R> ws = win_steps<R>(sp.a, sizeof(C), [](uint32_t u) { return Lay::p(u); });
     const WinSteps<R> we = win_steps<R>(sp.a, sizeof(T), [](uint32_t u) { return Lay::e(u); });
     const uint32_t ngroups = 1u << (t.tb - R);
@@ -395,36 +585,35 @@ __device__ __forceinline__ void subpass_adj(const TileRef<T>& t, const SubPass& 
         const uint32_t base = group_base<R>(g, sp.a);
         const uint32_t sb = Lay::p(base) * (uint32_t)sizeof(C), eb = Lay::e(base) * (uint32_t)sizeof(T);
         C v[1 << R], u[1 << R];
-        load_group<R>(t.psi, sb, sp.a == 0, ws, v);
+        load_group<R>(apsi, sb, sp.a == 0, ws, v);
         if (lam_from_E) {
-            for_energies<R>(t.E, eb, we, [&](int i, T e) {
+            for_energies<R, T>(aE, eb, we, [&](int i, T e) {
                 u[i].x = e * v[i].x;
                 u[i].y = e * v[i].y;
             });
         } else {
-            load_group<R>(t.lam, sb, sp.a == 0, ws, u);
+            load_group<R>(alam, sb, sp.a == 0, ws, u);
         }
 #pragma unroll 1
         for (int l = sp.lb; l >= sp.la; --l) {
-            const int j = sp.lb - l;
-            const T ab = mix_group_adj<R>(v, u, sp.mask, lc[l].c, lc[l].s);
-            if (j == 0) acc_b[0] += ab; else acc_b[1] += ab;
+            const T ab = mix_group_adj<R>(v, u, sp.mask, lc[l].t, lc[l].sn);
+            if (l == top) acc[0] += ab; else acc[1] += ab;
             if (l > sp.la || sp.ph_first) {
-                const T gp = -lc[l].gpi;
+                const PhaseK<T> ph = lc[l].ph;
                 T ag[4] = {T(0), T(0), T(0), T(0)};
-                for_energies<R>(t.E, eb, we, [&](int i, T e) {
+                for_energies<R, T>(aE, eb, we, [&](int i, T e) {
                     ag[i & 3] = fma(e, im_conj_mul(u[i], v[i]), ag[i & 3]);
                     T s, c;
-                    sincos_phase(gp, e, s, c);
-                    rot_neg(v[i], s, c);
-                    rot_neg(u[i], s, c);
+                    sincos_phase(ph, e, s, c);
+                    rot_neg(v[i], -s, c);
+                    rot_neg(u[i], -s, c);
                 });
                 const T agt = (ag[0] + ag[1]) + (ag[2] + ag[3]);
-                if (j == 0) acc_g[0] += agt; else acc_g[1] += agt;
+                if (l == top) acc[2] += agt; else acc[3] += agt;
             }
         }
-        store_group<R>(t.psi, sb, sp.a == 0, ws, v);
-        store_group<R>(t.lam, sb, sp.a == 0, ws, u);
+        store_group<R>(apsi, sb, sp.a == 0, ws, v);
+        store_group<R>(alam, sb, sp.a == 0, ws, u);
     }
 }
 
@@ -547,7 +736,8 @@ template <typename T>
 __device__ __forceinline__ void fused_init_store(const FusedInit<T>& fi, uint32_t u, uint32_t ix, T e) {
     typename Num<T>::C a;
     T s, c;
-    sincos_phase(fi.gpi0, e, s, c);
+    if constexpr (sizeof(T) == 4) sincos_gpi(fi.gpi0, e, s, c);
+    else sincospi(fi.gpi0 * e, &s, &c);
     a.x = fi.amp0 * c;          // amp0 e^{-i theta}
     a.y = -fi.amp0 * s;
     fi.psi[ix] = times_i_pow(a, fi.pc0 + __popc(u));
@@ -875,6 +1065,32 @@ __device__ __forceinline__ void rank_select(const TopEnt* cand, int count, int k
         }
         if (rank < k) out[rank] = me;
     }
+}
+
+// Block-wide FP64 sums of four values per thread, fixed order. In a warp the four reductions share
+// their first two steps (each lane hands over half of what it holds), six FP64 adds a lane
+// instead of twenty: FP64 issues at 1/64 of the FP32 rate. red: 4 * (blockDim / 32) doubles, at
+// most 16 warps. Lane j < 4 of warp 0 returns the sum of value j. Called by all threads.
+__device__ __forceinline__ double block_sum4(double v0, double v1, double v2, double v3, double* red) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    const bool o1 = lane & 1, o2 = lane & 2;
+    const double a = (o1 ? v2 : v0) + __shfl_xor_sync(0xffffffffu, o1 ? v0 : v2, 1);
+    const double b = (o1 ? v3 : v1) + __shfl_xor_sync(0xffffffffu, o1 ? v1 : v3, 1);
+    double c = (o2 ? b : a) + __shfl_xor_sync(0xffffffffu, o2 ? a : b, 2);   // lane & 3 holds v0, v2, v1, v3
+#pragma unroll
+    for (int o = 4; o <= 16; o <<= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    __syncthreads();
+    if (lane < 4) red[4 * w + (lane == 1 ? 2 : (lane == 2 ? 1 : lane))] = c;
+    __syncthreads();
+    double tot = 0.0;
+    if (w == 0) {   // lane 4 i + j: value j of warps i and i + 8
+        const int i = lane >> 2;
+        if (i < nw) tot = red[lane];
+        if (i + 8 < nw) tot += red[lane + 32];
+#pragma unroll
+        for (int o = 4; o <= 16; o <<= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    }
+    return tot;
 }
 
 // Block-wide sum of one value per thread into slot[0] (thread 0 only); red has blockDim/32

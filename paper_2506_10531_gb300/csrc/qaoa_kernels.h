@@ -47,10 +47,11 @@ size_t resident_smem_bytes(bool dbl, int n, int p, bool grad, int rmax = RES_RMA
 int resident_threads(bool dbl, int n, int rmax = RES_RMAX);
 // Launch a resident-tier kernel over `count` device descriptors (all with the same n).
 // queue: device int zeroed by the caller before the launch (work counter). With desc ==
-// nullptr the host descriptor `one` is passed by value and run by one block.
+// nullptr the host descriptor `one` is passed by value and run by one block. block5: the qubit
+// order of 5-qubit windows whatever rmax is (see WinSched).
 cudaError_t launch_resident(bool dbl, const void* desc, int count, int n, int pmax, bool grad,
                             int* queue, int grid, cudaStream_t st, const void* one = nullptr,
-                            int rmax = RES_RMAX);
+                            int rmax = RES_RMAX, bool block5 = false);
 int resident_max_blocks_per_sm(bool dbl, int n, int pmax, bool grad, int rmax = RES_RMAX);
 
 // ---- cluster tier: one cluster of 2^(n-L) CTAs per complex64 instance (15 <= n <= 18) ----

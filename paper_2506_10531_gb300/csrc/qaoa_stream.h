@@ -5,6 +5,13 @@
 
 namespace qaoa {
 
+// One sub-pass of a listed pass: window start, mask of its qubits, first and last layer (relative to
+// the pass's la), whether the cost phase of the first layer opens it.
+struct StreamSub {
+    int a, mask, l0, l1, phase;
+};
+constexpr int STREAM_MAX_SUB = 10;
+
 // One HBM pass over all tiles of the instances of a launch (uniform for the launch).
 struct StreamPass {
     int n;          // qubits of the instances of this launch
@@ -19,6 +26,8 @@ struct StreamPass {
     int need_e;     // the pass reads the energies
     int keep_frame; // fin pass of a gradient run: leave psi in the rotated frame for the adjoint
     int no_store;   // fin pass whose final state nobody reads: reductions only, no write-back
+    int nsub;       // > 0: the listed sub-passes (stream_plan_one), else the snake over the tile's windows
+    StreamSub sub[STREAM_MAX_SUB];
 };
 
 // One instance of a streaming launch (device pointers).
@@ -48,10 +57,15 @@ int stream_tile_bits(bool dbl);
 // Tile bits of the adjoint passes: one bit fewer than the forward tiles, so that two CTAs
 // (psi, lam and E tiles each) share an SM.
 int stream_adj_tile_bits(bool dbl);
+// A single state run outside a plan: the forward passes of qaoa_run_layers (the batched plan where it
+// has no tiles of its own), the most tiles any of its passes has, and the tile bits of qaoa_grad's
+// passes.
+int stream_plan_one(bool dbl, int n, int p, int k, StreamPass* out, int max_out);
+uint64_t stream_one_max_tiles(bool dbl, int n);
+int stream_one_grad_tile_bits(bool dbl, int n, bool adjoint);
 // Fill the pass list of a p-layer run on n qubits with tiles of tb bits (tb < 0: the forward
 // tile size); returns the number of passes or -1.
 int stream_plan(bool dbl, int n, int p, int k, StreamPass* out, int max_out, int tb = -1);
-size_t stream_smem_bytes(bool dbl);
 // insts: device array of `count` instances, or nullptr to pass the host instance `one` by value.
 cudaError_t launch_stream_pass(bool dbl, const StreamPass& P, const void* insts, int count,
                                int grid, cudaStream_t st, const void* one = nullptr);
@@ -70,7 +84,6 @@ cudaError_t launch_stream_adj_pass(bool dbl, const StreamPass& P, int si, bool l
 cudaError_t launch_stream_grad_reduce(bool dbl, const StreamPass* passes, int S, const void* insts,
                                       int count, uint64_t ntiles, cudaStream_t st,
                                       const void* one = nullptr);
-size_t stream_adj_smem_bytes(bool dbl);
 cudaError_t launch_energy(bool dbl, int n, const void* Q, void* E, cudaStream_t st);
 // Energies of `count` streaming instances (E written through insts[i].E from insts[i].Q).
 cudaError_t launch_energy_batch(bool dbl, int n, const void* insts, int count, cudaStream_t st);
