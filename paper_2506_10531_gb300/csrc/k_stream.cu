@@ -20,6 +20,14 @@ namespace qaoa {
 
 namespace {
 
+// Tiles of a single state (see the host side): windows, sizes with tiles of their own, first upper qubit.
+constexpr int SMALL_R = 3, SMALL_NMIN = 15, SMALL_NMAX = 21, SMALL_LOW = 13, SMALL_RA = 4;
+
+// Windows of a layer for tiles of tb bits whose kind-B chunks keep 2^cmin contiguous amplitudes.
+__host__ __device__ inline int stream_windows(int n, int tb, int cmin) {
+    return 1 + (n - tb + tb - cmin - 1) / (tb - cmin);
+}
+
 // Global index of tile-local index u for tile tau of pass P.
 __device__ __forceinline__ uint64_t global_index(const StreamPass& P, uint64_t tau, uint32_t u) {
     if (P.kind == 0) return (tau << P.tb) | u;
@@ -124,7 +132,7 @@ __device__ __forceinline__ void stream_stage(const StreamPass& P, const StreamIn
 // the instantiation serves passes with a top-k.
 template <typename T, int R, bool TOPK>
 __device__ void stream_tile(const StreamPass& P, const StreamInst<T>& I, uint64_t tau,
-                            const StreamSmem<T>& s, bool have_run, uint64_t prev_tau) {
+                            const StreamSmem<T>& s, bool have_run, uint64_t prev_tau, const StreamSubs& subs) {
     using C = typename Num<T>::C;
     const uint32_t TD = 1u << P.tb;
     C* gpsi = reinterpret_cast<C*>(I.psi);
@@ -134,10 +142,10 @@ __device__ void stream_tile(const StreamPass& P, const StreamInst<T>& I, uint64_
     const TileRef<T> tile{s.psi, nullptr, s.E, P.tb};
     const int m0 = (P.kind == 0) ? 0 : P.c;
     const T amp0 = (T)I.amp0;
-    if (P.nsub > 0) {              // listed sub-passes (a single state's small tiles)
-        for (int i = 0; i < P.nsub; ++i) {
-            const StreamSub& b = P.sub[i];
-            SubPass sp{b.a, b.mask, P.la + b.l0, P.la + b.l1, b.phase, P.fin && i == P.nsub - 1};
+    if (subs.n > 0) {              // listed sub-passes (a single state's small tiles)
+        for (int i = 0; i < subs.n; ++i) {
+            const StreamSub& b = subs.sub[i];
+            SubPass sp{b.a, b.mask, P.la + b.l0, P.la + b.l1, b.phase, P.fin && i == subs.n - 1};
             subpass_fwd<T, R>(tile, sp, s.lc, P.init && i == 0, amp0, __popcll(tau));
             __syncthreads();
         }
@@ -218,7 +226,7 @@ __device__ void stream_tile(const StreamPass& P, const StreamInst<T>& I, uint64_
 template <typename T, int R, int NTH, bool TOPK>
 __global__ void __launch_bounds__(NTH, 2) k_stream_pass(const StreamPass P,
                                                      const StreamInst<T>* __restrict__ insts,
-                                                     int count, const StreamInst<T> one) {
+                                                     int count, const StreamInst<T> one, const StreamSubs subs) {
     extern __shared__ __align__(16) unsigned char sm[];
     using C = typename Num<T>::C;
     const uint32_t TD = 1u << P.tb;
@@ -265,7 +273,7 @@ __global__ void __launch_bounds__(NTH, 2) k_stream_pass(const StreamPass P,
             cur_b = I.beta;
             cur_p = I.p;
         }
-        stream_tile<T, R, TOPK>(P, I, tau, s, run_ii == ii, run_tau);
+        stream_tile<T, R, TOPK>(P, I, tau, s, run_ii == ii, run_tau, subs);
         run_ii = ii;
         run_tau = tau;
     }
@@ -309,6 +317,11 @@ __global__ void __launch_bounds__(256) k_stream_finalize(const StreamInst<T>* __
     const int ii = blockIdx.x;
     if (ii >= count) return;
     const StreamInst<T>& I = insts ? insts[ii] : one;
+    if (ntiles == 0) {             // instances of several sizes
+        ntiles = 1ull << (I.n - (sizeof(T) == 8 ? 12 : 13));
+        k = I.k;
+        stride = k > 0 && ntiles > FIN_CHUNK ? FIN_CHUNK : 1;
+    }
     // sum: each thread a contiguous slice (fixed), then the block tree
     double acc = 0.0;
     const uint64_t per = (ntiles + blockDim.x - 1) / blockDim.x;
@@ -411,36 +424,32 @@ __global__ void __launch_bounds__(NTH, 2) k_stream_adj_pass(const StreamPass P, 
 // Block (i, l): dgamma_l = 2 sum of the gamma slots of layer l of instance i, dbeta_l = 2 sum of the
 // beta slots, over passes in order and tiles in fixed contiguous chunks per thread. (One block per
 // instance, its layers one after the other: 15 us at n = 20, p = 4; a layer per block: 6 us.)
-struct PassLayers {
-    int la[256], lb[256];
-};
 template <typename T>
-__global__ void __launch_bounds__(256) k_stream_grad_reduce(const PassLayers pl, int S,
-                                                            const StreamInst<T>* __restrict__ insts,
-                                                            int count, uint64_t ntiles,
+__global__ void __launch_bounds__(256) k_stream_grad_reduce(int tb, int cmin, const StreamInst<T>* __restrict__ insts, int count,
                                                             const StreamInst<T> one) {
     __shared__ double red[32];
-    const int ii = blockIdx.x;
+    const int ii = blockIdx.x, l = blockIdx.y;
     if (ii >= count) return;
     const StreamInst<T>& I = insts ? insts[ii] : one;
+    if (l >= I.p || !I.part_grad) return;   // (a mixed launch also meets instances without a gradient)
+    // the passes that hold layer l (stream_plan): the first shared with layer l - 1, the last with
+    // layer l + 1, W windows per layer
+    const int W = stream_windows(I.n, tb, cmin);
+    const uint64_t ntiles = 1ull << (I.n - tb);
     const uint64_t per = (ntiles + blockDim.x - 1) / blockDim.x;
-    const int l = blockIdx.y;
-    if (l < I.p) {
-        double gb = 0.0, gg = 0.0;
-        for (int s = 0; s < S; ++s) {
-            const bool hb = pl.lb[s] == l, ha = pl.la[s] == l && pl.lb[s] != pl.la[s];
-            if (!hb && !ha) continue;
-            const double* base = I.part_grad + ((uint64_t)s * ntiles) * 4;
-            for (uint64_t t = threadIdx.x * per; t < (threadIdx.x + 1) * per && t < ntiles; ++t) {
-                const double* q = base + t * 4;
-                if (hb) { gb += q[0]; gg += q[2]; }
-                if (ha) { gb += q[1]; gg += q[3]; }
-            }
+    double gb = 0.0, gg = 0.0;
+    for (int s = l * (W - 1); s <= (l + 1) * (W - 1); ++s) {
+        const bool ha = s == (l + 1) * (W - 1) && l + 1 < I.p;   // layer l is the pass's la, else its lb
+        const double* base = I.part_grad + ((uint64_t)s * ntiles) * 4 + (ha ? 1 : 0);
+        for (uint64_t t = threadIdx.x * per; t < (threadIdx.x + 1) * per && t < ntiles; ++t) {
+            const double* q = base + t * 4;
+            gb += q[0];
+            gg += q[2];
         }
-        const double v = block_sum4(gb, gg, 0.0, 0.0, red);
-        if (threadIdx.x == 0 && I.dbeta) I.dbeta[l] = 2.0 * v;
-        if (threadIdx.x == 1 && I.dgamma) I.dgamma[l] = 2.0 * v;
     }
+    const double v = block_sum4(gb, gg, 0.0, 0.0, red);
+    if (threadIdx.x == 0 && I.dbeta) I.dbeta[l] = 2.0 * v;
+    if (threadIdx.x == 1 && I.dgamma) I.dgamma[l] = 2.0 * v;
 }
 
 // ---- energy build into HBM, row form (n >= 2) ------------------------------------------
@@ -638,12 +647,30 @@ struct Acc {
     }
 };
 
+// Runs of instances of equal n in one launch: run i owns blocks [b0[i], b0[i + 1]).
+struct EnergyRuns {
+    int runs;
+    uint32_t b0[ENERGY_RUNS + 1];
+    int n[ENERGY_RUNS], first[ENERGY_RUNS];
+};
+
 template <typename T>
 __global__ void __launch_bounds__(256) k_energy_tile(int n, const T* __restrict__ Q, T* __restrict__ E,
-                                                     const StreamInst<T>* insts) {
+                                                     const StreamInst<T>* insts, const EnergyRuns er) {
     __shared__ T W[32 * 32];      // zero beyond n
     __shared__ Acc<T> d[16];
-    if (insts) {
+    uint32_t hi = blockIdx.x;
+    if (er.runs > 0) {
+        int r = 0;
+        while (hi >= er.b0[r + 1]) ++r;
+        n = er.n[r];
+        hi -= er.b0[r];
+        const int hb = n > ETB ? n - ETB : 0;
+        const StreamInst<T>& I = insts[er.first[r] + (hi >> hb)];
+        hi &= (1u << hb) - 1u;
+        Q = I.Q;
+        E = const_cast<T*>(I.E);
+    } else if (insts) {
         Q = insts[blockIdx.y].Q;
         E = const_cast<T*>(insts[blockIdx.y].E);
     }
@@ -654,7 +681,6 @@ __global__ void __launch_bounds__(256) k_energy_tile(int n, const T* __restrict_
         if (i < n && j < n) w = (i == j) ? Q[i * n + i] : Q[i * n + j] + Q[j * n + i];
         W[x] = w;
     }
-    const uint32_t hi = blockIdx.x;
     const int nhi = n > ETB ? n - ETB : 0, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __syncthreads();
     const bool on = lane < nhi && ((hi >> lane) & 1u);
@@ -732,14 +758,14 @@ __global__ void __launch_bounds__(256) k_energy_tile(int n, const T* __restrict_
 //   least 8 amplitudes, 16 amplitudes per thread.
 // GB300: qaoa_run_layers at n = 19, p = 3, passes of 22 to 29 us -> 14 to 18 (qubits 0..12) and 8 to
 // 10 us; qaoa_grad at n = 20, p = 4, forward passes 23 to 32 -> 10 to 15 us.
-constexpr int SMALL_R = 3, SMALL_NMIN = 15, SMALL_NMAX = 21, SMALL_LOW = 13, SMALL_RA = 4;
 static bool small_tiles(bool dbl, int n, int tb) { return !dbl && n >= 14 && n <= SMALL_NMAX && tb == (n + 4) / 2; }
 
 int stream_tile_bits(bool dbl) { return dbl ? 12 : 13; }
 int stream_adj_tile_bits(bool dbl) { return dbl ? 11 : 12; }
-int stream_one_grad_tile_bits(bool dbl, int n, bool adjoint) {
-    if (!dbl && n >= 14 && n <= SMALL_NMAX) return (n + 4) / 2;
-    return adjoint ? stream_adj_tile_bits(dbl) : stream_tile_bits(dbl);
+int stream_one_grad_tile_bits(bool dbl, int n, bool adjoint, int* cmin) {
+    const bool small = !dbl && n >= 14 && n <= SMALL_NMAX;
+    *cmin = small ? 3 : 4;
+    return small ? (n + 4) / 2 : (adjoint ? stream_adj_tile_bits(dbl) : stream_tile_bits(dbl));
 }
 uint64_t stream_one_max_tiles(bool dbl, int n) {
     if (!dbl && n >= SMALL_NMIN && n <= SMALL_NMAX) return 1ull << (n - 10);
@@ -747,7 +773,8 @@ uint64_t stream_one_max_tiles(bool dbl, int n) {
 }
 
 // The forward passes of a single state (see above); other sizes and types: the batched plan.
-int stream_plan_one(bool dbl, int n, int p, int k, StreamPass* out, int max_out) {
+int stream_plan_one(bool dbl, int n, int p, int k, StreamPass* out, StreamSubs* subs, int max_out) {
+    for (int i = 0; i < max_out; ++i) subs[i].n = 0;
     if (dbl || n < SMALL_NMIN || n > SMALL_NMAX || k > 0) return stream_plan(dbl, n, p, k, out, max_out);
     if (p + 1 > max_out) return -1;
     // blocks of qubits, each cut into windows of at most SMALL_R
@@ -781,12 +808,13 @@ int stream_plan_one(bool dbl, int n, int p, int k, StreamPass* out, int max_out)
                     StreamSub sb{a, ((1 << size) - 1) << (lo - a), l - P.la, l - P.la, 0};
                     const bool opens = i == 0 && q == b.q;
                     sb.phase = opens && (l > P.la || P.ph_first) ? 1 : 0;
-                    if (opens && l > P.la && P.sub[P.nsub - 1].a == sb.a && P.sub[P.nsub - 1].mask == sb.mask) {
-                        P.sub[P.nsub - 1].l1 = sb.l1;      // shared around the cost phase
+                    StreamSubs& L = subs[si];
+                    if (opens && l > P.la && L.sub[L.n - 1].a == sb.a && L.sub[L.n - 1].mask == sb.mask) {
+                        L.sub[L.n - 1].l1 = sb.l1;         // shared around the cost phase
                         continue;
                     }
-                    if (P.nsub == STREAM_MAX_SUB) return -1;
-                    P.sub[P.nsub++] = sb;
+                    if (L.n == STREAM_MAX_SUB) return -1;
+                    L.sub[L.n++] = sb;
                 }
             }
         out[si] = P;
@@ -795,14 +823,13 @@ int stream_plan_one(bool dbl, int n, int p, int k, StreamPass* out, int max_out)
 }
 
 // HBM windows of a layer: window 0 = kind A (qubits 0..tb-1); windows 1.. = kind B chunks of
-// the qubits [tb, n), as equal as possible, each at most tb - 4 qubits (tb - 3 for the small adjoint
-// tiles of a single state).
-int stream_plan(bool dbl, int n, int p, int k, StreamPass* out, int max_out, int tb) {
+// the qubits [tb, n), as equal as possible, each at most tb - cmin qubits (4: runs of at least 128
+// bytes; 3 for the small tiles of a single gradient).
+int stream_plan(bool dbl, int n, int p, int k, StreamPass* out, int max_out, int tb, int cmin) {
     if (tb < 0) tb = stream_tile_bits(dbl);
     if (n <= tb) return -1;
-    const int hmax = tb - (small_tiles(dbl, n, tb) ? 3 : 4);
     const int rest = n - tb;
-    const int nB = (rest + hmax - 1) / hmax;
+    const int nB = stream_windows(n, tb, cmin) - 1;
     int chunk_s[16], chunk_h[16];
     int s0 = tb;
     for (int i = 0; i < nB; ++i) {
@@ -861,18 +888,20 @@ static StreamInst<T> one_of(const void* one) {
 
 template <typename T, int R, int NTH, bool TOPK>
 static cudaError_t pass_t(const StreamPass& P, const void* insts, int count, int grid, int threads, cudaStream_t st,
-                          const void* one) {
+                          const void* one, const StreamSubs* subs = nullptr) {
     const size_t sm = stream_smem_bytes(sizeof(T) == 8, P.tb);
     const cudaError_t e = cudaFuncSetAttribute(k_stream_pass<T, R, NTH, TOPK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_stream_pass<T, R, NTH, TOPK><<<grid, threads, sm, st>>>(P, static_cast<const StreamInst<T>*>(insts), count, one_of<T>(one));
+    k_stream_pass<T, R, NTH, TOPK><<<grid, threads, sm, st>>>(P, static_cast<const StreamInst<T>*>(insts), count, one_of<T>(one),
+                                                            subs ? *subs : StreamSubs{});
     return cudaGetLastError();
 }
 
 cudaError_t launch_stream_pass(bool dbl, const StreamPass& P, const void* insts, int count,
-                               int grid, cudaStream_t st, const void* one) {
+                               int grid, cudaStream_t st, const void* one, const StreamSubs* subs) {
     if (dbl) return pass_t<double, Num<double>::RB, 256, true>(P, insts, count, grid, 256, st, one);
-    if (P.nsub > 0) return pass_t<float, SMALL_R, 256, false>(P, insts, count, grid, 1 << (P.tb - SMALL_R), st, one);
+    if (subs && subs->n > 0)
+        return pass_t<float, SMALL_R, 256, false>(P, insts, count, grid, 1 << (P.tb - SMALL_R), st, one, subs);
     if (small_tiles(dbl, P.n, P.tb) && P.k == 0)
         return pass_t<float, SMALL_RA, 256, false>(P, insts, count, grid, 1 << (P.tb - SMALL_RA), st, one);
     if (P.k == 0) return pass_t<float, Num<float>::RB, 256, false>(P, insts, count, grid, 256, st, one);
@@ -880,6 +909,17 @@ cudaError_t launch_stream_pass(bool dbl, const StreamPass& P, const void* insts,
 }
 
 bool stream_finalize_two_level(uint64_t ntiles, int k) { return k > 0 && ntiles > FIN_CHUNK; }
+
+cudaError_t launch_stream_topk_chunks(const void* insts, int count, uint64_t ntiles, int k, cudaStream_t st) {
+    const dim3 grid((unsigned)((ntiles + FIN_CHUNK - 1) / FIN_CHUNK), (unsigned)count);
+    k_stream_topk_chunks<float><<<grid, 256, 0, st>>>(static_cast<const StreamInst<float>*>(insts), count, ntiles, k, StreamInst<float>{});
+    return cudaGetLastError();
+}
+
+cudaError_t launch_stream_finalize_mixed(const void* insts, int count, cudaStream_t st) {
+    k_stream_finalize<float><<<count, 256, 0, st>>>(static_cast<const StreamInst<float>*>(insts), count, 0, 0, 1, StreamInst<float>{});
+    return cudaGetLastError();
+}
 
 cudaError_t launch_stream_finalize(bool dbl, const void* insts, int count, uint64_t ntiles, int k,
                                    cudaStream_t st, const void* one) {
@@ -925,8 +965,7 @@ static cudaError_t launch_rows(int n, int count, const void* Q, void* E, const v
     return cudaSuccess;
 }
 
-// Batches: tile form up to 2^22 energies per instance, row form above.
-constexpr int ENERGY_TILE_NMAX = 22;
+// Batches: tile form up to 2^22 energies per instance (ENERGY_TILE_NMAX), row form above.
 
 template <typename T>
 static cudaError_t launch_tiles(int n, int count, const void* Q, void* E, const void* insts, cudaStream_t st) {
@@ -935,11 +974,24 @@ static cudaError_t launch_tiles(int n, int count, const void* Q, void* E, const 
     for (int c0 = 0; c0 < count; c0 += 65535) {          // grid.y limit
         const int cy = count - c0 < 65535 ? count - c0 : 65535;
         k_energy_tile<T><<<dim3(gx, (unsigned)cy), 256, 0, st>>>(n, static_cast<const T*>(Q), static_cast<T*>(E),
-                                                                 in ? in + c0 : nullptr);
+                                                                 in ? in + c0 : nullptr, EnergyRuns{});
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+cudaError_t launch_energy_mixed(const void* insts, int runs, const int* n, const int* first, const int* count,
+                                cudaStream_t st) {
+    EnergyRuns er{};
+    for (int i = 0; i < runs; ++i) {
+        er.n[i] = n[i];
+        er.first[i] = first[i];
+        er.b0[i + 1] = er.b0[i] + ((uint32_t)count[i] << (n[i] > ETB ? n[i] - ETB : 0));
+    }
+    er.runs = runs;
+    k_energy_tile<float><<<er.b0[runs], 256, 0, st>>>(0, nullptr, nullptr, static_cast<const StreamInst<float>*>(insts), er);
+    return cudaGetLastError();
 }
 
 template <typename T>
@@ -994,14 +1046,11 @@ cudaError_t launch_stream_adj_pass(bool dbl, const StreamPass& P, int si, bool l
     return adj_t<float, Num<float>::RB_ADJ, ADJ_THREADS>(P, si, lam_first, store, insts, count, grid, ADJ_THREADS, st, one);
 }
 
-cudaError_t launch_stream_grad_reduce(bool dbl, const StreamPass* passes, int S, const void* insts,
-                                      int count, uint64_t ntiles, cudaStream_t st, const void* one) {
-    if (S > 256) return cudaErrorInvalidValue;
-    PassLayers pl;
-    int p = 1;   // layers of the group (uniform for a launch)
-    for (int i = 0; i < S; ++i) { pl.la[i] = passes[i].la; pl.lb[i] = passes[i].lb; p = pl.lb[i] + 1 > p ? pl.lb[i] + 1 : p; }
-    if (dbl) k_stream_grad_reduce<double><<<dim3((unsigned)count, (unsigned)p), 256, 0, st>>>(pl, S, static_cast<const StreamInst<double>*>(insts), count, ntiles, one_of<double>(one));
-    else k_stream_grad_reduce<float><<<dim3((unsigned)count, (unsigned)p), 256, 0, st>>>(pl, S, static_cast<const StreamInst<float>*>(insts), count, ntiles, one_of<float>(one));
+cudaError_t launch_stream_grad_reduce(bool dbl, int tb, int cmin, int pmax, const void* insts, int count, cudaStream_t st,
+                                      const void* one) {
+    const dim3 grid((unsigned)count, (unsigned)pmax);
+    if (dbl) k_stream_grad_reduce<double><<<grid, 256, 0, st>>>(tb, cmin, static_cast<const StreamInst<double>*>(insts), count, one_of<double>(one));
+    else k_stream_grad_reduce<float><<<grid, 256, 0, st>>>(tb, cmin, static_cast<const StreamInst<float>*>(insts), count, one_of<float>(one));
     return cudaGetLastError();
 }
 

@@ -2,8 +2,11 @@
 // passes walk the whole state in HBM; Section IV, Eq. 2: cost phase and mixer per layer, <C> and
 // the top-k bitstrings at the end).
 //
-// Each pass is one persistent launch, two CTAs per SM, walking the tiles of every instance of its
-// plan group. A tile is 2^13 amplitudes, moved between HBM and shared memory by TMA
+// A launch is persistent, two CTAs per SM, walking the tiles of one pass of every instance of its
+// plan groups: groups of other sizes and depths share the launches (segments, TsSeg), so that an
+// uneven batch takes as many launches as its longest group has passes and small states fill the
+// SMs that one group alone would leave idle (a launch per group and pass: 48 uneven training
+// instances 7.95 ms a step, 16 served jobs 800 us a tick; shared launches: 5.70 ms, 365 us). A tile is 2^13 amplitudes, moved between HBM and shared memory by TMA
 // (cp.async.bulk.tensor; the state with the 128-byte swizzle, its energies unswizzled, the
 // energies only in passes with a cost phase or the final reductions). A CTA loads its next tile
 // as soon as the bulk store of the current one has read the buffer, and the other CTA of the SM
@@ -35,17 +38,16 @@ using namespace tma;
 constexpr int TB = 13;
 constexpr uint32_t TD = 1u << TB;
 constexpr int NT = TMA_NT;
-constexpr int NSTAGE = 1;
 
 struct TsOff {
-    size_t stage[NSTAGE], estage[NSTAGE], lc, red, wbound, wb, cnt, cand, out, wlists, run, mbar, total;
+    size_t stage[1], estage[1], lc, red, wbound, wb, cnt, cand, out, wlists, run, mbar, total;
 };
 __host__ __device__ inline size_t ts_al(size_t x) { return (x + 15) & ~(size_t)15; }
 __host__ __device__ inline TsOff ts_offsets() {
     TsOff o{};
     size_t x = 0;
-    for (int s = 0; s < NSTAGE; ++s) { o.stage[s] = x; x += (size_t)TD * 8; }   // 1024-aligned at run time
-    for (int s = 0; s < NSTAGE; ++s) { o.estage[s] = x; x += (size_t)TD * 4; }
+    for (int s = 0; s < 1; ++s) { o.stage[s] = x; x += (size_t)TD * 8; }   // 1024-aligned at run time
+    for (int s = 0; s < 1; ++s) { o.estage[s] = x; x += (size_t)TD * 4; }
     o.lc = x; x = ts_al(x + 64 * sizeof(LayerConst<float>));
     o.red = x; x = ts_al(x + 32 * sizeof(float));
     o.wbound = x; x = ts_al(x + sizeof(float));
@@ -55,7 +57,7 @@ __host__ __device__ inline TsOff ts_offsets() {
     o.out = x; x = ts_al(x + 16 * sizeof(TopEnt));
     o.wlists = x; x = ts_al(x + (NT / 32) * 32 * sizeof(TopEnt));
     o.run = x; x = ts_al(x + 16 * sizeof(TopEnt));
-    o.mbar = x; x = ts_al(x + NSTAGE * sizeof(uint64_t));
+    o.mbar = x; x = ts_al(x + sizeof(uint64_t));
     o.total = x + 1024;
     return o;
 }
@@ -318,17 +320,80 @@ __device__ __forceinline__ void tile_store(const TsPass& T, const CUtensorMap* m
     }
 }
 
-__global__ void __launch_bounds__(NT, 2) k_tstream_pass(const StreamPass P, const TsPass T,
-                                                       const StreamInst<float>* __restrict__ insts, int count,
-                                                       const CUtensorMap* __restrict__ maps, unsigned* status) {
+// The segment a CTA works on: a group's pass, formed from the group's numbers by one thread.
+struct SegPass {
+    uint32_t tile0;
+    int si, lam_first;
+    StreamPass P;
+    TsPass T;
+    const StreamInst<float>* insts;
+    const CUtensorMap* maps;
+};
+__host__ __device__ __noinline__ void expand_segment(const TsGroup* groups, const TsSeg& seg, SegPass* x) {
+    const TsGroup& g = groups[seg.group];
+    const int s = seg.pass, W = g.W;
+    int l = 0, pos = s;
+    if (s >= W) {
+        l = 1 + (s - W) / (W - 1);
+        pos = 1 + (s - W) % (W - 1);
+    }
+    const int w = (l & 1) ? W - 1 - pos : pos;
+    StreamPass P{};
+    P.n = g.n;
+    P.tb = g.tb;
+    P.la = l;
+    P.lb = (pos == W - 1 && l + 1 < g.p) ? l + 1 : l;
+    P.ph_first = P.init = s == 0;
+    P.fin = s == g.S - 1;
+    P.k = P.fin ? g.k : 0;
+    P.kind = w > 0;
+    P.h = w > 0 ? g.ch[w - 1] : 0;
+    P.s = w > 0 ? g.cs[w - 1] : g.tb;
+    P.c = g.tb - P.h;
+    P.need_e = P.ph_first || P.lb > P.la || P.fin;
+    P.keep_frame = P.fin && g.keep_frame;
+    P.no_store = P.fin && g.no_store;
+    TsPass T{};
+    T.maps_per_inst = g.maps_per_inst;
+    T.map = g.adjoint ? 3 * w : w;
+    T.emap = g.adjoint ? T.map + 2 : W + w;
+    if (w == 0) {
+        T.bmode = g.adjoint ? TS_A3 : TS_A;
+    } else {
+        const bool top = P.s + P.h < P.n;
+        T.midbits = P.s - P.c;
+        T.bmode = P.h <= 8 ? (top ? TS_B5 : TS_B4) : (top ? TS_B9_5 : TS_B9_4);
+    }
+    x->tile0 = seg.tile0;
+    x->si = s;
+    x->lam_first = s == g.S - 1;
+    x->P = P;
+    x->T = T;
+    x->insts = g.insts;
+    x->maps = static_cast<const CUtensorMap*>(g.maps);
+}
+// Move on to the segment of tile q. All threads call it, behind a barrier that follows their last
+// use of the segment.
+__device__ __forceinline__ void advance_segment(const TsGroup* groups, const TsSeg* segs, int nseg, uint32_t total,
+                                                uint32_t q, int& sg, uint32_t& send, SegPass* cur) {
+    do {
+        ++sg;
+        send = sg + 1 < nseg ? segs[sg + 1].tile0 : total;
+    } while (q >= send);
+    if (threadIdx.x == 0) expand_segment(groups, segs[sg], cur);
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(NT, 2) k_tstream_pass(const TsGroup* __restrict__ groups,
+                                                       const TsSeg* __restrict__ segs, int nseg, uint32_t total,
+                                                       unsigned* status) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
+    __shared__ SegPass cur, nxt;   // nxt: thread 0's, for loads of the next segment's first tile
     const uint32_t raw = saddr(sm_raw);
     unsigned char* sm = sm_raw + (((raw + 1023u) & ~1023u) - raw);
     const TsOff o = ts_offsets();
-    // stage s at stage0 + s * TD (state) and estage0 + s * TD (energies): no arrays, so that no
-    // dynamic index sends them to local memory
-    float2* const stage0 = reinterpret_cast<float2*>(sm + o.stage[0]);
-    float* const estage0 = reinterpret_cast<float*>(sm + o.estage[0]);
+    float2* const sp = reinterpret_cast<float2*>(sm + o.stage[0]);
+    float* const sE = reinterpret_cast<float*>(sm + o.estage[0]);
     LayerConst<float>* lc = reinterpret_cast<LayerConst<float>*>(sm + o.lc);
     float* red = reinterpret_cast<float*>(sm + o.red);
     TileTopk ts;
@@ -338,70 +403,78 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const StreamPass P, cons
     ts.out = reinterpret_cast<TopEnt*>(sm + o.out);
     ts.wlists = reinterpret_cast<TopEnt*>(sm + o.wlists);
     uint64_t* mbar = reinterpret_cast<uint64_t*>(sm + o.mbar);
-    if (threadIdx.x == 0)
-        for (int s = 0; s < NSTAGE; ++s) mbar_init(&mbar[s], 1);
+    if (threadIdx.x == 0) mbar_init(mbar, 1);
     __syncthreads();
 
-    const int tbits = P.n - TB;                 // tiles of an instance: 2^tbits
-    const uint64_t ntiles = 1ull << tbits;
-    const uint64_t total = ntiles * (uint64_t)count;
-    const uint64_t first = blockIdx.x, step = gridDim.x;
-    const int nmine = first < total ? (int)((total - 1 - first) / step + 1) : 0;
-    const bool loads = !P.init || P.need_e;   // the init pass loads only the energies
-    const bool store = !P.fin || !P.no_store;
-    const bool pf = P.init || !store;
-    uint32_t parity = 0;   // bit s: parity of the next wait on stage s
+    const StreamPass& P = cur.P;
+    const TsPass& T = cur.T;
+    uint32_t parity = 0;
     bool ok = true;
-    // the energies first (their buffer is never stored from), then, once the last tile's store
-    // has read the state buffer (wait_store), the state
-    auto issue = [&](int k, bool wait_store) {
-        const uint64_t q = first + (uint64_t)k * step;
-        const int ii = (int)(q >> tbits);
-        const uint64_t tau = q & (ntiles - 1);
-        const int s = k % NSTAGE;
-        const CUtensorMap* m = maps + (size_t)ii * T.maps_per_inst;
-        mbar_expect_tx(&mbar[s], (P.init ? 0u : TD * 8) + (P.need_e ? TD * 4 : 0u));
-        if (P.need_e) tile_load(T, m + T.emap, estage0 + (size_t)s * TD, tau, &mbar[s]);
-        if (!P.init) {
+    int sg = -1;
+    uint32_t send = 0;        // first tile past the segment
+    if (blockIdx.x < total) advance_segment(groups, segs, nseg, total, blockIdx.x, sg, send, &cur);
+    // Thread 0: the loads of tile q (segment S). The energies first (their buffer is never stored
+    // from), then, once the last tile's store has read the state buffer (wait_store), the state.
+    auto issue = [&](uint32_t q, bool wait_store) {
+        const SegPass* S = &cur;
+        if (q >= send) {
+            int j = sg + 1;
+            while (j + 1 < nseg && q >= segs[j + 1].tile0) ++j;
+            expand_segment(groups, segs[j], &nxt);
+            S = &nxt;
+        }
+        const StreamPass& p = S->P;
+        const TsPass& t = S->T;
+        if (p.init && !p.need_e) return;
+        const int tbits = p.n - TB;
+        const uint32_t ql = q - S->tile0, tmask = (1u << tbits) - 1u;
+        const CUtensorMap* m = S->maps + (size_t)(ql >> tbits) * t.maps_per_inst;
+        mbar_expect_tx(mbar, (p.init ? 0u : TD * 8) + (p.need_e ? TD * 4 : 0u));
+        if (p.need_e) tile_load(t, m + t.emap, sE, ql & tmask, mbar);
+        if (!p.init) {
             if (wait_store) bulk_wait_read();
-            tile_load(T, m + T.map, stage0 + (size_t)s * TD, tau, &mbar[s]);
+            tile_load(t, m + t.map, sp, ql & tmask, mbar);
         }
         // the tile after it towards L2, a tile's compute ahead of its own load (in the passes
         // that store no state: with the state stores in flight it slowed the others down)
-        if (pf && k + 1 < nmine) {
-            const uint64_t q1 = q + step;
-            const CUtensorMap* m1 = maps + (size_t)(q1 >> tbits) * T.maps_per_inst;
-            if (P.need_e) tile_prefetch(T, m1 + T.emap, q1 & (ntiles - 1));
-            if (!P.init) tile_prefetch(T, m1 + T.map, q1 & (ntiles - 1));
+        const uint32_t q1 = ql + gridDim.x;
+        const uint32_t end = S == &cur ? send - S->tile0 : 0u;
+        if ((p.init || (p.fin && p.no_store)) && q1 < end) {
+            const CUtensorMap* m1 = S->maps + (size_t)(q1 >> tbits) * t.maps_per_inst;
+            if (p.need_e) tile_prefetch(t, m1 + t.emap, q1 & tmask);
+            if (!p.init) tile_prefetch(t, m1 + t.map, q1 & tmask);
         }
     };
-    if (loads && nmine > 0 && threadIdx.x == 0) issue(0, false);
+    if (blockIdx.x < total && threadIdx.x == 0) issue(blockIdx.x, false);
     const float *cur_g = nullptr, *cur_b = nullptr;
-    int cur_p = 0;
+    int cur_p = 0, cur_n = 0;
     TopEnt* run = reinterpret_cast<TopEnt*>(sm + o.run);
     bool run_valid = false;   // the run list holds this CTA's best k of the current instance so far
-    for (int k = 0; k < nmine; ++k) {
-        const uint64_t q = first + (uint64_t)k * step;
-        const int ii = (int)(q >> tbits);
-        const uint64_t tau = q & (ntiles - 1);
-        const int s = k % NSTAGE;
-        const StreamInst<float>& I = insts[ii];
-        if (I.gamma != cur_g || I.beta != cur_b || I.p != cur_p) {
+    for (uint32_t q = blockIdx.x; q < total; q += gridDim.x) {
+        if (q >= send) {
+            __syncthreads();
+            advance_segment(groups, segs, nseg, total, q, sg, send, &cur);
+        }
+        const int tbits = P.n - TB;                 // tiles of an instance: 2^tbits
+        const uint32_t ql = q - cur.tile0;
+        const int ii = (int)(ql >> tbits);
+        const uint64_t tau = ql & ((1u << tbits) - 1u);
+        const bool store = !P.fin || !P.no_store;
+        const StreamInst<float>& I = cur.insts[ii];
+        if (I.gamma != cur_g || I.beta != cur_b || I.p != cur_p || P.n != cur_n) {
             __syncthreads();
             set_layer_consts<float>(lc, I.gamma, I.beta, I.p, P.n, false);
             cur_g = I.gamma;
             cur_b = I.beta;
             cur_p = I.p;
+            cur_n = P.n;
         }
-        if (loads) {
-            if (ok) ok = mbar_wait_bounded(&mbar[s], (parity >> s) & 1u);
-            parity ^= 1u << s;
-            // the init pass loads only the energies, issued before the last tile's store had read
-            // the state buffer: that read must be over before this tile writes the buffer
-            if (P.init && k >= 1 && threadIdx.x == 0) bulk_wait_read();
-        } else if (k >= 1 && threadIdx.x == 0) {
-            bulk_wait_read();   // the buffer's earlier store has read it
+        if (!P.init || P.need_e) {
+            if (ok) ok = mbar_wait_bounded(mbar, parity);
+            parity ^= 1u;
         }
+        // a pass that loads no state may meet a store of the last tile still reading the buffer
+        if (P.init && threadIdx.x == 0) bulk_wait_read();
         ok = __syncthreads_and(ok);
         Geo geo;
         geo.kindA = P.kind == 0;
@@ -415,8 +488,6 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const StreamPass P, cons
             const uint64_t mid = tau & ((1ull << midbits) - 1ull), top = tau >> midbits;
             geo.zt = (mid << P.c) | (top << (P.s + P.h));
         }
-        float2* sp = stage0 + (size_t)s * TD;
-        const float* sE = estage0 + (size_t)s * TD;
         float accp = 0.0f, pmax = -1.0f;
         if (geo.kindA) tile_kind_a(sp, geo, P, lc, sE, (float)I.amp0, accp, pmax);
         else kind_b_dispatch(P.h, sp, geo, P, lc, sE, (float)I.amp0, accp, pmax);
@@ -503,8 +574,8 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const StreamPass P, cons
                     }
                 }
                 // this tile's slot: the list when it is the CTA's last tile of the instance
-                const uint64_t qn = q + step;
-                const bool last_of_inst = k + 1 >= nmine || (int)(qn >> tbits) != ii;
+                const uint32_t qn = q + gridDim.x;
+                const bool last_of_inst = qn >= send || (int)((qn - cur.tile0) >> tbits) != ii;
                 if (threadIdx.x < (unsigned)kk) {
                     const TopEnt e = last_of_inst ? run[threadIdx.x] : TopEnt{-1.0, 0xffffffffu};
                     I.part_topp[tau * kk + threadIdx.x] = e.p;
@@ -523,7 +594,7 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const StreamPass P, cons
             fence_async_smem();
             __syncthreads();
             if (threadIdx.x == 0) {
-                tile_store(T, maps + (size_t)ii * T.maps_per_inst + T.map, sp, tau);
+                tile_store(T, cur.maps + (size_t)ii * T.maps_per_inst + T.map, sp, tau);
                 bulk_commit();
             }
         } else {
@@ -532,7 +603,7 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const StreamPass P, cons
         }
         // the next tile's loads: the energies at once, the state once this tile's store has read
         // the buffer (the init pass loads only the energies)
-        if (loads && k + 1 < nmine && threadIdx.x == 0 && ok) issue(k + 1, true);
+        if (q + gridDim.x < total && threadIdx.x == 0 && ok) issue(q + gridDim.x, true);
     }
     if (threadIdx.x == 0) {
         bulk_wait_all();
@@ -568,11 +639,11 @@ __host__ __device__ inline TaOff ta_offsets() {
     return o;
 }
 
-__global__ void __launch_bounds__(NT, 2) k_tstream_adj_pass(const StreamPass P, const TsPass T, int si,
-                                                           int lam_first, int store,
-                                                           const StreamInst<float>* __restrict__ insts, int count,
-                                                           const CUtensorMap* __restrict__ maps, unsigned* status) {
+__global__ void __launch_bounds__(NT, 2) k_tstream_adj_pass(const TsGroup* __restrict__ groups,
+                                                           const TsSeg* __restrict__ segs, int nseg, uint32_t total,
+                                                           unsigned* status) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
+    __shared__ SegPass cur, nxt;   // nxt: thread 0's, for loads of the next segment's first tile
     const uint32_t raw = saddr(sm_raw);
     unsigned char* sm = sm_raw + (((raw + 1023u) & ~1023u) - raw);
     const TaOff o = ta_offsets();
@@ -582,45 +653,63 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_adj_pass(const StreamPass P, 
     LayerConst<float>* lc = reinterpret_cast<LayerConst<float>*>(sm + o.lc);
     double* red = reinterpret_cast<double*>(sm + o.red);
     uint64_t* mbar = reinterpret_cast<uint64_t*>(sm + o.mbar);
-    if (threadIdx.x == 0) mbar_init(mbar, 1);
-    __syncthreads();
-
-    constexpr int RA = Num<float>::RB_ADJ;
-    const int tbits = P.n - TSA_TB;             // tiles of an instance: 2^tbits (fewer than 2^32 in all)
-    const uint32_t total = (uint32_t)count << tbits, tmask = (1u << tbits) - 1u;
-    const bool need_e = lam_first || P.ph_first || P.lb > P.la;
-    uint32_t parity = 0;
-    bool ok = true;
-    // the energies first (never stored from), then, once the last tile's stores have read the
-    // state buffers (wait_store), psi and lam
-    auto issue = [&](uint32_t q, bool wait_store) {
-        const uint32_t tau = q & tmask;
-        const CUtensorMap* m = maps + (size_t)(q >> tbits) * T.maps_per_inst;
-        mbar_expect_tx(mbar, TDA * 8 + (lam_first ? 0u : TDA * 8) + (need_e ? TDA * 4 : 0u));
-        if (need_e) tile_load(T, m + T.emap, sE, tau, mbar);
-        if (wait_store) bulk_wait_read();
-        tile_load(T, m + T.map, spsi, tau, mbar);
-        if (!lam_first) tile_load(T, m + T.map + 1, slam, tau, mbar);
-        // the tile after it towards L2, a tile's compute ahead of its own loads
-        const uint32_t q1 = q + gridDim.x;
-        if (q1 < total) {
-            const CUtensorMap* m1 = maps + (size_t)(q1 >> tbits) * T.maps_per_inst;
-            if (need_e) tile_prefetch(T, m1 + T.emap, q1 & tmask);
-            tile_prefetch(T, m1 + T.map, q1 & tmask);
-            if (!lam_first) tile_prefetch(T, m1 + T.map + 1, q1 & tmask);
-        }
-    };
-    if (blockIdx.x < total && threadIdx.x == 0) issue(blockIdx.x, false);
     // the parameters the constants belong to, in shared memory: the sub-passes need the registers
     __shared__ const float *cur_g, *cur_b;
     __shared__ int cur_p;
-    if (threadIdx.x == 0) cur_p = 0;
+    if (threadIdx.x == 0) {
+        mbar_init(mbar, 1);
+        cur_p = 0;
+    }
     __syncthreads();
+
+    constexpr int RA = Num<float>::RB_ADJ;
+    const StreamPass& P = cur.P;
+    const TsPass& T = cur.T;
+    uint32_t parity = 0;
+    bool ok = true;
+    int sg = -1;
+    uint32_t send = 0;
+    if (blockIdx.x < total) advance_segment(groups, segs, nseg, total, blockIdx.x, sg, send, &cur);
+    // the energies first (never stored from), then, once the last tile's stores have read the
+    // state buffers (wait_store), psi and lam
+    auto issue = [&](uint32_t q, bool wait_store) {
+        const SegPass* S = &cur;
+        if (q >= send) {
+            int j = sg + 1;
+            while (j + 1 < nseg && q >= segs[j + 1].tile0) ++j;
+            expand_segment(groups, segs[j], &nxt);
+            S = &nxt;
+        }
+        const TsPass& t = S->T;
+        const bool lam_first = S->lam_first, need_e = lam_first || S->P.ph_first || S->P.lb > S->P.la;
+        const int tbits = S->P.n - TSA_TB;
+        const uint32_t ql = q - S->tile0, tmask = (1u << tbits) - 1u, tau = ql & tmask;
+        const CUtensorMap* m = S->maps + (size_t)(ql >> tbits) * t.maps_per_inst;
+        mbar_expect_tx(mbar, TDA * 8 + (lam_first ? 0u : TDA * 8) + (need_e ? TDA * 4 : 0u));
+        if (need_e) tile_load(t, m + t.emap, sE, tau, mbar);
+        if (wait_store) bulk_wait_read();
+        tile_load(t, m + t.map, spsi, tau, mbar);
+        if (!lam_first) tile_load(t, m + t.map + 1, slam, tau, mbar);
+        // the tile after it towards L2, a tile's compute ahead of its own loads
+        const uint32_t q1 = ql + gridDim.x;
+        if (S == &cur && q1 < send - S->tile0) {
+            const CUtensorMap* m1 = S->maps + (size_t)(q1 >> tbits) * t.maps_per_inst;
+            if (need_e) tile_prefetch(t, m1 + t.emap, q1 & tmask);
+            tile_prefetch(t, m1 + t.map, q1 & tmask);
+            if (!lam_first) tile_prefetch(t, m1 + t.map + 1, q1 & tmask);
+        }
+    };
+    if (blockIdx.x < total && threadIdx.x == 0) issue(blockIdx.x, false);
     const TileRef<float> tile{spsi, slam, sE, TSA_TB};
     for (uint32_t q = blockIdx.x; q < total; q += gridDim.x) {
-        const uint32_t tau = q & tmask;
-        const StreamInst<float>& I = insts[q >> tbits];
-        if (I.p != cur_p || I.gamma != cur_g || I.beta != cur_b) {
+        if (q >= send) {
+            __syncthreads();
+            advance_segment(groups, segs, nseg, total, q, sg, send, &cur);
+        }
+        const int tbits = P.n - TSA_TB;
+        const uint32_t ql = q - cur.tile0, tau = ql & ((1u << tbits) - 1u);
+        const StreamInst<float>& I = cur.insts[ql >> tbits];
+        if (I.p != cur_p || I.gamma != cur_g || I.beta != cur_b) {   // (the adjoint's constants do not depend on n)
             __syncthreads();
             set_layer_consts<float>(lc, I.gamma, I.beta, I.p, P.n, true);
             if (threadIdx.x == 0) { cur_g = I.gamma; cur_b = I.beta; cur_p = I.p; }
@@ -629,7 +718,7 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_adj_pass(const StreamPass P, 
         if (ok) ok = mbar_wait_bounded(mbar, parity);
         parity ^= 1u;
         float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        bool first_sub = lam_first;
+        bool first_sub = cur.lam_first;
         Snake sn(P.lb - P.la + 1, P.la, P.ph_first, P.kind == 0 ? 0 : P.c, TSA_TB, TSA_TB, RA, true);
         sn.to_last();
         for (;; sn.prev()) {
@@ -639,14 +728,14 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_adj_pass(const StreamPass P, 
             __syncthreads();
             if (sn.first()) break;
         }
-        double* out = I.part_grad + (((uint64_t)si << tbits) + tau) * 4;
+        double* out = I.part_grad + (((uint64_t)cur.si << tbits) + tau) * 4;
         const double v = block_sum4((double)acc[0], (double)acc[1], (double)acc[2], (double)acc[3], red);
         if (threadIdx.x < 4) out[threadIdx.x] = v;
-        if (store) {
+        if (cur.si > 0) {   // the first pass's states are not needed any more
             fence_async_smem();
             __syncthreads();
             if (threadIdx.x == 0) {
-                const CUtensorMap* m = maps + (size_t)(q >> tbits) * T.maps_per_inst;
+                const CUtensorMap* m = cur.maps + (size_t)(ql >> tbits) * T.maps_per_inst;
                 tile_store(T, m + T.map, spsi, tau);
                 tile_store(T, m + T.map + 1, slam, tau);
                 bulk_commit();
@@ -755,13 +844,25 @@ bool tstream_encode_maps(const StreamPass& P, void* psi, void* E, void* psi_map,
            encode_shape(P, E, 1, static_cast<CUtensorMap*>(e_map));
 }
 
-cudaError_t launch_tstream_pass(const StreamPass& P, const TsPass& T, const void* insts, int count,
-                                const void* maps, int grid, unsigned* status, cudaStream_t st) {
+void tstream_group_windows(const StreamPass* passes, int S, TsGroup* g) {
+    g->S = S;
+    g->W = 1;
+    for (int i = 0; i < 4; ++i) g->cs[i] = g->ch[i] = 0;
+    // the first pass of every window, in layer 0: contiguous, then the chunks by start qubit
+    for (int i = 0; i < S && passes[i].la == 0; ++i)
+        if (passes[i].kind == 1 && g->W <= 4) {
+            g->cs[g->W - 1] = passes[i].s;
+            g->ch[g->W - 1] = passes[i].h;
+            ++g->W;
+        }
+}
+
+cudaError_t launch_tstream_pass(const TsGroup* groups, const TsSeg* segs, int nseg, uint32_t total, int grid,
+                                unsigned* status, cudaStream_t st) {
     const size_t sm = tstream_smem_bytes();
     cudaError_t e = cudaFuncSetAttribute(k_tstream_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_tstream_pass<<<grid, NT, sm, st>>>(P, T, static_cast<const StreamInst<float>*>(insts), count,
-                                         static_cast<const CUtensorMap*>(maps), status);
+    k_tstream_pass<<<grid, NT, sm, st>>>(groups, segs, nseg, total, status);
     return cudaGetLastError();
 }
 
@@ -791,15 +892,12 @@ bool tstream_encode_adj_maps(const StreamPass& P, void* psi, void* lam, void* E,
            encode_shape(P, E, 1, reinterpret_cast<CUtensorMap*>(b + 2 * TS_MAP_BYTES));
 }
 
-cudaError_t launch_tstream_adj_pass(const StreamPass& P, const TsPass& T, int si, bool lam_first, bool store,
-                                    const void* insts, int count, const void* maps, int grid, unsigned* status,
-                                    cudaStream_t st) {
+cudaError_t launch_tstream_adj_pass(const TsGroup* groups, const TsSeg* segs, int nseg, uint32_t total, int grid,
+                                    unsigned* status, cudaStream_t st) {
     const size_t sm = tstream_adj_smem_bytes();
     cudaError_t e = cudaFuncSetAttribute(k_tstream_adj_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_tstream_adj_pass<<<grid, NT, sm, st>>>(P, T, si, lam_first ? 1 : 0, store ? 1 : 0,
-                                             static_cast<const StreamInst<float>*>(insts), count,
-                                             static_cast<const CUtensorMap*>(maps), status);
+    k_tstream_adj_pass<<<grid, NT, sm, st>>>(groups, segs, nseg, total, status);
     return cudaGetLastError();
 }
 

@@ -80,10 +80,11 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 // Workspace of a streaming gradient: psi and lam (2^n complex each), the forward scratch and the
 // per-pass, per-tile gradient partials of the adjoint plan (4 doubles).
 size_t stream_grad_bytes(bool dbl, int n, int p) {
-    const int tba = stream_one_grad_tile_bits(dbl, n, true);
     if (n <= stream_tile_bits(dbl)) return 0;
+    int cmin;
+    const int tba = stream_one_grad_tile_bits(dbl, n, true, &cmin);
     StreamPass tmp[256];
-    const int S = stream_plan(dbl, n, p, 0, tmp, 256, tba);
+    const int S = stream_plan(dbl, n, p, 0, tmp, 256, tba, cmin);
     if (S < 0) return 0;
     const size_t D = (size_t)1 << n, nta = (size_t)1 << (n - tba), cs = dbl ? 16 : 8;
     return 2 * align256(D * cs) + stream_scratch_bytes(dbl, n, 0) + align256((size_t)S * nta * 4 * sizeof(double));
@@ -126,12 +127,15 @@ qaoa_status run_stream_one(qaoa_ctx* c, int n, int p, const T* gamma, const T* b
     if (!init_plus)
         return fail(QAOA_E_UNSUPPORTED, "streaming tier (n=%d) starts from |+> only", n);
     StreamPass passes[256];
-    const int S = stream_plan_one(dbl, n, p, k, passes, 256);
+    StreamSubs subs[256];
+    const int S = stream_plan_one(dbl, n, p, k, passes, subs, 256);
     if (S < 0) return fail(QAOA_E_INVALID, "no streaming plan for n=%d p=%d", n, p);
     const uint64_t nt = 1ull << (n - passes[S - 1].tb);   // tiles of the last pass
     char* w = static_cast<char*>(c->ws) + ws_off;
     StreamInst<T> I{};
+    I.n = n;
     I.p = p;
+    I.k = 0;
     I.amp0 = exp2(-0.5 * n);
     I.gamma = gamma;
     I.beta = beta;
@@ -144,7 +148,8 @@ qaoa_status run_stream_one(qaoa_ctx* c, int n, int p, const T* gamma, const T* b
     I.expect = expect;
     I.topk_idx = tidx;
     I.topk_prob = tprob;
-    for (int s = 0; s < S; ++s) CK(launch_stream_pass(dbl, passes[s], nullptr, 1, one_grid(c, dbl, passes[s]), st, &I));
+    for (int s = 0; s < S; ++s)
+        CK(launch_stream_pass(dbl, passes[s], nullptr, 1, one_grid(c, dbl, passes[s]), st, &I, &subs[s]));
     if (expect || (k > 0 && tidx)) CK(launch_stream_finalize(dbl, nullptr, 1, nt, k, st, &I));
     return QAOA_OK;
 }
@@ -156,15 +161,18 @@ qaoa_status grad_stream_one(qaoa_ctx* c, int n, int p, const T* gamma, const T* 
     qaoa_status q = ensure_ws(c, stream_grad_bytes(dbl, n, p));
     if (q) return q;
     StreamPass passes[256];
-    const int tb = stream_one_grad_tile_bits(dbl, n, false);
-    const int S = stream_plan(dbl, n, p, 0, passes, 256, tb);
+    int cmin;
+    const int tb = stream_one_grad_tile_bits(dbl, n, false, &cmin);
+    const int S = stream_plan(dbl, n, p, 0, passes, 256, tb, cmin);
     if (S < 0) return fail(QAOA_E_INVALID, "no streaming plan for n=%d p=%d", n, p);
     passes[S - 1].keep_frame = 1;
     const uint64_t nt = 1ull << (n - tb), D = 1ull << n;
     const size_t cs = sizeof(typename qaoa::Num<T>::C);
     char* w = static_cast<char*>(c->ws);
     StreamInst<T> I{};
+    I.n = n;
     I.p = p;
+    I.k = 0;
     I.amp0 = exp2(-0.5 * n);
     I.gamma = gamma;
     I.beta = beta;
@@ -180,8 +188,8 @@ qaoa_status grad_stream_one(qaoa_ctx* c, int n, int p, const T* gamma, const T* 
     I.dgamma = dgamma;
     I.dbeta = dbeta;
     StreamPass apasses[256];
-    const int tba = stream_one_grad_tile_bits(dbl, n, true);
-    const int SA = stream_plan(dbl, n, p, 0, apasses, 256, tba);
+    const int tba = stream_one_grad_tile_bits(dbl, n, true, &cmin);
+    const int SA = stream_plan(dbl, n, p, 0, apasses, 256, tba, cmin);
     if (SA < 0) return fail(QAOA_E_INVALID, "no adjoint plan for n=%d p=%d", n, p);
     const uint64_t nta = 1ull << (n - tba);
     const int agrid = (int)std::min<uint64_t>(nta, (uint64_t)c->nsm * (tba < stream_adj_tile_bits(dbl) ? 4 : 2));
@@ -189,7 +197,7 @@ qaoa_status grad_stream_one(qaoa_ctx* c, int n, int p, const T* gamma, const T* 
     if (expect) CK(launch_stream_finalize(dbl, nullptr, 1, nt, 0, st, &I));
     for (int s = SA - 1; s >= 0; --s)
         CK(launch_stream_adj_pass(dbl, apasses[s], s, s == SA - 1, s > 0, nullptr, 1, agrid, st, &I));
-    CK(launch_stream_grad_reduce(dbl, apasses, SA, nullptr, 1, nta, st, &I));
+    CK(launch_stream_grad_reduce(dbl, tba, cmin, p, nullptr, 1, st, &I));
     return QAOA_OK;
 }
 
@@ -412,6 +420,19 @@ extern "C" qaoa_status qaoa_grad_z(qaoa_ctx* c, int n, int p, const double* g, c
 // Batched plans
 // =============================================================================================
 
+// What the launches of a mix, or of a group that runs by itself, move and count, in launch order.
+struct StrStep {
+    int g0, g1, mix;              // groups [g0, g1); mix < 0: one group by itself
+    bool grad = false;
+    double energy_bytes = 0.0, final_bytes = 0.0, reduce_bytes = 0.0;
+    std::vector<double> pass_bytes, adj_bytes;
+    int kernels = 0;
+};
+
+// Runs of equal n among the groups [g0, g1) for the energy launches: tile-form runs first.
+struct EnergyRun {
+    int n, first, count;
+};
 struct qaoa_plan {
     qaoa_ctx* ctx = nullptr;
     bool dbl = false;
@@ -431,11 +452,23 @@ struct qaoa_plan {
                       int tgrid = 0;   // TMA passes' persistent grid
                       // TMA adjoint passes: per instance three maps (psi, lam, E) per adjoint pass
                       // shape at amaps_off; atsp[i] is adjoint pass i's geometry
-                      bool tadj = false; size_t amaps_off = 0; int amaps_per_inst = 0; std::vector<TsPass> atsp; };
+                      size_t amaps_off = 0; int amaps_per_inst = 0; std::vector<TsPass> atsp; };
+    // Consecutive TMA groups that share their launches: pass s of every group that has one in one
+    // launch, likewise the adjoint passes (from each group's last), energies, finalize and gradient
+    // sums. Their instances follow one another at inst_off.
+    struct Mix { int g0, g1;            // groups [g0, g1) of str
+                 int count = 0, pmax = 0, tgrid = 0;
+                 bool grad = false;
+                 size_t inst_off = 0;
+                 size_t fgrp_off = 0, agrp_off = 0;   // TsGroup arrays, forward and adjoint
+                 struct Launch { size_t seg_off; int nseg; uint32_t total; };
+                 std::vector<Launch> fwd, adj; };
     std::vector<ResGroup> res;
     std::vector<CluGroup> clu;
     std::vector<CsGroup> cs;
     std::vector<StrGroup> str;
+    std::vector<Mix> mix;              // in the order of str; groups in none run by themselves
+    std::vector<StrStep> steps;        // the streaming launches in order
     int kernels = 0;
     bool timing = false;
     std::vector<cudaEvent_t> ev;       // 2 per kernel of one launch
@@ -444,6 +477,114 @@ struct qaoa_plan {
 };
 
 namespace {
+
+std::vector<EnergyRun> energy_runs(const qaoa_plan* P, int g0, int g1) {
+    std::vector<EnergyRun> r;
+    int at = 0;
+    for (int j = g0; j < g1; ++j) {
+        const auto& g = P->str[j];
+        if (!r.empty() && r.back().n == g.n) r.back().count += g.count;
+        else r.push_back(EnergyRun{g.n, at, g.count});
+        at += g.count;
+    }
+    return r;
+}
+
+std::vector<StrStep> str_steps(const qaoa_plan* P) {
+    std::vector<StrStep> out;
+    size_t mi = 0;
+    const int tb = stream_tile_bits(P->dbl), tba = stream_adj_tile_bits(P->dbl);
+    const double rs = P->dbl ? 8.0 : 4.0, cs = 2.0 * rs;
+    for (int i = 0; i < (int)P->str.size();) {
+        StrStep st{};
+        st.g0 = i;
+        st.g1 = i + 1;
+        st.mix = -1;
+        if (mi < P->mix.size() && P->mix[mi].g0 == i) {
+            st.mix = (int)mi;
+            st.g1 = P->mix[mi++].g1;
+        }
+        for (int j = st.g0; j < st.g1; ++j) {
+            const auto& g = P->str[j];
+            const double D = (double)(1ull << g.n), cnt = (double)g.count, nt = (double)(1ull << (g.n - tb));
+            st.energy_bytes += cnt * (D * rs + (double)g.n * g.n * rs);
+            st.pass_bytes.resize(std::max(st.pass_bytes.size(), g.passes.size()), 0.0);
+            for (size_t s = 0; s < g.passes.size(); ++s) {
+                const StreamPass& pass = g.passes[s];
+                st.pass_bytes[s] += cnt * D * ((pass.init ? 0.0 : cs) + (pass.no_store ? 0.0 : cs) + (pass.need_e ? rs : 0.0));
+            }
+            st.final_bytes += cnt * (nt * (sizeof(double) + std::max(g.k, 1) * 12.0) + 8.0 + g.k * 16.0);
+            if (stream_finalize_two_level(1ull << (g.n - tb), g.k)) ++st.kernels;
+            if (g.grad) {
+                // adjoint launches run from each group's last pass: psi and lam read (lam formed in
+                // the first), E read, both written back
+                const size_t SA = g.apasses.size();
+                st.grad = true;
+                st.adj_bytes.resize(std::max(st.adj_bytes.size(), SA), 0.0);
+                for (size_t t = 0; t < SA; ++t)
+                    st.adj_bytes[t] += cnt * D * ((t == 0 ? 1.0 : 2.0) * cs + rs + (t + 1 < SA ? 2.0 * cs : 0.0));
+                st.reduce_bytes += cnt * (double)SA * (double)(1ull << (g.n - tba)) * 32.0;
+            }
+        }
+        int energies = 1;
+        if (st.mix >= 0) {
+            energies = 0;
+            int tiles = 0;
+            for (const EnergyRun& r : energy_runs(P, st.g0, st.g1)) (r.n <= ENERGY_TILE_NMAX ? tiles : energies) += 1;
+            energies += (tiles + ENERGY_RUNS - 1) / ENERGY_RUNS;
+        }
+        st.kernels += energies + (int)st.pass_bytes.size() + 1 + (int)st.adj_bytes.size() + (st.grad ? 1 : 0);
+        out.push_back(st);
+        i = st.g1;
+    }
+    return out;
+}
+
+// The group and segment tables of the plan's shared launches, in the host image of its header
+// (base: the header's device address).
+void plan_mixes(qaoa_plan* P, char* img, char* base) {
+    const int tb = stream_tile_bits(false), tba = stream_adj_tile_bits(false);
+    for (auto& m : P->mix) {
+        TsGroup* fg = reinterpret_cast<TsGroup*>(img + m.fgrp_off);
+        TsGroup* ag = reinterpret_cast<TsGroup*>(img + m.agrp_off);
+        for (int j = m.g0; j < m.g1; ++j) {
+            const auto& g = P->str[j];
+            TsGroup x{};
+            x.n = g.n; x.p = g.p; x.k = g.k; x.tb = tb;
+            x.keep_frame = g.passes.back().keep_frame;
+            x.no_store = g.passes.back().no_store;
+            x.maps_per_inst = g.maps_per_inst;
+            x.insts = reinterpret_cast<const StreamInst<float>*>(base + g.inst_off);
+            x.maps = base + g.maps_off;
+            tstream_group_windows(g.passes.data(), (int)g.passes.size(), &x);
+            fg[j - m.g0] = x;
+            if (!g.grad) continue;
+            x.tb = tba;
+            x.adjoint = 1;
+            x.keep_frame = x.no_store = 0;
+            x.maps_per_inst = g.amaps_per_inst;
+            x.maps = base + g.amaps_off;
+            tstream_group_windows(g.apasses.data(), (int)g.apasses.size(), &x);
+            ag[j - m.g0] = x;
+        }
+        for (size_t s = 0; s < m.fwd.size() + m.adj.size(); ++s) {
+            const bool fwd = s < m.fwd.size();
+            auto& L = fwd ? m.fwd[s] : m.adj[s - m.fwd.size()];
+            TsSeg* seg = reinterpret_cast<TsSeg*>(img + L.seg_off);
+            int k = 0;
+            uint32_t at = 0;
+            for (int j = m.g0; j < m.g1; ++j) {
+                const auto& g = P->str[j];
+                const size_t t = fwd ? s : s - m.fwd.size(), n = fwd ? g.passes.size() : g.apasses.size();
+                if (t >= n) continue;
+                seg[k++] = TsSeg{at, (uint16_t)(j - m.g0), (uint16_t)(fwd ? t : n - 1 - t)};
+                at += (uint32_t)g.count << (g.n - (fwd ? tb : tba));
+            }
+            L.nseg = k;
+            L.total = at;
+        }
+    }
+}
 
 // Caller-provided placement of a plan: the device block lives in [base, base + bytes) and the
 // descriptor header is uploaded asynchronously on `st` from the pinned host buffer `staging`
@@ -604,6 +745,9 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
     // streaming: per instance its own E / psi / partial buffers inside the plan block
     struct SI { size_t e_off, psi_off, part_off, lam_off, grad_off; };
     std::vector<std::vector<SI>> sinfo;
+    size_t inst_at = hdr;              // the streaming instances of all groups, one array
+    for (auto& kv : sg) hdr += sizeof(StreamInst<T>) * kv.second.size();
+    hdr = align256(hdr);
     const int tb = stream_tile_bits(dbl), tba = stream_adj_tile_bits(dbl);
     for (auto& kv : sg) {
         qaoa_plan::StrGroup g{};
@@ -629,11 +773,15 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
             g.apasses.assign(atmp, atmp + SA);
         }
         const uint64_t nta = 1ull << (g.n - tba);
-        g.inst_off = hdr;
-        hdr = align256(hdr + sizeof(StreamInst<T>) * g.count);
+        g.inst_off = inst_at;
+        inst_at += sizeof(StreamInst<T>) * g.count;
         const int variant = dbl ? 2 : eff_stream_variant(c, g.n, g.p);
         g.tgrid = (variant == 1 ? 1 : 2) * c->nsm;
-        if (!dbl && variant != 2 && tstream_available()) {
+        // (energies the caller places at addresses TMA cannot take go through the cp.async passes)
+        bool e16 = true;
+        for (int i : kv.second)
+            e16 = e16 && (desc[i].e_off < 0 || (reinterpret_cast<uintptr_t>(epool + desc[i].e_off) & 15u) == 0);
+        if (!dbl && variant != 2 && tstream_available() && e16) {
             // map 0: the kind-A passes; map 1 + b: the kind-B passes of chunk b (by start qubit)
             std::vector<int> chunk_s;
             for (auto& ps : g.passes)
@@ -650,7 +798,8 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
             }
             g.maps_off = hdr;
             hdr = align256(hdr + TS_MAP_BYTES * (size_t)g.maps_per_inst * g.count);
-            if (g.grad && tba == TSA_TB) {
+            static_assert(TSA_TB == 12, "the adjoint's tile bits (stream_adj_tile_bits)");
+            if (g.grad) {
                 // adjoint shapes: kind A, then the kind-B chunks of the adjoint plan by start qubit
                 std::vector<int> achunk;
                 for (auto& ps : g.apasses)
@@ -665,7 +814,6 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
                 }
                 g.amaps_off = hdr;
                 hdr = align256(hdr + TS_MAP_BYTES * (size_t)g.amaps_per_inst * g.count);
-                g.tadj = true;
             }
         }
         std::vector<SI> v;
@@ -695,6 +843,46 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
         g.agrid = (int)std::min<uint64_t>(nta * (uint64_t)g.count, (uint64_t)c->nsm * 2);
         sinfo.push_back(v);
         P->str.push_back(std::move(g));
+    }
+    // shared launches of consecutive TMA groups (a launch counts its tiles in 32 bits)
+    for (size_t i = 0; i < P->str.size(); ++i) {
+        auto& g = P->str[i];
+        if (!g.tma) continue;
+        const uint64_t tiles = (uint64_t)g.count << (g.n - std::min(tb, tba));
+        uint64_t before = 0;
+        if (!P->mix.empty() && P->mix.back().g1 == (int)i)
+            for (int j = P->mix.back().g0; j < (int)i; ++j)
+                before += (uint64_t)P->str[j].count << (P->str[j].n - std::min(tb, tba));
+        if (P->mix.empty() || P->mix.back().g1 != (int)i || P->mix.back().tgrid != g.tgrid || before + tiles >= (1ull << 31) ||
+            (int)i - P->mix.back().g0 >= TS_MAX_GROUPS) {
+            qaoa_plan::Mix m{};
+            m.g0 = (int)i;
+            m.inst_off = g.inst_off;
+            m.tgrid = g.tgrid;
+            P->mix.push_back(m);
+        }
+        auto& m = P->mix.back();
+        m.g1 = (int)i + 1;
+        m.count += g.count;
+        m.pmax = std::max(m.pmax, g.p);
+    }
+    for (auto& m : P->mix) {
+        size_t smax = 0, amax = 0;
+        for (int j = m.g0; j < m.g1; ++j) {
+            smax = std::max(smax, P->str[j].passes.size());
+            amax = std::max(amax, P->str[j].apasses.size());
+        }
+        for (size_t s = 0; s < smax + amax; ++s) {
+            int nseg = 0;
+            for (int j = m.g0; j < m.g1; ++j) nseg += (s < smax ? s < P->str[j].passes.size() : s - smax < P->str[j].apasses.size());
+            (s < smax ? m.fwd : m.adj).push_back(qaoa_plan::Mix::Launch{hdr, nseg, 0});
+            hdr += sizeof(TsSeg) * nseg;
+        }
+        hdr = align256(hdr);
+        m.fgrp_off = hdr;
+        hdr = align256(hdr + sizeof(TsGroup) * (m.g1 - m.g0));
+        m.agrp_off = hdr;
+        if (amax) hdr = align256(hdr + sizeof(TsGroup) * (m.g1 - m.g0));
     }
     const size_t sbase = align256(hdr);
     const size_t bytes = sbase + scr;
@@ -770,7 +958,9 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
             const qaoa_inst& d = desc[i];
             const SI& s = sinfo[gi][j++];
             StreamInst<T> I{};
+            I.n = d.n;
             I.p = d.p;
+            I.k = d.k;
             I.amp0 = exp2(-0.5 * d.n);
             I.gamma = ppool + d.par_off;
             I.beta = ppool + d.par_off + d.p;
@@ -803,12 +993,13 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
                     char* row = img.data() + g.maps_off + TS_MAP_BYTES * (size_t)(j - 1) * g.maps_per_inst;
                     if (!tstream_encode_maps(g.passes[pi], I.psi, const_cast<T*>(I.E), row + TS_MAP_BYTES * mi,
                                              row + TS_MAP_BYTES * ei)) {
-                        g.tma = false;
-                        break;
+                        if (P->owns) cudaFree(P->dev);
+                        delete P;
+                        return fail(QAOA_E_CUDA, "instance %d: tensor maps of the streaming tier refused", i);
                     }
                 }
             }
-            if (g.tadj) {
+            if (g.tma && g.grad) {
                 std::vector<char> done(g.amaps_per_inst, 0);
                 for (size_t pi = 0; pi < g.apasses.size(); ++pi) {
                     const int mi = g.atsp[pi].map;
@@ -817,8 +1008,9 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
                     char* row = img.data() + g.amaps_off + TS_MAP_BYTES * (size_t)(j - 1) * g.amaps_per_inst;
                     if (!tstream_encode_adj_maps(g.apasses[pi], I.psi, I.lam, const_cast<T*>(I.E),
                                                  row + TS_MAP_BYTES * mi)) {
-                        g.tadj = false;
-                        break;
+                        if (P->owns) cudaFree(P->dev);
+                        delete P;
+                        return fail(QAOA_E_CUDA, "instance %d: tensor maps of the adjoint passes refused", i);
                     }
                 }
             }
@@ -827,10 +1019,9 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
             g.e.push_back(Ebuf);
         }
         std::memcpy(img.data() + g.inst_off, si.data(), sizeof(StreamInst<T>) * g.count);
-        P->kernels += 1 + (int)g.passes.size() + 1 + (g.grad ? (int)g.apasses.size() + 1 : 0) +
-                      (stream_finalize_two_level(1ull << (g.n - tb), g.k) ? 1 : 0);
         ++gi;
     }
+    if constexpr (sizeof(T) == 4) plan_mixes(P, img.data(), base);
     // upload the header: synchronously into the plan's own memory, else asynchronously on the
     // caller's stream from its pinned staging buffer
     if (mem && mem->staging) {
@@ -879,22 +1070,14 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
             ++gi;
         }
     }
-    for (auto& g : P->str) {
-        const double D = (double)(1ull << g.n), cnt = (double)g.count;
-        const double nt = (double)(1ull << (g.n - tb));
-        P->bytes.push_back(cnt * (D * sizeof(T) + (double)g.n * g.n * sizeof(T)));
-        for (auto& pass : g.passes)
-            P->bytes.push_back(cnt * D * ((pass.init ? 0.0 : sizeof(C2)) + (pass.no_store ? 0.0 : sizeof(C2)) +
-                                          (pass.need_e ? sizeof(T) : 0.0)));
-        P->bytes.push_back(cnt * (nt * (sizeof(double) + std::max(g.k, 1) * 12.0) + 8.0 + g.k * 16.0));
-        if (g.grad) {
-            const int SA = (int)g.apasses.size();
-            const double nta = (double)(1ull << (g.n - tba));
-            for (int s = SA - 1; s >= 0; --s)   // psi and lam read (lam formed in the first), E read, both written back
-                P->bytes.push_back(cnt * D * ((s == SA - 1 ? 1.0 : 2.0) * sizeof(C2) + sizeof(T) +
-                                              (s > 0 ? 2.0 * sizeof(C2) : 0.0)));
-            P->bytes.push_back(cnt * (double)SA * nta * 32.0);
-        }
+    P->steps = str_steps(P);
+    for (auto& m : P->steps) {
+        P->bytes.push_back(m.energy_bytes);
+        for (double b : m.pass_bytes) P->bytes.push_back(b);
+        P->bytes.push_back(m.final_bytes);
+        for (double b : m.adj_bytes) P->bytes.push_back(b);
+        if (m.grad) P->bytes.push_back(m.reduce_bytes);
+        P->kernels += m.kernels;
     }
     *out = P;
     return QAOA_OK;
@@ -948,7 +1131,10 @@ size_t plan_header_bound(int count) {
     // tensor maps per instance: the cluster-streaming tier's, or at n <= 30 the TMA streaming
     // tier's forward maps (at most 3 shapes x 2) and adjoint maps (at most 4 shapes x 3)
     const size_t maps = std::max<size_t>(CS_MAPS_BYTES, 18 * TS_MAP_BYTES);
-    return align256(256 + (size_t)count * (align256(d) + maps + 512));
+    // the shared launches' tables: groups by (n, p) with or without gradient, at most 2 * 17 * 64 of
+    // them, each with at most 129 forward and 193 adjoint passes
+    const size_t groups = std::min<size_t>(count, 2 * 17 * 64);
+    return align256(256 + (size_t)count * (align256(d) + maps + 512) + groups * (2 * sizeof(TsGroup) + 322 * sizeof(TsSeg)) + 4096);
 }
 
 // A complex64 plan placed in caller memory, its header uploaded on `st` from pinned `staging`.
@@ -1050,21 +1236,60 @@ qaoa_status plan_enqueue(qaoa_plan* P, cudaStream_t st) {
             return launch_cstream(g.n, base + g.desc_off, g.count, g.clusters,
                                   reinterpret_cast<unsigned*>(counters + PLAN_STATUS_SLOT), st);
         }));
-    const int tb = stream_tile_bits(P->dbl);
-    for (auto& g : P->str) {
-        CK(timed("energy", [&] { return launch_energy_batch(P->dbl, g.n, base + g.inst_off, g.count, st); }));
-        for (size_t pi = 0; pi < g.passes.size(); ++pi) {
-            const StreamPass& pass = g.passes[pi];
-            if (g.tma)
+    const int tb = stream_tile_bits(P->dbl), tba = stream_adj_tile_bits(P->dbl);
+    unsigned* status = reinterpret_cast<unsigned*>(counters + PLAN_STATUS_SLOT);
+    for (const StrStep& step : P->steps) {
+        if (step.mix >= 0) {
+            const auto& m = P->mix[step.mix];
+            char* insts = base + m.inst_off;
+            CK(timed("energy", [&]() -> cudaError_t {
+                int n[ENERGY_RUNS], first[ENERGY_RUNS], count[ENERGY_RUNS], k = 0;
+                cudaError_t e = cudaSuccess;
+                for (const EnergyRun& r : energy_runs(P, m.g0, m.g1)) {
+                    if (r.n > ENERGY_TILE_NMAX) {
+                        e = launch_energy_batch(false, r.n, insts + sizeof(StreamInst<float>) * r.first, r.count, st);
+                    } else {
+                        n[k] = r.n; first[k] = r.first; count[k] = r.count;
+                        if (++k == ENERGY_RUNS) {
+                            e = launch_energy_mixed(insts, k, n, first, count, st);
+                            k = 0;
+                        }
+                    }
+                    if (e != cudaSuccess) return e;
+                }
+                return k > 0 ? launch_energy_mixed(insts, k, n, first, count, st) : cudaSuccess;
+            }));
+            for (const auto& L : m.fwd)
                 CK(timed("tstream_pass", [&] {
-                    return launch_tstream_pass(pass, g.tsp[pi], base + g.inst_off, g.count, base + g.maps_off,
-                                               g.tgrid, reinterpret_cast<unsigned*>(counters + PLAN_STATUS_SLOT), st);
+                    return launch_tstream_pass(reinterpret_cast<const TsGroup*>(base + m.fgrp_off),
+                                               reinterpret_cast<const TsSeg*>(base + L.seg_off), L.nseg, L.total,
+                                               (int)std::min<uint32_t>(L.total, (uint32_t)m.tgrid), status, st);
                 }));
-            else
-                CK(timed("stream_pass", [&] {
-                    return launch_stream_pass(P->dbl, pass, base + g.inst_off, g.count, g.grid, st);
+            CK(timed("stream_finalize", [&]() -> cudaError_t {
+                for (int j = m.g0; j < m.g1; ++j) {
+                    const auto& g = P->str[j];
+                    if (!stream_finalize_two_level(1ull << (g.n - tb), g.k)) continue;
+                    const cudaError_t e = launch_stream_topk_chunks(base + g.inst_off, g.count, 1ull << (g.n - tb), g.k, st);
+                    if (e != cudaSuccess) return e;
+                }
+                return launch_stream_finalize_mixed(insts, m.count, st);
+            }));
+            for (const auto& L : m.adj)
+                CK(timed("stream_adjoint", [&] {
+                    return launch_tstream_adj_pass(reinterpret_cast<const TsGroup*>(base + m.agrp_off),
+                                                   reinterpret_cast<const TsSeg*>(base + L.seg_off), L.nseg, L.total,
+                                                   (int)std::min<uint32_t>(L.total, 2u * (uint32_t)P->ctx->nsm), status, st);
                 }));
+            if (step.grad)
+                CK(timed("stream_grad_reduce", [&] { return launch_stream_grad_reduce(false, tba, 4, m.pmax, insts, m.count, st); }));
+            continue;
         }
+        auto& g = P->str[step.g0];
+        CK(timed("energy", [&] { return launch_energy_batch(P->dbl, g.n, base + g.inst_off, g.count, st); }));
+        for (const StreamPass& pass : g.passes)
+            CK(timed("stream_pass", [&] {
+                return launch_stream_pass(P->dbl, pass, base + g.inst_off, g.count, g.grid, st);
+            }));
         CK(timed("stream_finalize", [&] {
             return launch_stream_finalize(P->dbl, base + g.inst_off, g.count, 1ull << (g.n - tb), g.k, st);
         }));
@@ -1072,16 +1297,11 @@ qaoa_status plan_enqueue(qaoa_plan* P, cudaStream_t st) {
             const int SA = (int)g.apasses.size();
             for (int s = SA - 1; s >= 0; --s)
                 CK(timed("stream_adjoint", [&] {
-                    if (g.tadj)
-                        return launch_tstream_adj_pass(g.apasses[s], g.atsp[s], s, s == SA - 1, s > 0, base + g.inst_off,
-                                                       g.count, base + g.amaps_off, 2 * P->ctx->nsm,
-                                                       reinterpret_cast<unsigned*>(counters + PLAN_STATUS_SLOT), st);
                     return launch_stream_adj_pass(P->dbl, g.apasses[s], s, s == SA - 1, s > 0, base + g.inst_off,
                                                   g.count, g.agrid, st);
                 }));
             CK(timed("stream_grad_reduce", [&] {
-                return launch_stream_grad_reduce(P->dbl, g.apasses.data(), SA, base + g.inst_off, g.count,
-                                                 1ull << (g.n - stream_adj_tile_bits(P->dbl)), st);
+                return launch_stream_grad_reduce(P->dbl, tba, 4, g.p, base + g.inst_off, g.count, st);
             }));
         }
     }

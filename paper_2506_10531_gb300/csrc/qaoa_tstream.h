@@ -34,19 +34,34 @@ TsPass tstream_pass_geometry(const StreamPass& P, int map, int emap, int maps_pe
 // a state at psi and its energies at E (both 16-byte aligned) into psi_map / e_map (host,
 // 64-byte aligned).
 bool tstream_encode_maps(const StreamPass& P, void* psi, void* E, void* psi_map, void* e_map);
-// One pass over `count` instances (device array of StreamInst<float>) whose maps start at `maps`
-// (device); a bounded wait that ran out sets bit 0 of *status.
-cudaError_t launch_tstream_pass(const StreamPass& P, const TsPass& T, const void* insts, int count,
-                                const void* maps, int grid, unsigned* status, cudaStream_t st);
+// A plan group's passes (forward or adjoint) for launches that hold passes of several groups: the
+// numbers stream_plan made them from, from which the kernels form the pass they are at.
+struct TsGroup {
+    int n, p, k, tb, S;          // S: passes
+    int W, cs[4], ch[4];         // windows of a layer: the contiguous one, then chunks [cs, cs + ch)
+    int adjoint, keep_frame, no_store, maps_per_inst;
+    const StreamInst<float>* insts;
+    const void* maps;
+};
+// One group's pass in a launch: its tiles are [tile0, the next segment's tile0).
+struct TsSeg {
+    uint32_t tile0;
+    uint16_t group, pass;
+};
+constexpr int TS_MAX_GROUPS = 65535;
+// Fill the windows of g (n, tb set) from its pass list.
+void tstream_group_windows(const StreamPass* passes, int S, TsGroup* g);
+// A launch over `nseg` segments (device array, `total` tiles in all) of the groups at `groups`; a
+// bounded wait that ran out sets bit 0 of *status.
+cudaError_t launch_tstream_pass(const TsGroup* groups, const TsSeg* segs, int nseg, uint32_t total, int grid,
+                                unsigned* status, cudaStream_t st);
 
 // Adjoint passes (tiles of TSA_TB bits, kind-B chunks of h <= 8 high qubits): per pass shape
 // three maps (state psi, adjoint state lam, energies) at indices T.map, T.map + 1, T.map + 2.
 size_t tstream_adj_smem_bytes();
 TsPass tstream_adj_geometry(const StreamPass& P, int map, int maps_per_inst);
 bool tstream_encode_adj_maps(const StreamPass& P, void* psi, void* lam, void* E, void* maps3);
-// Adjoint pass `si` of the adjoint plan over `count` instances (see launch_stream_adj_pass).
-cudaError_t launch_tstream_adj_pass(const StreamPass& P, const TsPass& T, int si, bool lam_first, bool store,
-                                    const void* insts, int count, const void* maps, int grid, unsigned* status,
-                                    cudaStream_t st);
+cudaError_t launch_tstream_adj_pass(const TsGroup* groups, const TsSeg* segs, int nseg, uint32_t total, int grid,
+                                    unsigned* status, cudaStream_t st);
 
 }  // namespace qaoa
