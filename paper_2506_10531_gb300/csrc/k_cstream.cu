@@ -535,8 +535,10 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
                             z = lo | (tau << CB) | (e << TB);
                         }
                     };
-                    const double tot = block_sum_df(accp, reinterpret_cast<float*>(red));   // its barriers end every energy read
-                    if (threadIdx.x == 0) my_ex += tot;
+                    __syncthreads();   // every energy has been read
+                    warp_sum_df(accp, reinterpret_cast<float*>(red));
+                    __syncthreads();
+                    if (threadIdx.x < 32) my_ex += sum_parts_df(reinterpret_cast<const float*>(red));
                     if (I.k > 0) {
                         if (!topk_own(sp, I.k, pmax, elem, ts, reinterpret_cast<float*>(sm + o.wbound))) {
                             // flat distribution: the tile-wide selection, with each thread's maximum

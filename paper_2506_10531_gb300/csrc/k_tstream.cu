@@ -6,18 +6,21 @@
 // plan groups: groups of other sizes and depths share the launches (segments, TsSeg), so that an
 // uneven batch takes as many launches as its longest group has passes and small states fill the
 // SMs that one group alone would leave idle (a launch per group and pass: 48 uneven training
-// instances 7.95 ms a step, 16 served jobs 800 us a tick; shared launches: 5.70 ms, 365 us). A tile is 2^13 amplitudes, moved between HBM and shared memory by TMA
-// (cp.async.bulk.tensor; the state with the 128-byte swizzle, its energies unswizzled, the
-// energies only in passes with a cost phase or the final reductions). A CTA loads its next tile
-// as soon as the bulk store of the current one has read the buffer, and the other CTA of the SM
-// works while it waits: measured on GB300 at n = 30 this beats one CTA per SM with a two-stage
-// ring (8 warps per SM leave the sub-passes latency-bound) by 12% over the passes of a solve.
+// instances 7.95 ms a step, 16 served jobs 800 us a tick; shared launches: 5.66 ms, 365 us). A tile is
+// 2^13 amplitudes, moved between HBM and shared memory by TMA (cp.async.bulk.tensor; the state with
+// the 128-byte swizzle). Phases and energies come from Q itself (qaoa_phase.cuh); instances whose
+// energies live in HBM anyway (gradient runs, returned energies) read them, unswizzled, in passes with
+// a cost phase or the final reductions. n = 30, p = 2: 16.19 ms, with energies built and read 16.74.
+// A CTA loads its next tile as soon as the bulk store of the current one has read the buffer, and the
+// other CTA of the SM works while it waits: measured on GB300 at n = 30 this beats one CTA per SM
+// with a two-stage ring (8 warps per SM leave the sub-passes latency-bound) by 12% over the passes
+// of a solve. What bounds the passes (n = 30): single-layer passes HBM (2.9 ms for 17.2 GB); the
+// others, at 2.8-3.8 ms, the latency of 16 warps per SM (0.35-0.45 of the issue slots).
 //
 // Tiles follow the streaming tier's pass plan (stream_plan): kind A holds qubits 0..12 (2^13
 // contiguous amplitudes), kind B the 2^c contiguous amplitudes of qubits 0..c-1 times the 2^h
 // values of qubits s..s+h-1 (c = 13 - h, 1 <= h <= 9). Inside a tile the qubits are mixed in
-// register windows of at most five bits: kind A in [0,4), [4,8), [8,13) (the cost phase in the
-// last), kind B in [c, c+h) or, for h > 5, [c, c+5) and [c+5, c+h) (the phase in the last). With
+// register windows of at most five bits (tile_pass; the cost phase in the one that reaches bit 12). With
 // the lanes of a warp on tile bits outside the window, the swizzle makes every shared access free
 // of bank conflicts. The final pass reduces each tile to an FP64 <C> partial and a top-k list;
 // the streaming tier's finalize kernel merges them per instance.
@@ -25,6 +28,7 @@
 
 #include "qaoa_engine.cuh"
 #include "qaoa_kernels.h"
+#include "qaoa_phase.cuh"
 #include "qaoa_stream.h"
 #include "qaoa_tma.cuh"
 #include "qaoa_tstream.h"
@@ -40,14 +44,15 @@ constexpr uint32_t TD = 1u << TB;
 constexpr int NT = TMA_NT;
 
 struct TsOff {
-    size_t stage[1], estage[1], lc, red, wbound, wb, cnt, cand, out, wlists, run, mbar, total;
+    size_t psi, E, lc, red, wbound, wb, cnt, cand, out, wlists, run, mbar, total;
 };
 __host__ __device__ inline size_t ts_al(size_t x) { return (x + 15) & ~(size_t)15; }
-__host__ __device__ inline TsOff ts_offsets() {
+// tab: the phase table in the place of the energy tile
+__host__ __device__ inline TsOff ts_offsets(bool tab) {
     TsOff o{};
     size_t x = 0;
-    for (int s = 0; s < 1; ++s) { o.stage[s] = x; x += (size_t)TD * 8; }   // 1024-aligned at run time
-    for (int s = 0; s < 1; ++s) { o.estage[s] = x; x += (size_t)TD * 4; }
+    o.psi = x; x += (size_t)TD * 8;   // 1024-aligned at run time
+    o.E = x; x = ts_al(x + (tab ? sizeof(PhaseTab) : (size_t)TD * 4));
     o.lc = x; x = ts_al(x + 64 * sizeof(LayerConst<float>));
     o.red = x; x = ts_al(x + 32 * sizeof(float));
     o.wbound = x; x = ts_al(x + sizeof(float));
@@ -114,171 +119,172 @@ __device__ __forceinline__ void wstore(float2* sp, uint32_t pb, const float2 (&v
     }
 }
 
-// What one sub-pass does to a group, in order: the mixer of layer la; then, with `phase`, the
-// cost phase of layer lb and its mixer; with `init`, the group starts as |+> (rotated frame)
-// followed by the cost phase of layer 0 and its mixer (la, phase unused); with `fin`, the
-// pending shear factor of the last layer and the thread's FP32 <C> terms and maximum |psi|^2.
-struct SubOps {
-    int la, lb;
-    bool mix_la, phase, init, fin;
-};
-
-// One sub-pass over window [A, A+R) of the tile in sp: every group of the thread (2^(13-R) /
-// 256 of them) is loaded, transformed and stored. zsh: shift of the window's bit 0 in the global
-// index (kind A: A; kind B: A - c + s).
-// The work of one group of window [A, A+R) (see wsub).
-template <int A, int R>
-__device__ __forceinline__ void wgroup(float2* sp, uint32_t g, const Geo& geo, const SubOps& op,
-                                       const LayerConst<float>* lc, const float* sE, float amp0, float& accp,
-                                       float& pmax) {
-    const uint32_t base = wbase<A, R>(g);
-    const uint32_t pb = psw(base);
-    float2 v[1 << R];
-    if (op.init) {
-        const int pc = __popcll(geo.z(base));
+// Phases and energies of a top window's elements (group r of the thread): from the tile's energies in
+// shared memory, or from the phase table.
+struct ValsMem {
+    const float* sE;
+    template <bool F>
+    __device__ __forceinline__ void load() {}
+    template <int A, int R, typename Fn>
+    __device__ __forceinline__ void phases(const PhaseK<float>& ph, uint32_t base, int, Fn&& fn) const {
 #pragma unroll
         for (int i = 0; i < (1 << R); ++i) {
             float s, c;
-            sincos_phase(lc[0].ph, sE[base + ((uint32_t)i << A)], s, c);
-            v[i] = times_i_pow(make_float2(amp0 * c, -amp0 * s), pc + __popc(i));
-        }
-        mix_layer<R>(v, (1 << R) - 1, lc[0]);
-    } else {
-        wload<A, R>(sp, pb, v);
-        if (op.mix_la) mix_layer<R>(v, (1 << R) - 1, lc[op.la]);
-        if (op.phase) {
-            const LayerConst<float>& k = lc[op.lb];
-            const Pending<float> pre(k.pre, k.pcot, __popc(base) + __popcll(geo.zt));
-#pragma unroll
-            for (int i = 0; i < (1 << R); ++i) {
-                float s, c;
-                sincos_phase(k.ph, sE[base + ((uint32_t)i << A)], s, c);
-                rot_neg(v[i], s * pre.f[__popc(i) & 1], c * pre.f[__popc(i) & 1]);
-            }
-            mix_layer<R>(v, (1 << R) - 1, k);
-        }
-        if (op.fin) {
-            scale_group<R>(v, Pending<float>(lc[op.la].post, lc[op.la].cot, __popc(base) + __popcll(geo.zt)));
-#pragma unroll
-            for (int i = 0; i < (1 << R); ++i) {
-                const float pr = v[i].x * v[i].x + v[i].y * v[i].y;
-                accp = fmaf(pr, sE[base + ((uint32_t)i << A)], accp);
-                pmax = fmaxf(pmax, pr);
-            }
+            sincos_phase(ph, sE[base + ((uint32_t)i << A)], s, c);
+            fn(i, s, c);
         }
     }
-    wstore<A, R>(sp, pb, v);
-}
+    template <int A, int R, typename Fn>
+    __device__ __forceinline__ void energies(uint32_t base, int, Fn&& fn) const {
+#pragma unroll
+        for (int i = 0; i < (1 << R); ++i) fn(i, sE[base + ((uint32_t)i << A)]);
+    }
+};
+struct ValsTab {
+    const PhaseTab* t;
+    TileVals x;
+    template <bool F>
+    __device__ __forceinline__ void load() {
+        x.init<F>(*t);
+    }
+    template <int A, int R, typename Fn>
+    __device__ __forceinline__ void phases(const PhaseK<float>&, uint32_t, int r, Fn&& fn) const {
+        tab_phases<A, R>(x, r, fn);
+    }
+    template <int A, int R, typename Fn>
+    __device__ __forceinline__ void energies(uint32_t, int r, Fn&& fn) const {
+        tab_energies<A, R>(x, r, fn);
+    }
+};
 
-// One sub-pass over window [A, A+R) of the tile in sp: every group of the thread (2^(13-R) /
-// 256 of them) is loaded, transformed and stored.
+// A pass takes a tile through the windows below its top one (upwards, mixing layer la), through the
+// top window, which reaches tile bit 12 (mixer of la; a pass that ends a layer and opens the next:
+// the cost phase of lb and its mixer; the opening pass: |+> in the rotated frame, phase and mixer of
+// layer 0; the final pass: the pending shear factor of the last layer and the thread's FP32 <C> terms
+// and maximum |psi|^2), and, where layer lb is mixed too, back down through the lower windows.
+//
+//   kind A:              [0,4) [4,8) | [8,13)
+//   kind B, h high bits: [13-h,8)    | [8,13)   (h > 5; h <= 5: [13-h,13) alone)
+//
+// One copy of each lower window's code serves both ways and both kinds; the top window has one per
+// thing it does (one body with run-time switches spilled 244 bytes: n = 30 18.6 ms, split 16.2). A
+// five-bit top window leaves a thread one group with one phase start (windows [c,c+5) and [c+5,13)
+// gave it up to eight: 13 shared loads per amplitude at h = 7; two-layer pass at n = 30 4.04 -> 3.82 ms).
+enum { TOP_ONE, TOP_TWO, TOP_INIT, TOP_FIN };   // what the top window does besides: nothing, phase and mixer of lb, ...
+
+// Window [A, A+R) below the top: the mixer of layer constants k on every group of the thread
+// (2^(13-R) / 256 of them).
 template <int A, int R>
-__device__ __forceinline__ void wsub(float2* sp, const Geo& geo, int zsh, const SubOps& op,
-                                     const LayerConst<float>* lc, const float* sE, float amp0,
-                                     float& accp, float& pmax) {
-    constexpr int NGT = (1 << (TB - R)) / NT;   // groups per thread
+__device__ __forceinline__ void low_window(float2* sp, const LayerConst<float>& k) {
+    constexpr int NGT = (1 << (TB - R)) / NT;
 #pragma unroll 1
-    for (int r = 0; r < NGT; ++r) wgroup<A, R>(sp, threadIdx.x + (uint32_t)(r * NT), geo, op, lc, sE, amp0, accp, pmax);
+    for (int r = 0; r < NGT; ++r) {
+        const uint32_t pb = psw(wbase<A, R>(threadIdx.x + (uint32_t)(r * NT)));
+        float2 v[1 << R];
+        wload<A, R>(sp, pb, v);
+        mix_layer<R>(v, (1 << R) - 1, k);
+        wstore<A, R>(sp, pb, v);
+    }
 }
 
-// Element i < 32 of the thread in the last sub-pass over window [A, A+R): shared and global index.
-template <int A, int R>
-__device__ __forceinline__ void welem(const Geo& geo, int zsh, int i, uint32_t& ix, uint64_t& z) {
-    const uint32_t g = threadIdx.x + (uint32_t)((i >> R) * NT);
+// The top window [A, 13), A >= 8: group r of the thread has base threadIdx.x + 256 r.
+template <int MODE, int A, typename Vals>
+__device__ __forceinline__ void top_window(float2* sp, const Geo& geo, const LayerConst<float>& ka,
+                                           const LayerConst<float>& kb, Vals vals, float amp0, float& accp, float& pmax) {
+    constexpr int R = TB - A, NGT = 1 << (A - 8);
+    const int pz = __popcll(geo.zt);
+    if (MODE != TOP_ONE) vals.template load<MODE == TOP_FIN>();
+#pragma unroll 1
+    for (int r = 0; r < NGT; ++r) {
+        const uint32_t base = threadIdx.x + (uint32_t)(r * NT);
+        const uint32_t pb = psw(base);
+        float2 v[1 << R];
+        if (MODE == TOP_INIT) {
+            const int pc = __popc(base) + pz;
+            vals.template phases<A, R>(ka.ph, base, r, [&](int i, float s, float c) {
+                v[i] = times_i_pow(make_float2(amp0 * c, -amp0 * s), pc + __popc(i));
+            });
+        } else {
+            wload<A, R>(sp, pb, v);
+        }
+        mix_layer<R>(v, (1 << R) - 1, ka);
+        if (MODE == TOP_TWO) {
+            const Pending<float> pre(kb.pre, kb.pcot, __popc(base) + pz);
+            vals.template phases<A, R>(kb.ph, base, r, [&](int i, float s, float c) {
+                rot_neg(v[i], s * pre.f[__popc(i) & 1], c * pre.f[__popc(i) & 1]);
+            });
+            mix_layer<R>(v, (1 << R) - 1, kb);
+        }
+        if (MODE == TOP_FIN) {
+            scale_group<R>(v, Pending<float>(ka.post, ka.cot, __popc(base) + pz));
+            vals.template energies<A, R>(base, r, [&](int i, float e) {
+                const float pr = v[i].x * v[i].x + v[i].y * v[i].y;
+                accp = fmaf(pr, e, accp);
+                pmax = fmaxf(pmax, pr);
+            });
+        }
+        wstore<A, R>(sp, pb, v);
+    }
+}
+template <int MODE, typename Vals>
+__device__ __forceinline__ void top_windows(int R, float2* sp, const Geo& geo, const LayerConst<float>& ka,
+                                            const LayerConst<float>& kb, const Vals& vals, float amp0, float& accp,
+                                            float& pmax) {
+    switch (R) {
+        case 1: top_window<MODE, 12>(sp, geo, ka, kb, vals, amp0, accp, pmax); break;
+        case 2: top_window<MODE, 11>(sp, geo, ka, kb, vals, amp0, accp, pmax); break;
+        case 3: top_window<MODE, 10>(sp, geo, ka, kb, vals, amp0, accp, pmax); break;
+        case 4: top_window<MODE, 9>(sp, geo, ka, kb, vals, amp0, accp, pmax); break;
+        default: top_window<MODE, 8>(sp, geo, ka, kb, vals, amp0, accp, pmax); break;
+    }
+}
+
+template <typename Vals>
+__device__ __forceinline__ void tile_pass(float2* sp, const Geo& geo, const StreamPass& P, const LayerConst<float>* lc,
+                                          const Vals& vals, float amp0, float& accp, float& pmax) {
+    const bool two = P.lb > P.la || P.init;
+    const int nlow = geo.kindA ? 2 : (P.h > 5 ? 1 : 0);
+    const int steps = two ? 2 * nlow : nlow;
+#pragma unroll 1
+    for (int i = P.init ? nlow : 0; i <= steps; ++i) {
+        if (i == nlow) {
+            const LayerConst<float>&ka = lc[P.la], &kb = lc[P.lb];
+            const int R = geo.kindA ? 5 : P.h;
+            if (P.init) top_window<TOP_INIT, 8>(sp, geo, ka, kb, vals, amp0, accp, pmax);   // a kind-A pass
+            else if (two) top_windows<TOP_TWO>(R, sp, geo, ka, kb, vals, amp0, accp, pmax);
+            else if (P.fin) top_windows<TOP_FIN>(R, sp, geo, ka, kb, vals, amp0, accp, pmax);
+            else top_windows<TOP_ONE>(R, sp, geo, ka, kb, vals, amp0, accp, pmax);
+        } else {
+            const LayerConst<float>& k = lc[i < nlow ? P.la : P.lb];
+            // kind A: [0,4) first and last; 0 and 4: the window's low bit
+            switch (geo.kindA ? ((i & 3) ? 4 : 0) : TB - P.h) {
+                case 0: low_window<0, 4>(sp, k); break;
+                case 4: low_window<4, 4>(sp, k); break;
+                case 5: low_window<5, 3>(sp, k); break;
+                case 6: low_window<6, 2>(sp, k); break;
+                default: low_window<7, 1>(sp, k); break;
+            }
+        }
+        if (i < steps) __syncthreads();
+    }
+}
+
+// Element i < 32 of the thread in the top window (reductions): shared and global index.
+template <int A>
+__device__ __forceinline__ void top_elem(const Geo& geo, int zsh, int i, uint32_t& ix, uint64_t& z) {
+    constexpr int R = TB - A;
+    const uint32_t base = threadIdx.x + (uint32_t)((i >> R) * NT);
     const int e = i & ((1 << R) - 1);
-    const uint32_t base = wbase<A, R>(g);
     ix = wix<A>(psw(base), e);
     z = geo.z(base) + ((uint64_t)e << zsh);
 }
-
-// Kind-A tile: the snake of the pass over the windows [0,4), [4,8), [8,13).
-__device__ __forceinline__ void tile_kind_a(float2* sp, const Geo& geo, const StreamPass& P,
-                                            const LayerConst<float>* lc, const float* sE, float amp0,
-                                            float& accp, float& pmax) {
-    if (P.init) {
-        // |+>, the cost phase and the mixer of layer 0 (the pass opens the state), then the mixer
-        // of layer 0 on the lower windows; a pass that also closes the layer is not planned
-        wsub<8, 5>(sp, geo, 8, SubOps{0, 0, false, false, true, false}, lc, sE, amp0, accp, pmax);
-        __syncthreads();
-        wsub<4, 4>(sp, geo, 4, SubOps{0, 0, true, false, false, false}, lc, sE, amp0, accp, pmax);
-        __syncthreads();
-        wsub<0, 4>(sp, geo, 0, SubOps{0, 0, true, false, false, false}, lc, sE, amp0, accp, pmax);
-        return;
-    }
-    const bool two = P.lb > P.la;
-    wsub<0, 4>(sp, geo, 0, SubOps{P.la, P.la, true, false, false, false}, lc, sE, amp0, accp, pmax);
-    __syncthreads();
-    wsub<4, 4>(sp, geo, 4, SubOps{P.la, P.la, true, false, false, false}, lc, sE, amp0, accp, pmax);
-    __syncthreads();
-    wsub<8, 5>(sp, geo, 8, SubOps{P.la, P.lb, true, two, false, (bool)P.fin}, lc, sE, amp0, accp, pmax);
-    if (two) {
-        __syncthreads();
-        wsub<4, 4>(sp, geo, 4, SubOps{P.lb, P.lb, true, false, false, false}, lc, sE, amp0, accp, pmax);
-        __syncthreads();
-        wsub<0, 4>(sp, geo, 0, SubOps{P.lb, P.lb, true, false, false, false}, lc, sE, amp0, accp, pmax);
-    }
-}
-
-// Kind-B tile with H high qubits: one window [c, c+H) for H <= 5, else [c, c+5) and [c+5, c+H).
-template <int H>
-__device__ __forceinline__ void tile_kind_b(float2* sp, const Geo& geo, const StreamPass& P,
-                                            const LayerConst<float>* lc, const float* sE, float amp0,
-                                            float& accp, float& pmax) {
-    constexpr int C = TB - H;
-    const bool two = P.lb > P.la;
-    if constexpr (H <= 5) {
-        wsub<C, H>(sp, geo, P.s, SubOps{P.la, P.lb, true, two, false, (bool)P.fin}, lc, sE, amp0, accp, pmax);
-    } else {
-        constexpr int A2 = C + 5, R2 = H - 5;
-        wsub<C, 5>(sp, geo, P.s, SubOps{P.la, P.la, true, false, false, false}, lc, sE, amp0, accp, pmax);
-        __syncthreads();
-        wsub<A2, R2>(sp, geo, P.s + 5, SubOps{P.la, P.lb, true, two, false, (bool)P.fin}, lc, sE, amp0, accp, pmax);
-        if (two) {
-            __syncthreads();
-            wsub<C, 5>(sp, geo, P.s, SubOps{P.lb, P.lb, true, false, false, false}, lc, sE, amp0, accp, pmax);
-        }
-    }
-}
-
-// Element accessor of the thread's 32 elements in the pass's last sub-pass (reductions).
-template <int H>
-__device__ __forceinline__ void last_elem_b(const Geo& geo, const StreamPass& P, int i, uint32_t& ix, uint64_t& z) {
-    constexpr int C = TB - H;
-    if constexpr (H <= 5) welem<C, H>(geo, P.s, i, ix, z);
-    else welem<C + 5, H - 5>(geo, P.s + 5, i, ix, z);
-}
-
-__device__ __forceinline__ void kind_b_dispatch(int h, float2* sp, const Geo& geo, const StreamPass& P,
-                                                const LayerConst<float>* lc, const float* sE, float amp0,
-                                                float& accp, float& pmax) {
-    switch (h) {
-        case 1: tile_kind_b<1>(sp, geo, P, lc, sE, amp0, accp, pmax); break;
-        case 2: tile_kind_b<2>(sp, geo, P, lc, sE, amp0, accp, pmax); break;
-        case 3: tile_kind_b<3>(sp, geo, P, lc, sE, amp0, accp, pmax); break;
-        case 4: tile_kind_b<4>(sp, geo, P, lc, sE, amp0, accp, pmax); break;
-        case 5: tile_kind_b<5>(sp, geo, P, lc, sE, amp0, accp, pmax); break;
-        case 6: tile_kind_b<6>(sp, geo, P, lc, sE, amp0, accp, pmax); break;
-        case 7: tile_kind_b<7>(sp, geo, P, lc, sE, amp0, accp, pmax); break;
-        case 8: tile_kind_b<8>(sp, geo, P, lc, sE, amp0, accp, pmax); break;
-        default: tile_kind_b<9>(sp, geo, P, lc, sE, amp0, accp, pmax); break;
-    }
-}
-
 __device__ __forceinline__ void last_elem(const Geo& geo, const StreamPass& P, int i, uint32_t& ix, uint64_t& z) {
-    if (P.kind == 0) {
-        welem<8, 5>(geo, 8, i, ix, z);
-        return;
-    }
-    switch (P.h) {
-        case 1: last_elem_b<1>(geo, P, i, ix, z); break;
-        case 2: last_elem_b<2>(geo, P, i, ix, z); break;
-        case 3: last_elem_b<3>(geo, P, i, ix, z); break;
-        case 4: last_elem_b<4>(geo, P, i, ix, z); break;
-        case 5: last_elem_b<5>(geo, P, i, ix, z); break;
-        case 6: last_elem_b<6>(geo, P, i, ix, z); break;
-        case 7: last_elem_b<7>(geo, P, i, ix, z); break;
-        case 8: last_elem_b<8>(geo, P, i, ix, z); break;
-        default: last_elem_b<9>(geo, P, i, ix, z); break;
+    switch (P.kind == 0 ? 5 : P.h) {
+        case 1: top_elem<12>(geo, P.s, i, ix, z); break;
+        case 2: top_elem<11>(geo, P.s, i, ix, z); break;
+        case 3: top_elem<10>(geo, P.s, i, ix, z); break;
+        case 4: top_elem<9>(geo, P.s, i, ix, z); break;
+        default: top_elem<8>(geo, P.kind == 0 ? 8 : 8 - P.c + P.s, i, ix, z); break;
     }
 }
 
@@ -384,6 +390,9 @@ __device__ __forceinline__ void advance_segment(const TsGroup* groups, const TsS
     __syncthreads();
 }
 
+// TAB: phases and energies come from Q (qaoa_phase.cuh), no energy vector exists; else from the energies
+// in HBM (gradient runs, whose adjoint reads them, and instances that return them).
+template <bool TAB>
 __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const TsGroup* __restrict__ groups,
                                                        const TsSeg* __restrict__ segs, int nseg, uint32_t total,
                                                        unsigned* status) {
@@ -391,9 +400,10 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const TsGroup* __restric
     __shared__ SegPass cur, nxt;   // nxt: thread 0's, for loads of the next segment's first tile
     const uint32_t raw = saddr(sm_raw);
     unsigned char* sm = sm_raw + (((raw + 1023u) & ~1023u) - raw);
-    const TsOff o = ts_offsets();
-    float2* const sp = reinterpret_cast<float2*>(sm + o.stage[0]);
-    float* const sE = reinterpret_cast<float*>(sm + o.estage[0]);
+    const TsOff o = ts_offsets(TAB);
+    float2* const sp = reinterpret_cast<float2*>(sm + o.psi);
+    float* const sE = reinterpret_cast<float*>(sm + o.E);
+    PhaseTab& tab = *reinterpret_cast<PhaseTab*>(sm + o.E);
     LayerConst<float>* lc = reinterpret_cast<LayerConst<float>*>(sm + o.lc);
     float* red = reinterpret_cast<float*>(sm + o.red);
     TileTopk ts;
@@ -425,12 +435,13 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const TsGroup* __restric
         }
         const StreamPass& p = S->P;
         const TsPass& t = S->T;
-        if (p.init && !p.need_e) return;
+        const bool need_e = !TAB && p.need_e;
+        if (p.init && !need_e) return;
         const int tbits = p.n - TB;
         const uint32_t ql = q - S->tile0, tmask = (1u << tbits) - 1u;
         const CUtensorMap* m = S->maps + (size_t)(ql >> tbits) * t.maps_per_inst;
-        mbar_expect_tx(mbar, (p.init ? 0u : TD * 8) + (p.need_e ? TD * 4 : 0u));
-        if (p.need_e) tile_load(t, m + t.emap, sE, ql & tmask, mbar);
+        mbar_expect_tx(mbar, (p.init ? 0u : TD * 8) + (need_e ? TD * 4 : 0u));
+        if (need_e) tile_load(t, m + t.emap, sE, ql & tmask, mbar);
         if (!p.init) {
             if (wait_store) bulk_wait_read();
             tile_load(t, m + t.map, sp, ql & tmask, mbar);
@@ -441,13 +452,16 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const TsGroup* __restric
         const uint32_t end = S == &cur ? send - S->tile0 : 0u;
         if ((p.init || (p.fin && p.no_store)) && q1 < end) {
             const CUtensorMap* m1 = S->maps + (size_t)(q1 >> tbits) * t.maps_per_inst;
-            if (p.need_e) tile_prefetch(t, m1 + t.emap, q1 & tmask);
+            if (need_e) tile_prefetch(t, m1 + t.emap, q1 & tmask);
             if (!p.init) tile_prefetch(t, m1 + t.map, q1 & tmask);
         }
     };
     if (blockIdx.x < total && threadIdx.x == 0) issue(blockIdx.x, false);
-    const float *cur_g = nullptr, *cur_b = nullptr;
-    int cur_p = 0, cur_n = 0;
+    // what the constants and the table belong to, in shared memory: the sub-passes need the registers
+    __shared__ const float *cur_g, *cur_b, *cur_q;
+    __shared__ int cur_p, cur_n, cur_l;
+    if (threadIdx.x == 0) cur_n = 0;
+    __syncthreads();
     TopEnt* run = reinterpret_cast<TopEnt*>(sm + o.run);
     bool run_valid = false;   // the run list holds this CTA's best k of the current instance so far
     for (uint32_t q = blockIdx.x; q < total; q += gridDim.x) {
@@ -461,21 +475,23 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const TsGroup* __restric
         const uint64_t tau = ql & ((1u << tbits) - 1u);
         const bool store = !P.fin || !P.no_store;
         const StreamInst<float>& I = cur.insts[ii];
-        if (I.gamma != cur_g || I.beta != cur_b || I.p != cur_p || P.n != cur_n) {
+        const bool same = P.n == cur_n && I.p == cur_p && I.gamma == cur_g && I.beta == cur_b;
+        const int layer = TAB && P.need_e ? (P.fin ? I.p : P.lb) + 64 * (P.kind ? P.s : 0) : -1;   // what the table holds
+        const bool retab = layer >= 0 && !(same && I.Q == cur_q && layer == cur_l);
+        if (!same || retab) {
             __syncthreads();
-            set_layer_consts<float>(lc, I.gamma, I.beta, I.p, P.n, false);
-            cur_g = I.gamma;
-            cur_b = I.beta;
-            cur_p = I.p;
-            cur_n = P.n;
+            if (!same) set_layer_consts<float>(lc, I.gamma, I.beta, I.p, P.n, false);
+            if (TAB && retab) {
+                if (P.fin) tab_build<true>(tab, I.Q, P.n, 0.0f, P.c, P.s);
+                else tab_build<false>(tab, I.Q, P.n, I.gamma[P.lb], P.c, P.s);
+            }
+            if (threadIdx.x == 0) {
+                cur_g = I.gamma; cur_b = I.beta; cur_p = I.p; cur_n = P.n;
+                if (retab) { cur_q = I.Q; cur_l = layer; }
+                if (!same && !retab) cur_q = nullptr;
+            }
+            __syncthreads();
         }
-        if (!P.init || P.need_e) {
-            if (ok) ok = mbar_wait_bounded(mbar, parity);
-            parity ^= 1u;
-        }
-        // a pass that loads no state may meet a store of the last tile still reading the buffer
-        if (P.init && threadIdx.x == 0) bulk_wait_read();
-        ok = __syncthreads_and(ok);
         Geo geo;
         geo.kindA = P.kind == 0;
         geo.c = P.c;
@@ -488,13 +504,27 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const TsGroup* __restric
             const uint64_t mid = tau & ((1ull << midbits) - 1ull), top = tau >> midbits;
             geo.zt = (mid << P.c) | (top << (P.s + P.h));
         }
+        if (TAB && P.need_e) {
+            if (P.fin) tab_tile<true>(tab, (uint32_t)geo.zt, P.c, P.s);
+            else tab_tile<false>(tab, (uint32_t)geo.zt, P.c, P.s);
+        }
+        if (!P.init || (!TAB && P.need_e)) {
+            if (ok) ok = mbar_wait_bounded(mbar, parity);
+            parity ^= 1u;
+        }
+        // a pass that loads no state may meet a store of the last tile still reading the buffer
+        if (P.init && threadIdx.x == 0) bulk_wait_read();
+        ok = __syncthreads_and(ok);
         float accp = 0.0f, pmax = -1.0f;
-        if (geo.kindA) tile_kind_a(sp, geo, P, lc, sE, (float)I.amp0, accp, pmax);
-        else kind_b_dispatch(P.h, sp, geo, P, lc, sE, (float)I.amp0, accp, pmax);
+        if constexpr (TAB) tile_pass(sp, geo, P, lc, ValsTab{&tab}, (float)I.amp0, accp, pmax);
+        else tile_pass(sp, geo, P, lc, ValsMem{sE}, (float)I.amp0, accp, pmax);
+        if (P.fin) warp_sum_df(accp, red);
         __syncthreads();
         if (P.fin) {
-            const double tot = block_sum_df(accp, red);
-            if (threadIdx.x == 0) I.part_expect[tau] = tot;
+            if (threadIdx.x < 32) {
+                const double tot = sum_parts_df(red);
+                if (threadIdx.x == 0) I.part_expect[tau] = tot;
+            }
             if (P.k > 0) {
                 // Top-k: the CTA carries one list (run) across its tiles of an instance and writes
                 // it into the slot of its last such tile (the other slots it owns stay empty); the
@@ -819,7 +849,7 @@ bool encode_shape(const StreamPass& P, void* base, int w, CUtensorMap* m) {
 
 bool tstream_available() { return encode_fn() != nullptr; }
 
-size_t tstream_smem_bytes() { return ts_offsets().total; }
+size_t tstream_smem_bytes(bool tab) { return ts_offsets(tab).total; }
 
 TsPass tstream_pass_geometry(const StreamPass& P, int map, int emap, int maps_per_inst) {
     TsPass T{};
@@ -841,7 +871,7 @@ TsPass tstream_pass_geometry(const StreamPass& P, int map, int emap, int maps_pe
 bool tstream_encode_maps(const StreamPass& P, void* psi, void* E, void* psi_map, void* e_map) {
     if (!encode_fn() || P.tb != TB || P.n <= TB || P.n > 34) return false;
     return encode_shape(P, psi, 2, static_cast<CUtensorMap*>(psi_map)) &&
-           encode_shape(P, E, 1, static_cast<CUtensorMap*>(e_map));
+           (!E || encode_shape(P, E, 1, static_cast<CUtensorMap*>(e_map)));
 }
 
 void tstream_group_windows(const StreamPass* passes, int S, TsGroup* g) {
@@ -857,13 +887,16 @@ void tstream_group_windows(const StreamPass* passes, int S, TsGroup* g) {
         }
 }
 
-cudaError_t launch_tstream_pass(const TsGroup* groups, const TsSeg* segs, int nseg, uint32_t total, int grid,
+cudaError_t launch_tstream_pass(bool tab, const TsGroup* groups, const TsSeg* segs, int nseg, uint32_t total, int grid,
                                 unsigned* status, cudaStream_t st) {
-    const size_t sm = tstream_smem_bytes();
-    cudaError_t e = cudaFuncSetAttribute(k_tstream_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    k_tstream_pass<<<grid, NT, sm, st>>>(groups, segs, nseg, total, status);
-    return cudaGetLastError();
+    const size_t sm = tstream_smem_bytes(tab);
+    const auto go = [&](auto kern) -> cudaError_t {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e != cudaSuccess) return e;
+        kern<<<grid, NT, sm, st>>>(groups, segs, nseg, total, status);
+        return cudaGetLastError();
+    };
+    return tab ? go(k_tstream_pass<true>) : go(k_tstream_pass<false>);
 }
 
 size_t tstream_adj_smem_bytes() { return ta_offsets().total; }

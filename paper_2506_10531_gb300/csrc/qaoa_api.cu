@@ -423,7 +423,7 @@ extern "C" qaoa_status qaoa_grad_z(qaoa_ctx* c, int n, int p, const double* g, c
 // What the launches of a mix, or of a group that runs by itself, move and count, in launch order.
 struct StrStep {
     int g0, g1, mix;              // groups [g0, g1); mix < 0: one group by itself
-    bool grad = false;
+    bool grad = false, tab = false;
     double energy_bytes = 0.0, final_bytes = 0.0, reduce_bytes = 0.0;
     std::vector<double> pass_bytes, adj_bytes;
     int kernels = 0;
@@ -448,7 +448,8 @@ struct qaoa_plan {
                       int grid, agrid; std::vector<const void*> q; std::vector<void*> e;
                       // TMA streaming passes (complex64): per instance one state tensor map per
                       // pass shape, at maps_off in the header; tsp[i] is pass i's geometry
-                      bool tma = false; size_t maps_off = 0; int maps_per_inst = 0; std::vector<TsPass> tsp;
+                      bool tma = false, tab = false;   // tab: phases from Q, no energies
+                      size_t maps_off = 0; int maps_per_inst = 0; std::vector<TsPass> tsp;
                       int tgrid = 0;   // TMA passes' persistent grid
                       // TMA adjoint passes: per instance three maps (psi, lam, E) per adjoint pass
                       // shape at amaps_off; atsp[i] is adjoint pass i's geometry
@@ -458,7 +459,7 @@ struct qaoa_plan {
     // sums. Their instances follow one another at inst_off.
     struct Mix { int g0, g1;            // groups [g0, g1) of str
                  int count = 0, pmax = 0, tgrid = 0;
-                 bool grad = false;
+                 bool tab = false;
                  size_t inst_off = 0;
                  size_t fgrp_off = 0, agrp_off = 0;   // TsGroup arrays, forward and adjoint
                  struct Launch { size_t seg_off; int nseg; uint32_t total; };
@@ -507,11 +508,12 @@ std::vector<StrStep> str_steps(const qaoa_plan* P) {
         for (int j = st.g0; j < st.g1; ++j) {
             const auto& g = P->str[j];
             const double D = (double)(1ull << g.n), cnt = (double)g.count, nt = (double)(1ull << (g.n - tb));
+            st.tab = g.tab;
             st.energy_bytes += cnt * (D * rs + (double)g.n * g.n * rs);
             st.pass_bytes.resize(std::max(st.pass_bytes.size(), g.passes.size()), 0.0);
             for (size_t s = 0; s < g.passes.size(); ++s) {
                 const StreamPass& pass = g.passes[s];
-                st.pass_bytes[s] += cnt * D * ((pass.init ? 0.0 : cs) + (pass.no_store ? 0.0 : cs) + (pass.need_e ? rs : 0.0));
+                st.pass_bytes[s] += cnt * D * ((pass.init ? 0.0 : cs) + (pass.no_store ? 0.0 : cs) + (pass.need_e && !g.tab ? rs : 0.0));
             }
             st.final_bytes += cnt * (nt * (sizeof(double) + std::max(g.k, 1) * 12.0) + 8.0 + g.k * 16.0);
             if (stream_finalize_two_level(1ull << (g.n - tb), g.k)) ++st.kernels;
@@ -527,7 +529,8 @@ std::vector<StrStep> str_steps(const qaoa_plan* P) {
             }
         }
         int energies = 1;
-        if (st.mix >= 0) {
+        if (st.tab) energies = 0;
+        else if (st.mix >= 0) {
             energies = 0;
             int tiles = 0;
             for (const EnergyRun& r : energy_runs(P, st.g0, st.g1)) (r.n <= ENERGY_TILE_NMAX ? tiles : energies) += 1;
@@ -646,7 +649,7 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
             csg[d.n].push_back(i);
         else if (!dbl && !grad && d.n >= CL_NMIN && d.n <= CL_NMAX && tier == QAOA_TIER_CLUSTER)
             cg[{d.n, qaoa::eff_cluster_L(c, d.n, d.p)}].push_back(i);
-        else sg[{d.n, d.p, d.k, grad ? 1 : 0}].push_back(i);
+        else sg[{grad ? 1 : 0, d.n, d.p, d.k}].push_back(i);   // gradient runs last: each kind shares launches
     }
     auto make_desc = [&](int i) {
         const qaoa_inst& d = desc[i];
@@ -751,10 +754,10 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
     const int tb = stream_tile_bits(dbl), tba = stream_adj_tile_bits(dbl);
     for (auto& kv : sg) {
         qaoa_plan::StrGroup g{};
-        g.n = std::get<0>(kv.first);
-        g.p = std::get<1>(kv.first);
-        g.k = std::get<2>(kv.first);
-        g.grad = std::get<3>(kv.first) != 0;
+        g.grad = std::get<0>(kv.first) != 0;
+        g.n = std::get<1>(kv.first);
+        g.p = std::get<2>(kv.first);
+        g.k = std::get<3>(kv.first);
         g.count = (int)kv.second.size();
         StreamPass tmp[256];
         const int S = stream_plan(dbl, g.n, g.p, g.k, tmp, 256);
@@ -778,7 +781,8 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
         const int variant = dbl ? 2 : eff_stream_variant(c, g.n, g.p);
         g.tgrid = (variant == 1 ? 1 : 2) * c->nsm;
         // (energies the caller places at addresses TMA cannot take go through the cp.async passes)
-        bool e16 = true;
+        bool e16 = true, e_out = false;
+        for (int i : kv.second) e_out = e_out || desc[i].e_off >= 0;
         for (int i : kv.second)
             e16 = e16 && (desc[i].e_off < 0 || (reinterpret_cast<uintptr_t>(epool + desc[i].e_off) & 15u) == 0);
         if (!dbl && variant != 2 && tstream_available() && e16) {
@@ -789,6 +793,7 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
                     chunk_s.push_back(ps.s);
             std::sort(chunk_s.begin(), chunk_s.end());
             g.tma = true;
+            g.tab = !g.grad && !e_out;
             const int nshape = 1 + (int)chunk_s.size();   // state maps, then the energy maps
             g.maps_per_inst = 2 * nshape;
             for (auto& ps : g.passes) {
@@ -822,7 +827,7 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
             SI s{};
             const qaoa_inst& d = desc[i];
             s.e_off = (d.e_off >= 0) ? (size_t)-1 : scr;
-            if (d.e_off < 0) scr = align256(scr + D * sizeof(T));
+            if (d.e_off < 0 && !g.tab) scr = align256(scr + D * sizeof(T));
             s.psi_off = (d.psi_off >= 0) ? (size_t)-1 : scr;
             if (d.psi_off < 0) scr = align256(scr + D * sizeof(C2));
             s.part_off = scr;
@@ -853,12 +858,13 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
         if (!P->mix.empty() && P->mix.back().g1 == (int)i)
             for (int j = P->mix.back().g0; j < (int)i; ++j)
                 before += (uint64_t)P->str[j].count << (P->str[j].n - std::min(tb, tba));
-        if (P->mix.empty() || P->mix.back().g1 != (int)i || P->mix.back().tgrid != g.tgrid || before + tiles >= (1ull << 31) ||
+        if (P->mix.empty() || P->mix.back().g1 != (int)i || P->mix.back().tgrid != g.tgrid || P->mix.back().tab != g.tab || before + tiles >= (1ull << 31) ||
             (int)i - P->mix.back().g0 >= TS_MAX_GROUPS) {
             qaoa_plan::Mix m{};
             m.g0 = (int)i;
             m.inst_off = g.inst_off;
             m.tgrid = g.tgrid;
+            m.tab = g.tab;
             P->mix.push_back(m);
         }
         auto& m = P->mix.back();
@@ -966,7 +972,7 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
             I.beta = ppool + d.par_off + d.p;
             I.Q = qpool + d.q_off;
             I.psi = (s.psi_off == (size_t)-1) ? (void*)(psipool + d.psi_off) : (void*)(sb + s.psi_off);
-            T* Ebuf = (s.e_off == (size_t)-1) ? epool + d.e_off : reinterpret_cast<T*>(sb + s.e_off);
+            T* Ebuf = g.tab ? nullptr : (s.e_off == (size_t)-1) ? epool + d.e_off : reinterpret_cast<T*>(sb + s.e_off);
             I.E = Ebuf;
             char* pw = sb + s.part_off;
             I.part_expect = reinterpret_cast<double*>(pw);
@@ -1072,7 +1078,7 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
     }
     P->steps = str_steps(P);
     for (auto& m : P->steps) {
-        P->bytes.push_back(m.energy_bytes);
+        if (!m.tab) P->bytes.push_back(m.energy_bytes);
         for (double b : m.pass_bytes) P->bytes.push_back(b);
         P->bytes.push_back(m.final_bytes);
         for (double b : m.adj_bytes) P->bytes.push_back(b);
@@ -1242,7 +1248,7 @@ qaoa_status plan_enqueue(qaoa_plan* P, cudaStream_t st) {
         if (step.mix >= 0) {
             const auto& m = P->mix[step.mix];
             char* insts = base + m.inst_off;
-            CK(timed("energy", [&]() -> cudaError_t {
+            if (!m.tab) CK(timed("energy", [&]() -> cudaError_t {
                 int n[ENERGY_RUNS], first[ENERGY_RUNS], count[ENERGY_RUNS], k = 0;
                 cudaError_t e = cudaSuccess;
                 for (const EnergyRun& r : energy_runs(P, m.g0, m.g1)) {
@@ -1261,7 +1267,7 @@ qaoa_status plan_enqueue(qaoa_plan* P, cudaStream_t st) {
             }));
             for (const auto& L : m.fwd)
                 CK(timed("tstream_pass", [&] {
-                    return launch_tstream_pass(reinterpret_cast<const TsGroup*>(base + m.fgrp_off),
+                    return launch_tstream_pass(m.tab, reinterpret_cast<const TsGroup*>(base + m.fgrp_off),
                                                reinterpret_cast<const TsSeg*>(base + L.seg_off), L.nseg, L.total,
                                                (int)std::min<uint32_t>(L.total, (uint32_t)m.tgrid), status, st);
                 }));

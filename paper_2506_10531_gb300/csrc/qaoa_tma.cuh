@@ -133,18 +133,19 @@ __device__ __forceinline__ void cluster_arrive_release() {
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
 
 // Block sum of one FP32 value per thread in double-float arithmetic (each partial an unevaluated
-// sum hi + lo of two floats, combined with Knuth's TwoSum), fixed order, returned to thread 0 as
-// one FP64 value: about 44 bits of precision without the FP64 pipe, whose latency on this part
-// would dominate a warp shuffle tree of FP64 adds. red: 2 * (TMA_NT / 32) floats.
+// sum hi + lo of two floats, combined with Knuth's TwoSum), fixed order: about 44 bits of precision
+// without the FP64 pipe, whose latency on this part would dominate a warp shuffle tree of FP64 adds.
+// warp_sum_df by every warp, a barrier (one the caller needs anyway), sum_parts_df by one warp; all
+// its lanes return the sum. red: 2 * (TMA_NT / 32) floats.
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = a + b;
     const float bb = s - a;
     e = (a - (s - bb)) + (b - bb);
 }
-__device__ __forceinline__ double block_sum_df(float v, float* red) {
-    float hi = v, lo = 0.0f;
+template <int O>
+__device__ __forceinline__ void tree_sum_df(float& hi, float& lo) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = O; o > 0; o >>= 1) {
         const float oh = __shfl_xor_sync(0xffffffffu, hi, o);
         const float ol = __shfl_xor_sync(0xffffffffu, lo, o);
         float s, e;
@@ -153,23 +154,19 @@ __device__ __forceinline__ double block_sum_df(float v, float* red) {
         hi = s + e;
         lo = e - (hi - s);
     }
+}
+__device__ __forceinline__ void warp_sum_df(float v, float* red) {
+    float hi = v, lo = 0.0f;
+    tree_sum_df<16>(hi, lo);
     const int w = threadIdx.x >> 5;
-    __syncthreads();
     if ((threadIdx.x & 31) == 0) { red[2 * w] = hi; red[2 * w + 1] = lo; }
-    __syncthreads();
-    double tot = 0.0;
-    if (threadIdx.x == 0) {
-        float th = 0.0f, tl = 0.0f;
-        for (int i = 0; i < TMA_NT / 32; ++i) {
-            float s, e;
-            two_sum(th, red[2 * i], s, e);
-            e += tl + red[2 * i + 1];
-            th = s + e;
-            tl = e - (th - s);
-        }
-        tot = (double)th + (double)tl;
-    }
-    return tot;
+}
+__device__ __forceinline__ double sum_parts_df(const float* red) {
+    constexpr int NW = TMA_NT / 32;
+    const int w = threadIdx.x & (NW - 1);
+    float hi = red[2 * w], lo = red[2 * w + 1];
+    tree_sum_df<NW / 2>(hi, lo);
+    return (double)hi + (double)lo;
 }
 
 // Top-k list of a tile whose amplitudes are in shared memory, given each thread's FP32

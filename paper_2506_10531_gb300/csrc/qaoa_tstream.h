@@ -28,10 +28,10 @@ constexpr size_t TS_MAP_BYTES = 128;   // one CUtensorMap, 64-byte aligned
 
 // The driver's tensor-map encoder could be found.
 bool tstream_available();
-size_t tstream_smem_bytes();
+size_t tstream_smem_bytes(bool tab);
 TsPass tstream_pass_geometry(const StreamPass& P, int map, int emap, int maps_per_inst);
 // Encode the tensor maps of pass P (any pass of the same kind and chunk gives the same maps) for
-// a state at psi and its energies at E (both 16-byte aligned) into psi_map / e_map (host,
+// a state at psi and its energies at E (both 16-byte aligned; E NULL: none) into psi_map / e_map (host,
 // 64-byte aligned).
 bool tstream_encode_maps(const StreamPass& P, void* psi, void* E, void* psi_map, void* e_map);
 // A plan group's passes (forward or adjoint) for launches that hold passes of several groups: the
@@ -51,9 +51,10 @@ struct TsSeg {
 constexpr int TS_MAX_GROUPS = 65535;
 // Fill the windows of g (n, tb set) from its pass list.
 void tstream_group_windows(const StreamPass* passes, int S, TsGroup* g);
-// A launch over `nseg` segments (device array, `total` tiles in all) of the groups at `groups`; a
-// bounded wait that ran out sets bit 0 of *status.
-cudaError_t launch_tstream_pass(const TsGroup* groups, const TsSeg* segs, int nseg, uint32_t total, int grid,
+// A launch over `nseg` segments (device array, `total` tiles in all) of the groups at `groups`, whose
+// phases come from Q (tab) or from the energies in HBM; a bounded wait that ran out sets bit 0 of
+// *status.
+cudaError_t launch_tstream_pass(bool tab, const TsGroup* groups, const TsSeg* segs, int nseg, uint32_t total, int grid,
                                 unsigned* status, cudaStream_t st);
 
 // Adjoint passes (tiles of TSA_TB bits, kind-B chunks of h <= 8 high qubits): per pass shape
