@@ -9,24 +9,25 @@
 // between L2 and shared memory, like the streaming tier. What differs is the order: the C CTAs
 // of one cluster run every pass of ONE instance, separated by cluster barriers, before taking
 // the next instance. With about 70 clusters of 4 CTAs in flight, two instances each, the working
-// set (state and energies of the instances in flight, 0.75-1.5 MiB each) stays below the 126 MB
-// L2, so the passes read and write L2, not HBM, and the whole batch is one launch.
+// set (the states of the instances in flight, 0.25-1 MiB each) stays below the 126 MB L2, so the
+// passes read and write L2, not HBM, and the whole batch is one launch. Phases and energies come from
+// Q in shared memory (qaoa_phase.cuh), a table per pass built while its first tile is on its way: with
+// energies built in pass 0 and moved with every tile, 128 instances of n = 17, p = 2 took 337 us,
+// without 325. What bounds the passes: the copies between L2 and shared memory and, with one instance
+// per cluster, the latency from pass to pass (63 us for one of n = 16, p = 3; 80 us for 74 at once).
 //
 // Passes (2^H tiles each, H = n - 13; CTA rank r takes tiles r, r + C, ...):
 //   kind A: tile bits 0..12 are qubits 0..12 (2^13 contiguous amplitudes);
 //   kind B: 2^c contiguous amplitudes (c = 13 - H) times the 2^H values of qubits 13..n-1.
-// Pass 0 (A) builds the tile's energies from Q, starts |+>, applies the first cost phase and
-// mixes qubits 0..12 of layer 0; pass j (0 < j < p) mixes the qubits of its kind for layer j-1,
+// Pass 0 (A) starts |+>, applies the first cost phase and mixes qubits 0..12 of layer 0; pass j (0 < j < p) mixes the qubits of its kind for layer j-1,
 // applies the cost phase of layer j and mixes them again for layer j; pass p finishes layer p-1
 // and reduces <C> (FP64 across tiles) and the top-k list. Kinds alternate A, B, A, ...
 //
 // Tiles move by TMA (cp.async.bulk.tensor) with completion on an mbarrier: the state with the
-// 128-byte swizzle (16-byte chunk index XOR 128-byte line index), the energies unswizzled. The
-// register windows of a kind-A tile are bits [0,4) (16-byte pair accesses), [4,8) and [8,13);
-// with the lanes of a warp on tile bits outside the window every shared access is free of bank
-// conflicts under that swizzle, and the cost phase runs in the [8,13) window, where the lanes
-// cover bits 0..4 and read the unswizzled energies conflict-free. A kind-B tile has one window
-// (its H high bits). Between passes the writer waits for its bulk stores, fences the async
+// 128-byte swizzle (16-byte chunk index XOR 128-byte line index). The register windows of a kind-A
+// tile are bits [0,4) (16-byte pair accesses), [4,8) and [8,13), the cost phase in the last; with the
+// lanes of a warp on tile bits outside the window every shared access is free of bank conflicts under
+// that swizzle. A kind-B tile has one window (its H high bits). Between passes the writer waits for its bulk stores, fences the async
 // proxy and arrives on the cluster barrier (release); the readers wait (acquire) and fence
 // before their next TMA loads. Every mbarrier wait is bounded; a wait that runs out sets bit 0
 // of the launch's status word and the kernel runs on to its end without further waits.
@@ -36,6 +37,7 @@
 #include "qaoa_cstream.h"
 #include "qaoa_engine.cuh"
 #include "qaoa_kernels.h"
+#include "qaoa_phase.cuh"
 #include "qaoa_tma.cuh"
 
 namespace cg = cooperative_groups;
@@ -57,12 +59,11 @@ constexpr uint32_t TD = 1u << TB;
 constexpr int NT = 256;
 
 // ---- shared-memory layout ------------------------------------------------------------------
-// One state tile and one energy tile, shared by the two instance slots of a CTA; the energy tile
-// doubles as the top-k scratch of the final pass (after the <C> partial has read it) and of the
-// merge on rank 0. Per slot: Q, layer constants, the CTA's top-k lists and <C> partial.
+// One state tile, one phase table (of the step's pass; the final pass's holds energies) and the top-k
+// scratch, shared by the two instance slots of a CTA. Per slot: Q, layer constants, the CTA's top-k
+// lists and <C> partial.
 struct CsOff {
-    size_t psi, E, red, escr, wbound, Q[2], lc[2], lists[2], cex[2], desc[2], mbar, total;
-    size_t wb, cnt, cand, out, wlists;   // inside the energy tile
+    size_t psi, tab, red, escr, wbound, Q[2], lc[2], lists[2], cex[2], desc[2], wb, cnt, cand, out, wlists, mbar, total;
 };
 __host__ __device__ inline size_t cs_al(size_t x) { return (x + 15) & ~(size_t)15; }
 constexpr size_t CS_DESC_BYTES = 128;   // a slot's copy of its instance descriptor
@@ -70,9 +71,9 @@ __host__ __device__ inline CsOff cs_offsets(int tpc) {
     CsOff o{};
     size_t x = 0;
     o.psi = x; x += (size_t)TD * 8;                        // 64 KiB, 1024-byte aligned at run time
-    o.E = x; x += (size_t)TD * 4;                          // 32 KiB
-    o.red = x; x = cs_al(x + 32 * sizeof(double));
-    o.escr = x; x = cs_al(x + 256 * sizeof(float));       // energy tables of pass 0
+    o.tab = x; x = cs_al(x + sizeof(PhaseTab));
+    o.red = x; x = cs_al(x + 2 * (NT / 32) * sizeof(float));
+    o.escr = x; x = cs_al(x + 256 * sizeof(float));       // staged parameters; energy tables of pass 0
     o.wbound = x; x = cs_al(x + (NT / 32) * sizeof(float));
     for (int s = 0; s < 2; ++s) {
         o.Q[s] = x; x = cs_al(x + (size_t)CS_NMAX * CS_NMAX * 4);
@@ -81,14 +82,13 @@ __host__ __device__ inline CsOff cs_offsets(int tpc) {
         o.cex[s] = x; x = cs_al(x + sizeof(double));
         o.desc[s] = x; x = cs_al(x + CS_DESC_BYTES);
     }
+    o.wb = x; x = cs_al(x + 16 * (NT / 32) * sizeof(float));
+    o.cnt = x; x = cs_al(x + 4 * sizeof(int));
+    o.cand = x; x = cs_al(x + TOPK_CAP * sizeof(TopEnt));
+    o.out = x; x = cs_al(x + 16 * sizeof(TopEnt));
+    o.wlists = x; x = cs_al(x + (NT / 32) * 32 * sizeof(TopEnt));
     o.mbar = x; x = cs_al(x + sizeof(uint64_t));
     o.total = x + 1024;                                    // room to align psi to 1024 bytes
-    size_t y = o.E;
-    o.wb = y; y = cs_al(y + 16 * (NT / 32) * sizeof(float));
-    o.cnt = y; y = cs_al(y + 4 * sizeof(int));
-    o.cand = y; y = cs_al(y + TOPK_CAP * sizeof(TopEnt));
-    o.out = y; y = cs_al(y + 16 * sizeof(TopEnt));
-    o.wlists = y;
     return o;
 }
 
@@ -122,16 +122,14 @@ __device__ __forceinline__ void w2_store(float2* sp, const float2 (&v)[32]) {
 #pragma unroll
     for (int i = 0; i < 32; ++i) sp[b + (i << 8)] = v[i];
 }
-template <int R>
-__device__ __forceinline__ void phase_group(float2 (&v)[1 << R], const float* sE, uint32_t e0, int eshift,
-                                            int parity, const LayerConst<float>& k) {
+// The cost phase of layer constants k on group r of the thread in window [A, 13).
+template <int A, int R>
+__device__ __forceinline__ void phase_group(float2 (&v)[1 << R], const TileVals& x, int r, int parity,
+                                            const LayerConst<float>& k) {
     const Pending<float> pre(k.pre, k.pcot, parity);
-#pragma unroll
-    for (int i = 0; i < (1 << R); ++i) {
-        float s, c;
-        sincos_phase(k.ph, sE[e0 + ((uint32_t)i << eshift)], s, c);
+    tab_phases<A, R>(x, r, [&](int i, float s, float c) {
         rot_neg(v[i], s * pre.f[__popc(i) & 1], c * pre.f[__popc(i) & 1]);
-    }
+    });
 }
 // W1: bits [4, 8). Group g < 512 (thread t: g = t and t + 256): base = (g & 15) | (g >> 4) << 8,
 // element i at (base ^ (i & 7) << 1) | (i << 4).
@@ -184,21 +182,22 @@ struct CsInstDev {
     const float* Q;
     const float* gamma;
     const float* beta;
+    float* E;                  // energies to return, or NULL
     double* expect;
     uint64_t* topk_idx;
     double* topk_prob;
-    const CUtensorMap* maps;   // psi kind A, psi kind B, E kind A, E kind B
+    const CUtensorMap* maps;   // psi kind A, psi kind B
 };
 static_assert(sizeof(CsInstDev) <= CS_DESC_BYTES && sizeof(CsInstDev) % 8 == 0, "descriptor copy");
 
-// Energies of kind-A tile tau of pass 0 in the W2 layout (thread t owns u = t | j << 8), with
+// Energies of kind-A tile tau (instances that return them) in the W2 layout (thread t owns u = t | j << 8), with
 // the tile's fixed global bits S = tau << 13. With P_ik = Q_ik + Q_ki (i < k, tile qubits),
 // d_i = Q_ii + sum_{s in S} (Q_is + Q_si) and E_S = sum_{s, s' in S} Q_ss',
 //   E(z) = E_S + sum_{i<8} t_i d_i + sum_{i<k<8} t_i t_k P_ik + Eh[j] + sum_{b in j} W_b(t),
 //   W_b(t) = sum_{i<8} t_i P_{i,8+b},   Eh[j] = sum_{b in j} d_{8+b} + sum_{b<c in j} P_{8+b,8+c},
 // every pair of set bits of z counted once with both Q_ik and Q_ki. The tables (scr: 256 floats)
 // are built once per tile; each thread's sums are unrolled with 0/1 weights (independent loads,
-// no serial chains). ev[j] receives the energies (the caller writes them to the energy tile).
+// no serial chains). ev[j] receives the energies.
 __device__ __forceinline__ void w2_energies(int n, uint32_t zfix, const float* Qs, float* scr, float (&ev)[32]) {
     float* P = scr;           // 13 x 13, upper triangle
     float* d = scr + 169;     // 13
@@ -287,8 +286,8 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
     unsigned char* sm = sm_raw + (((raw + 1023u) & ~1023u) - raw);
     const CsOff o = cs_offsets(TPC);
     float2* sp = reinterpret_cast<float2*>(sm + o.psi);
-    float* sE = reinterpret_cast<float*>(sm + o.E);
-    double* red = reinterpret_cast<double*>(sm + o.red);
+    PhaseTab& tab = *reinterpret_cast<PhaseTab*>(sm + o.tab);
+    float* red = reinterpret_cast<float*>(sm + o.red);
     TileTopk ts;
     ts.wb = reinterpret_cast<float*>(sm + o.wb);
     ts.cnt = reinterpret_cast<int*>(sm + o.cnt);
@@ -301,7 +300,7 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
     uint32_t parity = 0;
     bool ok = true;
     const int ncl = (int)(gridDim.x / C), cid = (int)(blockIdx.x / C);
-    const TileRef<float> tile{sp, nullptr, sE, TB};
+    const TileRef<float> tile{sp, nullptr, nullptr, TB};
 
     // Two instance slots per cluster, run in alternating steps: step j runs one pass of slot
     // j % 2. At the end of step j the stores of step j - 1 are complete and every CTA arrives at
@@ -349,15 +348,12 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
     };
     refill(0);
     refill(1);
-    // thread 0: TMA load of tile tau of a pass of instance I into the buffers: the energies at
-    // once (no store of a pass > 0 reads their buffer), the state once the last tile's store has
-    // read the state buffer (wait_store)
+    // thread 0: TMA load of tile tau of a pass of instance I, once the last tile's store has read
+    // the buffer (wait_store)
     const auto issue_load = [&](const CsInstDev& I, bool kindA, uint32_t tau, bool wait_store) {
         fence_async_global();
-        mbar_expect_tx(mbar, TD * 8 + TD * 4);
-        if (kindA) tma_load_3d(sE, &I.maps[2], 0, 0, (int)tau, mbar);
-        else tma_load_4d(sE, &I.maps[3], 0, 0, (int)tau, 0, mbar);
         if (wait_store) bulk_wait_read();
+        mbar_expect_tx(mbar, TD * 8);
         if (kindA) tma_load_4d(sp, &I.maps[0], 0, 0, 0, (int)tau, mbar);
         else tma_load_4d(sp, &I.maps[1], 0, 0, (int)tau, 0, mbar);
     };
@@ -398,7 +394,6 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
                     }
                 }
             }
-            fence_async_smem();   // the merge's writes to the energy tile before a TMA load refills it
             __syncthreads();
             refill(sl);
         }
@@ -412,39 +407,46 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
             const bool kindA = (pass & 1) == 0;
             const bool fin = pass == p;
             double my_ex = 0.0;
+            // the pass's table, while its first tile is on its way
+            const int c = kindA ? TB : CB;
+            if (fin) tab_build<true>(tab, sQ, n, 0.0, c, TB);
+            else tab_build<false>(tab, sQ, n, (double)lc[pass].ph.hi + (double)lc[pass].ph.lo, c, TB);
             for (int jt = 0; jt < TPC; ++jt) {
                 const uint32_t tau = rank + (uint32_t)(jt * C);
                 float accp = 0.0f, pmax = -1.0f;   // final pass: FP32 <C> terms (32 per thread) and max |psi|^2
-                // the bulk stores of the previous tile have read the buffers before they are
-                // refilled (by TMA in passes > 0, whose load waits for them itself; by the threads
-                // in pass 0, once the tile's energies are in registers; the first tile of a step
-                // follows the end-of-step wait)
+                if (fin) tab_tile<true>(tab, tau << c, c, TB);
+                else tab_tile<false>(tab, tau << c, c, TB);
+                // the bulk store of the previous tile has read the buffer before it is refilled (by
+                // TMA in passes > 0, whose load waits for it itself; by the threads in pass 0; the
+                // first tile of a step follows the end-of-step wait)
                 if (pass > 0) {
                     if (threadIdx.x == 0 && ok && !(jt == 0 && prefetched)) issue_load(I, kindA, tau, jt > 0);
                     if (ok) ok = mbar_wait_bounded(mbar, parity);
                     ok = __syncthreads_and(ok);
                     parity ^= 1u;
+                } else {
+                    if (jt > 0 && threadIdx.x == 0) bulk_wait_read();
+                    __syncthreads();
                 }
                 if (kindA) {
+                    const int par = __popc(threadIdx.x) + __popc(tau);
                     if (pass == 0) {
-                        // energies, |+>, the first cost phase and layer 0 on window [8, 13)
-                        float ev[32];
-                        w2_energies(n, tau << TB, sQ, reinterpret_cast<float*>(sm + o.escr), ev);
-                        if (jt > 0) {
-                            if (threadIdx.x == 0) bulk_wait_read();
-                            __syncthreads();
+                        if (I.E) {
+                            float ev[32];
+                            w2_energies(n, tau << TB, sQ, reinterpret_cast<float*>(sm + o.escr), ev);
+                            float* Eg = I.E + (tau << TB) + threadIdx.x;
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) Eg[i << 8] = ev[i];
+                            __syncthreads();   // the scratch is free for the next tile
                         }
-                        const uint32_t t = threadIdx.x;
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) sE[t + ((uint32_t)i << 8)] = ev[i];
-                        const int pc = __popc(tau) + __popc(t);
+                        // |+>, the first cost phase and layer 0 on window [8, 13)
                         float2 v[32];
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) {
-                            float s, c;
-                            sincos_phase(lc[0].ph, ev[i], s, c);
-                            float2 a = make_float2(I.amp0 * c, -I.amp0 * s);
-                            v[i] = times_i_pow(a, pc + __popc(i));
+                        {
+                            TileVals x;
+                            x.init<false>(tab);
+                            tab_phases<8, 5>(x, 0, [&](int i, float s, float c) {
+                                v[i] = times_i_pow(make_float2(I.amp0 * c, -I.amp0 * s), par + __popc(i));
+                            });
                         }
                         mix_layer<5>(v, 31, lc[0]);
                         w2_store(sp, v);
@@ -460,17 +462,19 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
                         float2 v[32];
                         w2_load(sp, v);
                         mix_layer<5>(v, 31, lc[pass - 1]);
+                        TileVals x;
                         if (!fin) {
-                            phase_group<5>(v, sE, threadIdx.x, 8, __popc(threadIdx.x) + __popc(tau), lc[pass]);
+                            x.init<false>(tab);
+                            phase_group<8, 5>(v, x, 0, par, lc[pass]);
                             mix_layer<5>(v, 31, lc[pass]);
                         } else {
-                            scale_group<5>(v, Pending<float>(lc[p - 1].post, lc[p - 1].cot, __popc(threadIdx.x) + __popc(tau)));
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) {
+                            scale_group<5>(v, Pending<float>(lc[p - 1].post, lc[p - 1].cot, par));
+                            x.init<true>(tab);
+                            tab_energies<8, 5>(x, 0, [&](int i, float e) {
                                 const float pr = v[i].x * v[i].x + v[i].y * v[i].y;
-                                accp = fmaf(pr, sE[threadIdx.x + (i << 8)], accp);
+                                accp = fmaf(pr, e, accp);
                                 pmax = fmaxf(pmax, pr);
-                            }
+                            });
                         }
                         w2_store(sp, v);
                         if (!fin) {
@@ -481,6 +485,9 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
                         }
                     }
                 } else {
+                    TileVals x;
+                    if (fin) x.init<true>(tab);
+                    else x.init<false>(tab);
 #pragma unroll 1
                     for (int r = 0; r < NB; ++r) {
                         const uint32_t lo = threadIdx.x + (uint32_t)(r * NT);
@@ -490,21 +497,21 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
                         for (int i = 0; i < (1 << H); ++i) v[i] = sp[b + ((uint32_t)i << CB)];
                         mix_layer<H>(v, (1 << H) - 1, lc[pass - 1]);
                         if (!fin) {
-                            phase_group<H>(v, sE, lo, CB, __popc(lo) + __popc(tau), lc[pass]);
+                            phase_group<CB, H>(v, x, r, __popc(lo) + __popc(tau), lc[pass]);
                             mix_layer<H>(v, (1 << H) - 1, lc[pass]);
                         } else {
                             scale_group<H>(v, Pending<float>(lc[p - 1].post, lc[p - 1].cot, __popc(lo) + __popc(tau)));
-#pragma unroll
-                            for (int i = 0; i < (1 << H); ++i) {
+                            tab_energies<CB, H>(x, r, [&](int i, float e) {
                                 const float pr = v[i].x * v[i].x + v[i].y * v[i].y;
-                                accp = fmaf(pr, sE[lo + ((uint32_t)i << CB)], accp);
+                                accp = fmaf(pr, e, accp);
                                 pmax = fmaxf(pmax, pr);
-                            }
+                            });
                         }
 #pragma unroll
                         for (int i = 0; i < (1 << H); ++i) sp[b + ((uint32_t)i << CB)] = v[i];
                     }
                 }
+                if (fin) warp_sum_df(accp, red);
                 __syncthreads();
                 if (!fin) {
                     fence_async_smem();
@@ -512,14 +519,11 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
                     if (threadIdx.x == 0) {
                         if (kindA) tma_store_4d(&I.maps[0], sp, 0, 0, 0, (int)tau);
                         else tma_store_4d(&I.maps[1], sp, 0, 0, (int)tau, 0);
-                        if (pass == 0) tma_store_3d(&I.maps[2], sE, 0, 0, (int)tau);
                         bulk_commit();
                         stored = true;
                     }
                 } else {
-                    // <C> partial and top-k list of the tile (the top-k scratch overlays the
-                    // energies once the partial has read them); the state leaves in the
-                    // standard frame
+                    // <C> partial and top-k list of the tile; the state leaves in the standard frame
                     const uint32_t cmask = (1u << CB) - 1u;
                     const auto zmap = [kindA, tau, cmask](uint32_t u) -> uint32_t {
                         return kindA ? (u | (tau << TB)) : ((u & cmask) | (tau << CB) | ((u >> CB) << TB));
@@ -535,10 +539,7 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
                             z = lo | (tau << CB) | (e << TB);
                         }
                     };
-                    __syncthreads();   // every energy has been read
-                    warp_sum_df(accp, reinterpret_cast<float*>(red));
-                    __syncthreads();
-                    if (threadIdx.x < 32) my_ex += sum_parts_df(reinterpret_cast<const float*>(red));
+                    if (threadIdx.x < 32) my_ex += sum_parts_df(red);
                     if (I.k > 0) {
                         if (!topk_own(sp, I.k, pmax, elem, ts, reinterpret_cast<float*>(sm + o.wbound))) {
                             // flat distribution: the tile-wide selection, with each thread's maximum
@@ -565,7 +566,7 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
                             stored = true;
                         }
                     }
-                    fence_async_smem();   // the top-k scratch writes before the next tile's TMA writes
+                    fence_async_smem();   // the sub-passes' shared writes before the next tile's TMA writes
                     __syncthreads();
                 }
             }
@@ -696,9 +697,9 @@ cudaError_t cstream_max_clusters(int n, int* out) {
 
 int cstream_cluster_size(int n) { return cs_cluster(1 << (n - TB)); }
 
-// The four tensor maps of one instance: state and energies (2^n values each, 16-byte aligned)
-// as kind-A and kind-B tiles. Returns false if the driver refuses one of them.
-bool cstream_encode_maps(int n, void* psi, void* E, void* maps_out) {
+// The tensor maps of one instance's state (16-byte aligned) as kind-A and kind-B tiles. Returns false
+// if the driver refuses one of them.
+bool cstream_encode_maps(int n, void* psi, void* maps_out) {
     if (!encode_fn() || n < CS_NMIN || n > CS_NMAX) return false;
     CUtensorMap* m = static_cast<CUtensorMap*>(maps_out);
     const int H = n - TB, c = TB - H;
@@ -715,23 +716,11 @@ bool cstream_encode_maps(int n, void* psi, void* E, void* maps_out) {
         const cuuint32_t b[4] = {32, 1u << (c - 4), 1, (cuuint32_t)NH};
         if (!encode(&m[1], psi, 4, d, s, b, true)) return false;
     }
-    {   // E, kind A: (256 floats, 32 lines, tile)
-        const cuuint64_t d[3] = {256, 32, NH};
-        const cuuint64_t s[2] = {1024, 32768};
-        const cuuint32_t b[3] = {256, 32, 1};
-        if (!encode(&m[2], E, 3, d, s, b, false)) return false;
-    }
-    {   // E, kind B: (256 floats, 2^(c-8) lines, tile = bits c..12, bits 13..n-1)
-        const cuuint64_t d[4] = {256, 1ull << (c - 8), NH, NH};
-        const cuuint64_t s[3] = {1024, (1ull << c) * 4, (1ull << TB) * 4};
-        const cuuint32_t b[4] = {256, 1u << (c - 8), 1, (cuuint32_t)NH};
-        if (!encode(&m[3], E, 4, d, s, b, false)) return false;
-    }
     return true;
 }
 
 void cstream_fill_inst(void* out, int n, int p, int k, bool out_psi, const float* Q, const float* gamma,
-                       const float* beta, double* expect, uint64_t* topk_idx, double* topk_prob,
+                       const float* beta, float* E, double* expect, uint64_t* topk_idx, double* topk_prob,
                        const void* maps_dev) {
     CsInstDev d{};
     d.n = n;
@@ -742,6 +731,7 @@ void cstream_fill_inst(void* out, int n, int p, int k, bool out_psi, const float
     d.Q = Q;
     d.gamma = gamma;
     d.beta = beta;
+    d.E = E;
     d.expect = expect;
     d.topk_idx = topk_idx;
     d.topk_prob = topk_prob;

@@ -482,8 +482,8 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const TsGroup* __restric
             __syncthreads();
             if (!same) set_layer_consts<float>(lc, I.gamma, I.beta, I.p, P.n, false);
             if (TAB && retab) {
-                if (P.fin) tab_build<true>(tab, I.Q, P.n, 0.0f, P.c, P.s);
-                else tab_build<false>(tab, I.Q, P.n, I.gamma[P.lb], P.c, P.s);
+                if (P.fin) tab_build<true>(tab, I.Q, P.n, 0.0, P.c, P.s);
+                else tab_build<false>(tab, I.Q, P.n, (double)I.gamma[P.lb] * 0.15915494309189533577, P.c, P.s);   // gamma / 2 pi
             }
             if (threadIdx.x == 0) {
                 cur_g = I.gamma; cur_b = I.beta; cur_p = I.p; cur_n = P.n;

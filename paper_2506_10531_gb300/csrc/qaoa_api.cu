@@ -715,9 +715,9 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
         g.clusters = std::min(g.count, mc);
         P->clu.push_back(g);
     }
-    // cluster-streaming: descriptors, then four tensor maps per instance (64-byte aligned);
-    // per-instance state and energies in the scratch unless the caller receives them
-    struct CsI { size_t psi_off, e_off; };
+    // cluster-streaming: descriptors, then the tensor maps of each instance (64-byte aligned); its
+    // state in the scratch unless the caller receives it
+    struct CsI { size_t psi_off; };
     std::vector<std::vector<CsI>> csinfo;
     std::vector<size_t> cs_maps_off;
     for (auto& kv : csg) {
@@ -737,8 +737,6 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
             CsI x{};
             x.psi_off = (desc[i].psi_off >= 0) ? (size_t)-1 : scr;
             if (desc[i].psi_off < 0) scr = align256(scr + D * sizeof(C2));
-            x.e_off = (desc[i].e_off >= 0) ? (size_t)-1 : scr;
-            if (desc[i].e_off < 0) scr = align256(scr + D * sizeof(T));
             v.push_back(x);
         }
         csinfo.push_back(v);
@@ -932,9 +930,8 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
                 const qaoa_inst& d = desc[i];
                 const CsI& x = csinfo[gi][j];
                 void* psi = (x.psi_off == (size_t)-1) ? (void*)(psipool + d.psi_off) : (void*)(sb + x.psi_off);
-                void* E = (x.e_off == (size_t)-1) ? (void*)(epool + d.e_off) : (void*)(sb + x.e_off);
                 const size_t moff = cs_maps_off[gi] + CS_MAPS_BYTES * j;
-                if (!cstream_encode_maps(d.n, psi, E, img.data() + moff)) {
+                if (!cstream_encode_maps(d.n, psi, img.data() + moff)) {
                     if (P->owns) cudaFree(P->dev);
                     delete P;
                     return fail(QAOA_E_CUDA, "instance %d: tensor maps of the cluster-streaming tier refused", i);
@@ -943,6 +940,7 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
                                   d.psi_off >= 0, reinterpret_cast<const float*>(qpool + d.q_off),
                                   reinterpret_cast<const float*>(ppool + d.par_off),
                                   reinterpret_cast<const float*>(ppool + d.par_off + d.p),
+                                  d.e_off >= 0 ? reinterpret_cast<float*>(epool + d.e_off) : nullptr,
                                   io->expect ? io->expect + i : nullptr,
                                   d.k > 0 ? io->topk_idx + (int64_t)i * io->k_stride : nullptr,
                                   (d.k > 0 && io->topk_prob) ? io->topk_prob + (int64_t)i * io->k_stride : nullptr,

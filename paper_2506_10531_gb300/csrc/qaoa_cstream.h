@@ -10,7 +10,7 @@ namespace qaoa {
 
 constexpr int CS_TILE_BITS = 13;
 constexpr int CS_NMIN = 15, CS_NMAX = 17;
-constexpr size_t CS_MAPS_BYTES = 4 * 128;   // four CUtensorMap per instance, 64-byte aligned
+constexpr size_t CS_MAPS_BYTES = 2 * 128;   // two CUtensorMap per instance, 64-byte aligned
 
 // The driver's tensor-map encoder could be found.
 bool cstream_available();
@@ -20,12 +20,13 @@ size_t cstream_inst_bytes();
 int cstream_cluster_size(int n);
 // Occupancy limit of active clusters for n qubits (0 when none fits).
 cudaError_t cstream_max_clusters(int n, int* out);
-// Encode the four tensor maps of an instance (state and energies at psi / E, 16-byte aligned)
-// into maps_out (host memory, CS_MAPS_BYTES, 64-byte aligned). False if the driver refuses.
-bool cstream_encode_maps(int n, void* psi, void* E, void* maps_out);
-// Host image of one device descriptor; maps_dev is the device address of its four maps.
+// Encode the two tensor maps of an instance (its state at psi, 16-byte aligned) into maps_out (host
+// memory, CS_MAPS_BYTES, 64-byte aligned). False if the driver refuses.
+bool cstream_encode_maps(int n, void* psi, void* maps_out);
+// Host image of one device descriptor; E receives the energies (NULL: not returned); maps_dev is the
+// device address of its maps.
 void cstream_fill_inst(void* out, int n, int p, int k, bool out_psi, const float* Q, const float* gamma,
-                       const float* beta, double* expect, uint64_t* topk_idx, double* topk_prob,
+                       const float* beta, float* E, double* expect, uint64_t* topk_idx, double* topk_prob,
                        const void* maps_dev);
 // One launch over `count` descriptors (device array, same n): `clusters` clusters walk them
 // round-robin; a bounded wait that ran out sets bit 0 of *status.

@@ -48,16 +48,16 @@ __device__ __forceinline__ uint32_t tab_term(double w, double g, bool& bad) {
 }
 __device__ __forceinline__ int tile_qubit(int a, int c, int s) { return a < c ? a : a - c + s; }
 
-// The table of an n-qubit instance (Q: n x n floats) for tiles with c low bits and s (kind A: c = 13).
-// All 256 threads call it; contains one barrier; the table may be read after the next one.
+// The table of an n-qubit instance (Q: n x n floats) for tiles with c low bits and s (kind A: c = 13);
+// g = gamma / 2 pi (unused with F). All 256 threads call it; contains one barrier; the table may be
+// read after the next one.
 template <bool F>
-__device__ __forceinline__ void tab_build(PhaseTab& t, const float* Q, int n, float gamma, int c, int s) {
-    const double g = (double)gamma * 0.15915494309189533577;   // gamma / 2 pi
+__device__ __forceinline__ void tab_build(PhaseTab& t, const float* Q, int n, double g, int c, int s) {
     bool bad = false;
-    for (int x = threadIdx.x; x < 32 * 32; x += 256) {
-        const int i = x >> 5, j = x & 31;
-        if (i > j || j >= n) continue;
-        const double w = i == j ? (double)Q[i * n + i] : (double)Q[i * n + j] + (double)Q[j * n + i];
+    for (int x = threadIdx.x; x < n * n; x += 256) {
+        const int i = x / n, j = x - i * n;
+        if (i > j) continue;
+        const double w = i == j ? (double)Q[x] : (double)Q[x] + (double)Q[j * n + i];
         t.W[i * 32 + j] = t.W[j * 32 + i] = tab_term<F>(w, g, bad);
     }
     bad = __syncthreads_or(bad);

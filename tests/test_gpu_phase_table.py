@@ -46,8 +46,8 @@ def run(q, n, p, Qs, par, energies, dbl=False):
 
 
 # (n, p, scale of Q): scale 1e3 takes phases through hundreds of turns, 1e7 through the reduction of
-# terms beyond 5e5 turns. n = 14..22 have one chunk of 1..9 high qubits, 23 two.
-@pytest.mark.parametrize("n,p,scale", [(18, 1, 1.0), (18, 3, 1.0), (19, 2, 1e3), (20, 1, 1e7), (21, 2, 1.0), (22, 2, 1.0),
+# terms beyond 5e5 turns. n = 14..22 have one chunk of 1..9 high qubits, 23 two; 15..17 run in clusters.
+@pytest.mark.parametrize("n,p,scale", [(15, 1, 1.0), (16, 3, 1e3), (17, 2, 1.0), (18, 1, 1.0), (18, 3, 1.0), (19, 2, 1e3), (20, 1, 1e7), (21, 2, 1.0), (22, 2, 1.0),
                                        (23, 1, 1.0), (24, 2, 1.0)])
 def test_table(q, n, p, scale):
     Qs = [scale * synth.symmetric_q(n, seed=60 + n + i) for i in range(2)]
@@ -56,11 +56,12 @@ def test_table(q, n, p, scale):
     par = [np.concatenate(synth.random_params(p, seed=90 + i)) for i in range(2)]
     ea, pa, ta, _ = run(q, n, p, Qs, par, False)
     eb, pb, tb, E = run(q, n, p, Qs, par, True)
-    ec, pc, tc, _ = run(q, n, p, Qs, par, False, True)
+    ec, pc, tc, Ec = run(q, n, p, Qs, par, True, True)
     for i in range(2):
         Emax = np.abs(E[i << n:(i + 1) << n]).max()
         W = np.abs(Qs[i].astype(np.float32)).sum()
         ref = pc[i]
+        assert np.abs(E[i << n:(i + 1) << n] - Ec[i << n:(i + 1) << n]).max() <= 32 * W * 2.0 ** -24
         # __sincosf 2^-21 and the angle's rounding 2^-23 a layer, n p mixer steps of 2^-22; the
         # FP32 sums of <C> 32 roundings
         tol = p * 2.0 ** -20 + n * p * 2.0 ** -22
