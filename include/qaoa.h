@@ -422,18 +422,18 @@ qaoa_status dqaoa_session_cycle_sampled(dqaoa_session* s, const double* Q, int q
 qaoa_status dqaoa_session_shots(dqaoa_session* s, uint64_t* shots_out, uint64_t* best_out, void* psi_out);
 /* Times of the last cycle in ms, out[4]: the host's decompose-and-enqueue time (index draw,
  * copies and launches), the device time from the first copy to the last chunk's results, the
- * host merge time (the first chunk's merge overlaps the device), and the whole call. */
+ * host merge time (all but the last chunk's merge overlaps the device), and the whole call. */
 qaoa_status dqaoa_session_timing(dqaoa_session* s, double* out);
 /* Device time of the last dqaoa_session_cycle's solve in ms: from the first chunk's launch to
  * the end of the last chunk's kernels (the chunks may overlap on the device). */
 qaoa_status dqaoa_session_solve_ms(dqaoa_session* s, double* ms);
 /* The batched plans the session launches, in order (for timing and kernel counts): the m
- * sub-QUBOs are solved in two chunks when m >= 128, else in one, the second on its own stream
- * (the two solves overlap on the device). The host merges the first chunk while the device
- * solves the second; the first holds floor(11 m / 16) sub-QUBOs (floor(9 m / 16) for N > 4096)
- * for the cluster-streaming tier,
- * else ceil(0.65 m) rounded up to a multiple of the instances whose tiles give each block of a
- * streaming launch one tile (at most m - 1). Returns NULL for i past the last plan. */
+ * sub-QUBOs are solved in several chunks when m >= 128, else in one, every other chunk on a second
+ * stream (the solves overlap on the device). The host merges a chunk while the device solves the
+ * next. For the cluster-streaming tier a chunk holds one sub-QUBO per cluster the device runs at a
+ * time (at most eight chunks; a remainder of less than a quarter chunk joins the last), else there
+ * are two, the first of ceil(0.65 m) rounded up to a multiple of the instances whose tiles give each
+ * block of a streaming launch one tile (at most m - 1). Returns NULL for i past the last plan. */
 qaoa_plan* dqaoa_session_plan(dqaoa_session* s, int i);
 void dqaoa_session_destroy(dqaoa_session* s);
 

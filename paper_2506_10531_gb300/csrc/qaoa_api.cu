@@ -1521,21 +1521,22 @@ struct dqaoa_session {
     double* mca_h = nullptr;
     // the sub-QUBOs are solved in chunks, one plan each, so that the host merges chunk c while
     // the device solves chunk c + 1 (the merge is sequential over sub-QUBOs in index order)
+    static constexpr int CHUNKS_MAX = 8;
     int chunks = 1;
-    int chunk_start[3] = {0, 0, 0};
-    qaoa_plan* plans[2] = {nullptr, nullptr};
-    cudaEvent_t chunk_solved[2] = {nullptr, nullptr};   // chunk's kernels done (main stream)
-    cudaEvent_t chunk_done[2] = {nullptr, nullptr};     // chunk's results on the host (side stream)
+    int chunk_start[CHUNKS_MAX + 1] = {};
+    qaoa_plan* plans[CHUNKS_MAX] = {};
+    cudaEvent_t chunk_solved[CHUNKS_MAX] = {};   // chunk's kernels done (its stream)
+    cudaEvent_t chunk_done[CHUNKS_MAX] = {};     // chunk's results on the host
     cudaEvent_t dev_begin = nullptr, dev_end = nullptr;   // device part of the last cycle
     // the FP64 blocks go to the host on a side stream, beside the first chunk's kernels
     cudaStream_t side = nullptr;
     cudaEvent_t sub_done = nullptr, qblk_done = nullptr, setup_done = nullptr;
-    cudaStream_t solve2 = nullptr;  // the second chunk's solve
+    cudaStream_t solve2 = nullptr;  // every other chunk's solve
     // per chunk one packed block (pair terms, candidates, <C>, status word) on the device and its
     // pinned copy: one copy per chunk brings back everything the merge reads
     char* pk_dev = nullptr;
     char* pk_h = nullptr;
-    size_t pk_off[2] = {0, 0};
+    size_t pk_off[CHUNKS_MAX] = {};
     bool last_sampled = false;      // the last cycle was dqaoa_session_cycle_sampled
     cudaEvent_t solve_begin = nullptr, solve_end = nullptr;   // span of the chunk solves
     double t_decompose = 0.0, t_merge = 0.0, t_cycle = 0.0; // host ms of the last cycle
@@ -1634,35 +1635,38 @@ extern "C" qaoa_status dqaoa_session_create(qaoa_ctx* c, int N, int m, int k, in
     for (int l = 0; l < p; ++l) { par[l] = (float)gamma[l]; par[p + l] = (float)(paper_mixer ? -beta[l] : beta[l]); }
     e = cudaMemcpy(s->params, par.data(), par.size() * sizeof(float), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) { dqaoa_session_destroy(s); return cuda_fail(e, "session params upload"); }
-    // Two chunks from m = 128 on, so that the host merges the first while the device solves the
-    // second. Streaming tier: about two thirds, rounded up to whole waves (instances whose tiles
-    // give every block of a launch one tile; measured on GB300 for 256 sub-QUBOs of n = 16: 190 /
-    // 66 beat 152 / 104, 128 / 128 and 114 / 142 by 4-8%). Cluster-streaming tier, whose two
-    // chunk launches overlap on the device: 11/16 of m for N <= 4096 (measured for 256
-    // sub-QUBOs at N = 1000: splits from 128 to 216 within 4%, 176 best, 232 8% slower), 9/16
-    // above (at N = 10^4 the merge costs about 0.8 of the solve).
+    // From m = 128 on several chunks, so that the host merges the first while the device solves the
+    // rest. Cluster-streaming tier: a chunk is one instance per cluster the device holds (74), whose
+    // launches, on two streams in turn, follow one another without a gap. One instance per cluster
+    // takes 80 us a chunk (n = 16, p = 3), two 150 us, so the chunks cost the device little, and
+    // the merge, which takes as long as the solve, starts after the first 74 instead of most of
+    // them; a remainder of less than a quarter chunk joins the last. 256 sub-QUBOs at N = 1000: two
+    // chunks (176 / 80; every split from 64 to 176 alike) 500 us a cycle, chunks of 74 420 us.
+    // Other tiers: two chunks. Streaming tier: about two thirds first, rounded up to whole waves
+    // (instances whose tiles give every block of a launch one tile; measured on GB300 for 256
+    // sub-QUBOs of n = 16: 190 / 66 beat 152 / 104, 128 / 128 and 114 / 142 by 4-8%).
     s->chunks = m >= 128 ? 2 : 1;
-    int m0 = m;
+    s->chunk_start[1] = m;
     if (s->chunks == 2) {
         const int tier = eff_tier(c, k, p);
         if (k >= CS_NMIN && k <= CS_NMAX && tier == QAOA_TIER_CSTREAM && cstream_usable(c, k)) {
-            // the first chunk's merge should end before the second chunk's solve does: with the
-            // merge's cost growing with N (the update of h per flipped variable), a larger N
-            // takes a smaller first chunk
-            m0 = N <= 4096 ? (m * 11) / 16 : (m * 9) / 16;
+            int w = 0;
+            cstream_max_clusters(k, &w);
+            w = std::max({1, w, (m + dqaoa_session::CHUNKS_MAX - 1) / dqaoa_session::CHUNKS_MAX});
+            s->chunks = std::max(1, (m + (3 * w) / 4) / w);
+            for (int ch = 1; ch < s->chunks; ++ch) s->chunk_start[ch] = ch * w;
         } else {
             int w = 1;
             if (k >= 16 && (k > 18 || tier == QAOA_TIER_STREAM)) {
                 const int tiles = 1 << (k - stream_tile_bits(false));
                 w = std::max(1, 2 * c->nsm / tiles);
             }
-            m0 = (m * 13 + 19) / 20;
+            int m0 = (m * 13 + 19) / 20;
             m0 = (m0 + w - 1) / w * w;
+            s->chunk_start[1] = std::max(1, std::min(m - 1, m0));
         }
-        m0 = std::max(1, std::min(m - 1, m0));
+        s->chunk_start[s->chunks] = m;
     }
-    s->chunk_start[1] = m0;
-    s->chunk_start[2] = m;
     for (int ch = 0; ch < s->chunks; ++ch) {
         const int j0 = s->chunk_start[ch], mc = s->chunk_start[ch + 1] - j0;
         std::vector<qaoa_inst> d(mc);
@@ -1764,9 +1768,9 @@ extern "C" qaoa_status dqaoa_session_cycle(dqaoa_session* s, const double* Q, in
     qaoa_status r = session_decompose(s, Q, q_changed, x, seed, cycle, st, nullptr, m);
     if (r) return r;
     CK(cudaEventRecord(s->sub_done, st));
-    // the second chunk's solve runs on its own stream: its clusters take the SMs the first
-    // chunk's clusters leave while that chunk's last instances finish
-    if (s->chunks == 2) CK(cudaStreamWaitEvent(s->solve2, s->sub_done, 0));
+    // every other chunk's solve runs on its own stream: its clusters take the SMs the chunk before
+    // it leaves while that chunk's last instances finish
+    if (s->chunks > 1) CK(cudaStreamWaitEvent(s->solve2, s->sub_done, 0));
     CK(cudaStreamWaitEvent(s->side, s->sub_done, 0));
     CK(cudaMemcpyAsync(s->qblk_h, s->qblk, (size_t)m * k * k * sizeof(double), cudaMemcpyDeviceToHost, s->side));
     CK(cudaEventRecord(s->qblk_done, s->side));
@@ -1780,7 +1784,7 @@ extern "C" qaoa_status dqaoa_session_cycle(dqaoa_session* s, const double* Q, in
     CK(cudaEventRecord(s->solve_begin, st));
     for (int ch = 0; ch < s->chunks; ++ch) {
         const int j0 = s->chunk_start[ch], mc = s->chunk_start[ch + 1] - j0;
-        cudaStream_t cs = ch == 0 ? st : s->solve2;
+        cudaStream_t cs = (ch & 1) ? s->solve2 : st;
         r = qaoa_plan_launch(s->plans[ch], (qaoa_stream_t)cs);
         if (r) return r;
         CK(cudaEventRecord(s->chunk_solved[ch], cs));
@@ -1798,7 +1802,7 @@ extern "C" qaoa_status dqaoa_session_cycle(dqaoa_session* s, const double* Q, in
     }
     for (int ch = 0; ch < s->chunks; ++ch) CK(cudaStreamWaitEvent(s->side, s->chunk_done[ch], 0));
     CK(cudaEventRecord(s->dev_end, s->side));
-    if (s->chunks == 2) CK(cudaStreamWaitEvent(st, s->chunk_solved[1], 0));   // the caller's stream covers the cycle
+    if (s->chunks > 1) CK(cudaStreamWaitEvent(st, s->chunk_solved[(s->chunks - 2) | 1], 0));   // the caller's stream covers the cycle
     CK(cudaEventRecord(s->solve_end, st));
     CK(cudaStreamWaitEvent(st, s->dev_end, 0));
     const double t1 = now_ms();
