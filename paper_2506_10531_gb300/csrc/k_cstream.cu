@@ -12,7 +12,7 @@
 // set (the states of the instances in flight, 0.25-1 MiB each) stays below the 126 MB L2, so the
 // passes read and write L2, not HBM, and the whole batch is one launch. Phases and energies come from
 // Q in shared memory (qaoa_phase.cuh), a table per pass built while its first tile is on its way: with
-// energies built in pass 0 and moved with every tile, 128 instances of n = 17, p = 2 took 337 us,
+// energies built in pass 0 and moved with every tile, 101 instances of n = 17, p = 5 took 337 us,
 // without 325. What bounds the passes: the copies between L2 and shared memory and, with one instance
 // per cluster, the latency from pass to pass (63 us for one of n = 16, p = 3; 80 us for 74 at once).
 //
@@ -49,12 +49,11 @@ namespace {
 using namespace tma;
 
 constexpr int TB = CS_TILE_BITS;
-// CTAs per cluster for a pass of `ntile` tiles (each CTA then takes ntile / C tiles per pass).
-// Measured on GB300 (batches of 128-256 instances): 4 CTAs beat 8 by 4-7% at n = 16 and 17 (twice
-// the clusters in flight, half the cluster barriers per tile), except where the instance count
-// falls just past a multiple of the slots in flight.
-constexpr int CS_CMAX = 4;
-__host__ __device__ constexpr int cs_cluster(int ntile) { return ntile < CS_CMAX ? ntile : CS_CMAX; }
+// CTAs per cluster: 4 for batches (4 beat 8 by 4-7% at n = 16 and 17: twice the clusters in flight,
+// half the cluster barriers per tile); 8, half the tiles per CTA and pass, for counts of instances
+// that are all in flight at once with 8 (36 of them) and leave half the device idle with 4: p = 3, 1 and 36
+// instances of n = 16 in 45 and 53 us against 63 and 76, 36 of n = 17 in 84 against 133.
+constexpr int CS_NARROW = 4, CS_WIDE = 8;
 constexpr uint32_t TD = 1u << TB;
 constexpr int NT = 256;
 
@@ -79,7 +78,7 @@ __host__ __device__ inline CsOff cs_offsets(int tpc) {
         o.Q[s] = x; x = cs_al(x + (size_t)CS_NMAX * CS_NMAX * 4);
         o.lc[s] = x; x = cs_al(x + 64 * sizeof(LayerConst<float>));
         o.lists[s] = x; x = cs_al(x + (size_t)tpc * 16 * sizeof(TopEnt));
-        o.cex[s] = x; x = cs_al(x + sizeof(double));
+        o.cex[s] = x; x = cs_al(x + (size_t)tpc * sizeof(double));
         o.desc[s] = x; x = cs_al(x + CS_DESC_BYTES);
     }
     o.wb = x; x = cs_al(x + 16 * (NT / 32) * sizeof(float));
@@ -271,11 +270,10 @@ __device__ __forceinline__ void w2_energies(int n, uint32_t zfix, const float* Q
     for (int j = 0; j < 32; ++j) ev[j] = base + (Eh[j] + X[j]);
 }
 
-template <int H>
+template <int H, int C>   // C: CTAs per cluster
 __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__ insts, int count,
                                                   unsigned* status) {
     constexpr int NTILE = 1 << H;                 // tiles per pass
-    constexpr int C = cs_cluster(NTILE);          // CTAs per cluster
     constexpr int TPC = NTILE / C;                // tiles per CTA per pass
     constexpr int CB = TB - H;                    // contiguous bits of a kind-B tile
     constexpr int NB = 1 << (CB - 8);             // kind-B groups per thread
@@ -365,19 +363,19 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
         bool stored = false;   // thread 0: this step committed a bulk store group
         if (sfin[sl] >= 0) {
             // the instance of this slot finished two steps ago (its final pass is visible to the
-            // cluster): rank 0 merges the CTAs' <C> partials (rank order) and top-k lists
+            // cluster): rank 0 merges the tiles' <C> partials (tile order) and the CTAs' top-k lists
             if (rank == 0) {
                 const CsInstDev& I = *reinterpret_cast<const CsInstDev*>(sm + o.desc[sl]);
                 double* cex = reinterpret_cast<double*>(sm + o.cex[sl]);
                 TopEnt* lists = reinterpret_cast<TopEnt*>(sm + o.lists[sl]);
                 if (threadIdx.x == 0 && I.expect) {
-                    // the C remote loads in flight together, then the sum in rank order
-                    double part[C];
+                    // the remote loads in flight together, then the sum in tile order
+                    double part[NTILE];
 #pragma unroll
-                    for (int r = 0; r < C; ++r) part[r] = *cl.map_shared_rank(cex, r);
+                    for (int t = 0; t < NTILE; ++t) part[t] = cl.map_shared_rank(cex, t % C)[t / C];
                     double acc = 0.0;
 #pragma unroll
-                    for (int r = 0; r < C; ++r) acc += part[r];
+                    for (int t = 0; t < NTILE; ++t) acc += part[t];
                     *I.expect = acc;
                 }
                 if (I.k > 0) {
@@ -406,7 +404,7 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
             const int n = I.n, p = I.p, pass = spass[sl];
             const bool kindA = (pass & 1) == 0;
             const bool fin = pass == p;
-            double my_ex = 0.0;
+            double* cex = reinterpret_cast<double*>(sm + o.cex[sl]);   // <C> partials of the CTA's tiles
             // the pass's table, while its first tile is on its way
             const int c = kindA ? TB : CB;
             if (fin) tab_build<true>(tab, sQ, n, 0.0, c, TB);
@@ -539,7 +537,10 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
                             z = lo | (tau << CB) | (e << TB);
                         }
                     };
-                    if (threadIdx.x < 32) my_ex += sum_parts_df(red);
+                    if (threadIdx.x < 32) {
+                        const double tot = sum_parts_df(red);
+                        if (threadIdx.x == 0) cex[jt] = tot;
+                    }
                     if (I.k > 0) {
                         if (!topk_own(sp, I.k, pmax, elem, ts, reinterpret_cast<float*>(sm + o.wbound))) {
                             // flat distribution: the tile-wide selection, with each thread's maximum
@@ -570,12 +571,8 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
                     __syncthreads();
                 }
             }
-            if (fin) {
-                if (threadIdx.x == 0) *reinterpret_cast<double*>(sm + o.cex[sl]) = my_ex;
-                sfin[sl] = j;
-            } else {
-                spass[sl] = pass + 1;
-            }
+            if (fin) sfin[sl] = j;
+            else spass[sl] = pass + 1;
         }
         // end of step j. Step j's bulk stores drain while step j + 1 computes: here only step
         // j - 1's stores must be complete (every group but the newest when step j committed one,
@@ -621,13 +618,11 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
     if (threadIdx.x == 0 && !ok) atomicOr(status, 1u);
 }
 
-template <int H>
-cudaError_t cs_launch_h(const void* insts, int count, int clusters, cudaStream_t st, int* max_clusters,
-                        unsigned* status) {
-    constexpr int NTILE = 1 << H;
-    constexpr int C = cs_cluster(NTILE);
-    const size_t smem = cs_offsets(NTILE / C).total;
-    cudaError_t e = cudaFuncSetAttribute(k_cstream<H>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <int H, int C>
+cudaError_t cs_launch_hc(const void* insts, int count, int clusters, cudaStream_t st, int* max_clusters,
+                         unsigned* status) {
+    const size_t smem = cs_offsets((1 << H) / C).total;
+    cudaError_t e = cudaFuncSetAttribute(k_cstream<H, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
@@ -643,14 +638,25 @@ cudaError_t cs_launch_h(const void* insts, int count, int clusters, cudaStream_t
     if (max_clusters) {
         cfg.gridDim = dim3(C);
         int mc = 0;
-        e = cudaOccupancyMaxActiveClusters(&mc, k_cstream<H>, &cfg);
+        e = cudaOccupancyMaxActiveClusters(&mc, k_cstream<H, C>, &cfg);
         *max_clusters = (e == cudaSuccess) ? mc : 0;
         return e;
     }
     cfg.gridDim = dim3((unsigned)(clusters * C));
-    e = cudaLaunchKernelEx(&cfg, k_cstream<H>, static_cast<const CsInstDev*>(insts), count, status);
+    e = cudaLaunchKernelEx(&cfg, k_cstream<H, C>, static_cast<const CsInstDev*>(insts), count, status);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
+}
+cudaError_t cs_launch(int n, bool wide, const void* insts, int count, int clusters, cudaStream_t st, int* max_clusters,
+                      unsigned* status) {
+    switch (2 * (n - TB) + (wide ? 1 : 0)) {
+        case 4: return cs_launch_hc<2, CS_NARROW>(insts, count, clusters, st, max_clusters, status);
+        case 6: return cs_launch_hc<3, CS_NARROW>(insts, count, clusters, st, max_clusters, status);
+        case 7: return cs_launch_hc<3, CS_WIDE>(insts, count, clusters, st, max_clusters, status);
+        case 8: return cs_launch_hc<4, CS_NARROW>(insts, count, clusters, st, max_clusters, status);
+        case 9: return cs_launch_hc<4, CS_WIDE>(insts, count, clusters, st, max_clusters, status);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 // cuTensorMapEncodeTiled, looked up once through the runtime (no link against the driver).
@@ -685,17 +691,10 @@ size_t cstream_inst_bytes() { return sizeof(CsInstDev); }
 
 bool cstream_available() { return encode_fn() != nullptr; }
 
-cudaError_t cstream_max_clusters(int n, int* out) {
+cudaError_t cstream_max_clusters(int n, bool wide, int* out) {
     *out = 0;
-    switch (n - TB) {
-        case 2: return cs_launch_h<2>(nullptr, 0, 0, nullptr, out, nullptr);
-        case 3: return cs_launch_h<3>(nullptr, 0, 0, nullptr, out, nullptr);
-        case 4: return cs_launch_h<4>(nullptr, 0, 0, nullptr, out, nullptr);
-        default: return cudaErrorInvalidValue;
-    }
+    return cs_launch(n, wide, nullptr, 0, 0, nullptr, out, nullptr);
 }
-
-int cstream_cluster_size(int n) { return cs_cluster(1 << (n - TB)); }
 
 // The tensor maps of one instance's state (16-byte aligned) as kind-A and kind-B tiles. Returns false
 // if the driver refuses one of them.
@@ -739,13 +738,8 @@ void cstream_fill_inst(void* out, int n, int p, int k, bool out_psi, const float
     *static_cast<CsInstDev*>(out) = d;
 }
 
-cudaError_t launch_cstream(int n, const void* insts, int count, int clusters, unsigned* status, cudaStream_t st) {
-    switch (n - TB) {
-        case 2: return cs_launch_h<2>(insts, count, clusters, st, nullptr, status);
-        case 3: return cs_launch_h<3>(insts, count, clusters, st, nullptr, status);
-        case 4: return cs_launch_h<4>(insts, count, clusters, st, nullptr, status);
-        default: return cudaErrorInvalidValue;
-    }
+cudaError_t launch_cstream(int n, bool wide, const void* insts, int count, int clusters, unsigned* status, cudaStream_t st) {
+    return cs_launch(n, wide, insts, count, clusters, st, nullptr, status);
 }
 
 }  // namespace qaoa

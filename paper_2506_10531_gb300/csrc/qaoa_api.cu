@@ -442,7 +442,7 @@ struct qaoa_plan {
     cudaGraphExec_t graph = nullptr;  // captured launch sequence (qaoa_plan_capture)
     struct ResGroup { int n, pmax, count; bool grad; size_t desc_off; int grid; int q_slot; int rmax; };
     struct CluGroup { int n, L, pmax, count; size_t desc_off; int clusters; };
-    struct CsGroup { int n, count; size_t desc_off; int clusters; };
+    struct CsGroup { int n, count; size_t desc_off; int clusters; bool wide; };
     struct StrGroup { int n, p, k, count; bool grad; size_t inst_off; std::vector<StreamPass> passes;
                       std::vector<StreamPass> apasses;   // adjoint plan (adjoint tile bits)
                       int grid, agrid; std::vector<const void*> q; std::vector<void*> e;
@@ -728,9 +728,9 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
         hdr = align256(hdr + cstream_inst_bytes() * g.count);
         cs_maps_off.push_back(hdr);
         hdr = align256(hdr + CS_MAPS_BYTES * g.count);
-        int mc = 0;
-        cstream_max_clusters(g.n, &mc);
-        g.clusters = std::max(1, std::min(g.count, mc));
+        // counts whose clusters of 8 CTAs are all in flight at once take those (k_cstream.cu)
+        g.wide = g.count <= c->cs_max_wide[g.n];
+        g.clusters = std::max(1, std::min(g.count, g.wide ? c->cs_max_wide[g.n] : c->cs_max[g.n]));
         std::vector<CsI> v;
         const size_t D = (size_t)1 << g.n;
         for (int i : kv.second) {
@@ -1097,7 +1097,9 @@ bool cstream_usable(qaoa_ctx* c, int n) {
         int mc = 0, dev = -1;
         cudaGetDevice(&dev);
         if (dev != c->device) cudaSetDevice(c->device);
-        const bool ok = cstream_available() && cstream_max_clusters(n, &mc) == cudaSuccess && mc >= 1;
+        const bool ok = cstream_available() && cstream_max_clusters(n, false, &mc) == cudaSuccess && mc >= 1;
+        c->cs_max[n] = mc;
+        if (ok && n > CS_NMIN) cstream_max_clusters(n, true, &c->cs_max_wide[n]);
         cudaGetLastError();
         if (dev >= 0 && dev != c->device) cudaSetDevice(dev);
         c->cs_ok[n] = ok ? 1 : -1;
@@ -1237,7 +1239,7 @@ qaoa_status plan_enqueue(qaoa_plan* P, cudaStream_t st) {
         }));
     for (auto& g : P->cs)
         CK(timed("cstream", [&] {
-            return launch_cstream(g.n, base + g.desc_off, g.count, g.clusters,
+            return launch_cstream(g.n, g.wide, base + g.desc_off, g.count, g.clusters,
                                   reinterpret_cast<unsigned*>(counters + PLAN_STATUS_SLOT), st);
         }));
     const int tb = stream_tile_bits(P->dbl), tba = stream_adj_tile_bits(P->dbl);
@@ -1650,9 +1652,7 @@ extern "C" qaoa_status dqaoa_session_create(qaoa_ctx* c, int N, int m, int k, in
     if (s->chunks == 2) {
         const int tier = eff_tier(c, k, p);
         if (k >= CS_NMIN && k <= CS_NMAX && tier == QAOA_TIER_CSTREAM && cstream_usable(c, k)) {
-            int w = 0;
-            cstream_max_clusters(k, &w);
-            w = std::max({1, w, (m + dqaoa_session::CHUNKS_MAX - 1) / dqaoa_session::CHUNKS_MAX});
+            const int w = std::max({1, c->cs_max[k], (m + dqaoa_session::CHUNKS_MAX - 1) / dqaoa_session::CHUNKS_MAX});
             s->chunks = std::max(1, (m + (3 * w) / 4) / w);
             for (int ch = 1; ch < s->chunks; ++ch) s->chunk_start[ch] = ch * w;
         } else {

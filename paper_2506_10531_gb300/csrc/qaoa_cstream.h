@@ -16,10 +16,8 @@ constexpr size_t CS_MAPS_BYTES = 2 * 128;   // two CUtensorMap per instance, 64-
 bool cstream_available();
 // Size of one device descriptor (plan header entry).
 size_t cstream_inst_bytes();
-// CTAs per cluster for n qubits.
-int cstream_cluster_size(int n);
-// Occupancy limit of active clusters for n qubits (0 when none fits).
-cudaError_t cstream_max_clusters(int n, int* out);
+// Occupancy limit of active clusters, of 4 CTAs or (wide, n > CS_NMIN) 8, for n qubits (0 when none fits).
+cudaError_t cstream_max_clusters(int n, bool wide, int* out);
 // Encode the two tensor maps of an instance (its state at psi, 16-byte aligned) into maps_out (host
 // memory, CS_MAPS_BYTES, 64-byte aligned). False if the driver refuses.
 bool cstream_encode_maps(int n, void* psi, void* maps_out);
@@ -30,6 +28,6 @@ void cstream_fill_inst(void* out, int n, int p, int k, bool out_psi, const float
                        const void* maps_dev);
 // One launch over `count` descriptors (device array, same n): `clusters` clusters walk them
 // round-robin; a bounded wait that ran out sets bit 0 of *status.
-cudaError_t launch_cstream(int n, const void* insts, int count, int clusters, unsigned* status, cudaStream_t st);
+cudaError_t launch_cstream(int n, bool wide, const void* insts, int count, int clusters, unsigned* status, cudaStream_t st);
 
 }  // namespace qaoa

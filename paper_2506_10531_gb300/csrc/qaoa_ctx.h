@@ -25,6 +25,7 @@ struct qaoa_ctx {
     int cluster_L[32] = {0};  // local qubits per CTA of the cluster tier by n (0: default 14)
     qaoa_tuned tuned[32][65]; // autotuner table by (n, p)
     int cs_ok[32] = {0};      // cluster-streaming tier: 0 unknown, 1 usable, -1 not on this device
+    int cs_max[32] = {0}, cs_max_wide[32] = {0};   // its clusters in flight, of 4 and of 8 CTAs (where usable)
 };
 
 namespace qaoa {
