@@ -129,9 +129,9 @@ def measured_peaks():
 # Source files that define each kernel family (the kernel itself and the headers it includes).
 KERNEL_SOURCES = {
     "stream": ["k_stream.cu", "qaoa_engine.cuh", "qaoa_common.cuh", "qaoa_stream.h", "qaoa_kernels.h"],
-    "tstream_pass": ["k_tstream.cu", "qaoa_tma.cuh", "qaoa_engine.cuh", "qaoa_common.cuh", "qaoa_tstream.h",
-                     "qaoa_stream.h", "qaoa_kernels.h"],
-    "cstream": ["k_cstream.cu", "qaoa_tma.cuh", "qaoa_engine.cuh", "qaoa_common.cuh", "qaoa_cstream.h",
+    "tstream_pass": ["k_tstream.cu", "qaoa_phase.cuh", "qaoa_tma.cuh", "qaoa_engine.cuh", "qaoa_common.cuh",
+                     "qaoa_tstream.h", "qaoa_stream.h", "qaoa_kernels.h"],
+    "cstream": ["k_cstream.cu", "qaoa_phase.cuh", "qaoa_tma.cuh", "qaoa_engine.cuh", "qaoa_common.cuh", "qaoa_cstream.h",
                 "qaoa_kernels.h"],
     "resident": ["k_resident.cu", "qaoa_engine.cuh", "qaoa_common.cuh", "qaoa_kernels.h"],
     "cluster": ["k_cluster.cu", "qaoa_engine.cuh", "qaoa_common.cuh", "qaoa_kernels.h"],

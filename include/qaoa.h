@@ -108,7 +108,8 @@ qaoa_status qaoa_tuning_load(qaoa_ctx* ctx, const char* path);
 
 /* E[z] = z^T Q z for z = 0..2^n-1 (Section IV, QUBO -> diagonal Hamiltonian).
  * Q: n*n floats, row-major; read as given (E uses Q_ij and Q_ji as separate terms).
- * E: 2^n floats. Built by Gray-code increments from direct FP32 evaluations. */
+ * E: 2^n floats, FP32 sums (direct up to n = 20, above by Gray-code increments of at most 256 steps
+ * from direct evaluations). */
 qaoa_status qaoa_build_energies(qaoa_ctx* ctx, int n, const float* Q, float* E,
                                 qaoa_stream_t stream);
 

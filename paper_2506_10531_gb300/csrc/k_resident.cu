@@ -1,8 +1,8 @@
 // k_resident.cu -- resident tier: one CTA per QAOA instance, the whole 2^n state (complex64
 // up to n = 14, complex128 up to n = 13) and its energy vector held in shared memory for all
 // p layers. One persistent launch walks a queue of instance descriptors; each CTA
-//   1. builds E(z) = z^T Q z for all z by Gray-code increments (Section IV, the QUBO mapped to
-//      the diagonal problem Hamiltonian),
+//   1. builds E(z) = z^T Q z for all z from small tables (Section IV, the QUBO mapped to the
+//      diagonal problem Hamiltonian),
 //   2. applies the p layers of Eq. 2 (cost phase, then exp(-i beta X_q) on every qubit) from
 //      |+> with the snake schedule of the tile engine,
 //   3. reduces <C> = sum |psi|^2 E (FP32 per-thread partials over at most 2^R terms, FP64

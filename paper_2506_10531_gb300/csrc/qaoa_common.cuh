@@ -197,14 +197,10 @@ __device__ __forceinline__ C times_i_pow(C v, int m) {
     return r;
 }
 
-// Im(conj(x) * y) and Re(conj(x) * y)
+// Im(conj(x) * y)
 template <typename C>
 __device__ __forceinline__ auto im_conj_mul(const C& x, const C& y) -> decltype(x.x) {
     return x.x * y.y - x.y * y.x;
-}
-template <typename C>
-__device__ __forceinline__ auto re_conj_mul(const C& x, const C& y) -> decltype(x.x) {
-    return x.x * y.x + x.y * y.y;
 }
 
 // ---- warp reductions (fixed order: deterministic) ----------------------------------------
@@ -224,22 +220,6 @@ __device__ __forceinline__ float warp_sort_desc(float v) {
         }
     }
     return v;
-}
-
-// The k-th largest (k = 1..32) of one float per lane.
-__device__ __forceinline__ float warp_kth_largest(float v, int k) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int size = 2; size <= 32; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            const float o = __shfl_xor_sync(0xffffffffu, v, stride);
-            const bool asc = (lane & size) == 0;
-            const bool lower = (lane & stride) == 0;
-            v = (lower != asc) ? fminf(v, o) : fmaxf(v, o);
-        }
-    }
-    return __shfl_sync(0xffffffffu, v, k - 1);
 }
 
 __device__ __forceinline__ double warp_sum(double v) {

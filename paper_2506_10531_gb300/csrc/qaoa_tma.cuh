@@ -108,10 +108,6 @@ __device__ __forceinline__ void tma_store_5d(const CUtensorMap* map, const void*
                  ::"l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(saddr(src))
                  : "memory");
 }
-// the shared-memory sources of all but the most recent committed bulk store have been read
-__device__ __forceinline__ void bulk_wait_read_all_but_one() {
-    asm volatile("cp.async.bulk.wait_group.read 1;\n" ::: "memory");
-}
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;\n" ::: "memory"); }
 // the shared-memory sources of every committed bulk store have been read
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
