@@ -591,9 +591,9 @@ def run_large(args):
                  amps * args.steps / tot_s, "amp-layer-updates/s", args, world, 1e3 * tot_s / args.steps,
                  "c64 state, f32 energies, f64 reductions",
                  {"workload": f"large instance: dense n={n} QUBO U[-1,1] (seed 5), p=2, gamma=(0.4,0.7), "
-                              f"beta=(0.6,0.3), complex64 ({(8 << n) / 2**30:g} GiB) + FP32 energies, top-8"
+                              f"beta=(0.6,0.3), complex64 ({(8 << n) / 2**30:g} GiB), top-8"
                               + (", with adjoint gradients (profiling case)" if args.large_grad else ""),
-                  "l2": "inputs larger than L2 (state + energies)", "parallelism": f"replicas x{world}"},
+                  "l2": "inputs larger than L2 (the state)", "parallelism": f"replicas x{world}"},
                  solves_per_s=args.steps * world / tot_s,
                  amp_gate_updates_per_s=amps * (n + 1) * args.steps / tot_s,
                  latency_ms={"p50": float(np.percentile(step_ms, 50)), "p99": float(np.percentile(step_ms, 99))},

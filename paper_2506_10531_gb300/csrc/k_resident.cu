@@ -24,7 +24,7 @@ struct Smem {
     typename Num<T>::C* lam;
     T* E;
     T* Q;
-    LayerConst<T>* lc;     // adjoint; the forward run's FwdConst<T> occupy the same place
+    LayerConst<T>* lc;     // adjoint; the forward run's constants occupy the same place
     double* red;       // 64 doubles
     TileTopk tk;       // top-k scratch
     T* escr;           // energy-build tables
@@ -57,14 +57,14 @@ __host__ __device__ inline size_t smem_layout(int n, int p, bool grad, int threa
     return o;
 }
 
-template <typename T, int R>
+template <typename T, int R, typename K>
 __device__ void forward_run(const InstDesc<T>& d, const Smem<T>& s, const WinSched& ws, bool started) {
     const int n = d.n, p = d.p;
     const TileRef<T> tile{s.psi, s.lam, s.E, n};
     // started: the energy build already wrote |+> after the first cost layer
     const bool init = !(d.flags & F_INIT_PSI) && !started;
     const T amp0 = (T)exp2(-0.5 * (double)n);
-    const FwdConst<T>* lc = reinterpret_cast<const FwdConst<T>*>(s.lc);
+    const K* lc = reinterpret_cast<const K*>(s.lc);
     // layer by layer through the windows in the schedule's order; when a layer's last window is the
     // next one's first, both share a sub-pass around the cost phase
     bool opens = !started, first = true;
@@ -180,7 +180,8 @@ __device__ void run_instance(const InstDesc<T>& d, unsigned char* sm, const WinS
     const uint32_t D = 1u << n;
 
     static_assert(sizeof(FwdConst<T>) <= sizeof(LayerConst<T>), "the forward constants share the adjoint's place");
-    set_fwd_consts(reinterpret_cast<FwdConst<T>*>(s.lc), d.gamma, d.beta, p, n);
+    using K = typename FwdFor<T, GRAD>::K;
+    set_fwd_consts(reinterpret_cast<K*>(s.lc), d.gamma, d.beta, p, n);
     bool started = false;
     if (d.Q) {
         for (int i = threadIdx.x; i < n * n; i += blockDim.x) s.Q[i] = d.Q[i];
@@ -190,6 +191,10 @@ __device__ void run_instance(const InstDesc<T>& d, unsigned char* sm, const WinS
             fi.psi = s.psi;
             fi.amp0 = (T)exp2(-0.5 * (double)n);
             fi.gpi0 = d.gamma[0] / T(3.14159265358979323846);
+            if constexpr (GRAD && sizeof(T) == 4) {
+                fi.two = true;
+                make_phase(d.gamma[0], fi.ph);
+            }
         }
         started = build_tile_energy_any<T>(n, n, 0u, s.Q, s.E, s.escr, fi);
     } else {
@@ -204,7 +209,7 @@ __device__ void run_instance(const InstDesc<T>& d, unsigned char* sm, const WinS
     if (d.E_out)
         for (uint32_t z = threadIdx.x; z < D; z += blockDim.x) d.E_out[z] = s.E[swz<T>(z)];
 
-    forward_run<T, R>(d, s, ws, started);
+    forward_run<T, R, K>(d, s, ws, started);
 
     if (d.psi_out) {              // back from the rotated frame: psi = (-i)^{|z|} psi~
         C* pout = reinterpret_cast<C*>(d.psi_out);

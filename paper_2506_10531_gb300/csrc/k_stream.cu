@@ -111,7 +111,7 @@ template <typename T>
 struct StreamSmem {
     typename Num<T>::C* psi;
     T* E;
-    FwdConst<T>* lc;
+    void* lc;        // forward constants: K[64]
     double* red;
     TileTopk tk;
     TopEnt* run;     // running top-k of the state's tiles this block reduced (last pass)
@@ -130,7 +130,7 @@ __device__ __forceinline__ void stream_stage(const StreamPass& P, const StreamIn
 // One staged tile. have_run: this block reduced tile prev_tau of the same state just before (last
 // pass, k >= 1); s.run then holds the top-k of all the state's tiles it reduced so far. TOPK:
 // the instantiation serves passes with a top-k.
-template <typename T, int R, bool TOPK>
+template <typename T, int R, bool TOPK, typename K>
 __device__ void stream_tile(const StreamPass& P, const StreamInst<T>& I, uint64_t tau,
                             const StreamSmem<T>& s, bool have_run, uint64_t prev_tau, const StreamSubs& subs) {
     using C = typename Num<T>::C;
@@ -146,7 +146,7 @@ __device__ void stream_tile(const StreamPass& P, const StreamInst<T>& I, uint64_
         for (int i = 0; i < subs.n; ++i) {
             const StreamSub& b = subs.sub[i];
             SubPass sp{b.a, b.mask, P.la + b.l0, P.la + b.l1, b.phase, P.fin && i == subs.n - 1};
-            subpass_fwd<T, R>(tile, sp, s.lc, P.init && i == 0, amp0, __popcll(tau));
+            subpass_fwd<T, R>(tile, sp, static_cast<const K*>(s.lc), P.init && i == 0, amp0, __popcll(tau));
             __syncthreads();
         }
     } else {
@@ -154,7 +154,7 @@ __device__ void stream_tile(const StreamPass& P, const StreamInst<T>& I, uint64_
         for (;; sn.next()) {
             SubPass sp = sn.get();
             sp.post = P.fin && sn.last();
-            subpass_fwd<T, R>(tile, sp, s.lc, P.init && sn.first(), amp0, __popcll(tau));
+            subpass_fwd<T, R>(tile, sp, static_cast<const K*>(s.lc), P.init && sn.first(), amp0, __popcll(tau));
             __syncthreads();
             if (sn.last()) break;
         }
@@ -223,18 +223,19 @@ __device__ void stream_tile(const StreamPass& P, const StreamInst<T>& I, uint64_
     __syncthreads();
 }
 
-template <typename T, int R, int NTH, bool TOPK>
+template <typename T, int R, int NTH, bool TOPK, bool GRAD>   // GRAD: the forward half of gradients
 __global__ void __launch_bounds__(NTH, 2) k_stream_pass(const StreamPass P,
                                                      const StreamInst<T>* __restrict__ insts,
                                                      int count, const StreamInst<T> one, const StreamSubs subs) {
     extern __shared__ __align__(16) unsigned char sm[];
     using C = typename Num<T>::C;
+    using K = typename FwdFor<T, GRAD>::K;
     const uint32_t TD = 1u << P.tb;
     StreamSmem<T> s;
     size_t o = 0;
     s.psi = reinterpret_cast<C*>(sm + o); o += (size_t)TD * sizeof(C);
     s.E = reinterpret_cast<T*>(sm + o); o += (size_t)TD * sizeof(T);
-    s.lc = reinterpret_cast<FwdConst<T>*>(sm + o); o += 64 * sizeof(LayerConst<T>);
+    s.lc = sm + o; o += 64 * sizeof(LayerConst<T>);
     o = (o + 15) & ~(size_t)15;
     s.red = reinterpret_cast<double*>(sm + o); o += 32 * sizeof(double);
     s.tk.wlists = reinterpret_cast<TopEnt*>(sm + o); o += 8 * 32 * sizeof(TopEnt);
@@ -268,12 +269,12 @@ __global__ void __launch_bounds__(NTH, 2) k_stream_pass(const StreamPass P,
         const StreamInst<T>& I = insts ? insts[ii] : one;
         stream_stage<T>(P, I, tau, s);   // the copies run while the constants are formed
         if (I.gamma != cur_g || I.beta != cur_b || I.p != cur_p) {
-            set_fwd_consts(s.lc, I.gamma, I.beta, I.p, P.n);
+            set_fwd_consts(static_cast<K*>(s.lc), I.gamma, I.beta, I.p, P.n);
             cur_g = I.gamma;
             cur_b = I.beta;
             cur_p = I.p;
         }
-        stream_tile<T, R, TOPK>(P, I, tau, s, run_ii == ii, run_tau, subs);
+        stream_tile<T, R, TOPK, K>(P, I, tau, s, run_ii == ii, run_tau, subs);
         run_ii = ii;
         run_tau = tau;
     }
@@ -886,20 +887,26 @@ static StreamInst<T> one_of(const void* one) {
     return o;
 }
 
-template <typename T, int R, int NTH, bool TOPK>
+template <typename T, int R, int NTH, bool TOPK, bool GRAD = false>
 static cudaError_t pass_t(const StreamPass& P, const void* insts, int count, int grid, int threads, cudaStream_t st,
                           const void* one, const StreamSubs* subs = nullptr) {
     const size_t sm = stream_smem_bytes(sizeof(T) == 8, P.tb);
-    const cudaError_t e = cudaFuncSetAttribute(k_stream_pass<T, R, NTH, TOPK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t e = cudaFuncSetAttribute(k_stream_pass<T, R, NTH, TOPK, GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_stream_pass<T, R, NTH, TOPK><<<grid, threads, sm, st>>>(P, static_cast<const StreamInst<T>*>(insts), count, one_of<T>(one),
+    k_stream_pass<T, R, NTH, TOPK, GRAD><<<grid, threads, sm, st>>>(P, static_cast<const StreamInst<T>*>(insts), count, one_of<T>(one),
                                                             subs ? *subs : StreamSubs{});
     return cudaGetLastError();
 }
 
 cudaError_t launch_stream_pass(bool dbl, const StreamPass& P, const void* insts, int count,
-                               int grid, cudaStream_t st, const void* one, const StreamSubs* subs) {
+                               int grid, cudaStream_t st, bool grad, const void* one, const StreamSubs* subs) {
     if (dbl) return pass_t<double, Num<double>::RB, 256, true>(P, insts, count, grid, 256, st, one);
+    if (grad) {
+        if (P.k > 0) return pass_t<float, Num<float>::RB, 256, true, true>(P, insts, count, grid, 256, st, one);
+        if (small_tiles(dbl, P.n, P.tb))
+            return pass_t<float, SMALL_RA, 256, false, true>(P, insts, count, grid, 1 << (P.tb - SMALL_RA), st, one);
+        return pass_t<float, Num<float>::RB, 256, false, true>(P, insts, count, grid, 256, st, one);
+    }
     if (subs && subs->n > 0)
         return pass_t<float, SMALL_R, 256, false>(P, insts, count, grid, 1 << (P.tb - SMALL_R), st, one, subs);
     if (small_tiles(dbl, P.n, P.tb) && P.k == 0)

@@ -149,7 +149,7 @@ qaoa_status run_stream_one(qaoa_ctx* c, int n, int p, const T* gamma, const T* b
     I.topk_idx = tidx;
     I.topk_prob = tprob;
     for (int s = 0; s < S; ++s)
-        CK(launch_stream_pass(dbl, passes[s], nullptr, 1, one_grid(c, dbl, passes[s]), st, &I, &subs[s]));
+        CK(launch_stream_pass(dbl, passes[s], nullptr, 1, one_grid(c, dbl, passes[s]), st, false, &I, &subs[s]));
     if (expect || (k > 0 && tidx)) CK(launch_stream_finalize(dbl, nullptr, 1, nt, k, st, &I));
     return QAOA_OK;
 }
@@ -193,7 +193,7 @@ qaoa_status grad_stream_one(qaoa_ctx* c, int n, int p, const T* gamma, const T* 
     if (SA < 0) return fail(QAOA_E_INVALID, "no adjoint plan for n=%d p=%d", n, p);
     const uint64_t nta = 1ull << (n - tba);
     const int agrid = (int)std::min<uint64_t>(nta, (uint64_t)c->nsm * (tba < stream_adj_tile_bits(dbl) ? 4 : 2));
-    for (int s = 0; s < S; ++s) CK(launch_stream_pass(dbl, passes[s], nullptr, 1, one_grid(c, dbl, passes[s]), st, &I));
+    for (int s = 0; s < S; ++s) CK(launch_stream_pass(dbl, passes[s], nullptr, 1, one_grid(c, dbl, passes[s]), st, true, &I));
     if (expect) CK(launch_stream_finalize(dbl, nullptr, 1, nt, 0, st, &I));
     for (int s = SA - 1; s >= 0; --s)
         CK(launch_stream_adj_pass(dbl, apasses[s], s, s == SA - 1, s > 0, nullptr, 1, agrid, st, &I));
@@ -1294,7 +1294,7 @@ qaoa_status plan_enqueue(qaoa_plan* P, cudaStream_t st) {
         CK(timed("energy", [&] { return launch_energy_batch(P->dbl, g.n, base + g.inst_off, g.count, st); }));
         for (const StreamPass& pass : g.passes)
             CK(timed("stream_pass", [&] {
-                return launch_stream_pass(P->dbl, pass, base + g.inst_off, g.count, g.grid, st);
+                return launch_stream_pass(P->dbl, pass, base + g.inst_off, g.count, g.grid, st, g.grad);
             }));
         CK(timed("stream_finalize", [&] {
             return launch_stream_finalize(P->dbl, base + g.inst_off, g.count, 1ull << (g.n - tb), g.k, st);

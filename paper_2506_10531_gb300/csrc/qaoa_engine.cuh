@@ -126,7 +126,11 @@ __device__ __forceinline__ void set_layer_consts(LayerConst<T>* lc, const T* gam
 // keep one arithmetic (gamma / pi in one float, shears where |cos| >= |sin| and scaled
 // rotations elsewhere, factors as powers of the rounded cosine) and one order of the qubits in a
 // layer (blocks of `block` qubits ascending in even layers, descending in odd ones, ascending
-// inside a block) whatever windows, tiles or block sizes a launch takes.
+// inside a block) whatever windows, tiles or block sizes a launch takes. The forward half of a
+// gradient takes LayerConst in complex64 too: the powers of a rounded cosine put a norm error of n 2^-25
+// a layer on psi and lam alike, and the adjoint undoes the phases of the two-float gamma (n = 20,
+// p = 4, medians of 24 gradients against 64 bits: dgamma 1.9e-6, dbeta 1.1e-6, <C> 6e-7; with
+// FwdConst32 on both sides 3.0e-6, 2.7e-6, 1.8e-6).
 struct FwdConst32 {
     float gpi;     // gamma_l / pi
     float c, s;    // cos(beta_l), sin(beta_l)
@@ -162,6 +166,12 @@ __device__ __forceinline__ void set_fwd_consts(LayerConst<double>* lc, const dou
                                                int n) {
     set_layer_consts<double>(lc, gamma, beta, p, n, false);
 }
+__device__ __forceinline__ void set_fwd_consts(LayerConst<float>* lc, const float* gamma, const float* beta, int p, int n) {
+    set_layer_consts<float>(lc, gamma, beta, p, n, false);
+}
+// The constants of a forward run, GRAD: that of a gradient.
+template <typename T, bool GRAD> struct FwdFor { using K = FwdConst<T>; };
+template <typename T> struct FwdFor<T, true> { using K = LayerConst<T>; };
 
 // One sub-pass: window start a, butterfly mask over the window bits, layers [la, lb]
 // (lb <= la + 1), whether the cost of layer la opens the sub-pass; post != 0 applies the
@@ -318,18 +328,20 @@ struct FwdPhase32 {
         rot_neg(v, s * pre, c * pre);
     }
 };
-struct FwdPhase64 {
-    PhaseK<double> ph;
-    Pending<double> pre;
-    __device__ __forceinline__ FwdPhase64(const LayerConst<double>& k, int parity) : ph(k.ph), pre(k.pre, k.pcot, parity) {}
-    __device__ __forceinline__ void apply(double2& v, int i, double e) const {
-        double s, c;
+template <typename T>
+struct FwdPhase {
+    PhaseK<T> ph;
+    Pending<T> pre;
+    __device__ __forceinline__ FwdPhase(const LayerConst<T>& k, int parity) : ph(k.ph), pre(k.pre, k.pcot, parity) {}
+    __device__ __forceinline__ void apply(typename Num<T>::C& v, int i, T e) const {
+        T s, c;
         sincos_phase(ph, e, s, c);
         rot_neg(v, s * pre.f[__popc(i) & 1], c * pre.f[__popc(i) & 1]);
     }
 };
 __device__ __forceinline__ FwdPhase32 fwd_phase(const FwdConst32& k, int parity) { return FwdPhase32(k, parity); }
-__device__ __forceinline__ FwdPhase64 fwd_phase(const LayerConst<double>& k, int parity) { return FwdPhase64(k, parity); }
+template <typename T>
+__device__ __forceinline__ FwdPhase<T> fwd_phase(const LayerConst<T>& k, int parity) { return FwdPhase<T>(k, parity); }
 
 // Apply a pending factor to every amplitude of a group.
 template <int R, typename C, typename T>
@@ -351,9 +363,9 @@ __device__ __forceinline__ void finish_group(float2 (&v)[1 << R], const FwdConst
         v[i].y *= k.post;
     }
 }
-template <int R>
-__device__ __forceinline__ void finish_group(double2 (&v)[1 << R], const LayerConst<double>& k, int parity) {
-    scale_group<R>(v, Pending<double>(k.post, k.cot, parity));
+template <int R, typename C, typename T>
+__device__ __forceinline__ void finish_group(C (&v)[1 << R], const LayerConst<T>& k, int parity) {
+    scale_group<R>(v, Pending<T>(k.post, k.cot, parity));
 }
 
 // Mixer inverse on two states with the accumulation of Im <lam| X_q |psi> over the masked
@@ -527,9 +539,9 @@ struct TileRef {
 // Forward sub-pass over all groups of the tile.
 //   init:  amplitudes start as |+> (amp0 i^{|z|} in the rotated frame; pc0 = number of set
 //          global bits that the tile index itself fixes) instead of being read
-template <typename T, int R>
+template <typename T, int R, typename K>
 __device__ __forceinline__ void subpass_fwd(const TileRef<T>& t, const SubPass& sp,
-                                            const FwdConst<T>* lc, bool init, T amp0, int pc0) {
+                                            const K* lc, bool init, T amp0, int pc0) {
     using C = typename Num<T>::C;
     const auto map = [](uint32_t u) { return swz<T>(u); };
     const uint32_t apsi = smem_addr(t.psi), aE = smem_addr(t.E);
@@ -730,14 +742,18 @@ struct FusedInit {
     typename Num<T>::C* psi;   // nullptr: energies only
     T amp0, gpi0;              // 2^{-n/2}, gamma_0 / pi
     int pc0;                   // set bits of zfix
+    bool two = false;          // the phase from the two-float ph instead of gpi0 (gradients, complex64)
+    PhaseK<T> ph{};
 };
 
 template <typename T>
 __device__ __forceinline__ void fused_init_store(const FusedInit<T>& fi, uint32_t u, uint32_t ix, T e) {
     typename Num<T>::C a;
     T s, c;
-    if constexpr (sizeof(T) == 4) sincos_gpi(fi.gpi0, e, s, c);
-    else sincospi(fi.gpi0 * e, &s, &c);
+    if constexpr (sizeof(T) == 4) {
+        if (fi.two) sincos_phase(fi.ph, e, s, c);
+        else sincos_gpi(fi.gpi0, e, s, c);
+    } else sincospi(fi.gpi0 * e, &s, &c);
     a.x = fi.amp0 * c;          // amp0 e^{-i theta}
     a.y = -fi.amp0 * s;
     fi.psi[ix] = times_i_pow(a, fi.pc0 + __popc(u));

@@ -71,8 +71,9 @@ int stream_one_grad_tile_bits(bool dbl, int n, bool adjoint, int* cmin);   // cm
 // tile size); returns the number of passes or -1.
 int stream_plan(bool dbl, int n, int p, int k, StreamPass* out, int max_out, int tb = -1, int cmin = 4);
 // insts: device array of `count` instances, or nullptr to pass the host instance `one` by value.
+// grad: the forward half of a gradient (its constants: FwdConst in qaoa_engine.cuh).
 cudaError_t launch_stream_pass(bool dbl, const StreamPass& P, const void* insts, int count,
-                               int grid, cudaStream_t st, const void* one = nullptr,
+                               int grid, cudaStream_t st, bool grad, const void* one = nullptr,
                                const StreamSubs* subs = nullptr);
 // <C> and top-k of each instance from its tile partials; with many tiles and k > 0 a first
 // merge level runs as its own kernel (stream_finalize_two_level: two launches instead of one).
