@@ -631,11 +631,15 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
     qaoa_plan* P = new qaoa_plan();
     P->ctx = c;
     P->dbl = dbl;
-    // group: resident by (n, grad); streaming by (n, p, k)
+    // group: resident by (n, grad); streaming by (gradient, energies, n, p, k). The energies' class
+    // decides the arithmetic (phases from Q, from an energy vector moved by TMA, or in the cp.async passes), so it
+    // is an instance's own: what a neighbour returns changes nothing for it. Gradient runs always keep
+    // the vector. They come last, so that each kind shares its launches.
+    enum { E_NONE, E_TMA, E_CPASYNC };   // E_CPASYNC: an unaligned vector, complex128, or the tier's variant 2
     std::map<std::pair<int, int>, std::vector<int>> rg;
     std::map<std::pair<int, int>, std::vector<int>> cg;   // cluster groups by (n, local qubits)
     std::map<int, std::vector<int>> csg;                   // cluster-streaming groups by n
-    std::map<std::tuple<int, int, int, int>, std::vector<int>> sg;
+    std::map<std::tuple<int, int, int, int, int>, std::vector<int>> sg;
     const int nres = dbl ? RES_NMAX_D : RES_NMAX_F;
     const int nres_adj = dbl ? RES_NMAX_D_ADJ : RES_NMAX_F_ADJ;
     for (int i = 0; i < count; ++i) {
@@ -649,7 +653,12 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
             csg[d.n].push_back(i);
         else if (!dbl && !grad && d.n >= CL_NMIN && d.n <= CL_NMAX && tier == QAOA_TIER_CLUSTER)
             cg[{d.n, qaoa::eff_cluster_L(c, d.n, d.p)}].push_back(i);
-        else sg[{grad ? 1 : 0, d.n, d.p, d.k}].push_back(i);   // gradient runs last: each kind shares launches
+        else {
+            const bool tma = !dbl && tstream_available() && eff_stream_variant(c, d.n, d.p) != 2 &&
+                             (d.e_off < 0 || (reinterpret_cast<uintptr_t>(epool + d.e_off) & 15u) == 0);
+            const int ecls = !tma ? E_CPASYNC : (grad || d.e_off >= 0) ? E_TMA : E_NONE;
+            sg[{grad ? 1 : 0, ecls, d.n, d.p, d.k}].push_back(i);
+        }
     }
     auto make_desc = [&](int i) {
         const qaoa_inst& d = desc[i];
@@ -753,9 +762,10 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
     for (auto& kv : sg) {
         qaoa_plan::StrGroup g{};
         g.grad = std::get<0>(kv.first) != 0;
-        g.n = std::get<1>(kv.first);
-        g.p = std::get<2>(kv.first);
-        g.k = std::get<3>(kv.first);
+        const int ecls = std::get<1>(kv.first);
+        g.n = std::get<2>(kv.first);
+        g.p = std::get<3>(kv.first);
+        g.k = std::get<4>(kv.first);
         g.count = (int)kv.second.size();
         StreamPass tmp[256];
         const int S = stream_plan(dbl, g.n, g.p, g.k, tmp, 256);
@@ -778,12 +788,7 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
         inst_at += sizeof(StreamInst<T>) * g.count;
         const int variant = dbl ? 2 : eff_stream_variant(c, g.n, g.p);
         g.tgrid = (variant == 1 ? 1 : 2) * c->nsm;
-        // (energies the caller places at addresses TMA cannot take go through the cp.async passes)
-        bool e16 = true, e_out = false;
-        for (int i : kv.second) e_out = e_out || desc[i].e_off >= 0;
-        for (int i : kv.second)
-            e16 = e16 && (desc[i].e_off < 0 || (reinterpret_cast<uintptr_t>(epool + desc[i].e_off) & 15u) == 0);
-        if (!dbl && variant != 2 && tstream_available() && e16) {
+        if (ecls != E_CPASYNC) {
             // map 0: the kind-A passes; map 1 + b: the kind-B passes of chunk b (by start qubit)
             std::vector<int> chunk_s;
             for (auto& ps : g.passes)
@@ -791,7 +796,7 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
                     chunk_s.push_back(ps.s);
             std::sort(chunk_s.begin(), chunk_s.end());
             g.tma = true;
-            g.tab = !g.grad && !e_out;
+            g.tab = ecls == E_NONE;
             const int nshape = 1 + (int)chunk_s.size();   // state maps, then the energy maps
             g.maps_per_inst = 2 * nshape;
             for (auto& ps : g.passes) {
