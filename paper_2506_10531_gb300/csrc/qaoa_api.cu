@@ -602,7 +602,7 @@ struct PlanMem {
 
 template <typename T>
 qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const qaoa_batch_io* io,
-                          const PlanMem* mem, qaoa_plan** out, size_t* need = nullptr) {
+                          const PlanMem* mem, qaoa_plan** out, size_t* need = nullptr, bool allow_tma = true) {
     using C2 = typename qaoa::Num<T>::C;
     const bool dbl = is_dbl<T>();
     const T* qpool = static_cast<const T*>(io->q);
@@ -654,7 +654,7 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
         else if (!dbl && !grad && d.n >= CL_NMIN && d.n <= CL_NMAX && tier == QAOA_TIER_CLUSTER)
             cg[{d.n, qaoa::eff_cluster_L(c, d.n, d.p)}].push_back(i);
         else {
-            const bool tma = !dbl && tstream_available() && eff_stream_variant(c, d.n, d.p) != 2 &&
+            const bool tma = !dbl && allow_tma && tstream_available() && eff_stream_variant(c, d.n, d.p) != 2 &&
                              (d.e_off < 0 || (reinterpret_cast<uintptr_t>(epool + d.e_off) & 15u) == 0);
             const int ecls = !tma ? E_CPASYNC : (grad || d.e_off >= 0) ? E_TMA : E_NONE;
             sg[{grad ? 1 : 0, ecls, d.n, d.p, d.k}].push_back(i);
@@ -910,6 +910,13 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
         if (e != cudaSuccess) { delete P; return fail(QAOA_E_NOMEM, "plan cudaMalloc(%zu): %s", bytes, cudaGetErrorString(e)); }
     }
     P->dev_bytes = bytes;
+    // a tensor map that the driver refuses: the same plan with the streaming tier's cp.async passes
+    // (another layout: their groups keep the energies)
+    const auto cp_async_plan = [&]() -> qaoa_status {
+        if (P->owns) cudaFree(P->dev);
+        delete P;
+        return plan_create_t<T>(c, desc, count, io, mem, out, need, false);
+    };
     char* base = static_cast<char*>(P->dev);
     char* sb = base + sbase;
     // host image of the header: zero counters, then the descriptor arrays
@@ -1002,9 +1009,7 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
                     char* row = img.data() + g.maps_off + TS_MAP_BYTES * (size_t)(j - 1) * g.maps_per_inst;
                     if (!tstream_encode_maps(g.passes[pi], I.psi, const_cast<T*>(I.E), row + TS_MAP_BYTES * mi,
                                              row + TS_MAP_BYTES * ei)) {
-                        if (P->owns) cudaFree(P->dev);
-                        delete P;
-                        return fail(QAOA_E_CUDA, "instance %d: tensor maps of the streaming tier refused", i);
+                        return cp_async_plan();
                     }
                 }
             }
@@ -1017,9 +1022,7 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
                     char* row = img.data() + g.amaps_off + TS_MAP_BYTES * (size_t)(j - 1) * g.amaps_per_inst;
                     if (!tstream_encode_adj_maps(g.apasses[pi], I.psi, I.lam, const_cast<T*>(I.E),
                                                  row + TS_MAP_BYTES * mi)) {
-                        if (P->owns) cudaFree(P->dev);
-                        delete P;
-                        return fail(QAOA_E_CUDA, "instance %d: tensor maps of the adjoint passes refused", i);
+                        return cp_async_plan();
                     }
                 }
             }
@@ -1390,9 +1393,9 @@ static qaoa_status batch_run(qaoa_ctx* c, const qaoa_inst* desc, int count, cons
         const PlanMem inws{c->ws, c->ws_bytes, (cudaStream_t)stream, nullptr, 0};
         s = dbl ? plan_create_t<double>(c, desc, count, io, &inws, &P)
                 : plan_create_t<float>(c, desc, count, io, &inws, &P);
-    } else {
-        s = qaoa_plan_create(c, desc, count, io, dbl, &P);
+        if (s && s != QAOA_E_NOMEM) return s;   // (a plan without the refused tensor maps may need more)
     }
+    if (!P) s = qaoa_plan_create(c, desc, count, io, dbl, &P);
     if (s) return s;
     s = qaoa_plan_launch(P, stream);
     cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
