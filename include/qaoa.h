@@ -393,7 +393,9 @@ qaoa_status dqaoa_session_create(qaoa_ctx* ctx, int N, int m, int k, int p, int 
  * first call needs); x: N host bytes, in/out (the global solution). seed/cycle select the
  * random index sets. energy_out: E(x') (may be NULL); accepted_out: accepted candidates (may
  * be NULL). Steps: index draw (host) -> sub-QUBO build, energies, p layers, <C> and top-K
- * (device, one stream) -> merge (host). Synchronous on `stream`. */
+ * (device, several streams behind `stream`) -> merge (host, chunk by chunk). Synchronous on `stream`.
+ * A cycle that returns an error leaves x as it was and none of its work in flight; the next cycle sends
+ * Q again if this one was to. */
 qaoa_status dqaoa_session_cycle(dqaoa_session* s, const double* Q, int q_changed, uint8_t* x,
                                 uint64_t seed, uint64_t cycle, double* energy_out,
                                 int* accepted_out, qaoa_stream_t stream);

@@ -1554,6 +1554,9 @@ struct dqaoa_session {
     StrongGraph graph;            // BFS / PFS strong-interaction graph of the current Q
     bool graph_valid = false;
     std::vector<uint8_t> x_last;  // the solution the cache belongs to
+    std::vector<uint8_t> x_begin; // the solution the running cycle began with
+    std::vector<double> h_begin;  // and the cache then
+    bool q_stale = false;         // a failed cycle leaves open whether the device holds its Q
     // random index sets of the next cycle, drawn on the host while the device works
     std::vector<int32_t> next_idx;
     bool next_valid = false;
@@ -1760,13 +1763,38 @@ qaoa_status session_decompose(dqaoa_session* s, const double* Q, int q_changed, 
     return QAOA_OK;
 }
 
-}  // namespace
+// Both cycle entry points run through this. A cycle that fails, wherever it does, leaves none of its
+// work in flight, and x and the session as if it had not been called: the chunks before the failure may
+// have been merged into x and h = Qx (their copies cost 9 N bytes a cycle), and the device may
+// hold the new Q or not, so that a retry sends it.
+template <typename Fn>
+qaoa_status session_guard(dqaoa_session* s, int q_changed, uint8_t* x, cudaStream_t st, Fn&& run) {
+    q_changed = q_changed || s->q_stale;
+    const bool keep = s->cache.valid && !q_changed;
+    const double energy = s->cache.energy, tau = s->cache.tau;
+    s->x_begin.assign(x, x + s->N);
+    if (keep) s->h_begin = s->cache.h;
+    const qaoa_status r = run(q_changed != 0);
+    if (r == QAOA_OK) {
+        s->q_stale = false;
+        return r;
+    }
+    cudaStreamSynchronize(st);
+    cudaStreamSynchronize(s->solve2);
+    cudaStreamSynchronize(s->side);
+    std::memcpy(x, s->x_begin.data(), (size_t)s->N);
+    s->cache.valid = keep;
+    if (keep) {
+        s->cache.h = s->h_begin;
+        s->cache.energy = energy;
+        s->cache.tau = tau;
+    }
+    s->q_stale = q_changed != 0;
+    return r;
+}
 
-extern "C" qaoa_status dqaoa_session_cycle(dqaoa_session* s, const double* Q, int q_changed, uint8_t* x,
-                                           uint64_t seed, uint64_t cycle, double* energy_out,
-                                           int* accepted_out, qaoa_stream_t stream) {
-    if (!s || !Q || !x) return fail(QAOA_E_INVALID, "session_cycle: NULL argument");
-    cudaStream_t st = (cudaStream_t)stream;
+qaoa_status session_cycle(dqaoa_session* s, const double* Q, bool q_changed, uint8_t* x, uint64_t seed, uint64_t cycle,
+                          double* energy_out, int* accepted_out, cudaStream_t st) {
     const int N = s->N, m = s->m, k = s->k, K = s->K;
     const double t0 = now_ms();
     // h = Qx from the last merge stays valid while Q is unchanged and x is the solution that
@@ -1840,8 +1868,7 @@ extern "C" qaoa_status dqaoa_session_cycle(dqaoa_session* s, const double* Q, in
         const uint64_t* cand_c = reinterpret_cast<const uint64_t*>(pair_c + (size_t)mcc * K);
         const unsigned status_c = *reinterpret_cast<const unsigned*>(reinterpret_cast<const double*>(cand_c + (size_t)mcc * K) + mcc);
         if (status_c) {
-            // a device-side wait of this chunk ran out: its results are not valid, x is left as is
-            cudaStreamSynchronize(st);
+            // a device-side wait of this chunk ran out: its results are not valid
             return fail(QAOA_E_TIMEOUT, "session_cycle: a device-side wait of chunk %d ran out of time", ch);
         }
         const double tm = now_ms();
@@ -1860,6 +1887,18 @@ extern "C" qaoa_status dqaoa_session_cycle(dqaoa_session* s, const double* Q, in
     s->t_merge = t_merge;
     s->t_cycle = now_ms() - t0;
     return QAOA_OK;
+}
+
+}  // namespace
+
+extern "C" qaoa_status dqaoa_session_cycle(dqaoa_session* s, const double* Q, int q_changed, uint8_t* x,
+                                           uint64_t seed, uint64_t cycle, double* energy_out,
+                                           int* accepted_out, qaoa_stream_t stream) {
+    if (!s || !Q || !x) return fail(QAOA_E_INVALID, "session_cycle: NULL argument");
+    const cudaStream_t st = (cudaStream_t)stream;
+    return session_guard(s, q_changed, x, st, [&](bool qc) {
+        return session_cycle(s, Q, qc, x, seed, cycle, energy_out, accepted_out, st);
+    });
 }
 
 extern "C" qaoa_status dqaoa_session_timing(dqaoa_session* s, double* out) {
@@ -1945,15 +1984,9 @@ qaoa_status session_sampling_setup(dqaoa_session* s, int shots) {
     return QAOA_OK;
 }
 
-}  // namespace
-
-extern "C" qaoa_status dqaoa_session_cycle_sampled(dqaoa_session* s, const double* Q, int q_changed, uint8_t* x,
-                                                   uint64_t seed, uint64_t cycle, int shots, const double* u,
-                                                   double* energy_out, int* accepted_out, qaoa_stream_t stream) {
-    if (!s || !Q || !x || !u || shots < 1 || shots > (1 << 20))
-        return fail(QAOA_E_INVALID, "session_cycle_sampled: bad arguments");
-    if (s->m > 65535) return fail(QAOA_E_INVALID, "session_cycle_sampled: m > 65535");
-    cudaStream_t st = (cudaStream_t)stream;
+qaoa_status session_cycle_sampled(dqaoa_session* s, const double* Q, bool q_changed, uint8_t* x, uint64_t seed,
+                                  uint64_t cycle, int shots, const double* u, double* energy_out, int* accepted_out,
+                                  cudaStream_t st) {
     const int N = s->N, m = s->m, k = s->k;
     CK(cudaSetDevice(s->ctx->device));
     qaoa_status r = session_sampling_setup(s, shots);
@@ -1975,7 +2008,7 @@ extern "C" qaoa_status dqaoa_session_cycle_sampled(dqaoa_session* s, const doubl
     }
     CK(cudaEventRecord(s->setup_done, s->side));
     CK(cudaMemcpyAsync(s->s_u, u, (size_t)m * shots * sizeof(double), cudaMemcpyHostToDevice, st));
-    r = qaoa_plan_launch(s->s_plan, stream);
+    r = qaoa_plan_launch(s->s_plan, (qaoa_stream_t)st);
     if (r) return r;
     CK(launch_sample(k, s->s_psi, m, shots, s->s_u, s->s_z, s->s_scratch, st));
     CK(launch_best_shot(m, k, shots, s->qblk, s->s_qdiag, s->s_z, s->s_best, st));
@@ -2000,6 +2033,20 @@ extern "C" qaoa_status dqaoa_session_cycle_sampled(dqaoa_session* s, const doubl
     s->t_merge = now_ms() - tm;
     s->t_cycle = now_ms() - t0;
     return QAOA_OK;
+}
+
+}  // namespace
+
+extern "C" qaoa_status dqaoa_session_cycle_sampled(dqaoa_session* s, const double* Q, int q_changed, uint8_t* x,
+                                                   uint64_t seed, uint64_t cycle, int shots, const double* u,
+                                                   double* energy_out, int* accepted_out, qaoa_stream_t stream) {
+    if (!s || !Q || !x || !u || shots < 1 || shots > (1 << 20))
+        return fail(QAOA_E_INVALID, "session_cycle_sampled: bad arguments");
+    if (s->m > 65535) return fail(QAOA_E_INVALID, "session_cycle_sampled: m > 65535");
+    const cudaStream_t st = (cudaStream_t)stream;
+    return session_guard(s, q_changed, x, st, [&](bool qc) {
+        return session_cycle_sampled(s, Q, qc, x, seed, cycle, shots, u, energy_out, accepted_out, st);
+    });
 }
 
 extern "C" qaoa_status dqaoa_session_shots(dqaoa_session* s, uint64_t* shots_out, uint64_t* best_out,
