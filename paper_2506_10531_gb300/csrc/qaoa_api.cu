@@ -77,17 +77,26 @@ size_t reduce_scratch_bytes(int n) {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// Workspace of a streaming gradient: psi and lam (2^n complex each), the forward scratch and the
-// per-pass, per-tile gradient partials of the adjoint plan (4 doubles).
-size_t stream_grad_bytes(bool dbl, int n, int p) {
-    if (n <= stream_tile_bits(dbl)) return 0;
+// Workspace of a streaming gradient: psi and lam (2^n complex each), the forward passes' <C> partials (one
+// per tile of their own size) and the per-pass, per-tile gradient partials of the adjoint plan (4
+// doubles). Offsets; bytes = 0: no such run.
+struct GradWs {
+    size_t lam = 0, expect = 0, grad = 0, bytes = 0;
+};
+GradWs stream_grad_ws(bool dbl, int n, int p) {
+    GradWs w;
+    if (n <= stream_tile_bits(dbl)) return w;
     int cmin;
-    const int tba = stream_one_grad_tile_bits(dbl, n, true, &cmin);
+    const int tb = stream_one_grad_tile_bits(dbl, n, false, &cmin), tba = stream_one_grad_tile_bits(dbl, n, true, &cmin);
     StreamPass tmp[256];
     const int S = stream_plan(dbl, n, p, 0, tmp, 256, tba, cmin);
-    if (S < 0) return 0;
-    const size_t D = (size_t)1 << n, nta = (size_t)1 << (n - tba), cs = dbl ? 16 : 8;
-    return 2 * align256(D * cs) + stream_scratch_bytes(dbl, n, 0) + align256((size_t)S * nta * 4 * sizeof(double));
+    if (S < 0) return w;
+    const size_t D = (size_t)1 << n, nt = (size_t)1 << (n - tb), nta = (size_t)1 << (n - tba), cs = dbl ? 16 : 8;
+    w.lam = align256(D * cs);
+    w.expect = 2 * w.lam;
+    w.grad = w.expect + align256(nt * sizeof(double));
+    w.bytes = w.grad + align256((size_t)S * nta * 4 * sizeof(double));
+    return w;
 }
 
 qaoa_status ensure_ws(qaoa_ctx* c, size_t bytes) {
@@ -158,7 +167,8 @@ template <typename T>
 qaoa_status grad_stream_one(qaoa_ctx* c, int n, int p, const T* gamma, const T* beta, const T* E,
                             double* expect, double* dgamma, double* dbeta, cudaStream_t st) {
     const bool dbl = is_dbl<T>();
-    qaoa_status q = ensure_ws(c, stream_grad_bytes(dbl, n, p));
+    const GradWs ws = stream_grad_ws(dbl, n, p);
+    qaoa_status q = ensure_ws(c, ws.bytes);
     if (q) return q;
     StreamPass passes[256];
     int cmin;
@@ -166,8 +176,7 @@ qaoa_status grad_stream_one(qaoa_ctx* c, int n, int p, const T* gamma, const T* 
     const int S = stream_plan(dbl, n, p, 0, passes, 256, tb, cmin);
     if (S < 0) return fail(QAOA_E_INVALID, "no streaming plan for n=%d p=%d", n, p);
     passes[S - 1].keep_frame = 1;
-    const uint64_t nt = 1ull << (n - tb), D = 1ull << n;
-    const size_t cs = sizeof(typename qaoa::Num<T>::C);
+    const uint64_t nt = 1ull << (n - tb);
     char* w = static_cast<char*>(c->ws);
     StreamInst<T> I{};
     I.n = n;
@@ -177,13 +186,10 @@ qaoa_status grad_stream_one(qaoa_ctx* c, int n, int p, const T* gamma, const T* 
     I.gamma = gamma;
     I.beta = beta;
     I.E = E;
-    I.psi = w; w += align256(D * cs);
-    I.lam = w; w += align256(D * cs);
-    I.part_expect = reinterpret_cast<double*>(w);
-    I.part_topp = reinterpret_cast<double*>(w + align256(nt * sizeof(double)));
-    I.part_topz = reinterpret_cast<uint32_t*>(w + align256(nt * sizeof(double)) + align256(nt * sizeof(double)));
-    w += stream_scratch_bytes(dbl, n, 0);
-    I.part_grad = reinterpret_cast<double*>(w);
+    I.psi = w;
+    I.lam = w + ws.lam;
+    I.part_expect = reinterpret_cast<double*>(w + ws.expect);   // (no top-k in a gradient run)
+    I.part_grad = reinterpret_cast<double*>(w + ws.grad);
     I.expect = expect;
     I.dgamma = dgamma;
     I.dbeta = dbeta;
@@ -356,7 +362,7 @@ extern "C" qaoa_status qaoa_set_tier(qaoa_ctx* c, int n, int tier, int param) {
 extern "C" size_t qaoa_workspace_bytes(int n, int dbl) {
     if (n < 1 || n > NMAX) return 0;
     return std::max({stream_scratch_bytes(dbl != 0, n, KMAX), reduce_scratch_bytes(n),
-                     stream_grad_bytes(dbl != 0, n, PMAX)});
+                     stream_grad_ws(dbl != 0, n, PMAX).bytes});
 }
 
 // =============================================================================================
