@@ -646,6 +646,8 @@ struct Acc {
         add(o.s);
         c += o.c;
     }
+    // (the error of a sum that has become infinite is NaN: its value is the sum's)
+    __device__ __forceinline__ T value() const { return c == c ? s + c : s; }
 };
 
 // Runs of instances of equal n in one launch: run i owns blocks [b0[i], b0[i + 1]).
@@ -704,22 +706,24 @@ __global__ void __launch_bounds__(256) k_energy_tile(int n, const T* __restrict_
         if (lane == 0) d[b] = v;
     }
     __syncthreads();
+    // terms of clear bits are masked out, not multiplied by 0: an infinite entry of Q reaches only the
+    // energies that hold its qubits
     const uint32_t t = threadIdx.x;
-    T f[8];
+    uint32_t m[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) f[i] = T((t >> i) & 1u);
+    for (int i = 0; i < 8; ++i) m[i] = 0u - ((t >> i) & 1u);
     Acc<T> base = d[ETB], w8[3];
 #pragma unroll
     for (int b = 0; b < 3; ++b) w8[b] = d[8 + b];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const Acc<T> di = d[i];
-        base.add(f[i] * di.s);
-        base.c = fma(f[i], di.c, base.c);
+        base.add(keep(di.s, m[i]));
+        base.c += keep(di.c, m[i]);
 #pragma unroll
-        for (int k = i + 1; k < 8; ++k) base.add(f[i] * f[k] * W[i * 32 + k]);
+        for (int k = i + 1; k < 8; ++k) base.add(keep(W[i * 32 + k], m[i] & m[k]));
 #pragma unroll
-        for (int b = 0; b < 3; ++b) w8[b].add(f[i] * W[i * 32 + 8 + b]);
+        for (int b = 0; b < 3; ++b) w8[b].add(keep(W[i * 32 + 8 + b], m[i]));
     }
     const T w01 = W[8 * 32 + 9], w02 = W[8 * 32 + 10], w12 = W[9 * 32 + 10];
     Acc<T> x[8];
@@ -737,7 +741,7 @@ __global__ void __launch_bounds__(256) k_energy_tile(int n, const T* __restrict_
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const uint64_t z = z0 + ((uint64_t)j << 8);
-        if (n >= ETB || z < (1ull << n)) E[z] = x[j].s + x[j].c;
+        if (n >= ETB || z < (1ull << n)) E[z] = x[j].value();
     }
 }
 
