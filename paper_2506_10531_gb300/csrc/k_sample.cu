@@ -186,7 +186,8 @@ __global__ void __launch_bounds__(NTS) k_sample_draw(const float2* __restrict__ 
     const int64_t s = HALF ? id >> 4 : id;
     const bool live = s < shots;
     if (!HALF && !live) return;
-    const double t = fmin(u[live ? s : shots - 1] * total, below(total));
+    // (+ 0: a target of -0 is 0, and lies behind leading amplitudes without probability like it)
+    const double t = fmin(__fma_rn(u[live ? s : shots - 1], total, 0.0), below(total));
     const uint32_t c = last_le(off, C, t);
     const double r = fmin(t - off[c], below(coarse[c]));
     const uint32_t f = last_le(pre + ((size_t)c << g.jb), J, r);
