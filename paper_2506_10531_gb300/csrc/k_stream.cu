@@ -564,32 +564,34 @@ __global__ void __launch_bounds__(256) k_energy_rows(int n, int nh, const T* __r
 }
 
 // ---- energy build into HBM, direct form ---------------------------------------------------
-// The row form without a walk (nh = 0: a single instance of up to 20 qubits), the same additions in
-// the same order: E is what qaoa_build_energies has always returned, and what states and shots
-// follow from. Bits 2..9 belong to the thread, the bits above to the block, so the loops over the
+// The row form without a walk (nh = 0: a single complex64 instance of up to 20 qubits), the same
+// additions in the same order: E is what qaoa_build_energies has always returned, and what states and
+// shots follow from. Bits 2..9 belong to the thread, the bits above to the block, so the loops over the
 // block's set bits are uniform and the thread's bits act as masks on unrolled additions, where
-// the row form tests every pair of bits (n = 19: 9.4 -> 6.8 us).
+// the row form tests every pair of bits (n = 19: 9.4 -> 6.8 us). FP64 keeps the row form: its issue
+// rate pays for every masked addition (n = 12: 8.8 us by rows, 10.3 so). Blocks have 256 threads at any n:
+// with 2^(n-2) of them a few threads fill W alone (n = 2: 30 us so, 3.7 now).
 __device__ __forceinline__ float keep(float x, uint32_t m) { return __uint_as_float(__float_as_uint(x) & m); }
 __device__ __forceinline__ double keep(double x, uint32_t m) { return m ? x : 0.0; }
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_energy_direct(int n, const T* __restrict__ Q, T* __restrict__ E) {
-    __shared__ T W[32 * 32];      // zero beyond n
-    for (int x = threadIdx.x; x < 32 * 32; x += blockDim.x) {
+__global__ void __launch_bounds__(256) k_energy_direct(int n, const float* __restrict__ Q, float* __restrict__ E) {
+    __shared__ float W[32 * 32];      // zero beyond n
+    for (int x = threadIdx.x; x < 32 * 32; x += 256) {
         const int i = x >> 5, j = x & 31;
-        T w = T(0);
+        float w = 0.0f;
         if (i < n && j < n) w = (i == j) ? Q[i * n + i] : Q[i * n + j] + Q[j * n + i];
         W[x] = w;
     }
     __syncthreads();
+    if (n < 10 && threadIdx.x >= 1u << (n - 2)) return;
     uint32_t m[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) m[i] = 0u - ((threadIdx.x >> i) & 1u);
-    T eb = T(0), f0 = W[0], f1 = W[33];
+    float eb = 0.0f, f0 = W[0], f1 = W[33];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-        const T* row = W + (2 + i) * 32;
-        T r = row[2 + i];
+        const float* row = W + (2 + i) * 32;
+        float r = row[2 + i];
 #pragma unroll
         for (int j = 0; j < i; ++j) r += keep(row[2 + j], m[j]);
         eb += keep(r, m[i]);
@@ -599,8 +601,8 @@ __global__ void __launch_bounds__(256) k_energy_direct(int n, const T* __restric
     const uint32_t hi = blockIdx.x;
     for (uint32_t b = hi; b; b &= b - 1u) {
         const int i = 10 + __ffs((int)b) - 1;
-        const T* row = W + i * 32;
-        T r = row[i];
+        const float* row = W + i * 32;
+        float r = row[i];
 #pragma unroll
         for (int j = 0; j < 8; ++j) r += keep(row[2 + j], m[j]);
         for (uint32_t d = hi & ((b & (0u - b)) - 1u); d; d &= d - 1u) r += row[10 + __ffs((int)d) - 1];
@@ -608,14 +610,9 @@ __global__ void __launch_bounds__(256) k_energy_direct(int n, const T* __restric
         f0 += row[0];
         f1 += row[1];
     }
-    T* dst = E + (((uint64_t)hi << 10) | ((uint64_t)threadIdx.x << 2));
-    const T e0 = eb, e1 = eb + f0, e2 = eb + f1, e3 = eb + f0 + f1 + W[1];
-    if constexpr (sizeof(T) == 4) {       // E is 8-byte aligned
-        reinterpret_cast<float2*>(dst)[0] = make_float2(e0, e1);
-        reinterpret_cast<float2*>(dst)[1] = make_float2(e2, e3);
-    } else {
-        dst[0] = e0; dst[1] = e1; dst[2] = e2; dst[3] = e3;
-    }
+    float2* dst = reinterpret_cast<float2*>(E + (((uint64_t)hi << 10) | ((uint64_t)threadIdx.x << 2)));   // E is 8-byte aligned
+    dst[0] = make_float2(eb, eb + f0);
+    dst[1] = make_float2(eb + f1, eb + f0 + f1 + W[1]);
 }
 
 // ---- energy build into HBM, tile form ----------------------------------------------------
@@ -1009,9 +1006,8 @@ template <typename T>
 static cudaError_t launch_one(int n, const void* Q, void* E, cudaStream_t st) {
     // one qubit, or an address the wider stores cannot take
     if (n < 2 || (reinterpret_cast<uintptr_t>(E) & 7u) != 0) return launch_tiles<T>(n, 1, Q, E, nullptr, st);
-    if (rows_nh(n, 1) > 0) return launch_rows<T>(n, 1, Q, E, nullptr, st);
-    const unsigned blocks = n > 10 ? 1u << (n - 10) : 1u, threads = n > 10 ? 256u : 1u << (n - 2);
-    k_energy_direct<T><<<blocks, threads, 0, st>>>(n, static_cast<const T*>(Q), static_cast<T*>(E));
+    if (sizeof(T) == 8 || rows_nh(n, 1) > 0) return launch_rows<T>(n, 1, Q, E, nullptr, st);
+    k_energy_direct<<<n > 10 ? 1u << (n - 10) : 1u, 256, 0, st>>>(n, static_cast<const float*>(Q), static_cast<float*>(E));
     return cudaGetLastError();
 }
 
