@@ -6,7 +6,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,first", [(3, 2), (6, 40), (12, 5), (12, 100), (12, 4095), (17, 70001), (21, 1500000), (25, 30000001)])
+@pytest.mark.parametrize("n,first", [(1, 1), (3, 2), (6, 40), (8, 200), (9, 300), (12, 5), (12, 100), (12, 4095), (17, 70001), (21, 1500000), (25, 30000001)])
 def test_zero_uniforms(n, first):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
