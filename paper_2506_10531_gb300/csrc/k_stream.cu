@@ -21,7 +21,7 @@ namespace qaoa {
 namespace {
 
 // Tiles of a single state (see the host side): windows, sizes with tiles of their own, first upper qubit.
-constexpr int SMALL_R = 3, SMALL_NMIN = 15, SMALL_NMAX = 21, SMALL_LOW = 13, SMALL_RA = 4;
+constexpr int SMALL_R = 3, SMALL_NMIN = 15, SMALL_NMAX = 20, SMALL_LOW = 13, SMALL_RA = 4, SMALL_GRAD_NMAX = 21;
 
 // Windows of a layer for tiles of tb bits whose kind-B chunks keep 2^cmin contiguous amplitudes.
 __host__ __device__ inline int stream_windows(int n, int tb, int cmin) {
@@ -748,11 +748,12 @@ __global__ void __launch_bounds__(256) k_energy_tile(int n, const T* __restrict_
 // host side
 // ---------------------------------------------------------------------------------------------
 
-// Passes of a single complex64 state of 15..21 qubits. With the batched tiles (2^13 forward, 2^12
+// Passes of a single complex64 state of up to 20 (forward) or 21 qubits (gradient). With the batched tiles (2^13 forward, 2^12
 // adjoint) such a state is a few dozen tiles, one per CTA and pass, and a pass lasts as long as
 // one tile does on a CTA of 256 threads that runs a thousand unrolled instructions once.
-//   qaoa_run_layers: qubits 0..12 in the batched tiles, qubits 13..n-1 in tiles of 2^10 or 2^11
-//   amplitudes (runs of at least 8), eight amplitudes per thread, the windows of a pass listed on
+//   qaoa_run_layers, n = 15..20: qubits 0..12 in the batched tiles, qubits 13..n-1 in tiles of 2^10
+//   amplitudes (runs of at least 8; at n = 21 such runs leave 2^11 and the pass loses to the batched tiles'
+//   256 blocks: p = 3, 88 us against 72; 2^11 at n = 19, 20 gave nothing), eight amplitudes per thread, the windows of a pass listed on
 //   the host so that the qubit order stays that of 5-qubit windows over 0..12 and 13..n-1 (see
 //   FwdConst: shots are drawn from these states, and that order is why the contiguous tiles
 //   keep 13 qubits; 1024 threads on one of them took as long as 256).
@@ -760,12 +761,12 @@ __global__ void __launch_bounds__(256) k_energy_tile(int n, const T* __restrict_
 //   least 8 amplitudes, 16 amplitudes per thread.
 // GB300: qaoa_run_layers at n = 19, p = 3, passes of 22 to 29 us -> 14 to 18 (qubits 0..12) and 8 to
 // 10 us; qaoa_grad at n = 20, p = 4, forward passes 23 to 32 -> 10 to 15 us.
-static bool small_tiles(bool dbl, int n, int tb) { return !dbl && n >= 14 && n <= SMALL_NMAX && tb == (n + 4) / 2; }
+static bool small_tiles(bool dbl, int n, int tb) { return !dbl && n >= 14 && n <= SMALL_GRAD_NMAX && tb == (n + 4) / 2; }
 
 int stream_tile_bits(bool dbl) { return dbl ? 12 : 13; }
 int stream_adj_tile_bits(bool dbl) { return dbl ? 11 : 12; }
 int stream_one_grad_tile_bits(bool dbl, int n, bool adjoint, int* cmin) {
-    const bool small = !dbl && n >= 14 && n <= SMALL_NMAX;
+    const bool small = !dbl && n >= 14 && n <= SMALL_GRAD_NMAX;
     *cmin = small ? 3 : 4;
     return small ? (n + 4) / 2 : (adjoint ? stream_adj_tile_bits(dbl) : stream_tile_bits(dbl));
 }
@@ -784,7 +785,7 @@ int stream_plan_one(bool dbl, int n, int p, int k, StreamPass* out, StreamSubs* 
     Blk up[2];
     int nu = 0;
     for (int q = SMALL_LOW; q < n; q += 5) up[nu++] = Blk{q, n - q < 5 ? n - q : 5};
-    const int tbA = SMALL_LOW, h = n - SMALL_LOW, tbB = n < 19 ? 10 : 11, c = tbB - h;
+    const int tbA = SMALL_LOW, h = n - SMALL_LOW, tbB = 10, c = tbB - h;
     for (int si = 0; si <= p; ++si) {
         StreamPass P{};
         P.n = n;
