@@ -221,30 +221,38 @@ __device__ void run_instance(const InstDesc<T>& d, unsigned char* sm, const WinS
     }
 }
 
-template <typename T, bool GRAD>
-__device__ void dispatch_instance(const InstDesc<T>& d, unsigned char* sm, int rmax, const WinSched& ws) {
+// WIDE: windows of RB (forward) and RB_ADJ (adjoint) qubits; else narrower ones (rmax, or fewer than RB
+// qubits): the same number for both.
+template <typename T, bool GRAD, bool WIDE>
+__device__ __forceinline__ void dispatch_instance(const InstDesc<T>& d, unsigned char* sm, int rmax, const WinSched& ws) {
     constexpr int RBF = Num<T>::RB, RBA = Num<T>::RB_ADJ;
-    // register windows: RB (forward, or rmax when the launch asks for narrower ones) and RB_ADJ
-    // (adjoint) qubits, fewer when n is smaller
-    const int rf = resident_window(d.n, RBF, rmax), ra = min(d.n, RBA);
-    if (rf == RBF && ra == RBA) run_instance<T, RBF, RBA, GRAD>(d, sm, ws);
-    else if (rf == 4 && ra == 4) run_instance<T, 4, 4, GRAD>(d, sm, ws);
-    else if (rf == 3) run_instance<T, 3, 3, GRAD>(d, sm, ws);
-    else if (rf == 2) run_instance<T, 2, 2, GRAD>(d, sm, ws);
-    else run_instance<T, 1, 1, GRAD>(d, sm, ws);
+    if constexpr (WIDE) {
+        run_instance<T, RBF, RBA, GRAD>(d, sm, ws);
+    } else {
+        const int rf = resident_window(d.n, RBF, rmax);
+        if constexpr (RBA >= 4) {
+            if (rf == 4) return run_instance<T, 4, 4, GRAD>(d, sm, ws);
+        }
+        if (rf == 3) run_instance<T, 3, 3, GRAD>(d, sm, ws);
+        else if (rf == 2) run_instance<T, 2, 2, GRAD>(d, sm, ws);
+        else run_instance<T, 1, 1, GRAD>(d, sm, ws);
+    }
 }
 
 // Persistent walk over `count` descriptors (queue: device counter zeroed before the launch);
 // with desc == nullptr the single instance `one` (passed by value) is run by block 0.
-// GRAD: a kernel of its own with the adjoint sweep, so that forward launches do not carry its
-// registers and code.
-template <typename T, bool GRAD>
+// GRAD: a kernel of its own with the adjoint sweep, and WIDE: one for windows of 5 (complex128: 4) qubits,
+// so that launches do not carry the registers and code of the others: in one kernel with the narrower
+// windows either the wide ones spilled (n = 13, 304 instances, p = 6: 74.3 us; 71.0 before the window starts
+// became run-time values; 68.8 now) or, with the spills mended, the narrow ones slowed down (n = 11, 1000
+// instances: 54.5 -> 56.9 us; 53.0 now). The launch picks by the size all its instances have.
+template <typename T, bool GRAD, bool WIDE>
 __global__ void __launch_bounds__(512) k_resident(const InstDesc<T>* __restrict__ desc, int count,
                                                   int* queue, const InstDesc<T> one, int rmax, const WinSched ws) {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ int s_next;
     if (desc == nullptr) {
-        if (blockIdx.x == 0) dispatch_instance<T, GRAD>(one, sm, rmax, ws);
+        if (blockIdx.x == 0) dispatch_instance<T, GRAD, WIDE>(one, sm, rmax, ws);
         return;
     }
     for (;;) {
@@ -254,15 +262,29 @@ __global__ void __launch_bounds__(512) k_resident(const InstDesc<T>* __restrict_
         __syncthreads();
         if (ii >= count) break;
         const InstDesc<T> d = desc[ii];
-        dispatch_instance<T, GRAD>(d, sm, rmax, ws);
+        dispatch_instance<T, GRAD, WIDE>(d, sm, rmax, ws);
         __syncthreads();
     }
+}
+
+int resident_r(bool dbl, int n, int rmax) { return resident_window(n, dbl ? Num<double>::RB : Num<float>::RB, rmax); }
+
+// fn(kernel, descriptor of its type) for the kernel that serves n-qubit instances
+template <typename T, typename Fn>
+auto with_kernel(bool grad, bool wide, Fn&& fn) {
+    if (grad) return wide ? fn(k_resident<T, true, true>, InstDesc<T>{}) : fn(k_resident<T, true, false>, InstDesc<T>{});
+    return wide ? fn(k_resident<T, false, true>, InstDesc<T>{}) : fn(k_resident<T, false, false>, InstDesc<T>{});
+}
+template <typename Fn>
+auto with_kernel(bool dbl, int n, bool grad, int rmax, Fn&& fn) {
+    const int R = resident_r(dbl, n, rmax);
+    return dbl ? with_kernel<double>(grad, R == Num<double>::RB, fn) : with_kernel<float>(grad, R == Num<float>::RB, fn);
 }
 
 }  // namespace
 
 int resident_threads(bool dbl, int n, int rmax) {
-    const int R = resident_window(n, dbl ? Num<double>::RB : Num<float>::RB, rmax);
+    const int R = resident_r(dbl, n, rmax);
     const int g = (n > R) ? (1 << (n - R)) : 1;
     return g < 32 ? 32 : (g > 512 ? 512 : g);
 }
@@ -279,13 +301,12 @@ int resident_max_blocks_per_sm(bool dbl, int n, int pmax, bool grad, int rmax) {
     const size_t sm = resident_smem_bytes(dbl, n, pmax, grad, rmax);
     // the occupancy query counts a block that needs more than 48 KB of dynamic shared memory only
     // once the kernel may use that much, so the limit is raised first (the launch sets it again)
-    const auto query = [&](auto kern) {
+    with_kernel(dbl, n, grad, rmax, [&](auto kern, auto) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, th, sm) != cudaSuccess)
             nb = 0;
-    };
-    if (dbl) { if (grad) query(k_resident<double, true>); else query(k_resident<double, false>); }
-    else { if (grad) query(k_resident<float, true>); else query(k_resident<float, false>); }
+        return nb;
+    });
     return nb;
 }
 
@@ -293,20 +314,18 @@ cudaError_t launch_resident(bool dbl, const void* desc, int count, int n, int pm
                             int* queue, int grid, cudaStream_t st, const void* one, int rmax, bool block5) {
     const int th = resident_threads(dbl, n, rmax);
     const size_t sm = resident_smem_bytes(dbl, n, pmax, grad, rmax);
-    const int R = resident_window(n, dbl ? Num<double>::RB : Num<float>::RB, rmax);
+    const int R = resident_r(dbl, n, rmax);
     // the qubit order of blocks of the window itself, or of 5 qubits for narrower windows of a
     // single complex64 instance
     const WinSched ws = win_sched(n, block5 ? Num<float>::RB : R, R);
-    const auto go = [&](auto kern, auto inst) -> cudaError_t {
+    return with_kernel(dbl, n, grad, rmax, [&](auto kern, auto inst) -> cudaError_t {
         using D = decltype(inst);
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
         if (one) inst = *static_cast<const D*>(one);
         kern<<<grid, th, sm, st>>>(static_cast<const D*>(desc), count, queue, inst, rmax, ws);
         return cudaGetLastError();
-    };
-    if (dbl) return grad ? go(k_resident<double, true>, InstDesc<double>{}) : go(k_resident<double, false>, InstDesc<double>{});
-    return grad ? go(k_resident<float, true>, InstDesc<float>{}) : go(k_resident<float, false>, InstDesc<float>{});
+    });
 }
 
 }  // namespace qaoa

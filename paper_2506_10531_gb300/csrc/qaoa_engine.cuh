@@ -561,7 +561,16 @@ struct TileRef {
     int tb;                    // tile bits
 };
 
-// Forward sub-pass over all groups of the tile.
+// A copy of x that the compiler cannot trace to it: what is formed from it is formed there.
+__device__ __forceinline__ int opaque(int x) {
+    asm volatile("" : "+r"(x));
+    return x;
+}
+
+// Forward sub-pass over all groups of the tile. Groups of 64 registers (5 complex64 qubits, 4 complex128)
+// form the steps of the energies' walk anew at each cost phase: held across the mixers they cost 112 bytes
+// of spills in the resident kernel (304 instances of n = 13, p = 6: 74.3 us so, 68.8 now; qaoa_run_layers at
+// n = 22, p = 5: 210 us, 187 now). Smaller groups have the registers (n = 11, 1000 instances: 54.7 us, 56.7 anew).
 //   init:  amplitudes start as |+> (amp0 i^{|z|} in the rotated frame; pc0 = number of set
 //          global bits that the tile index itself fixes) instead of being read
 template <typename T, int R, typename K>
@@ -570,7 +579,8 @@ __device__ __forceinline__ void subpass_fwd(const TileRef<T>& t, const SubPass& 
     using C = typename Num<T>::C;
     const auto map = [](uint32_t u) { return swz<T>(u); };
     const uint32_t apsi = smem_addr(t.psi), aE = smem_addr(t.E);
-    const WinSteps<R> ws = win_steps<R>(sp.a, sizeof(C), map), we = win_steps<R>(sp.a, sizeof(T), map);
+    constexpr bool tight = (sizeof(C) << R) >= 256;
+    const WinSteps<R> ws = win_steps<R>(sp.a, sizeof(C), map), we0 = win_steps<R>(sp.a, sizeof(T), map);
     const uint32_t ngroups = 1u << (t.tb - R);
     for (uint32_t g = threadIdx.x; g < ngroups; g += blockDim.x) {
         const uint32_t base = group_base<R>(g, sp.a);
@@ -596,6 +606,7 @@ __device__ __forceinline__ void subpass_fwd(const TileRef<T>& t, const SubPass& 
 #pragma unroll 1
         for (int l = sp.la; l <= sp.lb; ++l) {
             if (l > sp.la || sp.ph_first) {
+                const WinSteps<R> we = tight ? win_steps<R>(opaque(sp.a), sizeof(T), map) : we0;
                 const auto ph = fwd_phase(lc[l], pc0 + __popc(base));
                 for_energies<R, T>(aE, sb * (uint32_t)sizeof(T), we, [&](int i, T e) { ph.apply(v[i], i, e); });
             }
