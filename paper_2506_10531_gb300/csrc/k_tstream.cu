@@ -392,7 +392,12 @@ __device__ __forceinline__ void advance_segment(const TsGroup* groups, const TsS
 
 // TAB: phases and energies come from Q (qaoa_phase.cuh), no energy vector exists; else from the energies
 // in HBM (gradient runs, whose adjoint reads them, and instances that return them).
-template <bool TAB>
+// RUNS: a CTA takes its share of the tiles in a row instead of every gridDim.x-th, so that it meets few
+// instances: a table is an instance's, and rebuilding it for every tile took back what the tables give
+// (64 instances of n = 20, p = 3: 1218 us with energies, 1371 with a table per tile, 1067 in rows; 16 of n = 22:
+// 1295, 1313, 1072). Large instances stay with the stride, whose CTAs read neighbouring tiles at a time
+// (n = 30: 1% faster).
+template <bool TAB, bool RUNS>
 __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const TsGroup* __restrict__ groups,
                                                        const TsSeg* __restrict__ segs, int nseg, uint32_t total,
                                                        unsigned* status) {
@@ -422,7 +427,11 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const TsGroup* __restric
     bool ok = true;
     int sg = -1;
     uint32_t send = 0;        // first tile past the segment
-    if (blockIdx.x < total) advance_segment(groups, segs, nseg, total, blockIdx.x, sg, send, &cur);
+    const uint32_t per = total / gridDim.x, rem = total % gridDim.x;
+    const uint32_t q0 = RUNS ? blockIdx.x * per + min(blockIdx.x, rem) : blockIdx.x;
+    const uint32_t qend = RUNS ? q0 + per + (blockIdx.x < rem ? 1u : 0u) : total;
+    const uint32_t qstep = RUNS ? 1u : gridDim.x;
+    if (q0 < qend) advance_segment(groups, segs, nseg, total, q0, sg, send, &cur);
     // Thread 0: the loads of tile q (segment S). The energies first (their buffer is never stored
     // from), then, once the last tile's store has read the state buffer (wait_store), the state.
     auto issue = [&](uint32_t q, bool wait_store) {
@@ -448,15 +457,15 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const TsGroup* __restric
         }
         // the tile after it towards L2, a tile's compute ahead of its own load (in the passes
         // that store no state: with the state stores in flight it slowed the others down)
-        const uint32_t q1 = ql + gridDim.x;
-        const uint32_t end = S == &cur ? send - S->tile0 : 0u;
+        const uint32_t q1 = ql + qstep;
+        const uint32_t end = S == &cur ? (RUNS ? min(send, qend) : send) - S->tile0 : 0u;
         if ((p.init || (p.fin && p.no_store)) && q1 < end) {
             const CUtensorMap* m1 = S->maps + (size_t)(q1 >> tbits) * t.maps_per_inst;
             if (need_e) tile_prefetch(t, m1 + t.emap, q1 & tmask);
             if (!p.init) tile_prefetch(t, m1 + t.map, q1 & tmask);
         }
     };
-    if (blockIdx.x < total && threadIdx.x == 0) issue(blockIdx.x, false);
+    if (q0 < qend && threadIdx.x == 0) issue(q0, false);
     // what the constants and the table belong to, in shared memory: the sub-passes need the registers
     __shared__ const float *cur_g, *cur_b, *cur_q;
     __shared__ int cur_p, cur_n, cur_l;
@@ -464,7 +473,7 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const TsGroup* __restric
     __syncthreads();
     TopEnt* run = reinterpret_cast<TopEnt*>(sm + o.run);
     bool run_valid = false;   // the run list holds this CTA's best k of the current instance so far
-    for (uint32_t q = blockIdx.x; q < total; q += gridDim.x) {
+    for (uint32_t q = q0; q < qend; q += qstep) {
         if (q >= send) {
             __syncthreads();
             advance_segment(groups, segs, nseg, total, q, sg, send, &cur);
@@ -604,8 +613,8 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const TsGroup* __restric
                     }
                 }
                 // this tile's slot: the list when it is the CTA's last tile of the instance
-                const uint32_t qn = q + gridDim.x;
-                const bool last_of_inst = qn >= send || (int)((qn - cur.tile0) >> tbits) != ii;
+                const uint32_t qn = q + qstep;
+                const bool last_of_inst = (RUNS && qn >= qend) || qn >= send || (int)((qn - cur.tile0) >> tbits) != ii;
                 if (threadIdx.x < (unsigned)kk) {
                     const TopEnt e = last_of_inst ? run[threadIdx.x] : TopEnt{-1.0, 0xffffffffu};
                     I.part_topp[tau * kk + threadIdx.x] = e.p;
@@ -633,7 +642,7 @@ __global__ void __launch_bounds__(NT, 2) k_tstream_pass(const TsGroup* __restric
         }
         // the next tile's loads: the energies at once, the state once this tile's store has read
         // the buffer (the init pass loads only the energies)
-        if (q + gridDim.x < total && threadIdx.x == 0 && ok) issue(q + gridDim.x, true);
+        if (q + qstep < qend && threadIdx.x == 0 && ok) issue(q + qstep, true);
     }
     if (threadIdx.x == 0) {
         bulk_wait_all();
@@ -888,7 +897,7 @@ void tstream_group_windows(const StreamPass* passes, int S, TsGroup* g) {
 }
 
 cudaError_t launch_tstream_pass(bool tab, const TsGroup* groups, const TsSeg* segs, int nseg, uint32_t total, int grid,
-                                unsigned* status, cudaStream_t st) {
+                                bool runs, unsigned* status, cudaStream_t st) {
     const size_t sm = tstream_smem_bytes(tab);
     const auto go = [&](auto kern) -> cudaError_t {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -896,7 +905,8 @@ cudaError_t launch_tstream_pass(bool tab, const TsGroup* groups, const TsSeg* se
         kern<<<grid, NT, sm, st>>>(groups, segs, nseg, total, status);
         return cudaGetLastError();
     };
-    return tab ? go(k_tstream_pass<true>) : go(k_tstream_pass<false>);
+    if (!tab) return go(k_tstream_pass<false, false>);
+    return runs ? go(k_tstream_pass<true, true>) : go(k_tstream_pass<true, false>);
 }
 
 size_t tstream_adj_smem_bytes() { return ta_offsets().total; }

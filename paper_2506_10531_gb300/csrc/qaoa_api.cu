@@ -468,7 +468,7 @@ struct qaoa_plan {
                  bool tab = false;
                  size_t inst_off = 0;
                  size_t fgrp_off = 0, agrp_off = 0;   // TsGroup arrays, forward and adjoint
-                 struct Launch { size_t seg_off; int nseg; uint32_t total; };
+                 struct Launch { size_t seg_off; int nseg; uint32_t total; bool runs; };
                  std::vector<Launch> fwd, adj; };
     std::vector<ResGroup> res;
     std::vector<CluGroup> clu;
@@ -591,6 +591,16 @@ void plan_mixes(qaoa_plan* P, char* img, char* base) {
             }
             L.nseg = k;
             L.total = at;
+            // Tiles in a row (k_tstream_pass) where a launch of several instances has one that gives a CTA
+            // fewer than eight tiles by the stride: n <= 24 with two CTAs per SM (4 instances of n = 24: 1621 us
+            // by the stride, 1545 in rows; single ones of n = 25..30 lose 1% in rows).
+            int insts = 0, nmin = 99;
+            for (int j = m.g0; fwd && j < m.g1; ++j)
+                if (s < P->str[j].passes.size()) {
+                    insts += P->str[j].count;
+                    nmin = std::min(nmin, P->str[j].n);
+                }
+            L.runs = m.tab && insts > 1 && (1ull << (nmin - tb)) < 8ull * m.tgrid;
         }
     }
 }
@@ -890,7 +900,7 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
         for (size_t s = 0; s < smax + amax; ++s) {
             int nseg = 0;
             for (int j = m.g0; j < m.g1; ++j) nseg += (s < smax ? s < P->str[j].passes.size() : s - smax < P->str[j].apasses.size());
-            (s < smax ? m.fwd : m.adj).push_back(qaoa_plan::Mix::Launch{hdr, nseg, 0});
+            (s < smax ? m.fwd : m.adj).push_back(qaoa_plan::Mix::Launch{hdr, nseg, 0, false});
             hdr += sizeof(TsSeg) * nseg;
         }
         hdr = align256(hdr);
@@ -1283,7 +1293,7 @@ qaoa_status plan_enqueue(qaoa_plan* P, cudaStream_t st) {
                 CK(timed("tstream_pass", [&] {
                     return launch_tstream_pass(m.tab, reinterpret_cast<const TsGroup*>(base + m.fgrp_off),
                                                reinterpret_cast<const TsSeg*>(base + L.seg_off), L.nseg, L.total,
-                                               (int)std::min<uint32_t>(L.total, (uint32_t)m.tgrid), status, st);
+                                               (int)std::min<uint32_t>(L.total, (uint32_t)m.tgrid), L.runs, status, st);
                 }));
             CK(timed("stream_finalize", [&]() -> cudaError_t {
                 for (int j = m.g0; j < m.g1; ++j) {

@@ -52,10 +52,10 @@ constexpr int TS_MAX_GROUPS = 65535;
 // Fill the windows of g (n, tb set) from its pass list.
 void tstream_group_windows(const StreamPass* passes, int S, TsGroup* g);
 // A launch over `nseg` segments (device array, `total` tiles in all) of the groups at `groups`, whose
-// phases come from Q (tab) or from the energies in HBM; a bounded wait that ran out sets bit 0 of
-// *status.
+// phases come from Q (tab) or from the energies in HBM; runs (with tab): each CTA takes tiles in a row
+// instead of every grid-th; a bounded wait that ran out sets bit 0 of *status.
 cudaError_t launch_tstream_pass(bool tab, const TsGroup* groups, const TsSeg* segs, int nseg, uint32_t total, int grid,
-                                unsigned* status, cudaStream_t st);
+                                bool runs, unsigned* status, cudaStream_t st);
 
 // Adjoint passes (tiles of TSA_TB bits, kind-B chunks of h <= 8 high qubits): per pass shape
 // three maps (state psi, adjoint state lam, energies) at indices T.map, T.map + 1, T.map + 2.
