@@ -41,7 +41,7 @@ template <bool F>
 __device__ __forceinline__ uint32_t tab_term(float a, float b, double g, bool& bad) {
     if (F) return __float_as_uint(__fadd_rn(a, b));
     double x = g * ((double)a + (double)b);
-    if (((uint32_t)__double2hiint(x) & 0x7fffffffu) >= 0x411e8480u) {   // |x| >= 500000, or not a number
+    if (!(fabs(x) < 500000.0)) {
         bad = bad || !(fabs(x) <= 1.0e300);
         x -= rint(x);
     }
