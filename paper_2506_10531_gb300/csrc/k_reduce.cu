@@ -18,12 +18,51 @@ namespace {
 constexpr int RPT = 8;                     // amplitudes per thread and round
 constexpr uint64_t RCH = TK_NT * RPT;      // amplitudes per block and round
 
+// The round below after its collection overflowed (thousands of amplitudes tie with the bound): collections
+// above better bounds, then sorted insertion. A function of its own that reads the amplitudes again, so
+// that the round does not hold them for it (inlined, top-8 of a complex128 state of n = 26 took 422 us, 314 so).
+template <typename C>
+__device__ __noinline__ void topk_round_over(const C* __restrict__ psi, uint64_t z0, uint64_t D, int k, bool have_run,
+                                             float lo, TopScratch& s) {
+#pragma unroll 1
+    for (int t = 0; s.over && t < TK_RETRY; ++t) {
+        const TopEnt b = kth_collected(k, s);
+#pragma unroll 1
+        for (int i = 0; i < RPT; ++i) {
+            const uint64_t z = z0 + (uint64_t)i * TK_NT + threadIdx.x;
+            if (z >= D) break;
+            const C x = psi[z];
+            const float pf = (float)x.x * (float)x.x + (float)x.y * (float)x.y;
+            if (!(pf * 1.00000095367431640625f >= lo)) continue;
+            const double p = exact_prob(x);
+            if (!better(b.p, b.z, p, (uint32_t)z) && (!have_run || better(p, (uint32_t)z, s.run[k - 1].p, s.run[k - 1].z)))
+                collect_entry(p, (uint32_t)z, s);
+        }
+        __syncthreads();
+    }
+    if (!s.over) {
+        rank_collected(k, have_run, s);
+        return;
+    }
+    WarpTopK top;
+    top.init(k);
+#pragma unroll 1
+    for (int i = 0; i < RPT; ++i) {
+        const uint64_t z = z0 + (uint64_t)i * TK_NT + threadIdx.x;
+        C x;
+        x.x = x.y = 0;
+        if (z < D) x = psi[z];
+        top.offer(x, (uint32_t)z, z < D);
+    }
+    merge_warp_lists(top, k, have_run, s);
+}
+
 // One round of the selection over the block's RCH amplitudes: s.run (valid with have_run) becomes
 // the k best of itself and the amplitudes v[i] at z0 + i * TK_NT + tid (those < D). An FP32
 // test with the margins of WarpTopK::offer comes first; FP64 runs for the few that pass.
 template <typename C>
-__device__ __forceinline__ void topk_round(const C (&v)[RPT], uint64_t z0, uint64_t D, int k, bool have_run,
-                                           TopScratch& s) {
+__device__ __forceinline__ void topk_round(const C (&v)[RPT], const C* __restrict__ psi, uint64_t z0, uint64_t D, int k,
+                                           bool have_run, TopScratch& s) {
     float pf[RPT], pmax = -1.0f;
 #pragma unroll
     for (int i = 0; i < RPT; ++i) {
@@ -50,22 +89,8 @@ __device__ __forceinline__ void topk_round(const C (&v)[RPT], uint64_t z0, uint6
         }
     }
     __syncthreads();
-    if (!s.over) {
-        rank_collected(k, have_run, s);
-        return;
-    }
-    WarpTopK top;
-    top.init(k);
-#pragma unroll 1
-    for (int i = 0; i < RPT; ++i) {
-        C x = v[0];
-#pragma unroll
-        for (int j = 1; j < RPT; ++j)
-            if (j == i) x = v[j];
-        const uint64_t z = z0 + (uint64_t)i * TK_NT + threadIdx.x;
-        top.offer(x, (uint32_t)z, z < D);
-    }
-    merge_warp_lists(top, k, have_run, s);
+    if (s.over) topk_round_over(psi, z0, D, k, have_run, lo, s);
+    else rank_collected(k, have_run, s);
 }
 
 // expect / topk: what is wanted. One block (gridDim.x == 1) writes expect_out, idx_out, prob_out;
@@ -101,7 +126,7 @@ __global__ void __launch_bounds__(TK_NT) k_reduce_state(int n, const typename Nu
             ex += (double)acc;
         }
         if (TOPK) {
-            topk_round(v, z0, D, k, have_run, ts);
+            topk_round(v, psi, z0, D, k, have_run, ts);
             have_run = true;
         }
     }

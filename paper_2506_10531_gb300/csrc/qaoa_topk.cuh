@@ -9,16 +9,18 @@
 namespace qaoa {
 
 constexpr int TK_NT = 256;
-constexpr int TK_CAP = 256;   // collected entries; more (massive ties) take the sorted-insertion path
+constexpr int TK_CAP = 256;   // collected entries; more (massive ties): kth_collected
 
 struct __align__(16) TopScratch {
     float wb[16 * (TK_NT / 32)];
     TopEnt cand[TK_CAP];
     TopEnt wl[(TK_NT / 32) * 32];
     TopEnt run[16];             // the result: k entries, empty ones hold probability -1
+    TopEnt kth;
     float bound;
     int cnt, over;
 };
+constexpr int TK_RETRY = 4;   // collections after an overflow, each above a better bound, before sorted insertion
 
 // The k-th largest (1 <= k <= 16) of one value per thread of the block: every warp offers its k
 // largest and the k-th largest of those is found by rank. Also clears the collection counters.
@@ -53,6 +55,24 @@ __device__ __forceinline__ void collect_entry(double p, uint32_t z, TopScratch& 
     const int pos = atomicAdd(&s.cnt, 1);
     if (pos < TK_CAP) s.cand[pos] = TopEnt{p, z};
     else s.over = 1;
+}
+
+// After an overflow (s.over, behind a barrier): the k-th best of the TK_CAP entries that were kept, which
+// at least k of all entries are or beat, for another collection; clears the counters. Ties of one
+// probability are told apart by their index here, where the FP32 bound cannot, and a warp's sorted insertion
+// takes about 1 us per 32 of them (a flat state of n = 21, top-8: 260 us by insertion, 77 so). Called by
+// all threads; ends with a barrier.
+__device__ __forceinline__ TopEnt kth_collected(int k, TopScratch& s) {
+    static_assert(TK_CAP == TK_NT, "an entry per thread");
+    const TopEnt me = s.cand[threadIdx.x];
+    int rank = 0;
+    for (int j = 0; j < TK_CAP; ++j) rank += better(s.cand[j].p, s.cand[j].z, me.p, me.z) ? 1 : 0;
+    if (rank == k - 1) s.kth = me;
+    __syncthreads();
+    if (threadIdx.x == 0) { s.cnt = 0; s.over = 0; }
+    const TopEnt t = s.kth;
+    __syncthreads();
+    return t;
 }
 
 // s.run = the k best of the collected entries and, with have_run, the entries of s.run. Called by
@@ -118,6 +138,15 @@ __device__ __forceinline__ void merge_entries(uint64_t nent, int k, TopScratch& 
         }
     }
     __syncthreads();
+#pragma unroll 1
+    for (int t = 0; s.over && t < TK_RETRY; ++t) {
+        const TopEnt b2 = kth_collected(k, s);
+        for (uint64_t e = threadIdx.x; e < nent; e += TK_NT) {
+            const TopEnt x = at(e);
+            if (is_entry(x.p) && !better(b2.p, b2.z, x.p, x.z)) collect_entry(x.p, x.z, s);
+        }
+        __syncthreads();
+    }
     if (!s.over) {
         rank_collected(k, false, s);
         return;
