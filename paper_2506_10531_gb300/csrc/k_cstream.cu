@@ -581,8 +581,8 @@ __global__ void __launch_bounds__(NT, 2) k_cstream(const CsInstDev* __restrict__
         // a group per stored tile, so step j - 1's are older; else all) before the CTA arrives at
         // the cluster phase of step j - 1. While that phase completes (wait: every CTA's step
         // j - 1 data is complete), every store finishes reading the buffers, which the next
-        // step's prefetch of its first tile (the slot step j - 1 advanced), the pass-0 threads
-        // or rank 0's merge in the energy tile reuse once the barrier after the wait is passed.
+        // step's prefetch of its first tile (the slot step j - 1 advanced) or the pass-0 threads
+        // reuse once the barrier after the wait is passed.
         __syncthreads();
         if (threadIdx.x == 0 && j > 0) {
             if (stored) bulk_wait_all_but_one();

@@ -623,8 +623,8 @@ __global__ void __launch_bounds__(256) k_energy_direct(int n, const float* __res
 // of its low eight bits once and forms its eight energies by subset doubling over bits 8..10,
 // against a sum over all bit pairs per energy quadruple in the row form, whose walk over hi is
 // too short to pay for its start below about 2^23 energies (n = 20 on GB300: 14.6 us in the row form, 8.4 us
-// here). The energies of
-// batched instances; single instances keep the row form's sums (k_energy_direct). Sums are
+// here). The energies of batched instances; single instances keep the row form's sums (k_energy_direct).
+// Sums are
 // compensated (Acc: TwoSum, the rounding errors added separately), so that an energy is off by
 // little more than its own last rounding (relative 2-norm at n = 19: 9e-8 in the row form,
 // 2.5e-8 here): phases gamma E inherit that error. Stores are 4 (8) bytes per lane, coalesced: any
@@ -911,8 +911,6 @@ cudaError_t launch_stream_pass(bool dbl, const StreamPass& P, const void* insts,
     }
     if (subs && subs->n > 0)
         return pass_t<float, SMALL_R, 256, false>(P, insts, count, grid, 1 << (P.tb - SMALL_R), st, one, subs);
-    if (small_tiles(dbl, P.n, P.tb) && P.k == 0)
-        return pass_t<float, SMALL_RA, 256, false>(P, insts, count, grid, 1 << (P.tb - SMALL_RA), st, one);
     if (P.k == 0) return pass_t<float, Num<float>::RB, 256, false>(P, insts, count, grid, 256, st, one);
     return pass_t<float, Num<float>::RB, 256, true>(P, insts, count, grid, 256, st, one);
 }

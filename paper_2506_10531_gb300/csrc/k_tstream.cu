@@ -288,8 +288,19 @@ __device__ __forceinline__ void last_elem(const Geo& geo, const StreamPass& P, i
     }
 }
 
-// TMA coordinates of tile tau (TsPass::bmode, see qaoa_tstream.h); the energy maps have the same
-// coordinates as the state maps.
+// Shape of the tensor map of a pass (TMA coordinates of a tile): kind A; kind B with h <= 8 and
+// qubits above the chunk (5-D) or without (4-D); kind B with h = 9, whose 512 high values are
+// split over two box dimensions (at most 256 each), 5-D or 4-D; kind A of the adjoint's 12-bit tiles (3-D).
+enum : int { TS_A, TS_B5, TS_B4, TS_B9_5, TS_B9_4, TS_A3 };
+struct TsPass {
+    int bmode;          // TS_*
+    int midbits;        // kind B: tile-index bits below the chunk (s - c)
+    int map;            // index of this pass's state map among an instance's maps
+    int emap;           // index of its energy map
+    int maps_per_inst;  // maps per instance in the plan's map array
+};
+
+// TMA coordinates of tile tau; the energy maps have the same coordinates as the state maps.
 __device__ __forceinline__ void tile_load(const TsPass& T, const CUtensorMap* map, void* dst, uint64_t tau,
                                           uint64_t* bar) {
     const int mid = (int)(tau & ((1ull << T.midbits) - 1ull)), top = (int)(tau >> T.midbits);
@@ -860,23 +871,6 @@ bool tstream_available() { return encode_fn() != nullptr; }
 
 size_t tstream_smem_bytes(bool tab) { return ts_offsets(tab).total; }
 
-TsPass tstream_pass_geometry(const StreamPass& P, int map, int emap, int maps_per_inst) {
-    TsPass T{};
-    T.map = map;
-    T.emap = emap;
-    T.maps_per_inst = maps_per_inst;
-    if (P.kind == 0) {
-        T.bmode = TS_A;
-        T.midbits = 0;
-        return T;
-    }
-    T.midbits = P.s - P.c;
-    const bool top = P.s + P.h < P.n;
-    if (P.h <= 8) T.bmode = top ? TS_B5 : TS_B4;
-    else T.bmode = top ? TS_B9_5 : TS_B9_4;
-    return T;
-}
-
 bool tstream_encode_maps(const StreamPass& P, void* psi, void* E, void* psi_map, void* e_map) {
     if (!encode_fn() || P.tb != TB || P.n <= TB || P.n > 34) return false;
     return encode_shape(P, psi, 2, static_cast<CUtensorMap*>(psi_map)) &&
@@ -910,21 +904,6 @@ cudaError_t launch_tstream_pass(bool tab, const TsGroup* groups, const TsSeg* se
 }
 
 size_t tstream_adj_smem_bytes() { return ta_offsets().total; }
-
-TsPass tstream_adj_geometry(const StreamPass& P, int map, int maps_per_inst) {
-    TsPass T{};
-    T.map = map;
-    T.emap = map + 2;
-    T.maps_per_inst = maps_per_inst;
-    if (P.kind == 0) {
-        T.bmode = TS_A3;
-        T.midbits = 0;
-        return T;
-    }
-    T.midbits = P.s - P.c;
-    T.bmode = (P.s + P.h < P.n) ? TS_B5 : TS_B4;
-    return T;
-}
 
 bool tstream_encode_adj_maps(const StreamPass& P, void* psi, void* lam, void* E, void* maps3) {
     if (!encode_fn() || P.tb != TSA_TB || P.n <= TSA_TB || P.n > 34 || (P.kind == 1 && (P.h > 8 || P.c < 4)))

@@ -435,7 +435,7 @@ struct StrStep {
     int kernels = 0;
 };
 
-// Runs of equal n among the groups [g0, g1) for the energy launches: tile-form runs first.
+// A run of instances of equal n among a mix's groups, for the energy launches.
 struct EnergyRun {
     int n, first, count;
 };
@@ -453,13 +453,13 @@ struct qaoa_plan {
                       std::vector<StreamPass> apasses;   // adjoint plan (adjoint tile bits)
                       int grid, agrid; std::vector<const void*> q; std::vector<void*> e;
                       // TMA streaming passes (complex64): per instance one state tensor map per
-                      // pass shape, at maps_off in the header; tsp[i] is pass i's geometry
+                      // pass shape, then the energy maps, at maps_off in the header; map[i]: pass i's shape
                       bool tma = false, tab = false;   // tab: phases from Q, no energies
-                      size_t maps_off = 0; int maps_per_inst = 0; std::vector<TsPass> tsp;
+                      size_t maps_off = 0; int maps_per_inst = 0; std::vector<int> map;
                       int tgrid = 0;   // TMA passes' persistent grid
                       // TMA adjoint passes: per instance three maps (psi, lam, E) per adjoint pass
-                      // shape at amaps_off; atsp[i] is adjoint pass i's geometry
-                      size_t amaps_off = 0; int amaps_per_inst = 0; std::vector<TsPass> atsp; };
+                      // shape at amaps_off; amap[i]: adjoint pass i's shape
+                      size_t amaps_off = 0; int amaps_per_inst = 0; std::vector<int> amap; };
     // Consecutive TMA groups that share their launches: pass s of every group that has one in one
     // launch, likewise the adjoint passes (from each group's last), energies, finalize and gradient
     // sums. Their instances follow one another at inst_off.
@@ -662,10 +662,8 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
         const qaoa_inst& d = desc[i];
         const bool grad = (d.flags & QAOA_INST_GRAD) != 0;
         const int tier = (!dbl && !grad) ? qaoa::eff_tier(c, d.n, d.p) : QAOA_TIER_STREAM;
-        // the cluster-streaming tier moves the energies by TMA: an energy output must be 16-byte aligned
-        const bool e_ok = d.e_off < 0 || (reinterpret_cast<uintptr_t>(epool + d.e_off) & 15u) == 0;
         if (d.n <= nres && (!grad || d.n <= nres_adj)) rg[{d.n, grad ? 1 : 0}].push_back(i);
-        else if (tier == QAOA_TIER_CSTREAM && d.n >= CS_NMIN && d.n <= CS_NMAX && e_ok && cstream_usable(c, d.n))
+        else if (tier == QAOA_TIER_CSTREAM && d.n >= CS_NMIN && d.n <= CS_NMAX && cstream_usable(c, d.n))
             csg[d.n].push_back(i);
         else if (!dbl && !grad && d.n >= CL_NMIN && d.n <= CL_NMAX && tier == QAOA_TIER_CLUSTER)
             cg[{d.n, qaoa::eff_cluster_L(c, d.n, d.p)}].push_back(i);
@@ -815,11 +813,8 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
             g.tab = ecls == E_NONE;
             const int nshape = 1 + (int)chunk_s.size();   // state maps, then the energy maps
             g.maps_per_inst = 2 * nshape;
-            for (auto& ps : g.passes) {
-                const int mi = ps.kind == 0 ? 0
-                                            : 1 + (int)(std::find(chunk_s.begin(), chunk_s.end(), ps.s) - chunk_s.begin());
-                g.tsp.push_back(tstream_pass_geometry(ps, mi, nshape + mi, g.maps_per_inst));
-            }
+            for (auto& ps : g.passes)
+                g.map.push_back(ps.kind == 0 ? 0 : 1 + (int)(std::find(chunk_s.begin(), chunk_s.end(), ps.s) - chunk_s.begin()));
             g.maps_off = hdr;
             hdr = align256(hdr + TS_MAP_BYTES * (size_t)g.maps_per_inst * g.count);
             static_assert(TSA_TB == 12, "the adjoint's tile bits (stream_adj_tile_bits)");
@@ -831,11 +826,8 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
                         achunk.push_back(ps.s);
                 std::sort(achunk.begin(), achunk.end());
                 g.amaps_per_inst = 3 * (1 + (int)achunk.size());
-                for (auto& ps : g.apasses) {
-                    const int ai = ps.kind == 0 ? 0
-                                                : 1 + (int)(std::find(achunk.begin(), achunk.end(), ps.s) - achunk.begin());
-                    g.atsp.push_back(tstream_adj_geometry(ps, 3 * ai, g.amaps_per_inst));
-                }
+                for (auto& ps : g.apasses)
+                    g.amap.push_back(ps.kind == 0 ? 0 : 1 + (int)(std::find(achunk.begin(), achunk.end(), ps.s) - achunk.begin()));
                 g.amaps_off = hdr;
                 hdr = align256(hdr + TS_MAP_BYTES * (size_t)g.amaps_per_inst * g.count);
             }
@@ -1019,27 +1011,25 @@ qaoa_status plan_create_t(qaoa_ctx* c, const qaoa_inst* desc, int count, const q
                 // one map per pass shape, for this instance's state
                 std::vector<char> done(g.maps_per_inst, 0);
                 for (size_t pi = 0; pi < g.passes.size(); ++pi) {
-                    const int mi = g.tsp[pi].map, ei = g.tsp[pi].emap;
+                    const int mi = g.map[pi], ei = g.maps_per_inst / 2 + mi;
                     if (done[mi]) continue;
                     done[mi] = 1;
                     char* row = img.data() + g.maps_off + TS_MAP_BYTES * (size_t)(j - 1) * g.maps_per_inst;
                     if (!tstream_encode_maps(g.passes[pi], I.psi, const_cast<T*>(I.E), row + TS_MAP_BYTES * mi,
-                                             row + TS_MAP_BYTES * ei)) {
+                                             row + TS_MAP_BYTES * ei))
                         return cp_async_plan();
-                    }
                 }
             }
             if (g.tma && g.grad) {
                 std::vector<char> done(g.amaps_per_inst, 0);
                 for (size_t pi = 0; pi < g.apasses.size(); ++pi) {
-                    const int mi = g.atsp[pi].map;
+                    const int mi = 3 * g.amap[pi];
                     if (done[mi]) continue;
                     done[mi] = 1;
                     char* row = img.data() + g.amaps_off + TS_MAP_BYTES * (size_t)(j - 1) * g.amaps_per_inst;
                     if (!tstream_encode_adj_maps(g.apasses[pi], I.psi, I.lam, const_cast<T*>(I.E),
-                                                 row + TS_MAP_BYTES * mi)) {
+                                                 row + TS_MAP_BYTES * mi))
                         return cp_async_plan();
-                    }
                 }
             }
             si.push_back(I);

@@ -145,9 +145,10 @@ __device__ __forceinline__ void set_layer_consts(LayerConst<T>* lc, const T* gam
     __syncthreads();
 }
 
-// Constants of the engine's forward runs. complex128 uses LayerConst. complex64 states of the
-// resident tier and of the single-instance calls are what measured shots are drawn from, and
-// a shot is a whole number that moves when a probability moves by one rounding: these runs
+// Constants of the engine's forward runs. complex128 uses LayerConst. Measured shots are drawn from
+// complex64 states of the resident tier and of the single-instance calls (and, in sampled sessions of 15 and
+// more variables, from batched plans of the TMA tiers, which take LayerConst and phases from Q), and
+// a shot is a whole number that moves when a probability moves by one rounding: the engine's runs
 // keep one arithmetic (gamma / pi in one float, shears where |cos| >= |sin| and scaled
 // rotations elsewhere, factors as powers of the rounded cosine) and one order of the qubits in a
 // layer (blocks of `block` qubits ascending in even layers, descending in odd ones, ascending

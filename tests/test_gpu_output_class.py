@@ -44,3 +44,16 @@ def test_a_neighbours_energies_change_nothing(n, p, k, grad, e_off):
         assert none[1] == pair[1]
     finally:
         q.qaoa_destroy(ctx)
+
+
+@pytest.mark.parametrize("n", [15, 16, 17])
+def test_cluster_streaming_energies_at_any_address(n):
+    """15..17 qubits: the address energies are returned to decides nothing (they leave by 4-byte stores)."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2506_10531_gb300 as q
+    ctx = q.qaoa_create(0)
+    try:
+        assert launch(q, ctx, n, 2, 4, False, 2, [0]) == launch(q, ctx, n, 2, 4, False, 0, [0]) == launch(q, ctx, n, 2, 4, False, None, [0])
+    finally:
+        q.qaoa_destroy(ctx)
