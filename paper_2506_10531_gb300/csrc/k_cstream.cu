@@ -13,7 +13,7 @@
 // passes read and write L2, not HBM, and the whole batch is one launch. Phases and energies come from
 // Q in shared memory (qaoa_phase.cuh), a table per pass built while its first tile is on its way: with
 // energies built in pass 0 and moved with every tile, 101 instances of n = 17, p = 5 took 337 us,
-// without 325. What bounds the passes: the copies between L2 and shared memory and, with one instance
+// without 318. What bounds the passes: the copies between L2 and shared memory and, with one instance
 // per cluster, the latency from pass to pass (63 us for one of n = 16, p = 3; 80 us for 74 at once).
 //
 // Passes (2^H tiles each, H = n - 13; CTA rank r takes tiles r, r + C, ...):
@@ -72,7 +72,7 @@ __host__ __device__ inline CsOff cs_offsets(int tpc) {
     o.psi = x; x += (size_t)TD * 8;                        // 64 KiB, 1024-byte aligned at run time
     o.tab = x; x = cs_al(x + sizeof(PhaseTab));
     o.red = x; x = cs_al(x + 2 * (NT / 32) * sizeof(float));
-    o.escr = x; x = cs_al(x + 256 * sizeof(float));       // staged parameters; energy tables of pass 0
+    o.escr = x; x = cs_al(x + 256 * sizeof(float));       // staged parameters; tables of returned energies
     o.wbound = x; x = cs_al(x + (NT / 32) * sizeof(float));
     for (int s = 0; s < 2; ++s) {
         o.Q[s] = x; x = cs_al(x + (size_t)CS_NMAX * CS_NMAX * 4);

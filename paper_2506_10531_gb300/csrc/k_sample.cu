@@ -16,6 +16,7 @@
 // doubles as integers; a shot's walk is one thread over its 16 amplitudes (1.5 FP64 warp
 // instructions per shot; a warp per shot with shuffle scans needs 8 per 32 amplitudes walked).
 // Only for fb >= 7 half a warp walks a part together.
+// Up to 8 qubits the draw forms the sums itself (small_sums) and k_sample_sums does not run.
 // Every loop is bounded by the part length; nothing waits on another block. A batch of states of
 // equal n (a DQAOA cycle's sub-QUBO states, 2^n amplitudes apart) runs as one launch of each
 // kernel, the state index in blockIdx.y; each state has its own scratch (F + C doubles),

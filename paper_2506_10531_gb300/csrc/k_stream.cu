@@ -748,15 +748,15 @@ __global__ void __launch_bounds__(256) k_energy_tile(int n, const T* __restrict_
 // host side
 // ---------------------------------------------------------------------------------------------
 
-// Passes of a single complex64 state of up to 20 (forward) or 21 qubits (gradient). With the batched tiles (2^13 forward, 2^12
-// adjoint) such a state is a few dozen tiles, one per CTA and pass, and a pass lasts as long as
-// one tile does on a CTA of 256 threads that runs a thousand unrolled instructions once.
+// Passes of a single complex64 state of up to 20 (forward) or 21 qubits (gradient). With the batched
+// tiles (2^13 forward, 2^12 adjoint) such a state is a few dozen tiles, one per CTA and pass, and a pass
+// lasts as long as one tile does on a CTA of 256 threads that runs a thousand unrolled instructions once.
 //   qaoa_run_layers, n = 15..20: qubits 0..12 in the batched tiles, qubits 13..n-1 in tiles of 2^10
-//   amplitudes (runs of at least 8; at n = 21 such runs leave 2^11 and the pass loses to the batched tiles'
-//   256 blocks: p = 3, 88 us against 72; 2^11 at n = 19, 20 gave nothing), eight amplitudes per thread, the windows of a pass listed on
-//   the host so that the qubit order stays that of 5-qubit windows over 0..12 and 13..n-1 (see
-//   FwdConst: shots are drawn from these states, and that order is why the contiguous tiles
-//   keep 13 qubits; 1024 threads on one of them took as long as 256).
+//   amplitudes (runs of at least 8; at n = 21 such runs leave 2^11 and the pass loses to the batched
+//   tiles' 256 blocks: p = 3, 88 us against 72; 2^11 at n = 19, 20 gave nothing), eight amplitudes per
+//   thread, the windows of a pass listed on the host so that the qubit order stays that of 5-qubit
+//   windows over 0..12 and 13..n-1 (see FwdConst: shots are drawn from these states, and that order is
+//   why the contiguous tiles keep 13 qubits; 1024 threads on one of them took as long as 256).
 //   qaoa_grad (whose states stay inside): tb = (n + 4) / 2 bits forward and adjoint, runs of at
 //   least 8 amplitudes, 16 amplitudes per thread.
 // GB300: qaoa_run_layers at n = 19, p = 3, passes of 22 to 29 us -> 14 to 18 (qubits 0..12) and 8 to
